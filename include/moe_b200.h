@@ -120,8 +120,11 @@ int moe_permute(const void* x_bf16, const int32_t* topk_ids, const int32_t* expe
  * for batches that fill the chip (T*k >= 1024, at least 4 rows per expert on average, at least 128 (pass of tokens, tile
  * of weight rows) items; H and I multiples of 256, w13 and w2 32-byte aligned) the packed weights feed the block-scaled
  * 8-bit tensor-core instruction and each bf16 activation is two E4M3 terms with scales per 32 elements (exact for elements
- * within 2^-14 of their block's largest magnitude, off by at most 2^-22 of it otherwise; a token with a non-finite value
- * gives non-finite outputs);
+ * within 2^-14 of their block's largest magnitude, off by at most 2^-22 of it otherwise).  Where the shape would otherwise go
+ * to one of the last two, which take every bf16 value as it is, experts are done again by that one (same name reported) if they
+ * have a block that the terms hold too little of: a token block with 6 or more inexact elements of 32, a block of the
+ * intermediate with 8 or more of which at most 3 others reach 2^-10 of the largest, or one with a non-finite value.
+ * Elsewhere a token with a non-finite value gives non-finite outputs;
  * for other decode-sized batches (T*k <= 32*E and <= 6144; H and I multiples of 256 up to 4096 - so also the I = 256 shard of
  * the paper's TP8 layout; E up to about 400 at H = 4096, where shared memory runs out) the packed weights feed the block-scaled FP4
  * tensor-core instruction directly and each bf16 activation row is written as a sum of eight E2M1 rows with their

@@ -158,14 +158,17 @@ int expert_ffn_impl(const void* x_perm_bf16, const int32_t* expert_offsets, cons
   if (!twoterm && native_shape_ok(*choice, w.w13, w.w2))
     return launch_expert_ffn_native(xp, expert_offsets, w, *shape, act, y_perm, status, st, row_dst);
   if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
-  if (twoterm) return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr}, expert_offsets, w, *shape, *choice, act, y_perm, status.word, st, row_dst);
+  if (twoterm)
+    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr}, expert_offsets, w, *shape, *choice, twoterm_guarded(*choice, w),
+                                     act, y_perm, status.word, st, row_dst);
   if (umma_shape_ok(*choice) || w.blocked)
     return launch_expert_ffn_umma(xp, expert_offsets, w, *shape, act, y_perm, status.word, st, row_dst);
   return launch_expert_ffn_stream(xp, expert_offsets, w.w13, w.s13, w.w2, w.s2, *shape, act, y_perm, status.word, st, row_dst);
 }
 
 // Sort and expert FFN of a call that holds the tokens and their routing: moe_permute and moe_expert_ffn, or, where the
-// two-term kernel runs, the sort alone and that kernel fed from the unsorted rows (same bits; x_perm is then not written)
+// two-term kernel runs, the sort alone and that kernel fed from the unsorted rows (same bits; x_perm then only takes the rows of
+// experts that are done again)
 int permute_and_ffn(const void* x, const int32_t* ids, const int32_t* offsets, const ExpertWeights& w, const moe_shape_t* shape,
                     void* x_perm, int32_t* perm, int32_t* inv_perm, float* y_perm, int32_t* status_word, void* ws, size_t ws_bytes,
                     void* cuda_stream) {
@@ -187,7 +190,8 @@ int permute_and_ffn(const void* x, const int32_t* ids, const int32_t* offsets, c
   char* base = static_cast<char*>(ws);
   if ((rc = launch_permute(xb, ids, offsets, *shape, nullptr, perm, inv_perm, reinterpret_cast<int*>(base + L.permute_off), st)) != MOE_OK)
     return rc;
-  return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm}, offsets, w, *shape, *shape, base + L.act_off, y_perm, status.word, st);
+  return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, static_cast<__nv_bfloat16*>(x_perm)}, offsets, w, *shape, *shape,
+                                   twoterm_guarded(*shape, w), base + L.act_off, y_perm, status.word, st);
 }
 
 // the four tensors inside a buffer written by moe_prepack
@@ -620,7 +624,7 @@ int moe_debug_expert_ffn_variant(const void* x_perm_bf16, const int32_t* expert_
     if (!twoterm_shape_ok(*shape) || !twoterm_weights_ok(w13, w2)) return MOE_ERR_UNSUPPORTED_SHAPE;
     if (check_ws(ws, ws_bytes, L.act_off + twoterm_scratch(*shape).total) != MOE_OK) return MOE_ERR_WORKSPACE;
     if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
-    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr}, expert_offsets, w, *shape, *shape, act, y_perm, status.word, st);
+    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr}, expert_offsets, w, *shape, *shape, false, act, y_perm, status.word, st);
   }
   if (variant == 2) {
     if (!native_shape_ok(*shape, w13, w2)) return MOE_ERR_UNSUPPORTED_SHAPE;

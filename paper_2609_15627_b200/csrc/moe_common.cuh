@@ -66,7 +66,9 @@ inline TwoTermGeometry twoterm_geometry(const moe_shape_t& s) {
   return TwoTermGeometry{224, 2048};
 }
 struct TwoTermScratch {
-  size_t xq, aq, sfx, sfa, total;  // E4M3 pair rows of the tokens [2S, H] and of the intermediate [2S, I], scale factors
+  size_t xq, aq, sfx, sfa;  // E4M3 pair rows of the tokens [2S, H] and of the intermediate [2S, I], scale factors
+  size_t marks, flags;      // what the terms do not hold: a byte per token row and piece of it, an int per expert and one for any
+  size_t total;
 };
 inline TwoTermScratch twoterm_scratch(const moe_shape_t& s) {
   TwoTermScratch L;
@@ -83,6 +85,8 @@ inline TwoTermScratch twoterm_scratch(const moe_shape_t& s) {
   L.aq = take(2 * S * s.I);
   L.sfx = take(passes * (s.H / 128) * g.sf_step);
   L.sfa = take(passes * (s.I / 128) * g.sf_step);
+  L.marks = take(S * (s.H / 256));
+  L.flags = take((static_cast<size_t>(s.E) + 1) * 4);
   L.total = off;
   return L;
 }
@@ -215,22 +219,30 @@ int launch_permute(const __nv_bfloat16* x, const int* ids, const int* offsets, c
 // weight-streaming variant (any shape; the one for decode-sized batches)
 int launch_expert_ffn_stream(const __nv_bfloat16* x_perm, const int* offsets, const uint8_t* w13, const uint8_t* s13,
                              const uint8_t* w2, const uint8_t* s2, const moe_shape_t& s, __nv_bfloat16* act, float* y_perm,
-                             int* status_word, cudaStream_t st, float* const* row_dst = nullptr);
+                             int* status_word, cudaStream_t st, float* const* row_dst = nullptr, const int* only = nullptr);
+bool stream_shape_ok(const moe_shape_t& s);
+// (`only`, in this one and the next: null, or device flags [E + 1] of an earlier kernel - experts whose flag is zero are left
+// alone, and nothing is done where flag E is zero)
 // tcgen05 grouped-GEMM variant (prefill-sized batches); umma_shape_ok says whether it applies
 bool umma_shape_ok(const moe_shape_t& s);
 int launch_expert_ffn_umma(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
-                           __nv_bfloat16* act, float* y_perm, int* status_word, cudaStream_t st, float* const* row_dst = nullptr);
+                           __nv_bfloat16* act, float* y_perm, int* status_word, cudaStream_t st, float* const* row_dst = nullptr,
+                           const int* only = nullptr);
 // two-term E4M3 variant: packed codes and bf16 rows as two 8-bit terms on the block-scaled tensor-core path.  `choice` is the
-// shape that fixes the pass geometry and the scratch layout (`s`, or the unsharded shape of an expert-parallel rank)
+// shape that fixes the pass geometry and the scratch layout (`s`, or the unsharded shape of an expert-parallel rank).
+// `guard`: experts with blocks that two terms hold too little of are done again by a kernel that holds every bf16 value (see
+// kTtLossyTokens); set where such a kernel would take the shape without this one.
 bool twoterm_weights_ok(const void* w13, const void* w2);
 struct TwoTermInput {
   const __nv_bfloat16* x;  // rows in sorted order; or, with the two tables of the routing, the tokens' rows
   const int* ids;          // [T, k] expert of every slot
   const int* inv_perm;     // [T, k] sorted row of every slot
+  __nv_bfloat16* x_sorted; // with the tables: room for the rows in sorted order, of the experts that `guard` does again
 };
 int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
-                           const moe_shape_t& choice, void* scratch, float* y_perm, int* status_word, cudaStream_t st,
+                           const moe_shape_t& choice, bool guard, void* scratch, float* y_perm, int* status_word, cudaStream_t st,
                            float* const* row_dst = nullptr);
+bool twoterm_guarded(const moe_shape_t& choice, const ExpertWeights& w);
 // quantised activations, batches that fill the chip; scratch of q_pair_scratch
 int launch_expert_ffn_q_pair(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
                              void* scratch, float* y_perm, int* status_word, cudaStream_t st);

@@ -33,6 +33,7 @@ struct FfnArgs {
   float* y;                   // stage 2 output [S, Hout]
   float* const* row_dst;      // or null; else output row p goes to row_dst[p] (see y_row)
   int* status;
+  const int* only;            // or null; else [E + 1]: experts whose word is zero are skipped, all of them where word E is
   uint32_t k1, k2;         // 0x1040, 0x0104: multipliers of the E2M1 expansion, kept opaque to the compiler
   int E, K, R, I;             // R rows per expert (2I for stage 1, H for stage 2); I used by stage 1 only
   int n_stages;
@@ -53,6 +54,10 @@ MOE_DEVINL void mma_bf16_16x8x16(float (&c)[4], uint32_t a0, uint32_t a1, uint32
 template <bool STAGE1>
 __global__ void __launch_bounds__(kThreads, 1) ffn_stream_kernel(const FfnArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  if (a.only != nullptr) {  // (launched beside the kernel before it in this case)
+    pdl_wait();
+    if (__ldcg(a.only + a.E) == 0) return;
+  }
   const int K = a.K;
   const int code_half = 8 * (K / 2);   // bytes of 8 rows of codes
   const int scale_half = 8 * (K / 32); // bytes of 8 rows of scale bytes
@@ -73,11 +78,12 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_stream_kernel(const FfnArgs a
   {
     const int per = (a.E + kThreads - 1) / kThreads;
     const int base = tid * per;
+    auto has_work = [&](int e) {
+      return e < a.E && a.offsets[e + 1] > a.offsets[e] && (a.only == nullptr || __ldcg(a.only + e) != 0);
+    };
     int cnt = 0;
-    for (int i = 0; i < per; ++i) {
-      const int e = base + i;
-      if (e < a.E && a.offsets[e + 1] > a.offsets[e]) ++cnt;
-    }
+    for (int i = 0; i < per; ++i)
+      if (has_work(base + i)) ++cnt;
     int wtot;
     const int ex = warp_excl_scan(cnt, lane, &wtot);
     if (lane == 0) s_misc[wid] = wtot;
@@ -92,10 +98,8 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_stream_kernel(const FfnArgs a
     }
     __syncthreads();
     int pos = s_misc[wid] + ex;
-    for (int i = 0; i < per; ++i) {
-      const int e = base + i;
-      if (e < a.E && a.offsets[e + 1] > a.offsets[e]) touched[pos++] = e;
-    }
+    for (int i = 0; i < per; ++i)
+      if (has_work(base + i)) touched[pos++] = base + i;
     if (tid == 0) {
       for (int s = 0; s < n_stages; ++s) {
         mbar_init(&full_bar[s], 1);
@@ -272,10 +276,16 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_stream_kernel(const FfnArgs a
   }
 }
 
+namespace {
+constexpr int kSmemBudget = 200 * 1024;
+constexpr int stream_stage_bytes(int K) { return 16 * (K / 2 + K / 32); }
+}  // namespace
+// (the ring holds whole rows: at least two stages of 16)
+bool stream_shape_ok(const moe_shape_t& sh) { return kSmemBudget / stream_stage_bytes(sh.H > sh.I ? sh.H : sh.I) >= 2; }
+
 int launch_expert_ffn_stream(const __nv_bfloat16* x_perm, const int* offsets, const uint8_t* w13, const uint8_t* s13,
                       const uint8_t* w2, const uint8_t* s2, const moe_shape_t& sh, __nv_bfloat16* act, float* y_perm,
-                      int* status_word, cudaStream_t st, float* const* row_dst) {
-  constexpr int kSmemBudget = 200 * 1024;
+                      int* status_word, cudaStream_t st, float* const* row_dst, const int* only) {
   static PerDeviceFlag flag;
   if (!once_per_device(flag, [] {
         return cudaFuncSetAttribute(ffn_stream_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 24 * 1024) ==
@@ -292,8 +302,7 @@ int launch_expert_ffn_stream(const __nv_bfloat16* x_perm, const int* offsets, co
     a.y = y_perm;
     a.row_dst = row_dst;
     a.status = status_word;
-  a.k1 = 0x1040u;
-  a.k2 = 0x0104u;
+    a.only = only;
     a.k1 = 0x1040u;
     a.k2 = 0x0104u;
     a.E = sh.E;
@@ -311,13 +320,15 @@ int launch_expert_ffn_stream(const __nv_bfloat16* x_perm, const int* offsets, co
       a.K = sh.I;
       a.R = sh.H;
     }
-    const int stage_bytes = 16 * (a.K / 2 + a.K / 32);
+    const int stage_bytes = stream_stage_bytes(a.K);
     int n_stages = kSmemBudget / stage_bytes;
     if (n_stages > 12) n_stages = 12;
     if (n_stages < 2) return false;
     a.n_stages = n_stages;
     const size_t smem = static_cast<size_t>(n_stages) * stage_bytes + 2 * n_stages * 8 +
                         2 * kConsumerWarps * 128 * 4 + (static_cast<size_t>(sh.E) + 40) * 4;
+    if (only != nullptr)
+      return launch_pdl(stage1 ? ffn_stream_kernel<true> : ffn_stream_kernel<false>, dim3(grid), dim3(kThreads), smem, st, a) == cudaSuccess;
     if (stage1)
       ffn_stream_kernel<true><<<grid, kThreads, smem, st>>>(a);
     else

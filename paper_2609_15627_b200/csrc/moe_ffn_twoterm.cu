@@ -4,7 +4,11 @@
 // A bf16 value has 8 significant bits, an E4M3 value 4, so with one scale 2^s per 32 consecutive elements
 //   x = 2^s * hi + 2^(s-5) * lo,   hi = e4m3(x / 2^s),   lo = e4m3((x / 2^s - hi) * 32),   block maximum in [2^7, 2^8) * 2^s
 // is exact for every element within 2^14 of its block's maximum and off by at most 2^-22 of that maximum otherwise -
-// below what one fp32 addition of a 4096-long sum rounds away.  E2M1 x E4M3 products are exact and accumulate in fp32 in
+// below what one fp32 addition of a 4096-long sum rounds away, as long as that maximum is in the sum.  It need not be: its
+// weight may be zero, and where one element of a block is 2^12 (2^14, 2^18) times the others they then carry a relative error
+// of 3e-4 (7e-3, 0.5).  So where a kernel that holds every value would take the shape (twoterm_guarded), such blocks are
+// found where they are split, and their experts are done again by that kernel, in launches that end at once when there are none
+// (kTtLossyTokens, launch_again).  E2M1 x E4M3 products are exact and accumulate in fp32 in
 // tensor memory, so the result is that of the bf16 x expanded-weight product up to summation order, at the same
 // tensor-core time (two 8-bit MMAs of K = 32 take what two bf16 MMAs of K = 16 take) and without any expansion of
 // weights: what the bf16 kernel spends on that (about 1.9 ms for 256 experts of 4096 x 2048, whatever the batch) is
@@ -73,6 +77,9 @@ struct TtArgs {
   float* const* row_dst;   // or null; else output row p goes to row_dst[p] (see y_row)
   const int* offsets;      // [E + 1]
   int* status;
+  const uint4* marks;      // gate/up, guarded (else flags is null): bytes of the split kernel, `parts` per sorted row
+  int* flags;              //   [E + 1] out: experts to be done again
+  int parts;
   int E, K, R, I, S;       // R weight rows per expert (2I or H)
   int blocked;             // weights in moe_prepack's tile-contiguous layout (see ExpertWeights)
   int max_tok, sf_step;    // of the pass geometry (see TwoTermGeometry)
@@ -155,6 +162,22 @@ MOE_DEVINL int tt_sf_byte(int r, int k32) { return (r >> 7) * 512 + (r & 31) * 1
 // exists) and 1 / 2^s.  Blocks whose maximum is below 2^-115 lose bits at the bottom instead.
 MOE_DEVINL uint32_t tt_scale(uint32_t amax_bits) { return max(amax_bits >> 23, 12u) - 7u; }
 MOE_DEVINL float tt_inv(uint32_t sb) { return __uint_as_float((254u - sb) << 23); }
+// Smallest magnitude (bits of a float, at least 1) that is certain to be held exactly in a block with this maximum: the last bit
+// of a bf16 value 2^14 below the maximum's power of two is the lo term's last.  Smaller values lose their lowest
+// bits, 2^-22 of the maximum at most.  (A bf16 subnormal has the last bit of the smallest normal value.)
+MOE_DEVINL uint32_t tt_lossy_below(uint32_t amax_bits) {
+  const uint32_t eb = max(amax_bits >> 23, 12u);
+  return eb > 15u ? (eb - 14u) << 23 : 1u;
+}
+// Which experts are done again: those with a token block of at least kTtLossyTokens values below that bound, or a block of the
+// intermediate with at least kTtLossyInter of them and no more than kTtLarge that reach 2^-10 of the maximum; or with a value that is
+// not finite.  Batches of ordinary values have none: of normal values one in 10^4 is below the bound, of the products a
+// SwiGLU makes of them one in 10^3 (six, eight in one block: less than 1e-14 of the blocks), and where gates in the tens leave
+// half of a block next to zero the rest of it is large (four or fewer: 1e-6, so a block or so of a large batch).  With
+// one element of every block 2^10 times the others half a percent of the token blocks are found, 4 % of the
+// intermediate's; at 2^14 most.  What is left to the terms in an expert that is not done again is thus
+// an error of 1e-5 of a block's norm without its few largest elements, at most 2^-22 of its maximum per element.
+constexpr int kTtLossyTokens = 6, kTtLossyInter = 8, kTtLarge = 3;
 // Four values over their blocks' scales, as halves y (exact down to 2^-24, below the lo term's last bit) -> four hi and four lo
 // codes, one per byte.  E4M3 is a half without its last seven mantissa bits and 8 less of exponent bias, subnormals
 // included: the code of v is the half v / 2^8, rounded (half away from zero) by adding 0x40 to its bits, less the low
@@ -443,7 +466,9 @@ MOE_DEVINL TtSfPlace tt_sf_place(int p, int e, const TtTables& t, int H, int sf_
 // A warp's 256 consecutive values of a row, 16 bytes per lane -> 8 hi and 8 lo codes per lane, and the scale word of the K
 // step its half warp holds.  Four lanes share a block of 32.  Bound by issue where its input is in L2: the block maximum on
 // 16-bit pairs and the terms on pairs of halves.
-MOE_DEVINL void tt_split_256(const uint4& v, int lane, uint2* hi, uint2* lo, uint32_t* word) {
+// kGuard: says whether one of the eight blocks is to be done again (the same in all lanes).
+template <bool kGuard>
+MOE_DEVINL bool tt_split_256(const uint4& v, int lane, uint2* hi, uint2* lo, uint32_t* word) {
   uint32_t w[4] = {v.x, v.y, v.z, v.w};
   constexpr uint32_t kAbs = 0x7FFF7FFFu;
   uint32_t m2 = __vmaxu2(__vmaxu2(w[0] & kAbs, w[1] & kAbs), __vmaxu2(w[2] & kAbs, w[3] & kAbs));
@@ -466,6 +491,20 @@ MOE_DEVINL void tt_split_256(const uint4& v, int lane, uint2* hi, uint2* lo, uin
   sw |= __shfl_xor_sync(0xffffffffu, sw, 4);
   sw |= __shfl_xor_sync(0xffffffffu, sw, 8);
   *word = sw;
+  if constexpr (!kGuard) return false;
+  // magnitudes less one, so that zeros are the largest: the smallest against the bound, and a count only where it is below
+  uint32_t least = 0xFFFFFFFFu;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) least = __viaddmin_u16x2(w[j] & kAbs, 0xFFFFFFFFu, least);
+  const uint32_t below = max(tt_lossy_below(amax) >> 16, 1u) - 1u;
+  const bool finite = amax < 0x7F800000u;
+  if (!__any_sync(0xffffffffu, min(least & 0xFFFFu, least >> 16) < below || !finite)) return false;
+  int n = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) n += ((w[j] & 0x7FFFu) - 1u < below) + (((w[j] >> 16) & 0x7FFFu) - 1u < below);
+  n += __shfl_xor_sync(0xffffffffu, n, 1);
+  n += __shfl_xor_sync(0xffffffffu, n, 2);
+  return __any_sync(0xffffffffu, n >= kTtLossyTokens || !finite);
 }
 
 // The quantised-activation variant's counterpart: 8 E2M1 codes per lane (native_quant_rows_kernel's arithmetic), scale word likewise
@@ -496,15 +535,18 @@ MOE_DEVINL uint32_t tt_quant_256(const uint4& v, int lane, uint32_t* word) {
 // issue (2 bytes read and 2 written per element; 12288 rows of 4096: 41 us, 54 with
 // conversion instructions and a look-up per four pieces). ----
 // kQ (quantised activations): one E2M1 term instead, rows of H / 2 bytes, two scale words per K step of 256.
-template <bool kQ>
+// kGuard: a byte per task into `marks` (see tt_split_256), and the experts' flags start at zero.
+template <bool kQ, bool kGuard>
 __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ offsets,
                                                               uint8_t* __restrict__ xq, uint8_t* __restrict__ sfx, int S, int H, int E,
-                                                              int max_tok, int sf_step) {
+                                                              int max_tok, int sf_step, uint8_t* __restrict__ marks, int* __restrict__ flags) {
   extern __shared__ int s_tt_tables[];
   pdl_launch_dependents();  // the gate/up grid may set up and start its weight stream; it waits before it reads rows
   // (expert_offsets was complete before the kernel in front of this one could start)
   const TtTables tab = tt_tables<kQ>(s_tt_tables, offsets, E, max_tok);
   pdl_wait();
+  if (kGuard && blockIdx.x == 0)
+    for (int e = threadIdx.x; e <= E; e += blockDim.x) flags[e] = 0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int n_chunk = H / 256, parts = (n_chunk + 7) / 8;
   const int p_begin = tab.off[0], n_task = (tab.off[E] - p_begin) * parts;
@@ -523,6 +565,7 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
     uint32_t* dst_q = reinterpret_cast<uint32_t*>(xq + static_cast<size_t>(p) * (H / 2)) + c0 * 32 + lane;
     uint8_t* sf = kQ ? sfx + at.hi + (lane >> 4) * at.lo + static_cast<size_t>(c0) * sf_step
                      : sfx + at.hi + (sf_is_lo ? at.lo : 0) + static_cast<size_t>(2 * c0 + (lane >> 4)) * sf_step;
+    bool again = false;
 #pragma unroll 1
     for (int cb = 0; cb < 8 && cb < left; cb += 4) {
       uint4 v[4];
@@ -539,7 +582,7 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
             sf += sf_step;
           } else {
             uint2 hi, lo;
-            tt_split_256(v[u], lane, &hi, &lo, &word);
+            again |= tt_split_256<kGuard>(v[u], lane, &hi, &lo, &word);
             dst_hi[u * 32] = hi;
             dst_lo[u * 32] = lo;
             if (sf_lane) *reinterpret_cast<uint32_t*>(sf) = word - sf_less;
@@ -551,6 +594,7 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
       dst_lo += 128;
       dst_q += 128;
     }
+    if (kGuard && lane == 0) marks[static_cast<size_t>(p) * parts + (task - row * parts)] = again;
   }
 }
 
@@ -558,14 +602,18 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
 // once and stored at its k sorted places, so the bf16 copy in sorted order is neither written nor read and a value is
 // converted once, not k times.  Warp task: (token, `chunks` pieces of 256 values).  Bound by the k * H * 2 bytes written per
 // token. ----
+template <bool kGuard>
 __global__ void __launch_bounds__(256) twoterm_scatter_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ ids,
                                                              const int* __restrict__ inv_perm, const int* __restrict__ offsets,
                                                              uint8_t* __restrict__ xq, uint8_t* __restrict__ sfx, int T, int k, int H,
-                                                             int E, int max_tok, int sf_step, int chunks) {
+                                                             int E, int max_tok, int sf_step, int chunks, uint8_t* __restrict__ marks,
+                                                             int* __restrict__ flags) {
   extern __shared__ int s_tt_tables[];
   pdl_launch_dependents();  // as above
   const TtTables tab = tt_tables<false>(s_tt_tables, offsets, E, max_tok);
   pdl_wait();
+  if (kGuard && blockIdx.x == 0)
+    for (int e = threadIdx.x; e <= E; e += blockDim.x) flags[e] = 0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const size_t S = static_cast<size_t>(T) * k;
   const int n_chunk = H / 256, parts = (n_chunk + chunks - 1) / chunks;
@@ -582,11 +630,12 @@ __global__ void __launch_bounds__(256) twoterm_scatter_kernel(const __nv_bfloat1
     }
     __syncwarp();
     const uint4* src = reinterpret_cast<const uint4*>(x + static_cast<size_t>(t) * H);
+    bool again = false;
 #pragma unroll 2
     for (int c = c0; c < c1; ++c) {
       uint2 hi, lo;
       uint32_t word;
-      tt_split_256(__ldg(src + c * 32 + lane), lane, &hi, &lo, &word);
+      again |= tt_split_256<kGuard>(__ldg(src + c * 32 + lane), lane, &hi, &lo, &word);
       const size_t step = static_cast<size_t>(2 * c + (lane >> 4)) * sf_step;
       for (int j = 0; j < k; ++j) {
         const size_t row = static_cast<size_t>(__shfl_sync(0xffffffffu, p, j));
@@ -598,6 +647,22 @@ __global__ void __launch_bounds__(256) twoterm_scatter_kernel(const __nv_bfloat1
         if ((lane & 15) == 1) *reinterpret_cast<uint32_t*>(sfx + at + step + d) = word - 0x05050505u;
       }
     }
+    if (kGuard && lane < k) marks[static_cast<size_t>(p) * parts + task % parts] = again;
+  }
+}
+
+// Rows in sorted order of the experts that are done again, where the split above left them where they were
+__global__ void __launch_bounds__(256) twoterm_gather_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ ids,
+                                                            const int* __restrict__ inv_perm, const int* only, int T, int k, int H,
+                                                            int E, __nv_bfloat16* __restrict__ x_sorted) {
+  pdl_wait();
+  if (__ldcg(only + E) == 0) return;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (size_t s = static_cast<size_t>(blockIdx.x) * 8 + wid; s < static_cast<size_t>(T) * k; s += static_cast<size_t>(gridDim.x) * 8) {
+    if (__ldcg(only + __ldg(ids + s)) == 0) continue;
+    const uint4* src = reinterpret_cast<const uint4*>(x + s / k * H);
+    uint4* dst = reinterpret_cast<uint4*>(x_sorted + static_cast<size_t>(__ldg(inv_perm + s)) * H);
+    for (int i = lane; i < H / 8; i += 32) dst[i] = __ldg(src + i);
   }
 }
 
@@ -913,10 +978,32 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     int tog = 0, g_known = -1;
     TtPass p = {};
     uint32_t acc_ph[2] = {0u, 0u};
+    const bool guard = STAGE1 && !kQ && a.flags != nullptr;
+    if (guard) {
+      // the split kernel's marks -> flags of their experts, 16 at a time, while the first MMAs run
+      pdl_wait();  // the marks are complete and the flags zero
+      const size_t n_marks = (static_cast<size_t>(a.S) * a.parts + 15) / 16;
+      for (size_t i = static_cast<size_t>(blockIdx.x) * (kTtEpiWarps * 32) + (tid - kTtFirstEpi * 32); i < n_marks;
+           i += static_cast<size_t>(gridDim.x) * (kTtEpiWarps * 32)) {
+        const uint4 v = __ldcg(a.marks + i);
+        if ((v.x | v.y | v.z | v.w) == 0u) continue;
+        const uint32_t m[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int b = 0; b < 16; ++b) {
+          if (((m[b >> 2] >> (8 * (b & 3))) & 0xFFu) == 0u) continue;
+          const int row = static_cast<int>((i * 16 + b) / a.parts);
+          if (row < s_off[0] || row >= s_off[a.E]) continue;  // (rows of other ranks' experts: their marks are not written)
+          a.flags[tt_find_expert(s_off, a.E, row)] = 1;
+          a.flags[a.E] = 1;
+        }
+      }
+      __syncwarp();
+    }
+    int e = 0;
     for (int w = first; w < total; w = next_item(w)) {
       const int g = w / tiles, rt = w % tiles;
       if (g != g_known) {
-        const int e = tt_find_expert(prefix, a.E, g);
+        e = tt_find_expert(prefix, a.E, g);
         p = tt_pass<kQ>(s_off[e], s_off[e + 1], g - prefix[e], a.max_tok);
         g_known = g;
       }
@@ -1020,6 +1107,7 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
           const int kstep = rt * 2 + rank;
           const int i0 = kstep * 128 + q * 32 + 4 * (lane >> 2);
           uint8_t* sf = a.sfa + (static_cast<size_t>(g) * (a.I / kTtK) + kstep) * a.sf_step;
+          bool again = false;  // a block of this item that the terms hold too little of
   #pragma unroll
           for (int ch = 0; ch < kChunks; ++ch) {
             const int c0 = ch * 32 + sub * 8;
@@ -1038,6 +1126,13 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
                   v[t] = __uint_as_float(vb);
                   inv[t] = tt_inv(sb);
                   bad |= amax >= 0x7F800000u;
+                  if (guard) {
+                    const uint32_t abs_v = vb & 0x7FFFFFFFu;
+                    bool found = __popc(__ballot_sync(0xffffffffu, abs_v - 1u < tt_lossy_below(amax) - 1u)) >= kTtLossyInter;
+                    if (found)  // (its maximum is above 2^-111 then)
+                      found = __popc(__ballot_sync(0xffffffffu, abs_v >= (amax & 0x7F800000u) - (10u << 23))) <= kTtLarge;
+                    again |= (found || amax >= 0x7F800000u) && c0 + jj + t < p.n;
+                  }
                   if (lane == jj + t) my_sb = sb;
                 }
                 uint32_t hw, lw, h1, l1;
@@ -1061,6 +1156,10 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
                 sf[p.stacked ? tt_sf_byte(p.nr + r, q) : 1024 + tt_sf_byte(r, q)] = static_cast<uint8_t>(my_sb - 5u);
               }
             }
+          }
+          if (again && lane == 0) {
+            a.flags[e] = 1;
+            a.flags[a.E] = 1;
           }
         }
       } else {
@@ -1145,8 +1244,28 @@ bool tt_launch(const CUtensorMap& tm_w, const CUtensorMap& tm_sc, const TtTokMap
 
 }  // namespace
 
+bool twoterm_guarded(const moe_shape_t& choice, const ExpertWeights& w) {
+  return !native_shape_ok(choice, w.w13, w.w2) && (umma_shape_ok(choice) || w.blocked || stream_shape_ok(choice));
+}
+
+// The experts that `flags` names, by the kernel that would take the shape without this one; their rows of the output are
+// written again.  The bf16 intermediate lies over the two-term one, which no kernel reads any more.
+static int launch_again(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh, const moe_shape_t& choice,
+                        void* act, float* y_perm, int* status_word, cudaStream_t st, float* const* row_dst, const int* flags) {
+  const __nv_bfloat16* rows = in.x;
+  if (in.inv_perm != nullptr) {
+    if (launch_pdl(twoterm_gather_kernel, dim3(static_cast<unsigned>(sm_count()) * 8), dim3(256), 0, st, in.x, in.ids, in.inv_perm, flags,
+                   sh.T, sh.k, sh.H, sh.E, in.x_sorted) != cudaSuccess)
+      return MOE_ERR_CUDA;
+    rows = in.x_sorted;
+  }
+  __nv_bfloat16* a = static_cast<__nv_bfloat16*>(act);
+  if (umma_shape_ok(choice) || w.blocked) return launch_expert_ffn_umma(rows, offsets, w, sh, a, y_perm, status_word, st, row_dst, flags);
+  return launch_expert_ffn_stream(rows, offsets, w.w13, w.s13, w.w2, w.s2, sh, a, y_perm, status_word, st, row_dst, flags);
+}
+
 int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
-                              const moe_shape_t& choice, void* scratch, float* y_perm, int* status_word, cudaStream_t st,
+                              const moe_shape_t& choice, bool guard, void* scratch, float* y_perm, int* status_word, cudaStream_t st,
                               float* const* row_dst) {
   const TwoTermGeometry geo = twoterm_geometry(choice);
   const TwoTermScratch L = twoterm_scratch(choice);
@@ -1161,23 +1280,28 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
   for (int b = 0; b < kTtBoxes; ++b)
     if (!term_row_map(&tm_x.box[b], base + L.xq, sh.H, 2 * S, 64u >> b) || !term_row_map(&tm_a.box[b], base + L.aq, sh.I, 2 * S, 64u >> b))
       return MOE_ERR_CUDA;
-  if (!byte_map_2d(&tm_x.sf, base + L.sfx, 128, (L.sfa - L.sfx) / 128, 128, 4) || !byte_map_2d(&tm_a.sf, base + L.sfa, 128, (L.total - L.sfa) / 128, 128, 4))
+  if (!byte_map_2d(&tm_x.sf, base + L.sfx, 128, (L.sfa - L.sfx) / 128, 128, 4) || !byte_map_2d(&tm_a.sf, base + L.sfa, 128, (L.marks - L.sfa) / 128, 128, 4))
     return MOE_ERR_CUDA;
+  uint8_t* marks = base + L.marks;
+  int* flags = reinterpret_cast<int*>(base + L.flags);
+  const int n_chunk = sh.H / 256;
+  int parts = (n_chunk + 7) / 8;  // pieces of a row, a mark each
   const size_t most = static_cast<size_t>(sm_count()) * 8;  // CTAs of eight warps that fit the chip
   const size_t table_bytes = static_cast<size_t>(kTtTableInts * (sh.E + 1)) * 4;
   cudaError_t rc;
   if (in.inv_perm != nullptr) {
     // whole rows per warp where there are tokens enough to fill the chip, pieces of them otherwise
-    const int n_chunk = sh.H / 256;
     const size_t per_token = most * 8 / static_cast<size_t>(sh.T);
     const int chunks = per_token >= static_cast<size_t>(n_chunk) ? 1 : (per_token <= 1 ? n_chunk : (n_chunk + static_cast<int>(per_token) - 1) / static_cast<int>(per_token));
-    const size_t want = (static_cast<size_t>(sh.T) * ((n_chunk + chunks - 1) / chunks) + 7) / 8;
-    rc = launch_pdl(twoterm_scatter_kernel, dim3(static_cast<unsigned>(want < most ? want : most)), dim3(256), table_bytes, st, in.x,
-                    in.ids, in.inv_perm, offsets, base + L.xq, base + L.sfx, sh.T, sh.k, sh.H, sh.E, geo.max_tok, geo.sf_step, chunks);
+    parts = (n_chunk + chunks - 1) / chunks;
+    const size_t want = (static_cast<size_t>(sh.T) * parts + 7) / 8;
+    rc = launch_pdl(guard ? twoterm_scatter_kernel<true> : twoterm_scatter_kernel<false>, dim3(static_cast<unsigned>(want < most ? want : most)), dim3(256), table_bytes, st, in.x,
+                    in.ids, in.inv_perm, offsets, base + L.xq, base + L.sfx, sh.T, sh.k, sh.H, sh.E, geo.max_tok, geo.sf_step, chunks,
+                    marks, flags);
   } else {
-    const size_t want = (S * ((sh.H / 256 + 7) / 8) + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
-    rc = launch_pdl(twoterm_split_kernel<false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256), table_bytes, st, in.x,
-                    offsets, base + L.xq, base + L.sfx, static_cast<int>(S), sh.H, sh.E, geo.max_tok, geo.sf_step);
+    const size_t want = (S * parts + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
+    rc = launch_pdl(guard ? twoterm_split_kernel<false, true> : twoterm_split_kernel<false, false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256), table_bytes, st, in.x,
+                    offsets, base + L.xq, base + L.sfx, static_cast<int>(S), sh.H, sh.E, geo.max_tok, geo.sf_step, marks, flags);
   }
   if (rc != cudaSuccess) return MOE_ERR_CUDA;
   TtArgs a = {};
@@ -1197,6 +1321,11 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
   a.t_bytes = a.sf_off + (geo.sf_step > 1024 ? 2048 : 1024);
   a.aq = base + L.aq;
   a.sfa = base + L.sfa;
+  if (guard) {
+    a.marks = reinterpret_cast<const uint4*>(marks);
+    a.flags = flags;
+    a.parts = parts;
+  }
   a.sc = w.s13;
   a.K = sh.H;
   a.R = 2 * sh.I;
@@ -1206,7 +1335,11 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
   a.R = sh.H;
   const bool two = geo.max_tok == 64 && sh.H % 512 == 0;
   if (!(two ? tt_launch<false, 2, false>(tm_w2, tm_s2, tm_a, a, st) : tt_launch<false, 1, false>(tm_w2, tm_s2, tm_a, a, st))) return MOE_ERR_CUDA;
-  note_kernel("ffn_mxf8_two_term_cta_pair", 3);
+  if (guard) {
+    const int again = launch_again(in, offsets, w, sh, choice, base + L.aq, y_perm, status_word, st, row_dst, flags);
+    if (again != MOE_OK) return again;
+  }
+  note_kernel("ffn_mxf8_two_term_cta_pair", 3 + (guard && in.inv_perm != nullptr ? 1 : 0));
   return MOE_OK;
 }
 
@@ -1224,9 +1357,9 @@ int launch_expert_ffn_q_pair(const __nv_bfloat16* x_perm, const int* offsets, co
   if (!byte_map_2d(&tm_x.sf, base + L.sfx, 128, (L.sfa - L.sfx) / 128, 128, 4) || !byte_map_2d(&tm_a.sf, base + L.sfa, 128, (L.total - L.sfa) / 128, 128, 4))
     return MOE_ERR_CUDA;
   const size_t want = (S * ((sh.H / 256 + 7) / 8) + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
-  if (launch_pdl(twoterm_split_kernel<true>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256),
+  if (launch_pdl(twoterm_split_kernel<true, false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256),
                  static_cast<size_t>(kTtTableInts * (sh.E + 1)) * 4, st, x_perm, offsets, base + L.xq, base + L.sfx, static_cast<int>(S), sh.H,
-                 sh.E, kQPairTok, 2048) != cudaSuccess)
+                 sh.E, kQPairTok, 2048, nullptr, nullptr) != cudaSuccess)
     return MOE_ERR_CUDA;
   TtArgs a = {};
   a.offsets = offsets;

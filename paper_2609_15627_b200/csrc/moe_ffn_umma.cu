@@ -53,6 +53,7 @@ struct UmmaArgs {
   float* y;                // stage 2 output [S, R]
   float* const* row_dst;   // or null; else output row p goes to row_dst[p] (see y_row)
   int* status;
+  const int* only;         // or null; else [E + 1]: experts whose word is zero are skipped, all of them where word E is
   uint32_t k1, k2;         // 0x1040, 0x0104: multipliers of the E2M1 expansion, kept opaque to the compiler
   int E, K, R, I;          // R weight rows per expert (2I or H)
 };
@@ -106,6 +107,10 @@ template <bool STAGE1>
 __global__ void __launch_bounds__(kThreadsUmma, 1)
 ffn_umma_kernel(const __grid_constant__ CUtensorMap tmap_tok, const __grid_constant__ CUtensorMap tmap_w, const UmmaArgs a) {
   extern __shared__ unsigned char smem_dyn[];
+  if (a.only != nullptr) {  // (launched beside the kernel before it in this case)
+    pdl_wait();
+    if (__ldcg(a.only + a.E) == 0) return;
+  }
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
   const SmemMap sm = smem_map(a.E);
   unsigned char* sA = smem + sm.a;
@@ -132,7 +137,7 @@ ffn_umma_kernel(const __grid_constant__ CUtensorMap tmap_tok, const __grid_const
     int run = 0;
     for (int e0 = 0; e0 < a.E; e0 += 32) {
       const int e = e0 + lane;
-      const int rows = (e < a.E) ? a.offsets[e + 1] - a.offsets[e] : 0;
+      const int rows = (e < a.E && (a.only == nullptr || __ldcg(a.only + e) != 0)) ? a.offsets[e + 1] - a.offsets[e] : 0;
       const int passes = (rows + kMaxTok - 1) / kMaxTok;
       int tot;
       const int ex = warp_excl_scan(passes, lane, &tot);
@@ -397,7 +402,8 @@ bool umma_shape_ok(const moe_shape_t& sh) {
 }
 
 int launch_expert_ffn_umma(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
-                           __nv_bfloat16* act, float* y_perm, int* status_word, cudaStream_t st, float* const* row_dst) {
+                           __nv_bfloat16* act, float* y_perm, int* status_word, cudaStream_t st, float* const* row_dst,
+                           const int* only) {
   const size_t smem = smem_map(sh.E).total + 1024;
   static PerDeviceFlag flag;
   if (!once_per_device(flag, [] {
@@ -423,6 +429,7 @@ int launch_expert_ffn_umma(const __nv_bfloat16* x_perm, const int* offsets, cons
   a.y = y_perm;
   a.row_dst = row_dst;
   a.status = status_word;
+  a.only = only;
   a.k1 = 0x1040u;
   a.k2 = 0x0104u;
   a.E = sh.E;
@@ -432,14 +439,17 @@ int launch_expert_ffn_umma(const __nv_bfloat16* x_perm, const int* offsets, cons
   a.sc = w.s13;
   a.K = sh.H;
   a.R = 2 * sh.I;
-  ffn_umma_kernel<true><<<grid, kThreadsUmma, smem, st>>>(tm_x, tm_w13, a);
-  if (cudaGetLastError() != cudaSuccess) return MOE_ERR_CUDA;
+  auto run = [&](auto kernel, const CUtensorMap& tok, const CUtensorMap& wt) {
+    if (only != nullptr) return launch_pdl(kernel, dim3(grid), dim3(kThreadsUmma), smem, st, tok, wt, a) == cudaSuccess;
+    kernel<<<grid, kThreadsUmma, smem, st>>>(tok, wt, a);
+    return cudaGetLastError() == cudaSuccess;
+  };
+  if (!run(ffn_umma_kernel<true>, tm_x, tm_w13)) return MOE_ERR_CUDA;
   a.w = w.w2;
   a.sc = w.s2;
   a.K = sh.I;
   a.R = sh.H;
-  ffn_umma_kernel<false><<<grid, kThreadsUmma, smem, st>>>(tm_act, tm_w2, a);
-  if (cudaGetLastError() != cudaSuccess) return MOE_ERR_CUDA;
+  if (!run(ffn_umma_kernel<false>, tm_act, tm_w2)) return MOE_ERR_CUDA;
   note_kernel("ffn_umma_tcgen05_grouped", 2);
   return MOE_OK;
 }

@@ -121,3 +121,144 @@ def test_quantised_activations_on_cta_pairs(T, H, I, E, k, packed):
     torch.cuda.synchronize()
     assert int(status.item()) == 0 and moe.moe_last_kernel_name() == "ffn_mxf4_quantised_cta_pair"
     _check_rows(y.cpu().numpy(), O.expert_ffn_q(x_perm, off, *w, k), "quantised, CTA pairs")
+
+
+# ---- blocks that two terms hold too little of: their experts are done again by the kernel that holds every value ----
+_UMMA, _STREAM = "ffn_umma_tcgen05_grouped", "ffn_stream_bulk_ring_mma16816"
+_AGAIN = [(2048, 1024, _UMMA, False), (2048, 1024, _UMMA, True), (2048, 1280, _STREAM, False)]
+
+
+def _at_16(t):
+    """A copy at an address that is a multiple of 16 bytes and not of 32."""
+    room = torch.empty(t.numel() + 48, dtype=torch.uint8, device="cuda")
+    lead = (16 - room.data_ptr()) % 32
+    return room[lead:lead + t.numel()].copy_(t.reshape(-1)).view(t.shape)
+
+
+def _bits(t):
+    return t.contiguous().view(torch.int32)
+
+
+def _three_ways(x, off, wdev, sh, kernel, packed):
+    """y_perm of the public call, of the kernel that takes the shape without this one, and of this one alone."""
+    xd, offd = dev(x), dev(off)
+    buf = moe.LayerBuffers(sh)
+    ys = []
+
+    def run(call, *args, name=NAME):
+        buf.y_perm.fill_(float("nan"))
+        call(xd, offd, *args)
+        torch.cuda.synchronize()
+        assert int(buf.status.item()) == 0 and moe.moe_last_kernel_name() == name
+        ys.append(buf.y_perm.clone())
+
+    if packed:
+        run(moe.moe_expert_ffn_packed, moe.moe_prepack(*wdev, sh), sh, buf.y_perm, buf.status, buf.ws)
+    else:
+        run(moe.moe_expert_ffn, *wdev, sh, buf.y_perm, buf.status, buf.ws)
+    w16 = (_at_16(wdev[0]), wdev[1], _at_16(wdev[2]), wdev[3])
+    run(moe.moe_expert_ffn, *w16, sh, buf.y_perm, buf.status, buf.ws, name=kernel)
+    run(moe.moe_debug_expert_ffn_variant, *wdev, sh, buf.y_perm, buf.status, buf.ws, moe.VARIANT_TWOTERM)
+    return ys
+
+
+def _done_again(ys, off):
+    """Experts whose rows are the other kernel's bits; every expert's rows are either that or this kernel's."""
+    got, other, alone = (_bits(y) for y in ys)
+    again = []
+    for e in range(len(off) - 1):
+        r = slice(int(off[e]), int(off[e + 1]))
+        if torch.equal(got[r], other[r]) and not torch.equal(other[r], alone[r]):
+            again.append(e)
+        else:
+            assert torch.equal(got[r], alone[r]), e
+    return again
+
+
+@pytest.mark.parametrize("H,I,kernel,packed", _AGAIN)
+def test_experts_done_again(H, I, kernel, packed):
+    E, counts = 16, [66 + (7 * e) % 11 for e in range(16)]
+    S = sum(counts)
+    off = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    w = [a.copy() for a in _weights(H, I, E, seed=21)]
+    xf = inputs.bf16_bits_to_f32(inputs.make_x(S, H, seed=22))
+
+    def block(row, c0, n_small, edge):
+        """2^15, n_small values below 2^-14 of it, `edge` at that bound, the rest between"""
+        xf[row, c0:c0 + 32] = 64.0
+        xf[row, c0 + 5] = 2.0 ** 15
+        xf[row, c0 + 8:c0 + 8 + n_small] = 1.0 + 2.0 ** -7
+        xf[row, c0 + 20:c0 + 20 + edge] = 2.0
+
+    block(int(off[1]), 0, 6, 0)                    # six: the first row of expert 1
+    block(int(off[4]) - 1, H - 32, 5, 3)           # five, and three at the bound: not enough
+    block(int(off[5]) + 3, 256 - 32, 9, 0)
+    xf[int(off[7]) + 1, 300] = np.inf
+    xf[int(off[9]) - 1, 17] = np.nan
+    w[1][10, I:, :] = 105                          # up rows of expert 10: one of a block 2^15 times the others
+    w[1][10, I + 101, :] = 120
+    w[1][12, I:, :] = 105                          # of expert 12: half of a block
+    w[1][12, I + 96:I + 112, :] = 120
+    x = inputs.f32_to_bf16_bits(xf)
+    sh = moe.shape(S, H, I, E, 1)
+    ys = _three_ways(x, off, [dev(a) for a in w], sh, kernel, packed)
+    assert _done_again(ys, off) == [1, 5, 7, 8, 10]
+
+
+@pytest.mark.parametrize("where", ["tokens", "intermediate"])
+@pytest.mark.parametrize("p", [10, 14, 18])
+def test_rows_keep_their_precision_beside_an_outlier_of_every_block(where, p):
+    """One element of every block of 32 is 2^p times the others and meets zero weights only, so every output is a sum over
+    the others.  By the median over rows (a row in ten holds a bf16 rounding of the intermediate that falls the other way,
+    2^-9 of one value): an fp32 sum of 2048 terms is off by 5e-7 of its norm, the two terms would be by 5e-5 (2^10) to 0.5."""
+    H, I, E, counts = 2048, 1024, 16, [66] * 16
+    S = sum(counts)
+    off = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    w = [a.copy() for a in _weights(H, I, E, seed=31)]
+    xf = inputs.bf16_bits_to_f32(inputs.make_x(S, H, seed=32))
+    if where == "tokens":
+        xf[:, 5::32] *= 2.0 ** p
+        w[0][:, :, 2::16] &= 0x0F                  # element 5 of a block: the high nibble of byte 2
+    else:
+        w[1][:, I:, :] = 108
+        w[1][:, I + 5::32, :] = 108 + p
+        w[2][:, :, 2::16] &= 0x0F
+    x = inputs.f32_to_bf16_bits(xf)
+    sh = moe.shape(S, H, I, E, 1)
+    buf = moe.LayerBuffers(sh)
+    moe.moe_expert_ffn(dev(x), dev(off), *[dev(a) for a in w], sh, buf.y_perm, buf.status, buf.ws)
+    torch.cuda.synchronize()
+    assert int(buf.status.item()) == 0 and moe.moe_last_kernel_name() == NAME
+    rows = np.concatenate([np.arange(off[e], off[e] + 8) for e in (0, 7, 15)])
+    sub = np.zeros(E + 1, np.int32)
+    sub[1:] = np.cumsum([8 if e in (0, 7, 15) else 0 for e in range(E)])
+    ref = O.expert_ffn(x[rows], sub, *w, 1).astype(np.float64)
+    got = buf.y_perm.cpu().numpy()[rows].astype(np.float64)
+    err = np.linalg.norm(got - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert np.median(err) <= 5e-6 and err.max() <= 5e-3, (np.median(err), err.max())
+
+
+@pytest.mark.parametrize("I,kernel", [(1024, _UMMA), (1280, _STREAM)])
+def test_whole_layer_and_expert_parallel_ranks_do_experts_again(I, kernel):
+    T, k, H, E = 536, 2, 2048, 16
+    wdev = tuple(dev(a) for a in _weights(H, I, E, seed=41))
+    xf = inputs.bf16_bits_to_f32(inputs.make_x(T, H, 42))
+    xf[::3, 64] = 2.0 ** 20                        # tokens of every expert
+    logits, x = dev(inputs.make_logits(T, E, 43)), dev(inputs.f32_to_bf16_bits(xf))
+    sh = moe.shape(T, H, I, E, k)
+    buf = moe.LayerBuffers(sh)
+    w16 = (_at_16(wdev[0]), wdev[1], _at_16(wdev[2]), wdev[3])
+    want = moe.moe_layer(logits, x, w16, buf).clone()
+    moe.moe_expert_ffn(buf.x_perm, buf.expert_offsets, *w16, sh, buf.y_perm, buf.status, buf.ws)
+    assert moe.moe_last_kernel_name() == kernel
+    assert torch.equal(moe.moe_layer(logits, x, wdev, buf), want)
+    out = torch.empty_like(want)
+    fws = moe.alloc_forward_workspace(sh)
+    fws[moe.moe_forward_sync_bytes():].fill_(0xFF)
+    for call, weights in ((moe.moe_forward, wdev), (moe.moe_forward_packed, (moe.moe_prepack(*wdev, sh),))):
+        out.fill_(float("nan"))
+        call(logits, x, *weights, sh, out, None, None, buf.status, fws)
+        assert torch.equal(out, want)
+    out, ranks = ep.run_emulated(torch, moe, sh, 2, logits, x, wdev)
+    assert all(int(b.layer.status.item()) == 0 for b in ranks) and torch.equal(out, want)
+    assert int(buf.status.item()) == 0
