@@ -86,7 +86,7 @@ uint64_t moe_launch_count(void);
  *   fixed fp32 sequence: d = max(d,-80); n = rint(d*0x1.715476p+0f); r = fma(n,-0x1.62e4p-1f,d);
  *   r = fma(n,-0x1.7f7d1cp-20f,r); p = Horner/fma over 1/720,1/120,1/24,1/6,1/2,1,1 in r; EXP = p*2^n.
  *   expert_offsets [E+1] int32: exclusive prefix sum of the per-expert slot counts, [E] = T*k.
- * Launch order: for T <= 128 the kernel uses programmatic dependent launch.  It reads logits before it waits
+ * Launch order: for T <= 32 the kernel uses programmatic dependent launch.  It reads logits before it waits
  * for the kernel launched just before it on the stream, and writes its outputs only after that kernel has
  * completed (so the outputs of one layer call may be the buffers the previous call's moe_combine still reads).
  * If that preceding kernel releases its dependents early (cudaTriggerProgrammaticLaunchCompletion /
@@ -132,9 +132,10 @@ int moe_permute(const void* x_bf16, const int32_t* topk_ids, const int32_t* expe
  * less than 2^-16 of that magnitude);
  * for other prefill-sized batches (T*k >= 1024, H and I multiples of 512) weights are expanded to bf16 exactly on chip for a bf16 grouped GEMM;
  * every other supported shape uses a register-expansion streaming kernel.
- * Launch order: the first two use programmatic dependent launch.  They read expert_offsets and the
- * weights before waiting for the kernel launched just before them on the stream, and x_perm only after it has
- * completed: expert_offsets must not be written by that immediately preceding kernel (moe_permute does not).
+ * Launch order: the second (T*k <= 32*E and <= 6144) reads expert_offsets and the weights before waiting for the kernel
+ * launched just before it on the stream (programmatic dependent launch), and x_perm only after that has completed:
+ * expert_offsets must not be written by that immediately preceding kernel (moe_permute does not).  The others read
+ * nothing before everything in front of them has completed.
  */
 int moe_expert_ffn(const void* x_perm_bf16 /* [T*k,H] */, const int32_t* expert_offsets,
                    const uint8_t* w13, const uint8_t* w13_scale, const uint8_t* w2, const uint8_t* w2_scale,

@@ -541,10 +541,12 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
                                                               uint8_t* __restrict__ xq, uint8_t* __restrict__ sfx, int S, int H, int E,
                                                               int max_tok, int sf_step, uint8_t* __restrict__ marks, int* __restrict__ flags) {
   extern __shared__ int s_tt_tables[];
-  pdl_launch_dependents();  // the gate/up grid may set up and start its weight stream; it waits before it reads rows
-  // (expert_offsets was complete before the kernel in front of this one could start)
-  const TtTables tab = tt_tables<kQ>(s_tt_tables, offsets, E, max_tok);
+  // The first launch of a public call, so the kernel in front of it may be the one that writes expert_offsets: wait before
+  // they are read here, and before the gate/up grid, which reads them as it starts, may start (it waits again before it
+  // reads rows).
   pdl_wait();
+  pdl_launch_dependents();
+  const TtTables tab = tt_tables<kQ>(s_tt_tables, offsets, E, max_tok);
   if (kGuard && blockIdx.x == 0)
     for (int e = threadIdx.x; e <= E; e += blockDim.x) flags[e] = 0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -609,7 +611,8 @@ __global__ void __launch_bounds__(256) twoterm_scatter_kernel(const __nv_bfloat1
                                                              int E, int max_tok, int sf_step, int chunks, uint8_t* __restrict__ marks,
                                                              int* __restrict__ flags) {
   extern __shared__ int s_tt_tables[];
-  pdl_launch_dependents();  // as above
+  // (behind the sort of the same call, which waited for the router before it let this kernel start: expert_offsets is complete)
+  pdl_launch_dependents();
   const TtTables tab = tt_tables<false>(s_tt_tables, offsets, E, max_tok);
   pdl_wait();
   if (kGuard && blockIdx.x == 0)
@@ -702,7 +705,7 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
   const bool sf_tma = (K % 512) == 0, sf_bulk = K == 256;
   const int grp_steps = (sf_tma ? 512 : 256) / step_k;
 
-  // ---- setup ----  (expert_offsets was complete before the kernel in front of this one could start)
+  // ---- setup ----  (expert_offsets was complete before the split kernel let this chain start)
   if (wid == 2) tt_prefix(a.offsets, a.E, a.max_tok, prefix, lane);
   if (wid >= kTtFirstEpi)
     for (int e = tid - kTtFirstEpi * 32; e <= a.E; e += kTtEpiWarps * 32) s_off[e] = __ldg(a.offsets + e);

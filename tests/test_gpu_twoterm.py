@@ -262,3 +262,42 @@ def test_whole_layer_and_expert_parallel_ranks_do_experts_again(I, kernel):
     out, ranks = ep.run_emulated(torch, moe, sh, 2, logits, x, wdev)
     assert all(int(b.layer.status.item()) == 0 for b in ranks) and torch.equal(out, want)
     assert int(buf.status.item()) == 0
+
+
+# (33 and 97 rows per expert: passes of 64 and of 224 tokens; the quantised variant above 64)
+@pytest.mark.parametrize("T,k,H,I,quantised", [(2112, 2, 512, 512, False), (3100, 4, 512, 512, False), (3100, 4, 512, 512, True)])
+def test_offsets_may_come_from_the_launch_in_front(T, k, H, I, quantised):
+    """moe_route lets its dependents start before it has written expert_offsets; a call right behind it on rows sorted
+    earlier has to see the new ones.  (The old ones in the buffer are valid too, so a call that read them too early would
+    give other rows, not stray ones.)"""
+    E = 128
+    w = tuple(dev(a) for a in _weights(H, I, E, seed=51))
+    logits, x = dev(inputs.make_logits(T, E, 52)), dev(inputs.make_x(T, H, 53))
+    sh = moe.shape(T, H, I, E, k)
+    buf = moe.LayerBuffers(sh)
+    qws = moe.alloc_ffn_q_workspace(sh)
+    moe.moe_route(logits, k, buf.topk_ids, buf.topk_w, buf.expert_offsets, buf.ws)
+    moe.moe_permute(x, buf.topk_ids, buf.expert_offsets, sh, buf.x_perm, buf.perm, buf.inv_perm, buf.ws)
+
+    def ffn():
+        if quantised:
+            moe.moe_expert_ffn_q(buf.x_perm, buf.expert_offsets, w, sh, buf.y_perm, buf.status, qws)
+            assert moe.moe_last_kernel_name() == "ffn_mxf4_quantised_cta_pair"
+        else:
+            moe.moe_expert_ffn(buf.x_perm, buf.expert_offsets, *w, sh, buf.y_perm, buf.status, buf.ws)
+            assert moe.moe_last_kernel_name() == NAME
+
+    torch.cuda.synchronize()
+    ffn()
+    torch.cuda.synchronize()
+    want = buf.y_perm.clone()
+    stale = torch.full_like(buf.expert_offsets, T * k)
+    stale[0] = 0
+    for _ in range(5):
+        buf.expert_offsets.copy_(stale)
+        buf.y_perm.fill_(float("nan"))
+        torch.cuda.synchronize()
+        moe.moe_route(logits, k, buf.topk_ids, buf.topk_w, buf.expert_offsets, buf.ws)
+        ffn()
+        torch.cuda.synchronize()
+        assert int(buf.status.item()) == 0 and torch.equal(buf.y_perm, want)
