@@ -42,10 +42,10 @@ int moe_debug_forward_one_launch(const float* logits, const void* x_bf16, const 
 
 /*
  * moe_expert_ffn with the kernel variant chosen by the caller instead of by the shape: 0 = register-expansion
- * streaming kernel (any supported shape), 1 = the tensor-core kernel for prefill-sized batches (H and I multiples of 512:
- * bf16 grouped GEMM), 2 = the one for decode-sized batches (the shapes moe_expert_ffn gives it: eight E2M1 terms) - both
- * the two-term kernel where the shape selects that -, 3 = the two-term kernel on any shape it can take (H and I multiples
- * of 256; workspace: enough for its E4M3 rows and scale factors).  Same arguments, workspace and meaning as moe_expert_ffn.
+ * streaming kernel (any supported shape), 1 = bf16 grouped GEMM (H and I multiples of 512), 2 = eight E2M1 terms on the
+ * block-scaled FP4 path (T*k <= 32*E and <= 6144, and the other limits moe_expert_ffn states for it), 3 = two E4M3 terms
+ * (H and I multiples of 256; workspace: enough for its E4M3 rows and scale factors), alone: no expert is done again.  Same
+ * arguments, workspace and meaning as moe_expert_ffn.
  * MOE_ERR_UNSUPPORTED_SHAPE if the variant cannot take the shape.  For tests that compare two variants on the same
  * inputs over a whole tensor, at sizes where the oracle can only be sampled.
  */

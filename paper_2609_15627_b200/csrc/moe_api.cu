@@ -619,8 +619,7 @@ int moe_debug_expert_ffn_variant(const void* x_perm_bf16, const int32_t* expert_
   const ExpertWeights w{w13, w13_scale, w2, w2_scale, false};
   StatusRef status;
   if ((rc = resolve_status(status_word, &status)) != MOE_OK) return rc;
-  const bool twoterm = twoterm_batch_ok(*shape) && twoterm_weights_ok(w13, w2);
-  if (variant == 3 || (variant != 0 && twoterm)) {
+  if (variant == 3) {
     if (!twoterm_shape_ok(*shape) || !twoterm_weights_ok(w13, w2)) return MOE_ERR_UNSUPPORTED_SHAPE;
     if (check_ws(ws, ws_bytes, L.act_off + twoterm_scratch(*shape).total) != MOE_OK) return MOE_ERR_WORKSPACE;
     if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;

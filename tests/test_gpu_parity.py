@@ -863,12 +863,19 @@ def test_layer_prefill_sampled(name, n_tokens, prod_weights):
     assert 4.0 < rms < 20.0, rms
 
 
-@pytest.mark.parametrize("name,variant", [("prefill_8k", moe.VARIANT_UMMA), ("decode_c64", moe.VARIANT_NATIVE),
-                                          ("decode_c768", moe.VARIANT_NATIVE)])
-def test_ffn_variants_agree_over_the_whole_tensor(name, variant, prod_weights):
-    """Where the oracle can only be sampled: every element of y_perm from the variant the shape selects against the
+_VARIANT_NAMES = {moe.VARIANT_STREAM: "ffn_stream_bulk_ring_mma16816", moe.VARIANT_UMMA: "ffn_umma_tcgen05_grouped",
+                  moe.VARIANT_NATIVE: "ffn_native_mxf4_block_scaled", moe.VARIANT_TWOTERM: "ffn_mxf8_two_term_cta_pair"}
+
+
+@pytest.mark.parametrize("name,selected,variant", [
+    ("prefill_8k", moe.VARIANT_TWOTERM, moe.VARIANT_TWOTERM), ("prefill_8k", moe.VARIANT_TWOTERM, moe.VARIANT_UMMA),
+    ("decode_c64", moe.VARIANT_NATIVE, moe.VARIANT_NATIVE),
+    ("decode_c768", moe.VARIANT_TWOTERM, moe.VARIANT_TWOTERM), ("decode_c768", moe.VARIANT_TWOTERM, moe.VARIANT_NATIVE)])
+def test_ffn_variants_agree_over_the_whole_tensor(name, selected, variant, prod_weights):
+    """Where the oracle can only be sampled: every element of y_perm from the variant the shape selects, and from the one
+    that takes the shape where that one cannot (weights aligned to 16 bytes only), against the
     streaming variant on the same inputs (the streaming variant is checked against the oracle in full on the small
-    shapes and shares no tile scheduler with the other two), within the tolerance of the fp32 per-slot rows.  A fault
+    shapes and shares no tile scheduler with the others), within the tolerance of the fp32 per-slot rows.  A fault
     confined to particular work shares, passes or row tiles of the full-size launch shows up here."""
     wl = inputs.WORKLOADS[name] if name in inputs.WORKLOADS else _EXTRA[name]
     (w13, s13, w2, s2), wdev = prod_weights
@@ -879,11 +886,14 @@ def test_ffn_variants_agree_over_the_whole_tensor(name, variant, prod_weights):
     moe.moe_permute(x, buf.topk_ids, buf.expert_offsets, sh, buf.x_perm, buf.perm, buf.inv_perm, buf.ws)
     moe.moe_expert_ffn(buf.x_perm, buf.expert_offsets, *wdev, sh, buf.y_perm, buf.status, buf.ws)
     torch.cuda.synchronize()
-    chosen = moe.moe_last_kernel_name()
+    assert moe.moe_last_kernel_name() == _VARIANT_NAMES[selected]
     y_sel = buf.y_perm.clone()
     moe.moe_debug_expert_ffn_variant(buf.x_perm, buf.expert_offsets, *wdev, sh, buf.y_perm, buf.status, buf.ws, variant)
     torch.cuda.synchronize()
-    assert moe.moe_last_kernel_name() == chosen and torch.equal(buf.y_perm, y_sel)   # the named variant IS the chosen one
+    assert moe.moe_last_kernel_name() == _VARIANT_NAMES[variant]
+    # the named variant IS the chosen one, or another one: equal bits then would be one kernel under two names
+    assert torch.equal(buf.y_perm, y_sel) == (variant == selected)
+    y_sel = buf.y_perm.clone()
     moe.moe_debug_expert_ffn_variant(buf.x_perm, buf.expert_offsets, *wdev, sh, buf.y_perm, buf.status, buf.ws,
                                      moe.VARIANT_STREAM)
     torch.cuda.synchronize()
