@@ -345,8 +345,8 @@ int moe_ep_expert_ffn(const void* x_perm_bf16 /* [T*k,H] */, const int32_t* expe
  * the library holds those 16 MiB until the process exits).
  *
  *   - Sizes: the bf16 intermediate (2*T*k*I bytes) - for the decode-sized kernel variant the E2M1 term rows of
- *     both projections' inputs, 4.25*T*k*(H+I) bytes, for the two-term variant its E4M3 rows where they fit - must fit the array, else MOE_ERR_WORKSPACE and nothing is
- *     launched (up to 640 slots at H = 4096, I = 2048).  Other argument rules as moe_expert_ffn.
+ *     both projections' inputs, 4.25*T*k*(H+I) bytes - of the kernel that takes the shape, or would without the two-term
+ *     one, must fit the array, else MOE_ERR_WORKSPACE and nothing is launched (up to 640 slots at H = 4096, I = 2048).  Other argument rules as moe_expert_ffn.
  *   - The call allocates and frees nothing and calls no allocating library routine.  Its first call on a
  *     device looks up the array's device address (one runtime query, cached per device): make that first
  *     call outside any stream capture.
@@ -354,8 +354,9 @@ int moe_ep_expert_ffn(const void* x_perm_bf16 /* [T*k,H] */, const int32_t* expe
  *     at zero (each call writes every row it later reads), but two calls that overlap on the GPU - other
  *     streams, other host threads - race on it: keep calls on one stream or order them yourself.
  *   - Result: identical to moe_expert_ffn on the same inputs (same kernels, same kernel choice), except where the
- *     two-term kernel's scratch does not fit the array: such a call runs the kernel that would take the shape without
- *     it, and its result is the same up to the summation order of fp32 dot products.
+ *     two-term kernel's scratch (2*T*k*(H+I) bytes and its scale factors) does not fit the array: such a call runs the
+ *     kernel that would take the shape without it, and its result is the same up to the summation order of fp32 dot
+ *     products and the bf16 roundings of the intermediate that turn on it.
  */
 size_t moe_expert_ffn_noalloc_max_bytes(void);
 int moe_expert_ffn_noalloc(const void* x_perm_bf16 /* [T*k,H] */, const int32_t* expert_offsets, const uint8_t* w13,

@@ -131,7 +131,6 @@ int moe_permute(const void* x_bf16, const int32_t* topk_ids, const int32_t* expe
 }
 
 namespace {
-bool twoterm_chosen(const moe_shape_t& s, const ExpertWeights& w) { return twoterm_batch_ok(s) && twoterm_weights_ok(w.w13, w.w2); }
 int expert_ffn_impl(const void* x_perm_bf16, const int32_t* expert_offsets, const ExpertWeights& w, const moe_shape_t* shape,
                     float* y_perm, int32_t* status_word, void* ws, size_t ws_bytes, void* cuda_stream,
                     float* const* row_dst = nullptr, const moe_shape_t* choice = nullptr) {

@@ -242,6 +242,9 @@ struct TwoTermInput {
 int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
                            const moe_shape_t& choice, bool guard, void* scratch, float* y_perm, int* status_word, cudaStream_t st,
                            float* const* row_dst = nullptr);
+// chosen by the batch and the weights' alignment, where another kernel takes the shape as well: what one of those refuses
+// (rows too long for the streaming kernel, its only one) stays refused
+bool twoterm_chosen(const moe_shape_t& choice, const ExpertWeights& w);
 bool twoterm_guarded(const moe_shape_t& choice, const ExpertWeights& w);
 // quantised activations, batches that fill the chip; scratch of q_pair_scratch
 int launch_expert_ffn_q_pair(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,

@@ -1247,9 +1247,11 @@ bool tt_launch(const CUtensorMap& tm_w, const CUtensorMap& tm_sc, const TtTokMap
 
 }  // namespace
 
-bool twoterm_guarded(const moe_shape_t& choice, const ExpertWeights& w) {
-  return !native_shape_ok(choice, w.w13, w.w2) && (umma_shape_ok(choice) || w.blocked || stream_shape_ok(choice));
+bool twoterm_chosen(const moe_shape_t& choice, const ExpertWeights& w) {
+  return twoterm_batch_ok(choice) && twoterm_weights_ok(w.w13, w.w2) &&
+         (native_shape_ok(choice, w.w13, w.w2) || umma_shape_ok(choice) || w.blocked || stream_shape_ok(choice));
 }
+bool twoterm_guarded(const moe_shape_t& choice, const ExpertWeights& w) { return !native_shape_ok(choice, w.w13, w.w2); }
 
 // The experts that `flags` names, by the kernel that would take the shape without this one; their rows of the output are
 // written again.  The bf16 intermediate lies over the two-term one, which no kernel reads any more.

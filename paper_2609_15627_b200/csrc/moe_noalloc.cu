@@ -54,11 +54,12 @@ int moe_expert_ffn_noalloc(const void* x_perm_bf16, const int32_t* expert_offset
   // what the chosen kernel keeps between its launches must fit the fixed array: the bf16 intermediate act[T*k, I],
   // or for the native variant the E2M1 term rows and scale bytes of both projections' inputs (4.25 (H + I) bytes per slot)
   const unsigned long long S = static_cast<unsigned long long>(s.T) * s.k;
-  // (the two-term variant where its own scratch fits, else the kernel that would take the shape without it)
-  const bool twoterm = twoterm_batch_ok(s) && twoterm_weights_ok(w13, w2) && twoterm_scratch(s).total + kAlign <= kStaticScratchBytes;
   const unsigned long long need =
-      twoterm ? 0ULL : (native_shape_ok(s, w13, w2) ? static_cast<unsigned long long>(native_scratch_bytes(s)) : S * s.I * 2ULL) + kAlign;
+      (native_shape_ok(s, w13, w2) ? static_cast<unsigned long long>(native_scratch_bytes(s)) : S * s.I * 2ULL) + kAlign;
   if (need > kStaticScratchBytes) return MOE_ERR_WORKSPACE;
+  // (the two-term variant only where its own scratch fits as well)
+  const ExpertWeights w{w13, w13_scale, w2, w2_scale, false};
+  const bool twoterm = twoterm_chosen(s, w) && twoterm_scratch(s).total + kAlign <= kStaticScratchBytes;
   void* scratch = nullptr;
   int rc = static_scratch(&scratch);  // first call on a device looks the address up
   if (rc != MOE_OK) return rc;
@@ -68,7 +69,6 @@ int moe_expert_ffn_noalloc(const void* x_perm_bf16, const int32_t* expert_offset
   // to start at zero.  Same kernels as moe_expert_ffn.
   __nv_bfloat16* act = static_cast<__nv_bfloat16*>(scratch);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const ExpertWeights w{w13, w13_scale, w2, w2_scale, false};
   if (!twoterm && native_shape_ok(s, w13, w2))
     return launch_expert_ffn_native(static_cast<const __nv_bfloat16*>(x_perm_bf16), expert_offsets, w, s, scratch, y_perm,
                                     status, st);

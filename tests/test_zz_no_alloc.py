@@ -34,6 +34,7 @@ def _case(T, H, I, E, k, seed):
 
 
 _NATIVE, _UMMA, _STREAM = "ffn_native_mxf4_block_scaled", "ffn_umma_tcgen05_grouped", "ffn_stream_bulk_ring_mma16816"
+_TWOTERM = "ffn_mxf8_two_term_cta_pair"
 
 # Every kernel variant behind the entry point, each carving its own kind of scratch out of the fixed array: the
 # decode-sized variant its E2M1 term rows, scale bytes and per-expert counters (read back through TMA tensor maps),
@@ -42,7 +43,9 @@ _NATIVE, _UMMA, _STREAM = "ffn_native_mxf4_block_scaled", "ffn_umma_tcgen05_grou
 # decode-sized batch at the production H and I whose scratch (26,112 bytes per slot) still fits the 16 MiB.
 _CASES = [(64, 512, 384, 8, 2, 0, _STREAM), (8, 1024, 512, 32, 6, 3, _NATIVE), (16, 256, 128, 8, 2, 1, _STREAM),
           (256, 512, 512, 8, 6, 4, _UMMA), (4, 512, 512, 8, 2, 5, _NATIVE), (64, 512, 256, 8, 2, 2, _NATIVE),
-          (80, 4096, 2048, 32, 8, 6, _NATIVE)]
+          (80, 4096, 2048, 32, 8, 6, _NATIVE),
+          # the two-term variant: its E4M3 rows and scale factors; 16 rows per expert, and 35 (experts may be done again)
+          (512, 512, 512, 64, 2, 7, _TWOTERM), (1120, 512, 512, 64, 2, 8, _TWOTERM)]
 
 
 def test_noalloc_matches_regular_entry_point_on_two_calls_in_a_row():
@@ -75,6 +78,36 @@ def test_noalloc_matches_regular_entry_point_on_two_calls_in_a_row():
         assert np.linalg.norm(g - r) / np.linalg.norm(r) <= 5e-4 and np.abs(g - r).max() <= 2e-2 * rms
 
 
+# The two-term variant's rows (2*T*k*(H+I) bytes) are beyond the array, the bf16 intermediate is not
+@pytest.mark.parametrize("T,H,I,E,k,kernel", [(1400, 1536, 512, 32, 3, _UMMA), (2048, 2048, 256, 64, 2, _STREAM)])
+def test_noalloc_runs_the_other_kernel_where_the_two_term_scratch_does_not_fit(T, H, I, E, k, kernel):
+    w, x_perm, off, sh = _case(T, H, I, E, k, 9)
+    buf = moe.LayerBuffers(sh)
+    moe.moe_expert_ffn(x_perm, off, *w, sh, buf.y_perm, buf.status, buf.ws)
+    torch.cuda.synchronize()
+    assert moe.moe_last_kernel_name() == _TWOTERM
+    want = buf.y_perm.double()
+    got = torch.full_like(buf.y_perm, float("nan"))
+    moe.moe_expert_ffn_noalloc(x_perm, off, *w, sh, got, buf.status)
+    torch.cuda.synchronize()
+    assert int(buf.status.item()) == 0 and moe.moe_last_kernel_name() == kernel
+    diff = got.double() - want                      # the tolerance of the fp32 per-slot rows
+    assert float(diff.norm() / want.norm()) <= 5e-4 and float(diff.abs().max()) <= 2e-2 * float(want.pow(2).mean().sqrt())
+
+
+def test_what_no_other_kernel_takes_stays_refused():
+    """Rows of 12,544 elements: too long for the streaming kernel's ring, no multiple of 512 for the grouped GEMM."""
+    T, H, I, E, k = 1024, 12544, 256, 64, 1
+    w = [torch.zeros(n, dtype=torch.uint8, device="cuda") for n in (E * I * H, E * I * H // 16, E * I * H // 2, E * I * H // 32)]
+    sh = moe.shape(T, H, I, E, k)
+    buf = moe.LayerBuffers(sh)
+    buf.x_perm.zero_()
+    off = torch.arange(E + 1, dtype=torch.int32, device="cuda") * (T // E)
+    with pytest.raises(moe.MoeError):
+        moe.moe_expert_ffn(buf.x_perm, off, *w, sh, buf.y_perm, buf.status, buf.ws)
+    torch.cuda.synchronize()
+
+
 def test_noalloc_rejects_a_misaligned_status_word():
     L = moe.lib()
     w, x_perm, off, sh = _case(16, 256, 128, 8, 2, 1)
@@ -90,4 +123,7 @@ def test_noalloc_rejects_sizes_beyond_the_fixed_array():
     fake = C.c_void_p(0x1000)  # never dereferenced: the size check comes first
     big = moe.shape(4096, 4096, 2048, 256, 8)   # 2*T*k*I = 128 MiB > 16 MiB
     assert L.moe_expert_ffn_noalloc(fake, fake, fake, fake, fake, fake, C.byref(big), fake, None, None) == 3
+    # 1024 slots: the two-term variant's rows would fit (12.6 MB), the eight-term kernel's (26.7 MB) never did
+    mid = moe.shape(512, 4096, 2048, 64, 2)
+    assert L.moe_expert_ffn_noalloc(fake, fake, fake, fake, fake, fake, C.byref(mid), fake, None, None) == 3
     assert L.moe_expert_ffn_noalloc(fake, fake, fake, fake, fake, fake, None, fake, None, None) == 1
