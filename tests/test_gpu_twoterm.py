@@ -301,3 +301,23 @@ def test_offsets_may_come_from_the_launch_in_front(T, k, H, I, quantised):
         ffn()
         torch.cuda.synchronize()
         assert int(buf.status.item()) == 0 and torch.equal(buf.y_perm, want)
+
+
+@pytest.mark.parametrize("T,I,kernel", [(512, 512, "ffn_native_mxf4_block_scaled"), (1120, 512, _UMMA), (1120, 256, _STREAM)])
+def test_weights_aligned_to_16_bytes_take_the_other_kernels(T, I, kernel):
+    """16 and 35 rows per expert, where 32-byte aligned weights take the two-term kernel."""
+    H, E, k = 512, 64, 2
+    w = _weights(H, I, E, seed=61)
+    x, ids = inputs.make_x(T, H, 62), O.route(inputs.make_logits(T, E, 63), k)
+    x_perm, _, _ = O.permute(x, ids[0], ids[2])
+    want = O.expert_ffn(x_perm, ids[2], *w, k)
+    sh = moe.shape(T, H, I, E, k)
+    buf = moe.LayerBuffers(sh)
+    wdev = [dev(a) for a in w]
+    for weights, name in ((wdev, NAME), ([_at_16(wdev[0]), wdev[1], wdev[2], wdev[3]], kernel),
+                          ([wdev[0], wdev[1], _at_16(wdev[2]), wdev[3]], kernel)):
+        buf.y_perm.fill_(float("nan"))
+        moe.moe_expert_ffn(dev(x_perm), dev(ids[2]), *weights, sh, buf.y_perm, buf.status, buf.ws)
+        torch.cuda.synchronize()
+        assert int(buf.status.item()) == 0 and moe.moe_last_kernel_name() == name
+        check_y(buf.y_perm.cpu().numpy(), want, name)
