@@ -164,10 +164,10 @@ MOE_DEVINL uint32_t tt_scale(uint32_t amax_bits) { return max(amax_bits >> 23, 1
 MOE_DEVINL float tt_inv(uint32_t sb) { return __uint_as_float((254u - sb) << 23); }
 // Smallest magnitude (bits of a float, at least 1) that is certain to be held exactly in a block with this maximum: the last bit
 // of a bf16 value 2^14 below the maximum's power of two is the lo term's last.  Smaller values lose their lowest
-// bits, 2^-22 of the maximum at most.  (A bf16 subnormal has the last bit of the smallest normal value.)
+// bits, 2^-22 of the maximum at most.
 MOE_DEVINL uint32_t tt_lossy_below(uint32_t amax_bits) {
-  const uint32_t eb = max(amax_bits >> 23, 12u);
-  return eb > 15u ? (eb - 14u) << 23 : 1u;
+  constexpr uint32_t k14 = (14u << 23) + 1u;
+  return max(amax_bits & 0x7F800000u, k14) - k14 + 1u;
 }
 // Which experts are done again: those with a token block of at least kTtLossyTokens values below that bound, or a block of the
 // intermediate with at least kTtLossyInter of them and no more than kTtLarge that reach 2^-10 of the maximum; or with a value that is
@@ -178,6 +178,22 @@ MOE_DEVINL uint32_t tt_lossy_below(uint32_t amax_bits) {
 // intermediate's; at 2^14 most.  What is left to the terms in an expert that is not done again is thus
 // an error of 1e-5 of a block's norm without its few largest elements, at most 2^-22 of its maximum per element.
 constexpr int kTtLossyTokens = 6, kTtLossyInter = 8, kTtLarge = 3;
+// The decision for eight blocks of the intermediate, value t of a lane in half t & 1 of word t / 2, of which the first n count
+// (the others are columns beyond the pass).  By a whole warp, after a cheaper look has found one of the eight suspect.
+MOE_DEVINL bool tt_again(const uint32_t (&pk)[4], int n) {
+  bool again = false;
+#pragma unroll 1
+  for (int t = 0; t < 8 && t < n; ++t) {
+    const uint32_t w = t < 2 ? pk[0] : t < 4 ? pk[1] : t < 6 ? pk[2] : pk[3];
+    const uint32_t v = ((t & 1) ? w & 0xFFFF0000u : w << 16) & 0x7FFFFFFFu;
+    const uint32_t amax = __reduce_max_sync(0xffffffffu, v);
+    const int lossy = __popc(__ballot_sync(0xffffffffu, v - 1u < tt_lossy_below(amax) - 1u));
+    // (with an inexact value in it the maximum is above 2^-112)
+    const int large = lossy > 0 ? __popc(__ballot_sync(0xffffffffu, v >= (amax & 0x7F800000u) - (10u << 23))) : 32;
+    again |= amax >= 0x7F800000u || (lossy >= kTtLossyInter && large <= kTtLarge);
+  }
+  return again;
+}
 // Four values over their blocks' scales, as halves y (exact down to 2^-24, below the lo term's last bit) -> four hi and four lo
 // codes, one per byte.  E4M3 is a half without its last seven mantissa bits and 8 less of exponent bias, subnormals
 // included: the code of v is the half v / 2^8, rounded (half away from zero) by adding 0x40 to its bits, less the low
@@ -502,7 +518,7 @@ MOE_DEVINL bool tt_split_256(const uint4& v, int lane, uint2* hi, uint2* lo, uin
   uint32_t least = 0xFFFFFFFFu;
 #pragma unroll
   for (int j = 0; j < 4; ++j) least = __viaddmin_u16x2(w[j] & kAbs, 0xFFFFFFFFu, least);
-  const uint32_t below = max(tt_lossy_below(amax) >> 16, 1u) - 1u;
+  const uint32_t below = (tt_lossy_below(amax) - 1u) >> 16;  // (a value v of 1 .. bound - 1: v - 1 < below)
   const bool finite = amax < 0x7F800000u;
   if (!__any_sync(0xffffffffu, min(least & 0xFFFFu, least >> 16) < below || !finite)) return false;
   int n = 0;
@@ -678,11 +694,13 @@ __global__ void __launch_bounds__(256) twoterm_gather_kernel(const __nv_bfloat16
 // kM: M tiles per item (gate/up: always 2)
 // kQ: quantised activations (moe_expert_ffn_q), one E2M1 term per value: dense 4-bit operands (kind::mxf4, K = 64), K steps of
 // 256, two scale words per row and step; every pass is of the separate form with one operand
-template <bool STAGE1, int kM, bool kQ>
+// kGuard (gate/up): blocks that the terms hold too little of are looked for
+template <bool STAGE1, int kM, bool kQ, bool kGuard>
 __global__ void __launch_bounds__(kTtThreads, 1)
 ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_sc,
                    const __grid_constant__ TtTokMaps tmap_t, const TtArgs a) {
   static_assert(!STAGE1 || kM == 2, "gate and up");
+  static_assert(!kGuard || (STAGE1 && !kQ), "gate/up on two terms");
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
   const TtSmem sm = tt_smem(a.E, kM, a.stages, a.t_bytes);
@@ -987,8 +1005,7 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     int tog = 0, g_known = -1;
     TtPass p = {};
     uint32_t acc_ph[2] = {0u, 0u};
-    const bool guard = STAGE1 && !kQ && a.flags != nullptr;
-    if (guard) {
+    if constexpr (kGuard) {
       // the split kernel's marks -> flags of their experts, 16 at a time, while the first MMAs run
       pdl_wait();  // the marks are complete and the flags zero
       const size_t n_marks = (static_cast<size_t>(a.S) * a.parts + 15) / 16;
@@ -1116,12 +1133,14 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
           const int kstep = rt * 2 + rank;
           const int i0 = kstep * 128 + q * 32 + 4 * (lane >> 2);
           uint8_t* sf = a.sfa + (static_cast<size_t>(g) * (a.I / kTtK) + kstep) * a.sf_step;
-          bool again = false;  // a block of this item that the terms hold too little of
+          bool again = false;  // (kGuard) a block of this item that the terms hold too little of
   #pragma unroll
           for (int ch = 0; ch < kChunks; ++ch) {
             const int c0 = ch * 32 + sub * 8;
             if (c0 < p.n) {
               uint32_t my_sb = 0u;
+              int lossy = 0;           // most inexact values in one of the eight blocks
+              bool not_finite = false;
   #pragma unroll
               for (int jj = 0; jj < 8; jj += 4) {
                 float v[4], inv[4];
@@ -1135,13 +1154,7 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
                   v[t] = __uint_as_float(vb);
                   inv[t] = tt_inv(sb);
                   bad |= amax >= 0x7F800000u;
-                  if (guard) {
-                    const uint32_t abs_v = vb & 0x7FFFFFFFu;
-                    bool found = __popc(__ballot_sync(0xffffffffu, abs_v - 1u < tt_lossy_below(amax) - 1u)) >= kTtLossyInter;
-                    if (found)  // (its maximum is above 2^-111 then)
-                      found = __popc(__ballot_sync(0xffffffffu, abs_v >= (amax & 0x7F800000u) - (10u << 23))) <= kTtLarge;
-                    again |= (found || amax >= 0x7F800000u) && c0 + jj + t < p.n;
-                  }
+                  if (kGuard) lossy = max(lossy, __popc(__ballot_sync(0xffffffffu, (vb & 0x7FFFFFFFu) - 1u < tt_lossy_below(amax) - 1u)));
                   if (lane == jj + t) my_sb = sb;
                 }
                 uint32_t hw, lw, h1, l1;
@@ -1150,6 +1163,7 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
                 hw |= h1 << 16;
                 lw |= l1 << 16;
                 if (bad) hw = tt_nan_codes(hw, v[0], v[1], v[2], v[3]);
+                not_finite |= bad;
                 hw = transpose_4x4(hw, lane);
                 lw = transpose_4x4(lw, lane);
                 const int tok = c0 + jj + (lane & 3);
@@ -1164,9 +1178,10 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
                 sf[tt_sf_byte(r, q)] = static_cast<uint8_t>(my_sb);
                 sf[p.stacked ? tt_sf_byte(p.nr + r, q) : 1024 + tt_sf_byte(r, q)] = static_cast<uint8_t>(my_sb - 5u);
               }
+              if (kGuard && (lossy >= kTtLossyInter || not_finite)) again |= tt_again(pk[ch], p.n - c0);
             }
           }
-          if (again && lane == 0) {
+          if (kGuard && again && lane == 0) {
             a.flags[e] = 1;
             a.flags[a.E] = 1;
           }
@@ -1225,13 +1240,13 @@ bool twoterm_weights_ok(const void* w13, const void* w2) {  // the 4-bit tensor 
 
 namespace {
 
-template <bool STAGE1, int kM, bool kQ>
+template <bool STAGE1, int kM, bool kQ, bool kGuard = false>
 bool tt_launch(const CUtensorMap& tm_w, const CUtensorMap& tm_sc, const TtTokMaps& tm_t, TtArgs a, cudaStream_t st) {
   a.stages = 1;
   while (a.stages < kTtMaxStages && tt_smem(a.E, kM, a.stages + 1, a.t_bytes).total + 1024 <= 227 * 1024) ++a.stages;
   static PerDeviceFlag flag;
   if (!once_per_device(flag, [] {
-        return cudaFuncSetAttribute(ffn_twoterm_kernel<STAGE1, kM, kQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
+        return cudaFuncSetAttribute(ffn_twoterm_kernel<STAGE1, kM, kQ, kGuard>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
       }))
     return false;
   cudaLaunchConfig_t cfg = {};
@@ -1248,7 +1263,7 @@ bool tt_launch(const CUtensorMap& tm_w, const CUtensorMap& tm_sc, const TtTokMap
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, ffn_twoterm_kernel<STAGE1, kM, kQ>, tm_w, tm_sc, tm_t, a) == cudaSuccess;
+  return cudaLaunchKernelEx(&cfg, ffn_twoterm_kernel<STAGE1, kM, kQ, kGuard>, tm_w, tm_sc, tm_t, a) == cudaSuccess;
 }
 
 }  // namespace
@@ -1340,7 +1355,8 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
   a.sc = w.s13;
   a.K = sh.H;
   a.R = 2 * sh.I;
-  if (!tt_launch<true, 2, false>(tm_w13, tm_s13, tm_x, a, st)) return MOE_ERR_CUDA;
+  if (!(guard ? tt_launch<true, 2, false, true>(tm_w13, tm_s13, tm_x, a, st) : tt_launch<true, 2, false>(tm_w13, tm_s13, tm_x, a, st)))
+    return MOE_ERR_CUDA;
   a.sc = w.s2;
   a.K = sh.I;
   a.R = sh.H;
