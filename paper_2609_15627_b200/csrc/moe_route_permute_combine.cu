@@ -147,10 +147,13 @@ MOE_DEVINL void warp_copy_row(const __nv_bfloat16* src, __nv_bfloat16* dst, int 
   }
 }
 
-// Up to kPermuteDirect slots: a CTA takes eight consecutive slots, counts the earlier slots of each one's expert directly
+// Up to permute_direct slots: a CTA takes eight consecutive slots, counts the earlier slots of each one's expert directly
 // (an id is loaded once per CTA and compared with the eight experts) and copies their rows, one warp each; the sort is
-// stable by construction.  One launch where the chunked sort takes four.
-constexpr int kPermuteDirect = 16384;
+// stable by construction.  One launch where the chunked sort takes three, and a fourth for the rows.
+// The count is quadratic and the launches are not: the line lies where the two meet (256 experts, direct / chunked).  Short
+// rows or none to copy: 4096 slots 10 us and 15, 8192 13 and 17, 12288 21 and 17, 16384 29 and 19; with long ones beside
+// the count later (H = 4096): 8192 slots 21 and 31, 12288 29 and 36, 16384 37 and 42, 24576 59 and 56.
+constexpr int permute_direct(bool rows, int H) { return rows && H >= 2048 ? 16384 : 8192; }
 __global__ void __launch_bounds__(256, 8) permute_small_kernel(const __nv_bfloat16* __restrict__ x,
                                                             const int* __restrict__ ids,
                                                             const int* __restrict__ offsets, int S, int H, int k,
@@ -302,7 +305,7 @@ int launch_permute(const __nv_bfloat16* x, const int* ids, const int* offsets, c
                    __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st, const int* range_lo,
                    const int* range_hi) {
   const int S = sh.T * sh.k;
-  if (S <= kPermuteDirect) {
+  if (S <= permute_direct(x_perm != nullptr, sh.H)) {
     if (launch_pdl(permute_small_kernel, dim3((S + 7) / 8), dim3(256), 0, st, x, ids, offsets, S, sh.H, sh.k, x_perm, perm,
                    inv_perm, range_lo, range_hi) != cudaSuccess)
       return MOE_ERR_CUDA;
