@@ -82,9 +82,10 @@ __global__ void __launch_bounds__(kGemvWarps * 32) router_gemv_kernel(const __nv
 constexpr int kRM = 128, kRK = 64;  // K per stage: one 128-byte row of bf16
 constexpr int kRStages = 8;
 constexpr int kRABytes = kRM * kRK * 2;
-// Experts per CTA.  What a CTA pays is the chain of K stages, so few tokens are spread over many CTAs of 16 experts (48
-// tokens, 256 experts, H = 4096: @R@); with tokens enough for a CTA per SM, 64 experts read the tokens a quarter as often.  The
-// order of a logit's sum is the same in both.
+// Experts per CTA.  What a CTA pays is the chain of K stages, a little less of it with 16 experts than with 64 (256 experts, up
+// to 512 tokens: 18.4-19.5 us and 18.4-19.6 at H = 4096, 26.6-27.5 and 26.7-28.7 at H = 7168); with tokens enough for
+// a CTA per SM, 64 read the tokens a quarter as often (2048 tokens: 20.5 us and 31.7).  The order of a logit's sum is the
+// same in both.
 constexpr int router_cols(int T) { return T <= 1024 ? 16 : 64; }
 constexpr int kRThreads = 6 * 32;
 
