@@ -117,8 +117,10 @@ int moe_permute(const void* x_bf16, const int32_t* topk_ids, const int32_t* expe
  * The summation order inside a dot product is the kernel's; everything else is as written.
  *   status_word: device int32, may be NULL; see the common rules.
  * Four kernel variants, chosen by the shape and the weights' alignment (moe_last_kernel_name names the one that ran):
- * for batches that fill the chip (T*k >= 1024, at least 4 rows per expert on average, at least 128 (pass of tokens, tile
- * of weight rows) items; H and I multiples of 256, w13 and w2 32-byte aligned) the packed weights feed the block-scaled
+ * for batches that fill the chip (T*k >= 1024, at least 4 rows per expert on average - more than 6 where H >= 4096 and
+ * I >= 1024 and the second kernel takes the shape -, at least 128 items of (pass of tokens, tile of weight rows), but for
+ * layers of small experts with more than 112 rows each), or for more than 32 rows per expert of large ones (H >= 4096, I >=
+ * 2048); H and I multiples of 256, w13 and w2 32-byte aligned: the packed weights feed the block-scaled
  * 8-bit tensor-core instruction and each bf16 activation is two E4M3 terms with scales per 32 elements (exact for elements
  * within 2^-14 of their block's largest magnitude, off by at most 2^-22 of it otherwise).  Where the shape would otherwise go
  * to one of the last two, which take every bf16 value as it is, experts are done again by that one (same name reported) if they
@@ -175,7 +177,7 @@ int moe_validate_scales(const uint8_t* scales, size_t n_bytes, int32_t* bad_coun
  *     with nothing packed - if there is one.  Because of that read-back this call, unlike the others, WAITS for the
  *     stream and cannot be captured into a CUDA graph.  The caller may free the four tensors afterwards.
  *   - moe_expert_ffn_packed: moe_expert_ffn with `packed` in place of the four weight arguments; same arithmetic, same
- *     result bit for bit.  Kernel choice as moe_expert_ffn, except that shapes with the tiled layout that would fall to
+ *     result bit for bit (as with w13 and w2 aligned to 32 bytes).  Kernel choice as moe_expert_ffn, except that shapes with the tiled layout that would fall to
  *     the row-streaming fallback kernel (neither decode-sized nor prefill-sized) run the grouped-GEMM kernel.
  */
 size_t moe_prepack_bytes(const moe_shape_t* shape);

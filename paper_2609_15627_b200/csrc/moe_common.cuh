@@ -102,9 +102,13 @@ inline bool twoterm_batch_ok(const moe_shape_t& s) {
   const long long groups = S / 224 > s.E ? S / 224 : (S < s.E ? S : s.E);
   const int tiles = s.I / 128 < s.H / 256 ? s.I / 128 : s.H / 256;
   if (!twoterm_shape_ok(s)) return false;
+  // at least 128 items of (pass, 128 values of i or 256 output columns), that is 64 gate/up items of 256 i for the 74 CTA
+  // pairs.  Where the layer is small as well the launches decide, and the kernels meet (this call / bf16 kernel, L2 cold: 64
+  // experts of 512 x 512, 33 rows each 42 us and 42, 64 rows 45 and 48, 96 rows 51 and 50; 128 of them, 64 rows 66 and 81).
   if (S >= 1024 && S >= 4LL * s.E && groups * tiles >= 128) return true;
-  // few large experts (a block's shared expert: 48 rows of one expert of 4096 x 2048 take @S@ us, 71 on the streaming kernel
-  // that was left for more than 32 rows per expert)
+  // few large experts (a block's shared expert), whatever the number of items: one expert of 4096 x 2048, this call / the kernel
+  // that takes it otherwise: 48 rows 51 us and 73 (streaming), 192 rows 84 and 241, 1024 rows 90 and 110 (bf16), 2048 rows 111
+  // and 114, 3000 rows 154 and 202.
   return S > 32LL * s.E && tiles >= 16;
 }
 

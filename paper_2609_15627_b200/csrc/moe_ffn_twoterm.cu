@@ -1269,6 +1269,21 @@ bool tt_launch(const CUtensorMap& tm_w, const CUtensorMap& tm_sc, const TtTokMap
 }  // namespace
 
 bool twoterm_chosen(const moe_shape_t& choice, const ExpertWeights& w) {
+  const long long S = static_cast<long long>(choice.T) * choice.k;
+  // Few rows per expert of large ones: this kernel loses more than the eight-term one where the weights' rows lie 2 KB apart,
+  // and both read moe_prepack's tiles alike (256 experts of 4096 x 2048, 4 / 5 / 6 / 7 / 8 rows, eight terms and two: rows of
+  // weights 595 us and 632, 611 and 636, 618 and 640, 636 and 649, 884 and 646; the whole call on tiles 568 and 567, 577 and
+  // 577, 598 and 580; with rows of 2048 elements two terms are ahead from 4 on, 374 us and 321).  One line for both layouts,
+  // so that they give the same bits.
+  if (choice.H >= 4096 && choice.I >= 1024 && S <= 6LL * choice.E && native_shape_ok(choice, w.w13, w.w2)) return false;
+  // A layer of small experts is done in a few rounds of either kernel, and the launches that look for experts to be done again
+  // decide (L2 cold, this call / bf16 kernel: 64 experts of 512 x 512, 128 rows 59 us and 56, 200 rows 74 and 65; 32 of 1024 x
+  // 512, 128 rows 57 and 50; with fewer rows or more experts the other way: 64 of 512 x 512, 64 rows 45 and 48, 128 of them,
+  // 128 rows 79 and 97).
+  const long long expert = static_cast<long long>(choice.H) * choice.I;
+  if (umma_shape_ok(choice) && !native_shape_ok(choice, w.w13, w.w2) && S > 112LL * choice.E && expert <= (1 << 19) &&
+      expert * choice.E < (1 << 25))
+    return false;
   return twoterm_batch_ok(choice) && twoterm_weights_ok(w.w13, w.w2) &&
          (native_shape_ok(choice, w.w13, w.w2) || umma_shape_ok(choice) || w.blocked || stream_shape_ok(choice));
 }

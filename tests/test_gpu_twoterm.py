@@ -321,3 +321,54 @@ def test_weights_aligned_to_16_bytes_take_the_other_kernels(T, I, kernel):
         torch.cuda.synchronize()
         assert int(buf.status.item()) == 0 and moe.moe_last_kernel_name() == name
         check_y(buf.y_perm.cpu().numpy(), want, name)
+
+
+@pytest.mark.parametrize("T,H,I,E,name,other", [
+    (768, 4096, 1024, 256, "ffn_native_mxf4_block_scaled", moe.VARIANT_TWOTERM),   # 6 rows per expert
+    (769, 4096, 1024, 256, NAME, moe.VARIANT_NATIVE),
+    (1792, 1024, 512, 32, NAME, moe.VARIANT_UMMA),                                  # 112
+    (1793, 1024, 512, 32, _UMMA, moe.VARIANT_TWOTERM)])
+def test_lines_of_the_choice(T, H, I, E, name, other):
+    k = 2
+    g = torch.Generator(device="cuda").manual_seed(71)
+    w = [torch.randint(lo, hi, (E, rows, cols), dtype=torch.uint8, device="cuda", generator=g)
+         for lo, hi, rows, cols in ((0, 256, 2 * I, H // 2), (119, 123, 2 * I, H // 32), (0, 256, H, I // 2), (119, 123, H, I // 32))]
+    sh = moe.shape(T, H, I, E, k)
+    buf = moe.LayerBuffers(sh)
+    moe.moe_route(dev(inputs.make_logits(T, E, 72)), k, buf.topk_ids, buf.topk_w, buf.expert_offsets, buf.ws)
+    moe.moe_permute(dev(inputs.make_x(T, H, 73)), buf.topk_ids, buf.expert_offsets, sh, buf.x_perm, buf.perm, buf.inv_perm, buf.ws)
+    moe.moe_expert_ffn(buf.x_perm, buf.expert_offsets, *w, sh, buf.y_perm, buf.status, buf.ws)
+    assert moe.moe_last_kernel_name() == name
+    got = buf.y_perm.clone()
+    packed = moe.moe_prepack(*w, sh)
+    buf.y_perm.fill_(float("nan"))
+    moe.moe_expert_ffn_packed(buf.x_perm, buf.expert_offsets, packed, sh, buf.y_perm, buf.status, buf.ws)
+    torch.cuda.synchronize()
+    assert moe.moe_last_kernel_name() == name and torch.equal(buf.y_perm, got)     # the same choice, the same bits
+    ws = torch.empty(buf.ws.numel() + 9 * T * k * (H + I), dtype=torch.uint8, device="cuda")
+    moe.moe_debug_expert_ffn_variant(buf.x_perm, buf.expert_offsets, *w, sh, buf.y_perm, buf.status, ws, other)
+    torch.cuda.synchronize()
+    want = buf.y_perm.double()
+    diff = got.double() - want                       # the tolerance of the fp32 per-slot rows
+    assert int(buf.status.item()) == 0
+    assert float(diff.norm() / want.norm()) <= 5e-4 and float(diff.abs().max()) <= 2e-2 * float(want.pow(2).mean().sqrt())
+
+
+@pytest.mark.parametrize("S,H", [(8192, 1024), (8200, 1024), (8200, 2048), (16384, 2048), (16392, 2048)])
+def test_sort_at_the_lines_between_its_forms(S, H):
+    """The direct count and the chunked sort give the one stable order, rows copied along (the whole layer sorts without
+    them: the line for short rows)."""
+    k, E = 8, 40
+    T = S // k
+    logits, x = inputs.make_logits(T, E, 81), inputs.make_x(T, H, 82)
+    sh = moe.shape(T, H, 256, E, k)
+    buf = moe.LayerBuffers(sh)
+    moe.moe_route(dev(logits), k, buf.topk_ids, buf.topk_w, buf.expert_offsets, buf.ws)
+    moe.moe_permute(dev(x), buf.topk_ids, buf.expert_offsets, sh, buf.x_perm, buf.perm, buf.inv_perm, buf.ws)
+    torch.cuda.synchronize()
+    direct = S <= (16384 if H >= 2048 else 8192)
+    assert moe.moe_last_kernel_name() == ("permute_rank_by_count" if direct else "permute_chunked_scan")
+    ids, off = buf.topk_ids.cpu().numpy(), buf.expert_offsets.cpu().numpy()
+    x_perm, perm, inv = O.permute(x, ids, off)
+    assert np.array_equal(buf.perm.cpu().numpy(), perm) and np.array_equal(buf.inv_perm.cpu().numpy().reshape(-1), inv.reshape(-1))
+    assert np.array_equal(buf.x_perm.view(torch.int16).cpu().numpy().view(np.uint16), x_perm)
