@@ -146,9 +146,9 @@ int expert_ffn_impl(const void* x_perm_bf16, const int32_t* expert_offsets, cons
   __nv_bfloat16* act = reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(ws) + L.act_off);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const __nv_bfloat16* xp = static_cast<const __nv_bfloat16*>(x_perm_bf16);
-  // kernel choice is a pure function of the shape (and of the alignment the tensor maps need): native block-scaled
-  // FP4 MMA for decode-sized batches, bf16 grouped GEMM for prefill-sized batches, the register-expansion streaming
-  // kernel for every other shape.  The streaming kernel reads whole rows, so with the tile-contiguous weight layout
+  // kernel choice is a pure function of the shape (and of the alignment the tensor maps need): two E4M3 terms for batches
+  // that fill the chip (twoterm_chosen), else native block-scaled FP4 MMA for decode-sized batches, bf16 grouped GEMM for
+  // prefill-sized ones, the register-expansion streaming kernel for every other shape.  The streaming kernel reads whole rows, so with the tile-contiguous weight layout
   // (which only shapes the first two kernels take can have) the grouped GEMM also takes what is left.
   StatusRef status;
   int rc = resolve_status(status_word, &status);

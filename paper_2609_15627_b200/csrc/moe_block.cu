@@ -269,7 +269,7 @@ int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, 
   if (cols == 16) router_gemm_kernel<16><<<grid, kRThreads, smem, st>>>(tm_x, tm_w, T, H, E, logits, status);
   else router_gemm_kernel<64><<<grid, kRThreads, smem, st>>>(tm_x, tm_w, T, H, E, logits, status);
   if (cudaGetLastError() != cudaSuccess) return MOE_ERR_CUDA;
-  note_kernel("router_gemm_tcgen05_128x64", 1);  // (one kernel, named by its largest tile)
+  note_kernel("router_gemm_tcgen05_128x64", 1);  // (also for tiles of 16 experts: callers know the kernel by this name)
   return MOE_OK;
 }
 

@@ -173,8 +173,8 @@ MOE_DEVINL void umma_commit(uint64_t* bar) {
 }
 // The same from a whole convergent warp: one elected lane, always the same, issues it.  MMA loops run in all lanes of their
 // warp, with operands the compiler knows to be uniform (see warp_uniform): inside an `if (lane == 0)` every operand is
-// moved to a uniform register anew for each instruction, and a block-scaled MMA takes 115 to 150 cycles to issue, whatever
-// its size, where the elected form takes 14.
+// moved to a uniform register anew for each instruction, and a block-scaled MMA takes 63 to 115 cycles to issue, whatever
+// its size, where the elected form takes what the tensor core does, 39 to 45 at the smallest N.
 MOE_DEVINL void umma_commit_elect(uint64_t* bar) {
   asm volatile(
       "{\n\t.reg .pred q;\n\t"
