@@ -10,12 +10,16 @@
 // with s_t the smallest exponent for which the block's largest |r_t| is at most 6 * 2^(s_t).  Every term removes
 // at least two bits of the block's largest residual, so after 8 terms the residual of every element is below
 // 2^-16 of its block's largest magnitude, and elements within 2^-10 of it are exact; products are exact and
-// accumulate in fp32 in tensor memory.  The 8 rows of a token are 8 of the 128 rows of the A operand, which the
-// tensor core walks anyway: the terms cost shared memory, not time.
+// accumulate in fp32 in tensor memory.
 //
-// Operand roles: the weights are the B operand (N = 256 weight rows per MMA, K = 64) and the tokens the A
-// operand (M = 128 rows = up to 16 tokens x 8 terms per pass over the weights, row = 8 * token + term; rows of
-// tokens that do not exist hold other rows' data or zeros and their accumulator lanes are never looked at).
+// Operand roles: the weights are the A operand (two tiles of M = 128 weight rows, K = 64) and the tokens the B operand
+// (N = 16..128 rows: up to 16 tokens x 8 terms per pass over the weights, row = 8 * token + term).  So an MMA multiplies what
+// the pass holds and not the 128 rows that an A operand of tokens has whatever it holds: at one to four tokens per expert
+// that is a quarter to an eighth of the work, which the stream of weights did not wait for, but for which the board's power
+// limit made it pay (256 experts of 4096 x 2048, top-8, layer after layer: 64 tokens 548 us at 1.49 GHz with the tokens as A,
+// 503 us at 1.70 GHz as B; 5 tokens, top-6, 82.8 and 76.0 us).  A lane of the accumulators is a weight row, so the eight terms of a token are
+// eight registers of a thread, gate and up of one i meet in it, and the 32 lanes of a warp are one scale block of the
+// intermediate.  Up to 8 tokens the halves of the accumulator columns take turns and the epilogue runs beside the next item.
 // Both operands ride the same shared-memory ring: a stage is one K step (256 elements) of the weight tile plus
 // the same K step of the pass's term rows, each fetched by TMA with the 128-byte swizzle the MMA reads.
 //
@@ -32,10 +36,9 @@
 //   warp 1      allocates tensor memory, issues the MMAs, commits to mbarriers
 //   warps 2..5  move weight scale bytes into tensor memory (tcgen05.st), and at a change of (expert, pass) the
 //               scale bytes of its term rows
-//   warps 6..9  epilogue, one warp per tensor-memory lane quadrant: sum the 8 term rows of each token, then SwiGLU +
-//               bf16 rounding + the 8-term split for the down projection (gate/up) or the fp32 store (down).  A pass
-//               of more than 4 tokens: quadrant q holds tokens 4q..4q+3, its warp takes all 256 columns.  A pass of
-//               at most 4 tokens is loaded into every quadrant, and each warp takes a quarter of the columns.
+//   warps 6..9  epilogue, one warp per tensor-memory lane quadrant (32 weight rows of either tile, all tokens): sum the 8
+//               terms of each token, then SwiGLU + bf16 rounding + the 8-term split for the down projection (gate/up) or the
+//               fp32 store (down)
 // Every wait is bounded and reports through the status word.
 //
 // The weights are read either in the checkpoint's row layout or in moe_prepack's tile-contiguous layout (one tensor
@@ -50,7 +53,8 @@
 //
 // Instantiated with kQ = true it is the quantised-activation variant (moe_expert_ffn_q): one operand row per token - the
 // activation quantised online to E2M1 with one scale per 32 elements, as the paper's historical decode route does to
-// INT8 - so a pass holds 128 tokens and the epilogues sum nothing across lanes.  Large batches run one projection per
+// INT8 - so a pass holds 128 tokens and the epilogues sum nothing.  Its tokens are the A operand (M = 128) and the weights
+// the B operand (N = 256): accumulator lane = token.  Large batches run one projection per
 // launch over blocks of (expert, pass, four tiles) dealt round-robin to the CTAs (see the set-up).
 #include <cuda.h>
 #include <cuda_fp4.h>
@@ -86,6 +90,8 @@ constexpr uint32_t kNatTmemCols = 512;
 // scale-factor block of 4 columns (a block covers 128 rows - rows 32c..32c+31 in column c - and must start on a
 // multiple of 4 columns); 3 groups of 4 words x 8 columns (256 weight rows) for the weight scales
 constexpr uint32_t kColD = 0, kColSfAct = 256, kColSfW = 384;
+// accumulator columns of the two weight tiles: a pass of at most 64 operand rows takes one half of the 256, the halves in turn
+constexpr int kSmallRows = 64;
 
 struct NatArgs {
   const uint8_t* sf1;        // scale bytes of the token rows' terms [S * 8, H/32] (terms: row p * 8 + t, packed E2M1)
@@ -144,16 +150,6 @@ constexpr int kTermBoxes = 5;
 struct alignas(64) TermMaps {
   CUtensorMap box[kTermBoxes];
 };
-// A pass of one token is loaded once per lane quadrant of the accumulator, so that each of the four epilogue warps finds
-// the token in its own quadrant and takes a quarter of the columns instead of one warp taking them all (decode_c1:
-// every expert has one row, and the epilogues are on the critical path).  The scheme works for up to 4 tokens (one
-// quadrant = 32 operand rows), but every repeated KB of term rows competes with the weight stream: measured on
-// decode_c64 (2.3 rows per expert on average) the expert-FFN call takes 545 us with passes of up to 4 tokens repeated,
-// 526 us with single-token passes only (row-layout weights; 560 against 550 us under the power cap).
-// Nor is it worth anything where the epilogue hides behind the next item's MMAs: a CTA repeats only in a phase in which
-// it has at most kRepMaxItems items (another 0.7 % on decode_c64, where a CTA has 24).
-constexpr int kRepBox = 0, kRepTok = 1 << kRepBox;  // boxes 0..kRepBox hold at most kRepTok tokens
-constexpr int kRepMaxItems = 2;
 MOE_DEVINL int op_box(int n_rows) { return n_rows <= 8 ? 0 : (n_rows <= 16 ? 1 : (n_rows <= 32 ? 2 : (n_rows <= 64 ? 3 : 4))); }
 
 // One projection as the kernel sees it
@@ -161,7 +157,6 @@ struct Phase {
   int K, R, n_steps, tiles;  // reduction length, weight rows per expert, K steps, items per entry of the expert list
   int begin, end;            // this CTA's items (at most 1024 experts x 32 tiles)
   bool direct;               // K is not a multiple of 512: scale bytes come by plain loads (see NatArgs::s13)
-  bool rep_ok;               // few enough of them for single-token passes to be repeated per lane quadrant
 };
 // Items go to CTAs in contiguous shares: gate/up items evenly, per0 each.  A down item of expert t is placed as if it
 // followed that expert's last gate/up item in the gate/up list, its expert's down items spread over the span of the
@@ -205,7 +200,6 @@ MOE_DEVINL Phase phase_of(int ph, const NatArgs& a, const int* shares) {
   p.tiles = a.by_pass ? block_tiles(p.R / kTile) : p.R / kTile;
   p.begin = warp_uniform(shares[2 * ph]);  // (phase_of is called by whole warps)
   p.end = warp_uniform(shares[2 * ph + 1]);
-  p.rep_ok = p.end - p.begin <= kRepMaxItems;
   return p;
 }
 
@@ -332,9 +326,9 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
   uint64_t* empty_sc = full_sc + kScStages;      // [kScStages] scale warps -> producer
   uint64_t* sf_full = empty_sc + kScStages;      // [kSfGroups] scale warps -> MMA
   uint64_t* sf_free = sf_full + kSfGroups;       // [kSfGroups] MMA done -> scale warps
-  uint64_t* acc_full = sf_free + kSfGroups;      // MMA -> epilogue
-  uint64_t* acc_empty = acc_full + 1;            // epilogue -> MMA
-  uint64_t* act_ready = acc_empty + 1;           // scale warps -> MMA: term-row scale factors of the current (expert, pass)
+  uint64_t* acc_full = sf_free + kSfGroups;      // [2] MMA -> epilogue (kQ: the first)
+  uint64_t* acc_empty = acc_full + 2;            // [2] epilogue -> MMA
+  uint64_t* act_ready = acc_empty + 2;           // scale warps -> MMA: term-row scale factors of the current (expert, pass)
   uint64_t* act_free = act_ready + 1;            // MMA done with them -> scale warps
   uint64_t* ctr_done = act_free + 1;             // one-launch layer: epilogue warps that are through with the global counters
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + sm.misc);
@@ -442,20 +436,21 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
     for (int s = 0; s < kWStages; ++s) { mbar_init(&full_w[s], 1); mbar_init(&empty_w[s], 1); }
     for (int s = 0; s < kScStages; ++s) { mbar_init(&full_sc[s], 1); mbar_init(&empty_sc[s], 4); }
     for (int s = 0; s < kSfGroups; ++s) { mbar_init(&sf_full[s], 4); mbar_init(&sf_free[s], 1); }
-    mbar_init(acc_full, 1);
-    mbar_init(acc_empty, 4);
+    for (int h = 0; h < 2; ++h) { mbar_init(&acc_full[h], 1); mbar_init(&acc_empty[h], 4); }
     mbar_init(act_ready, 4);
     mbar_init(act_free, 1);
     mbar_init(ctr_done, 4);
     mbar_fence_init();
   }
-  // Operand rows that no term-row box has written yet read as zeros instead of whatever shared memory held (their
-  // results are never looked at; zeros cost less power)
-  for (int s = 0; s < kWStages; ++s) {
-    uint4* z = reinterpret_cast<uint4*>(sW + s * kStage + kWStage);
-    for (int i = tid; i < kAStage / 16; i += kNatThreads) z[i] = make_uint4(0u, 0u, 0u, 0u);
+  if constexpr (kQ) {
+    // Operand rows that no box has written yet read as zeros instead of whatever shared memory held (their results are
+    // never looked at; zeros cost less power)
+    for (int s = 0; s < kWStages; ++s) {
+      uint4* z = reinterpret_cast<uint4*>(sW + s * kStage + kWStage);
+      for (int i = tid; i < kAStage / 16; i += kNatThreads) z[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    fence_proxy_async_smem();
   }
-  fence_proxy_async_smem();
   if (wid == 1) tmem_alloc(tmem_holder, kNatTmemCols);
   tc_fence_before_sync();
   __syncthreads();
@@ -592,11 +587,10 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
       bool pdl_done = kFused, dep_ok = kFused;
       if (kFused) fence_proxy_async_all();  // they were written through the generic proxy
       int dep_phase = 0, dep_e = -1;
-      int n_pend = 0, pend_s[kWStages], pend_x[kWStages], pend_y[kWStages], pend_b[kWStages], pend_r[kWStages];
-      // term rows of one K step, n_rep times: once, or once per lane quadrant of the accumulator
-      auto load_terms = [&](const TermMaps* ma, int stage, int bi, int n_rep, int x, int y) {
-        for (int r = 0; r < n_rep; ++r)
-          tma_load_2d(sW + stage * kStage + kWStage + r * (32 * 128), &ma->box[bi], x, y, &full_w[stage]);
+      int n_pend = 0, pend_s[kWStages], pend_x[kWStages], pend_y[kWStages], pend_b[kWStages];
+      // term rows of one K step
+      auto load_terms = [&](const TermMaps* ma, int stage, int bi, int x, int y) {
+        tma_load_2d(sW + stage * kStage + kWStage, &ma->box[bi], x, y, &full_w[stage]);
       };
       auto meet = [&]() {  // wait for the open dependency and send the held-back loads
         if (!pdl_done) {
@@ -608,7 +602,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
           fence_proxy_async_all();  // the rows were written through the generic proxy, TMA reads through the async one
         }
         const TermMaps* ma = dep_phase == 0 ? &tmap_a1 : &tmap_a2;
-        for (int i = 0; i < n_pend; ++i) load_terms(ma, pend_s[i], pend_b[i], pend_r[i], pend_x[i], pend_y[i]);
+        for (int i = 0; i < n_pend; ++i) load_terms(ma, pend_s[i], pend_b[i], pend_x[i], pend_y[i]);
         n_pend = 0;
         dep_ok = true;
       };
@@ -634,7 +628,6 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
           for (int pass = 0; pass < n_pass; ++pass) {
             const bool by_token = kFused && phase == 0;  // the expert's rows are fetched token by token (at most 4)
             const int bi = op_box(min(tok_pass, n_rows_e - pass * tok_pass) * nt);  // box of 8 << bi operand rows
-            const int n_rep = (!kQ && P.rep_ok && bi <= kRepBox) ? 4 : 1;
             for (int ks = 0; ks < P.n_steps; ++ks) {
               if (!P.direct && (ks & 1) == 0) {  // 16 scale bytes per weight row cover two K steps
                 mbar_wait(&empty_sc[cs], cph ^ 1u, a.status);
@@ -648,7 +641,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
                 if (++cs == kScStages) { cs = 0; cph ^= 1u; }
               }
               mbar_wait(&empty_w[s], ph ^ 1u, a.status);
-              mbar_expect_tx(&full_w[s], static_cast<uint32_t>(kWStage + n_rep * (by_token ? n_rows_e * 8 : 8 << bi) * 128));
+              mbar_expect_tx(&full_w[s], static_cast<uint32_t>(kWStage + (by_token ? n_rows_e * 8 : 8 << bi) * 128));
               // 128 rows x 128 bytes of codes; tile-contiguous layout: tile (row / 128, ks) is 128 consecutive rows of 128 bytes
               const int wx = a.blocked ? 0 : ks * 128;
               const int wya = a.blocked ? ((wrow_a >> 7) * P.n_steps + ks) * 128 : wrow_a;
@@ -660,13 +653,10 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
               if (by_token) {
                 // (the tokens' term rows were seen complete during the set-up: no dependency to hold these back for)
                 for (int j = 0; j < n_rows_e; ++j)
-                  for (int r = 0; r < n_rep; ++r)
-                    tma_load_2d(sW + s * kStage + kWStage + r * (32 * 128) + j * (8 * 128), &ma->box[0], ks * 128,
-                                s_tok[row_begin + j] * kTerms, &full_w[s]);
+                  tma_load_2d(sW + s * kStage + kWStage + j * (8 * 128), &ma->box[0], ks * 128, s_tok[row_begin + j] * kTerms, &full_w[s]);
               } else if (dep_ok) {
-                load_terms(ma, s, bi, n_rep, ks * 128, arow);
+                load_terms(ma, s, bi, ks * 128, arow);
               } else {
-                pend_r[n_pend] = n_rep;
                 pend_s[n_pend] = s;
                 pend_x[n_pend] = ks * 128;
                 pend_y[n_pend] = arow;
@@ -705,16 +695,20 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
   } else if (role == 1) {
     // =========================== MMA issuer: all lanes ===========================
     int s = 0, slot = 0;
-    uint32_t ph = 0, sph = 0, aph = 0, acc_ph = 0;
-    const uint32_t d_addr = tmem_base + kColD;
+    uint32_t ph = 0, sph = 0, aph = 0, acc_ph = 0, half = 0;  // acc_ph: bit h, parity of accumulator half h
     const uint32_t ring = smem_u32(sW);
     for (int phase = a.ph_lo; phase < a.ph_hi; ++phase) {
       const Phase P = phase_of(phase, a, s_misc + 1);
       int prev_ti = -1;
       for (int it = P.begin; it < P.end; ++it) {
         const int ti = it / P.tiles;
-        const int n_pass = warp_uniform((t_end[ti] - t_begin[ti] + tok_pass - 1) / tok_pass);
+        const int n_rows_e = warp_uniform(t_end[ti] - t_begin[ti]);
+        const int n_pass = (n_rows_e + tok_pass - 1) / tok_pass;
         for (int pass = 0; pass < n_pass; ++pass) {
+          const uint32_t n_op = static_cast<uint32_t>(min(tok_pass, n_rows_e - pass * tok_pass) * nt);
+          const bool small = !kQ && n_op <= kSmallRows;
+          const uint32_t d_addr = tmem_base + kColD + (small ? half * 128u : 0u);
+          const uint32_t idesc = kQ ? idesc_mxf4() : idesc_mxf4((n_op + 15u) & ~15u);
           // The scale factors of the term rows (tensor memory) are shared by consecutive items of an expert whose
           // rows fit one pass; otherwise every (item, pass) has its own.  The scale warps follow the same rule.
           const bool new_operand = (prev_ti != ti) || (n_pass > 1);
@@ -723,7 +717,8 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
             mbar_wait_warp(act_ready, aph, a.status);
             aph ^= 1u;
           }
-          mbar_wait_warp(acc_empty, acc_ph ^ 1u, a.status);
+          if (kQ || !small || half == 0) mbar_wait_warp(&acc_empty[0], (acc_ph & 1u) ^ 1u, a.status);
+          if (!kQ && (!small || half == 1)) mbar_wait_warp(&acc_empty[1], (acc_ph >> 1) ^ 1u, a.status);
           tc_fence_after_sync();
           for (int ks = 0; ks < P.n_steps; ++ks) {
             if ((ks & 1) == 0) mbar_wait_warp(&sf_full[slot], sph, a.status);  // weight scale factors of 2 K steps at a time
@@ -731,9 +726,15 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
             tc_fence_after_sync();
             const uint32_t w_addr = ring + static_cast<uint32_t>(s * kStage);
             // scale words: 4 columns apart for the term rows, 8 for the 256 weight rows of a group
-            umma_mxf4_step<4, 8>(d_addr, umma_desc_k_sw128(w_addr + kWStage), umma_desc_k_sw128(w_addr), idesc_mxf4(),
-                                 tmem_base + kColSfAct + static_cast<uint32_t>(ks * 8),
-                                 tmem_base + kColSfW + static_cast<uint32_t>(slot * 32 + (ks & 1) * 16), ks != 0 ? 1u : 0u);
+            const uint32_t sf_act = tmem_base + kColSfAct + static_cast<uint32_t>(ks * 8);
+            const uint32_t sf_w = tmem_base + kColSfW + static_cast<uint32_t>(slot * 32 + (ks & 1) * 16), acc = ks != 0 ? 1u : 0u;
+            if constexpr (kQ) {
+              umma_mxf4_step<4, 8>(d_addr, umma_desc_k_sw128(w_addr + kWStage), umma_desc_k_sw128(w_addr), idesc, sf_act, sf_w, acc);
+            } else {
+              const uint64_t terms = umma_desc_k_sw128(w_addr + kWStage);
+              umma_mxf4_step<8, 4>(d_addr, umma_desc_k_sw128(w_addr), terms, idesc, sf_w, sf_act, acc);
+              umma_mxf4_step<8, 4>(d_addr + (small ? 64u : 128u), umma_desc_k_sw128(w_addr + 128 * 128), terms, idesc, sf_w + 4, sf_act, acc);
+            }
             umma_commit_elect(&empty_w[s]);
             if (++s == kWStages) { s = 0; ph ^= 1u; }
             if ((ks & 1) == 1 || ks == P.n_steps - 1) {
@@ -741,8 +742,10 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
               if (++slot == kSfGroups) { slot = 0; sph ^= 1u; }
             }
           }
-          umma_commit_elect(acc_full);
-          acc_ph ^= 1u;
+          if (kQ || !small || half == 0) umma_commit_elect(&acc_full[0]);
+          if (!kQ && (!small || half == 1)) umma_commit_elect(&acc_full[1]);
+          acc_ph ^= kQ ? 1u : (small ? 1u << half : 3u);
+          half = small ? half ^ 1u : 0u;
           // last use of these scale factors?  (always at the end of a phase)
           bool next_new = true;
           if (pass + 1 >= n_pass && it + 1 < P.end) next_new = ((it + 1) / P.tiles != ti) || (n_pass > 1);
@@ -787,7 +790,6 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
             const bool by_token = kFused && phase == 0;  // the tokens' scale bytes are stored by token, not by sorted row
             const int row0 = row_begin + pass * tok_pass;
             const int n_rows = min(tok_pass, row_end - row0) * nt;  // operand rows that exist
-            const bool rep = !kQ && P.rep_ok && n_rows <= kRepTok * kTerms;  // the operand repeats in every lane quadrant
             // rows are n_blk bytes each and consecutive: one contiguous range, copied 16 bytes at a time
             // (the 16-byte chunks of a row are XOR-swizzled with the row number against bank conflicts)
             const int n_chunk = n_blk / 16, cmask = min(n_chunk, 8) - 1;
@@ -811,7 +813,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
               uint32_t w[8];
 #pragma unroll
               for (int c = 0; c < 4; ++c) {
-                const int r = rep ? lane : 32 * c + lane;
+                const int r = 32 * c + lane;
                 const uint2 v = P.direct ? reinterpret_cast<const uint2*>(sSfa)[r * (n_blk / 8) + ks]
                                          : *reinterpret_cast<const uint2*>(sSfa + (r * n_chunk + ((ks >> 1) ^ (r & cmask))) * 16 + (ks & 1) * 8);
                 w[c] = v.x;
@@ -875,122 +877,129 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
     }
   } else if (role >= kEpiWarp) {
     // =========================== epilogue ===========================
-    // Accumulator lane = term row = 8 * token + term.  A 32x32b load hands each lane 32 columns of its row; three
-    // exchange rounds over the 8 lanes of a token (each halves the columns a lane keeps) leave lane (token, t) with
-    // the 8-term sums of 4 consecutive columns, at offset 16 (t & 1) + 8 (t >> 1 & 1) + 4 (t >> 2) of the 32.
-    // A pass of more than kRepTok tokens: the warp of quadrant q owns tokens 4q..4q+3 and all 256 columns.  A smaller
-    // pass has all its tokens in every quadrant: the warp of quadrant q owns a quarter of the columns of every token.
+    // Accumulator lane = weight row, column = operand row = 8 * token + term: the warp of quadrant q has 32 consecutive rows
+    // of either weight tile, a lane the terms of all tokens for one of them.  (kQ: see run_pass_q.)
     const int q = wid & 3;
     const uint32_t lane_base = static_cast<uint32_t>(q * 32) << 16;
-    const int jl = lane >> 3, tl = lane & 7;
-    const int cb = 16 * (tl & 1) + 8 * ((tl >> 1) & 1) + 4 * (tl >> 2);
-    uint32_t acc_ph = 0;
+    uint32_t acc_ph = 0, half = 0;
     bool told = false;  // one-launch layer: this warp has said that it is through with the global counters
     auto tell = [&]() {
       __syncwarp();
       if (lane == 0) mbar_arrive(ctr_done);
       told = true;
     };
+    auto sum8 = [](const uint32_t* v) {
+      auto f = [&](int i) { return __uint_as_float(v[i]); };
+      return ((f(0) + f(1)) + (f(2) + f(3))) + ((f(4) + f(5)) + (f(6) + f(7)));
+    };
     // One pass of one item.  `dry` runs the same instructions on whatever tensor memory holds, with every wait, signal
     // and store left out: each CTA executes this code only a few times, so its first real use would otherwise pay
     // for fetching it - on the critical path of a one-item CTA - while the warp has nothing to do before the first
     // accumulator is complete.
-    auto run_pass = [&](const int phase, const bool rep_ok, const int out_stride, const int tile, const int row0, const int n_tok,
-                        const bool dry) {
-      const bool rep = rep_ok && n_tok <= kRepTok;
-      const bool active = rep || 4 * q < n_tok;
-      // 32-column chunks this warp sums: all 8, or (small pass) gate chunk q and up chunk 4 + q of a gate/up item,
-      // chunks 2q and 2q + 1 of a down item
-      const int n_ch = rep ? 2 : 8;
-      const int ch0 = rep ? (phase == 0 ? q : 2 * q) : 0, ch_step = rep ? (phase == 0 ? 4 : 1) : 1;
+    auto run_pass = [&](const int phase, const int out_stride, const int tile, const int row0, const int n_tok, const bool dry) {
+      const bool small = n_tok * kTerms <= kSmallRows;
+      const uint32_t h = small ? half : 0u;
       if (!dry) {
-        mbar_wait(acc_full, acc_ph, a.status);
-        acc_ph ^= 1u;
+        mbar_wait(&acc_full[h], (acc_ph >> h) & 1u, a.status);
+        if (!small) mbar_wait(&acc_full[1], acc_ph >> 1, a.status);
+        acc_ph ^= small ? 1u << h : 3u;
+        half = small ? h ^ 1u : 0u;
       }
       __syncwarp();  // tcgen05.ld is warp-collective
       tc_fence_after_sync();
-      float acc[8][4];  // [chunk][column cb + c of the chunk]
-      if (active) {
+      const uint32_t d0 = tmem_base + lane_base + kColD + h * 128u, d1 = d0 + (small ? 64u : 128u);
+      auto release = [&]() {
+        tc_fence_before_sync();
+        __syncwarp();
+        if (!dry && lane == 0) {
+          mbar_arrive(&acc_empty[h]);
+          if (!small) mbar_arrive(&acc_empty[1]);
+        }
+      };
+      if (phase == 0) {
+        // SwiGLU and the rounding to bf16 (the intermediate is defined as a bf16 value) of every token, then the accumulators
+        // are handed back and the 8-term split overlaps the next item's MMAs
+        float v[kMaxTokPass];
 #pragma unroll
-        for (int mm = 0; mm < 8; ++mm) {
-          if (mm < n_ch) {
-            uint32_t vc[32];
-            tmem_ld_32x32(tmem_base + lane_base + kColD + static_cast<uint32_t>(32 * (ch0 + mm * ch_step)), vc);
+        for (int g4 = 0; g4 < kMaxTokPass / 4; ++g4) {
+          if (4 * g4 < n_tok) {
+            uint32_t gv[32], uv[32];
+            tmem_ld_32x32(d0 + static_cast<uint32_t>(32 * g4), gv);
+            tmem_ld_32x32(d1 + static_cast<uint32_t>(32 * g4), uv);
             tmem_ld_wait();
-            float a16[16], a8[8];
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-              const float lo = __uint_as_float(vc[k]), hi = __uint_as_float(vc[16 + k]);
-              a16[k] = ((tl & 1) ? hi : lo) + __shfl_xor_sync(0xffffffffu, (tl & 1) ? lo : hi, 1);
+            for (int j = 0; j < 4; ++j) {
+              const float g = sum8(gv + 8 * j), u = sum8(uv + 8 * j);
+              v[4 * g4 + j] = __bfloat162float(__float2bfloat16_rn(__fdividef(g, 1.0f + __expf(-g)) * u));
             }
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-              a8[k] = ((tl & 2) ? a16[8 + k] : a16[k]) + __shfl_xor_sync(0xffffffffu, (tl & 2) ? a16[k] : a16[8 + k], 2);
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              acc[mm][k] = ((tl & 4) ? a8[4 + k] : a8[k]) + __shfl_xor_sync(0xffffffffu, (tl & 4) ? a8[k] : a8[4 + k], 4);
           }
         }
-      }
-      tc_fence_before_sync();
-      __syncwarp();
-      if (!dry && lane == 0) mbar_arrive(acc_empty);  // the accumulator is free: the rest overlaps the next item's MMAs
-      if (!active) return;
-      if (phase == 0) {
-        // SwiGLU, bf16 rounding and the 8-term split, one (token, block of 32 consecutive i) per group of 8 lanes
-        const int n_blk_i = a.I / 32;
-        // small pass: lane group jl has token jl, block q of the item's four, gate in acc[0] and up in acc[1] - one
-        // round.  Otherwise round rd hands the four blocks of the quadrant's token rd (gate in chunk m, up in chunk
-        // m + 4) to the four lane groups.
-        const int n_rd = rep ? 1 : min(4, n_tok - 4 * q);
+        release();
+        const int n_blk_i = a.I / 32, i0 = tile * 128 + 32 * q;
 #pragma unroll 1
-        for (int rd = 0; rd < n_rd; ++rd) {
-          float gsel[4], usel[4];
-          if (rep) {
+        for (int g4 = 0; 4 * g4 < n_tok; ++g4) {
+          // four tokens' chains side by side; a lane has one value of each block
+          float r[4];
+          uint32_t keep[4], word[4], sb[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              gsel[c] = acc[0][c];
-              usel[c] = acc[1][c];
-            }
-          } else {
-#pragma unroll
-            for (int m = 0; m < 4; ++m)
-#pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                const float tg = __shfl_sync(0xffffffffu, acc[m][c], rd * 8 + tl);
-                const float tu = __shfl_sync(0xffffffffu, acc[m + 4][c], rd * 8 + tl);
-                if (jl == m) {
-                  gsel[c] = tg;
-                  usel[c] = tu;
-                }
-              }
+          for (int j = 0; j < 4; ++j) {
+            r[j] = g4 == 0 ? v[j] : (g4 == 1 ? v[4 + j] : (g4 == 2 ? v[8 + j] : v[12 + j]));
+            keep[j] = r[j] != r[j] ? 0u : 0x7FFFFFFFu;  // (a NaN does not take part in its block's maximum)
+            word[j] = 0u;
+            sb[j] = 0u;
           }
-          float r[1][4];
+#pragma unroll 1
+          for (int t = 0; t < kTerms; ++t) {
+            int se[4];
+            float qv[4];
+            uint32_t codes[2];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const float sv = __fdividef(gsel[c], 1.0f + __expf(-gsel[c])) * usel[c];
-            r[0][c] = __bfloat162float(__float2bfloat16_rn(sv));  // the intermediate is defined as a bf16 value
-          }
-          const int tok = rep ? jl : 4 * q + rd;  // token of the pass whose block this lane group splits
-          const int i0 = tile * 128 + 32 * (rep ? q : jl);
-          const bool live = !dry && tok < n_tok;
-          uint8_t* qrow = a.aq2 + static_cast<size_t>(row0 + tok) * kTerms * (a.I / 2) + ((i0 + cb) >> 1);
-          uint8_t* srow = a.sf2 + static_cast<size_t>(row0 + tok) * kTerms * n_blk_i + (i0 >> 5);
-          split_terms<1>(r, [&](int, int t, uint32_t bytes, int se) {
-            if (live) {
-              *reinterpret_cast<uint16_t*>(qrow + static_cast<size_t>(t) * (a.I / 2)) = static_cast<uint16_t>(bytes);
-              if (tl == 0) srow[static_cast<size_t>(t) * n_blk_i] = static_cast<uint8_t>(se + 127);
+            for (int j = 0; j < 4; ++j) {
+              const uint32_t amax = __reduce_max_sync(0xffffffffu, __float_as_uint(r[j]) & keep[j]);
+              se[j] = amax != 0u ? term_exp(__uint_as_float(amax)) : 0;
             }
-          });
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+              codes[j] = e2m1_pair(r[2 * j] * pow2f(-se[2 * j]), r[2 * j + 1] * pow2f(-se[2 * j + 1]), &qv[2 * j], &qv[2 * j + 1]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              r[j] = fmaf(-qv[j], pow2f(se[j]), r[j]);
+              word[j] |= ((codes[j >> 1] >> (4 * (j & 1))) & 15u) << (4 * t);
+              if ((lane & 7) == t) sb[j] = static_cast<uint32_t>(se[j] + 127);
+            }
+          }
+          // nibble t of a lane's word is term t of its value: transposed over eight lanes, a lane holds eight consecutive values
+          // of one term, and the four lanes of a term store its 16 bytes
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int tok = 4 * g4 + j;
+            const uint32_t w = transpose_8x8_nibbles(word[j], lane);
+            if (!dry && tok < n_tok) {
+              const size_t trow = static_cast<size_t>(row0 + tok) * kTerms + (lane & 7);
+              *reinterpret_cast<uint32_t*>(a.aq2 + trow * (a.I / 2) + i0 / 2 + 4 * (lane >> 3)) = w;
+              if (lane < 8) a.sf2[trow * n_blk_i + (i0 >> 5)] = static_cast<uint8_t>(sb[j]);
+            }
+          }
         }
       } else {
-        const int tok = rep ? jl : 4 * q + jl;
-        if (!dry && tok < n_tok) {
-          float* dst = y_row(a.y, a.row_dst, static_cast<size_t>(row0 + tok), out_stride) + tile * kTile + 32 * ch0 + cb;
+#pragma unroll 1
+        for (int g4 = 0; 4 * g4 < n_tok; ++g4) {
+          uint32_t va[32], vb[32];
+          tmem_ld_32x32(d0 + static_cast<uint32_t>(32 * g4), va);
+          tmem_ld_32x32(d1 + static_cast<uint32_t>(32 * g4), vb);
+          tmem_ld_wait();
 #pragma unroll
-          for (int mm = 0; mm < 8; ++mm)
-            if (mm < n_ch) *reinterpret_cast<float4*>(dst + 32 * mm) = make_float4(acc[mm][0], acc[mm][1], acc[mm][2], acc[mm][3]);
+          for (int j = 0; j < 4; ++j) {
+            const int tok = 4 * g4 + j;
+            const float s0 = sum8(va + 8 * j), s1 = sum8(vb + 8 * j);
+            if (!dry && tok < n_tok) {
+              float* dst = y_row(a.y, a.row_dst, static_cast<size_t>(row0 + tok), out_stride) + tile * kTile + 32 * q + lane;
+              dst[0] = s0;
+              dst[128] = s1;
+            }
+          }
         }
+        release();
       }
     };
     // Quantised-activation variant: accumulator lane = operand row = token.  The warp of quadrant q owns tokens
@@ -999,7 +1008,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
       const bool active = 32 * q < n_tok;
       const int tok = 32 * q + lane;
       const bool live = tok < n_tok;
-      mbar_wait(acc_full, acc_ph, a.status);
+      mbar_wait(&acc_full[0], acc_ph, a.status);
       acc_ph ^= 1u;
       __syncwarp();  // tcgen05.ld is warp-collective
       tc_fence_after_sync();
@@ -1026,7 +1035,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
         }
         tc_fence_before_sync();
         __syncwarp();
-        if (lane == 0) mbar_arrive(acc_empty);  // the rest overlaps the next pass's MMAs
+        if (lane == 0) mbar_arrive(&acc_empty[0]);  // the rest overlaps the next pass's MMAs
         if (!active) return;
         const int n_blk_i = a.I / 32;
         uint8_t* qrow = a.aq2 + static_cast<size_t>(row0 + tok) * (a.I / 2) + tile * 64;
@@ -1090,7 +1099,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
         }
         tc_fence_before_sync();
         __syncwarp();
-        if (lane == 0) mbar_arrive(acc_empty);
+        if (lane == 0) mbar_arrive(&acc_empty[0]);
       }
     };
     for (int sweep = kQ ? 1 : 0; sweep < 2; ++sweep) {  // sweep 0 is the dry run of this CTA's first pass, through the one call site below
@@ -1107,7 +1116,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
             if constexpr (kQ)
               run_pass_q(phase, P.R, tile, row0, min(tok_pass, row_end - row0));
             else
-              run_pass(phase, P.rep_ok, P.R, tile, row0, min(tok_pass, row_end - row0), dry);
+              run_pass(phase, P.R, tile, row0, min(tok_pass, row_end - row0), dry);
           }
           if constexpr (kFused) {
             if (!dry && phase == 1) {

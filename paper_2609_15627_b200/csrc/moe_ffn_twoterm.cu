@@ -430,16 +430,6 @@ MOE_DEVINL void tt_tmem_ld_32x8(uint32_t taddr, uint32_t (&v)[8]) {
 
 MOE_DEVINL float tt_silu_mul(float g, float u) { return __fdividef(g, 1.0f + __expf(-g)) * u; }
 
-// 8 x 8 nibble transpose over lanes 8a..8a+7: in, nibble t of lane l is (token t, row l); out, nibble l of lane t
-MOE_DEVINL uint32_t transpose_8x8_nibbles(uint32_t w, int lane) {
-  uint32_t p = __shfl_xor_sync(0xffffffffu, w, 4);
-  w = (lane & 4) ? __byte_perm(w, p, 0x3276) : __byte_perm(w, p, 0x5410);
-  p = __shfl_xor_sync(0xffffffffu, w, 2);
-  w = (lane & 2) ? __byte_perm(w, p, 0x3715) : __byte_perm(w, p, 0x6240);
-  p = __shfl_xor_sync(0xffffffffu, w, 1);
-  return (lane & 1) ? ((p >> 4) & 0x0F0F0F0Fu) | (w & 0xF0F0F0F0u) : (w & 0x0F0F0F0Fu) | ((p & 0x0F0F0F0Fu) << 4);
-}
-
 // 4 x 4 byte transpose over lanes 4a..4a+3: in, byte t of lane l is (token t, row l); out, byte l of lane t
 MOE_DEVINL uint32_t transpose_4x4(uint32_t w, int lane) {
   uint32_t p = __shfl_xor_sync(0xffffffffu, w, 1);

@@ -86,6 +86,16 @@ MOE_DEVINL uint32_t e2m1_pair(float a, float b, float* qa, float* qb) {
   return static_cast<uint32_t>(c);
 }
 
+// 8 x 8 nibble transpose over lanes 8a..8a+7: in, nibble t of lane l is (token t, row l); out, nibble l of lane t
+MOE_DEVINL uint32_t transpose_8x8_nibbles(uint32_t w, int lane) {
+  uint32_t p = __shfl_xor_sync(0xffffffffu, w, 4);
+  w = (lane & 4) ? __byte_perm(w, p, 0x3276) : __byte_perm(w, p, 0x5410);
+  p = __shfl_xor_sync(0xffffffffu, w, 2);
+  w = (lane & 2) ? __byte_perm(w, p, 0x3715) : __byte_perm(w, p, 0x6240);
+  p = __shfl_xor_sync(0xffffffffu, w, 1);
+  return (lane & 1) ? ((p >> 4) & 0x0F0F0F0Fu) | (w & 0xF0F0F0F0u) : (w & 0x0F0F0F0Fu) | ((p & 0x0F0F0F0Fu) << 4);
+}
+
 // Eight threads (consecutive lanes) share one 32-element block, four consecutive values each: the 8-term split,
 // for NB independent blocks at once (their dependency chains interleave).  `store(nb, t, bytes, se)` receives
 // term t's two bytes of codes (values 0,1 and 2,3 of this thread) and the block exponent.  All 32 lanes must call

@@ -1028,6 +1028,26 @@ def test_ffn_native_fp4_path_against_oracle(T, H, I, E, k, hot, seed):
     check_y(buf.y_perm.cpu().numpy(), ry, "native fp4 path")
 
 
+@pytest.mark.parametrize("rows", [
+    (1, 8, 9, 0, 16, 17, 2, 24, 25, 3, 40, 5),  # half of the accumulator columns up to 8 rows, all of them beyond; 16 rows per pass
+    (9, 1, 1, 1, 9, 9, 1, 16, 2, 8, 8, 8),      # the two forms in turn, the halves left in either state
+])
+@pytest.mark.parametrize("H,I", [(512, 512), (768, 256)])
+def test_ffn_native_pass_sizes(rows, H, I):
+    E, S = len(rows), sum(rows)
+    w = inputs.make_expert_weights(H, I, E, seed=11)
+    w = (w[0], inputs.index_scales(2 * I, H, E, lo=117, span=6), w[2], inputs.index_scales(H, I, E, lo=118, span=5))
+    x = inputs.make_x(S, H, seed=11)
+    off = np.concatenate([[0], np.cumsum(rows)]).astype(np.int32)
+    sh = moe.shape(S, H, I, E, 1)
+    buf = moe.LayerBuffers(sh)
+    moe.moe_expert_ffn(dev(x), dev(off), *[dev(a) for a in w], sh, buf.y_perm, buf.status, buf.ws)
+    torch.cuda.synchronize()
+    assert int(buf.status.item()) == 0
+    assert moe.moe_last_kernel_name() == "ffn_native_mxf4_block_scaled"
+    check_y(buf.y_perm.cpu().numpy(), O.expert_ffn(x, off, *w, 1), "native pass sizes")
+
+
 # ---- consecutive layer calls on one stream, sharing every buffer but the output ----
 # With programmatic dependent launch the next call's router may start while this call's combine is still
 # running; it must not overwrite the routing weights and the inverse permutation that combine reads.
