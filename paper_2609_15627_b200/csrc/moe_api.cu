@@ -158,7 +158,7 @@ int expert_ffn_impl(const void* x_perm_bf16, const int32_t* expert_offsets, cons
     return launch_expert_ffn_native(xp, expert_offsets, w, *shape, act, y_perm, status, st, row_dst);
   if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
   if (twoterm)
-    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr}, expert_offsets, w, *shape, *choice, twoterm_guarded(*choice, w),
+    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr, false}, expert_offsets, w, *shape, *choice, twoterm_guarded(*choice, w),
                                      act, y_perm, status.word, st, row_dst);
   if (umma_shape_ok(*choice) || w.blocked)
     return launch_expert_ffn_umma(xp, expert_offsets, w, *shape, act, y_perm, status.word, st, row_dst);
@@ -189,8 +189,44 @@ int permute_and_ffn(const void* x, const int32_t* ids, const int32_t* offsets, c
   char* base = static_cast<char*>(ws);
   if ((rc = launch_permute(xb, ids, offsets, *shape, nullptr, perm, inv_perm, reinterpret_cast<int*>(base + L.permute_off), st)) != MOE_OK)
     return rc;
-  return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, static_cast<__nv_bfloat16*>(x_perm)}, offsets, w, *shape, *shape,
+  return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, static_cast<__nv_bfloat16*>(x_perm), false}, offsets, w, *shape, *shape,
                                    twoterm_guarded(*shape, w), base + L.act_off, y_perm, status.word, st);
+}
+
+// Routing, sort and expert FFN of such a call.  Where one cluster routes and the expert FFN is the two-term or the native
+// kernel, routing and sort are one launch, and the native kernel takes the tokens' rows as that launch splits them beside it, once
+// per token and not per slot; otherwise moe_route and the above.  Same bits.  `offsets2` (may be null) receives {0, T}; `late`:
+// the kernel in front may be the one that writes the logits.
+int route_and_ffn(const float* logits, const void* x, int32_t* ids, float* topk_w, int32_t* offsets, int32_t* offsets2, bool late,
+                  const ExpertWeights& w, const moe_shape_t* shape, void* x_perm, int32_t* perm, int32_t* inv_perm, float* y_perm,
+                  int32_t* status_word, void* ws, size_t ws_bytes, void* cuda_stream) {
+  int rc;
+  const moe_shape_t& s = *shape;
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  const bool twoterm = twoterm_chosen(s, w), native = !twoterm && native_shape_ok(s, w.w13, w.w2) && s.H % 512 == 0;
+  if (!route_sort_ok(s.T, s.E) || !(twoterm || native)) {
+    if (offsets2 != nullptr && (rc = launch_shared_offsets(offsets2, s.T, st)) != MOE_OK) return rc;
+    if ((rc = moe_route(logits, s.T, s.E, s.k, ids, topk_w, offsets, ws, ws_bytes, cuda_stream)) != MOE_OK) return rc;
+    return permute_and_ffn(x, ids, offsets, w, shape, x_perm, perm, inv_perm, y_perm, status_word, ws, ws_bytes, cuda_stream);
+  }
+  if (!aligned(w.w13, 16) || !aligned(w.s13, 16) || !aligned(w.w2, 16) || !aligned(w.s2, 16) ||
+      (status_word != nullptr && !aligned(status_word, 4)))
+    return MOE_ERR_INVALID_ARG;
+  const WsLayout L = ws_layout(s);
+  if (check_ws(ws, ws_bytes, L.total) != MOE_OK) return MOE_ERR_WORKSPACE;
+  StatusRef status;
+  if ((rc = resolve_status(status_word, &status)) != MOE_OK) return rc;
+  const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(x);
+  char* scratch = static_cast<char*>(ws) + L.act_off;
+  if (twoterm) {
+    if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
+    if ((rc = launch_route_sort(logits, s.T, s.E, s.k, ids, topk_w, offsets, perm, inv_perm, false, offsets2, nullptr, late, st)) != MOE_OK) return rc;
+    return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, static_cast<__nv_bfloat16*>(x_perm), true}, offsets, w, s, s,
+                                     twoterm_guarded(s, w), scratch, y_perm, status.word, st);
+  }
+  const FrontSplit split = native_front_split(xb, s, scratch, status);
+  if ((rc = launch_route_sort(logits, s.T, s.E, s.k, ids, topk_w, offsets, perm, inv_perm, true, offsets2, &split, late, st)) != MOE_OK) return rc;
+  return launch_expert_ffn_native_tokens(perm, offsets, w, s, scratch, y_perm, status, st);
 }
 
 // the four tensors inside a buffer written by moe_prepack
@@ -468,10 +504,8 @@ int moe_ffn_block(const void* x_bf16, const void* w_router_bf16, const uint8_t* 
                              base + L.one_scratch, status, st, &shared);
   }
   if ((rc = moe_router_logits(x_bf16, w_router_bf16, s.T, s.H, s.E, d_logits, status_word, st)) != MOE_OK) return rc;
-  if ((rc = launch_shared_offsets(d_off2, s.T, st)) != MOE_OK) return rc;
-  if ((rc = moe_route(d_logits, s.T, s.E, s.k, d_ids, d_w, d_off, inner, L.inner_bytes, st)) != MOE_OK) return rc;
-  if ((rc = permute_and_ffn(x_bf16, d_ids, d_off, ExpertWeights{w13, w13_scale, w2, w2_scale, false}, shape, d_xp, d_perm, d_inv, d_y,
-                            status_word, inner, L.inner_bytes, st)) != MOE_OK)
+  if ((rc = route_and_ffn(d_logits, x_bf16, d_ids, d_w, d_off, d_off2, true, ExpertWeights{w13, w13_scale, w2, w2_scale, false}, shape, d_xp,
+                          d_perm, d_inv, d_y, status_word, inner, L.inner_bytes, st)) != MOE_OK)
     return rc;
   if ((rc = moe_expert_ffn(x_bf16, d_off2, shared_w13, shared_w13_scale, shared_w2, shared_w2_scale, &sh1, d_ys, status_word, inner,
                            L.inner_bytes, st)) != MOE_OK)
@@ -562,9 +596,8 @@ int forward_impl(const float* logits, const void* x_bf16, const ExpertWeights& w
   float* d_y = reinterpret_cast<float*>(base + L.y_perm);
   void* inner = base + L.inner;
   const size_t inner_bytes = ws_bytes - L.inner;
-  const moe_shape_t& s = *shape;
-  if ((rc = moe_route(logits, s.T, s.E, s.k, d_ids, d_w, d_off, inner, inner_bytes, st)) != MOE_OK) return rc;
-  if ((rc = permute_and_ffn(x_bf16, d_ids, d_off, w, shape, d_xp, d_perm, d_inv, d_y, status_word, inner, inner_bytes, st)) != MOE_OK)
+  if ((rc = route_and_ffn(logits, x_bf16, d_ids, d_w, d_off, nullptr, false, w, shape, d_xp, d_perm, d_inv, d_y, status_word, inner, inner_bytes,
+                          st)) != MOE_OK)
     return rc;
   return moe_combine(d_y, d_inv, d_w, shape, out_bf16, st);
 }
@@ -622,7 +655,7 @@ int moe_debug_expert_ffn_variant(const void* x_perm_bf16, const int32_t* expert_
     if (!twoterm_shape_ok(*shape) || !twoterm_weights_ok(w13, w2)) return MOE_ERR_UNSUPPORTED_SHAPE;
     if (check_ws(ws, ws_bytes, L.act_off + twoterm_scratch(*shape).total) != MOE_OK) return MOE_ERR_WORKSPACE;
     if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
-    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr}, expert_offsets, w, *shape, *shape, false, act, y_perm, status.word, st);
+    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr, false}, expert_offsets, w, *shape, *shape, false, act, y_perm, status.word, st);
   }
   if (variant == 2) {
     if (!native_shape_ok(*shape, w13, w2)) return MOE_ERR_UNSUPPORTED_SHAPE;

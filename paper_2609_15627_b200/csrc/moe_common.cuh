@@ -216,6 +216,20 @@ void note_kernel(const char* name, int launches);
 // ---- launchers implemented in the .cu files --------------------------------------------------
 int launch_route(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* counters,
                  cudaStream_t st);
+// Routing and stable sort in one launch, for batches that one thread-block cluster routes; beside it, where `split` is given, the
+// tokens' rows are split into E2M1 term rows, stored by token (split->n_done counters are cleared).  `order` (null: the
+// routing alone) receives slot t * k + j of every sorted row, or with `order_tokens` its token; offsets2 (may be null) {0, T};
+// `late`: the kernel in front may be the one that writes the logits.
+struct FrontSplit {
+  const __nv_bfloat16* x;
+  uint8_t *aq, *sf;   // [T * 8, H / 2], [T * 8, H / 32]
+  int* done;
+  int n_done, H;
+  int* status_clear;  // the library's own status word, or null
+};
+bool route_sort_ok(int T, int E);
+int launch_route_sort(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* order, int* inv_perm,
+                      bool order_tokens, int* offsets2, const FrontSplit* split, bool late, cudaStream_t st);
 // (x_perm null: the sort alone, no rows are copied)
 int launch_permute(const __nv_bfloat16* x, const int* ids, const int* offsets, const moe_shape_t& s,
                    __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st,
@@ -242,6 +256,7 @@ struct TwoTermInput {
   const int* ids;          // [T, k] expert of every slot
   const int* inv_perm;     // [T, k] sorted row of every slot
   __nv_bfloat16* x_sorted; // with the tables: room for the rows in sorted order, of the experts that `guard` does again
+  bool offsets_late;       // with the tables: the kernel in front is the one that writes the offsets
 };
 int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
                            const moe_shape_t& choice, bool guard, void* scratch, float* y_perm, int* status_word, cudaStream_t st,
@@ -265,6 +280,12 @@ int launch_expert_ffn_native_q(const __nv_bfloat16* x_perm, const int* offsets, 
                                void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst = nullptr);
 int launch_expert_ffn_native(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
                              void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst = nullptr);
+
+// the native variant behind launch_route_sort: token rows by token (native_front_split says where that launch leaves them),
+// `tok` the token of every sorted row.  H a multiple of 512.
+FrontSplit native_front_split(const __nv_bfloat16* x, const moe_shape_t& s, void* scratch, StatusRef status);
+int launch_expert_ffn_native_tokens(const int* tok, const int* offsets, const ExpertWeights& w, const moe_shape_t& s, void* scratch,
+                                    float* y_perm, StatusRef status, cudaStream_t st);
 
 // the whole layer in one launch, for a handful of tokens on shapes the native variant takes (moe_forward);
 // `sync` is the zeroed block of kForwardSyncBytes, `scratch` holds forward_fused_scratch_bytes

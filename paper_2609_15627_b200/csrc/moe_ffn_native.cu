@@ -32,13 +32,17 @@
 // No gate/up item ever waits for another CTA, and a down item waits only for gate/up items of CTAs with a lower or
 // equal index (see cta_shares), so the waits cannot form a cycle and do not need the whole grid to be resident.
 // Warp roles:
-//   warp 0      producer: TMA loads of the weight tile, of the term rows and of the weight scale bytes
+//   warp 0      producer of the weight tiles and their scale bytes (TMA), which depend on nothing
 //   warp 1      allocates tensor memory, issues the MMAs, commits to mbarriers
 //   warps 2..5  move weight scale bytes into tensor memory (tcgen05.st), and at a change of (expert, pass) the
 //               scale bytes of its term rows
 //   warps 6..9  epilogue, one warp per tensor-memory lane quadrant (32 weight rows of either tile, all tokens): sum the 8
 //               terms of each token, then SwiGLU + bf16 rounding + the 8-term split for the down projection (gate/up) or the
 //               fp32 store (down)
+//   warp 10     producer of the term rows (TMA): waits for the split, and in phase 1 for the expert's gate/up items, while the
+//               weights of the next steps are on their way
+// The producing warps run convergent and an elected lane issues: from lane 0 of a branch a load takes so long that a second
+// one per step and expert was felt (64 tokens whose rows are fetched one by one: 746 us a layer, now 478).
 // Every wait is bounded and reports through the status word.
 //
 // The weights are read either in the checkpoint's row layout or in moe_prepack's tile-contiguous layout (one tensor
@@ -83,8 +87,9 @@ constexpr int kSfGroups = 3;          // tensor-memory groups for the weight sca
 constexpr int kMaxTokPass = 16;       // tokens per pass (16 x 8 = 128 operand rows)
 constexpr int kQOneLaunchRows = 64;   // quantised-activation variant: up to this many rows per expert on average, one launch
 constexpr int kMaxK = 4096;           // scale factors of one pass's term rows stay in tensor memory: 8 columns per K step
-constexpr int kNatThreads = 10 * 32;
+constexpr int kNatThreads = 11 * 32;
 constexpr int kEpiWarp = 6;           // warps 6..9: warp % 4 = 2, 3, 0, 1 -> one tensor-memory lane quadrant each
+constexpr int kTermWarp = 10;
 constexpr uint32_t kNatTmemCols = 512;
 // tensor-memory columns: one 256-column accumulator; per K step two scale words per operand row, each its own
 // scale-factor block of 4 columns (a block covers 128 rows - rows 32c..32c+31 in column c - and must start on a
@@ -95,6 +100,8 @@ constexpr int kSmallRows = 64;
 
 struct NatArgs {
   const uint8_t* sf1;        // scale bytes of the token rows' terms [S * 8, H/32] (terms: row p * 8 + t, packed E2M1)
+  const int* tok;            // null; or the token of every sorted row: then the token rows' terms are stored by token, once each,
+                             //   and the kernel in front of this one is the one that routes, sorts and splits (launch_route_sort)
   uint8_t* aq2;              // terms of the bf16 intermediate [S * 8, I/2]: written by phase 0, read by phase 1
   uint8_t* sf2;              //   and their scale bytes [S * 8, I/32]
   int* done;                 // [E] epilogue warps that have published a gate/up item of the expert
@@ -240,26 +247,12 @@ __global__ void __launch_bounds__(1024) native_split_kernel(const __nv_bfloat16*
                                                            int E, int* __restrict__ status_clear) {
   pdl_launch_dependents();  // the FFN grid may set up and start its weight stream; it waits before it reads aq or done
   pdl_wait();               // the sorted token rows of moe_permute are complete, and every earlier kernel on the stream
-  const int n_blk = H / 32;
   const long long gt = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (gt < E) done[gt] = 0;
   // the library's own status word (caller passed none): whatever an earlier call left there is over, and the FFN grid
   // of this call looks at the word only in waits that have lasted a millisecond
   if (gt == 0 && status_clear != nullptr) *status_clear = 0;
-  const long long task = gt >> 3;  // (row, block); the grid is padded to whole warps, so whole tasks are in or out
-  const int sub = static_cast<int>(gt & 7);
-  const bool live = task < static_cast<long long>(S) * n_blk;
-  const int p = live ? static_cast<int>(task / n_blk) : 0, b = live ? static_cast<int>(task % n_blk) : 0;
-  const uint2 v = __ldcg(reinterpret_cast<const uint2*>(x + static_cast<size_t>(p) * H + b * 32 + sub * 4));
-  float r[1][4] = {{__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
-                   __uint_as_float(v.y & 0xFFFF0000u)}};
-  split_terms<1>(r, [&](int, int t, uint32_t bytes, int se) {
-    if (live) {
-      const size_t row = static_cast<size_t>(p) * kTerms + t;
-      *reinterpret_cast<uint16_t*>(aq + row * (H / 2) + b * 16 + sub * 2) = static_cast<uint16_t>(bytes);
-      if (sub == 0) aq_sf[row * n_blk + b] = static_cast<uint8_t>(se + 127);
-    }
-  });
+  split_row_blocks(x, aq, aq_sf, S, H, gt);
 }
 
 // ---- the quantised-activation variant's split: bf16 token rows -> one E2M1 row with its scale bytes.  Four threads per
@@ -403,7 +396,9 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
     }
   } else if (!kFused && wid == 2) {
     // lane l looks at experts l, l + 32, ...: all loads are issued before any is used (one memory round trip);
-    // the second loop's loads hit L1.  expert_offsets was complete before the permute kernel let this chain start.
+    // the second loop's loads hit L1.  expert_offsets was complete before the permute kernel let this chain start - where there
+    // is none, it is the kernel in front's.
+    if (a.tok != nullptr) pdl_wait();
     const int n_it = (a.E + 31) / 32;
     unsigned has_mask = 0u;
 #pragma unroll 8
@@ -433,7 +428,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
     }
   }
   if (tid == 0) {
-    for (int s = 0; s < kWStages; ++s) { mbar_init(&full_w[s], 1); mbar_init(&empty_w[s], 1); }
+    for (int s = 0; s < kWStages; ++s) { mbar_init(&full_w[s], 2); mbar_init(&empty_w[s], 1); }
     for (int s = 0; s < kScStages; ++s) { mbar_init(&full_sc[s], 1); mbar_init(&empty_sc[s], 4); }
     for (int s = 0; s < kSfGroups; ++s) { mbar_init(&sf_full[s], 4); mbar_init(&sf_free[s], 1); }
     for (int h = 0; h < 2; ++h) { mbar_init(&acc_full[h], 1); mbar_init(&acc_empty[h], 4); }
@@ -502,7 +497,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
           if (blockIdx.x == 0 && f.w_out != nullptr) f.w_out[t * f.k + lane] = wt;
         }
       }
-    } else if (wid != 0 && static_cast<int>(blockIdx.x) < n_split) {
+    } else if (wid != 0 && wid != kTermWarp && static_cast<int>(blockIdx.x) < n_split) {
       // warps 1 and 6..9 of the first CTAs: token rows -> term rows, one 32-element block per group of 8 lanes;
       // CTA c takes blocks c, c + n_split, ..., 20 of them per round (one round up to two 4096-wide rows)
       const int sw = wid == 1 ? 0 : wid - 5;  // 0..4
@@ -573,102 +568,50 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
 
   const int role = warp_uniform((kFused && s_misc[5] != 0) ? -1 : wid);  // a sync block that was never cleared: no work at all
   if (role == 0) {
-    // =========================== producer ===========================
+    // =========================== weights: all lanes, issued by an elected one ===========================
     const Phase P0 = phase_of(0, a, s_misc + 1), P1 = phase_of(1, a, s_misc + 1);
-    if (lane == 0) {
-      int s = 0, cs = 0;
-      uint32_t ph = 0, cph = 0;
-      // every weight byte is read once per call - unless items have several passes, each of which reads it again
-      const uint64_t stream_once = a.by_pass ? l2_policy_evict_normal() : l2_policy_evict_first();
-      // The weights depend on nothing, the term rows do: on the split kernel (phase 0) or on the gate/up items of
-      // their expert (phase 1).  While a dependency is open, the weight loads go out and the term-row loads of up to
-      // kWStages steps are held back; they follow once the dependency is met.
-      // (one-launch layer: the tokens' term rows were seen complete during the set-up)
-      bool pdl_done = kFused, dep_ok = kFused;
-      if (kFused) fence_proxy_async_all();  // they were written through the generic proxy
-      int dep_phase = 0, dep_e = -1;
-      int n_pend = 0, pend_s[kWStages], pend_x[kWStages], pend_y[kWStages], pend_b[kWStages];
-      // term rows of one K step
-      auto load_terms = [&](const TermMaps* ma, int stage, int bi, int x, int y) {
-        tma_load_2d(sW + stage * kStage + kWStage, &ma->box[bi], x, y, &full_w[stage]);
-      };
-      auto meet = [&]() {  // wait for the open dependency and send the held-back loads
-        if (!pdl_done) {
-          pdl_wait();  // the split kernel is complete: term rows of the tokens, cleared counters
-          pdl_done = true;
-        }
-        if (dep_phase == 1) {
-          counter_wait_ge(a.done + dep_e, need_done, a.status);
-          fence_proxy_async_all();  // the rows were written through the generic proxy, TMA reads through the async one
-        }
-        const TermMaps* ma = dep_phase == 0 ? &tmap_a1 : &tmap_a2;
-        for (int i = 0; i < n_pend; ++i) load_terms(ma, pend_s[i], pend_b[i], pend_x[i], pend_y[i]);
-        n_pend = 0;
-        dep_ok = true;
-      };
-      for (int phase = a.ph_lo; phase < a.ph_hi; ++phase) {
-        const Phase P = phase == 0 ? P0 : P1;
-        const CUtensorMap* mw = phase == 0 ? &tmap_w13 : &tmap_w2;
-        const CUtensorMap* msc = phase == 0 ? &tmap_s13 : &tmap_s2;
-        const TermMaps* ma = phase == 0 ? &tmap_a1 : &tmap_a2;
-        for (int it = P.begin; it < P.end; ++it) {
-          const int ti = it / P.tiles, e = touched[ti];
-          const int tile = t_tile[ti] + it % P.tiles;
-          const int row_begin = t_begin[ti];
-          const int n_rows_e = t_end[ti] - row_begin;
-          const int n_pass = (n_rows_e + tok_pass - 1) / tok_pass;
-          const int wrow_a = phase == 0 ? e * P.R + tile * 128 : e * P.R + tile * kTile;
-          const int wrow_b = phase == 0 ? e * P.R + a.I + tile * 128 : wrow_a + 128;
-          if (phase == 1 && (dep_phase != 1 || dep_e != e)) {  // a new dependency: settle the old one first
-            if (n_pend > 0) meet();
-            dep_phase = 1;
-            dep_e = e;
-            dep_ok = false;
-          }
-          for (int pass = 0; pass < n_pass; ++pass) {
-            const bool by_token = kFused && phase == 0;  // the expert's rows are fetched token by token (at most 4)
-            const int bi = op_box(min(tok_pass, n_rows_e - pass * tok_pass) * nt);  // box of 8 << bi operand rows
-            for (int ks = 0; ks < P.n_steps; ++ks) {
-              if (!P.direct && (ks & 1) == 0) {  // 16 scale bytes per weight row cover two K steps
-                mbar_wait(&empty_sc[cs], cph ^ 1u, a.status);
-                mbar_expect_tx(&full_sc[cs], kScStage);
-                // 128 rows x 16 scale bytes; tile-contiguous layout: tile (row / 128, ks / 2) is 128 consecutive rows of 16 bytes
-                const int sx = a.blocked ? 0 : ks * 8;
-                const int sya = a.blocked ? ((wrow_a >> 7) * (P.n_steps >> 1) + (ks >> 1)) * 128 : wrow_a;
-                const int syb = a.blocked ? ((wrow_b >> 7) * (P.n_steps >> 1) + (ks >> 1)) * 128 : wrow_b;
-                tma_load_2d_hint(sSc + cs * kScStage, msc, sx, sya, &full_sc[cs], stream_once);
-                tma_load_2d_hint(sSc + cs * kScStage + 128 * 16, msc, sx, syb, &full_sc[cs], stream_once);
-                if (++cs == kScStages) { cs = 0; cph ^= 1u; }
-              }
-              mbar_wait(&empty_w[s], ph ^ 1u, a.status);
-              mbar_expect_tx(&full_w[s], static_cast<uint32_t>(kWStage + (by_token ? n_rows_e * 8 : 8 << bi) * 128));
-              // 128 rows x 128 bytes of codes; tile-contiguous layout: tile (row / 128, ks) is 128 consecutive rows of 128 bytes
-              const int wx = a.blocked ? 0 : ks * 128;
-              const int wya = a.blocked ? ((wrow_a >> 7) * P.n_steps + ks) * 128 : wrow_a;
-              const int wyb = a.blocked ? ((wrow_b >> 7) * P.n_steps + ks) * 128 : wrow_b;
-              tma_load_2d_hint(sW + s * kStage, mw, wx, wya, &full_w[s], stream_once);
-              tma_load_2d_hint(sW + s * kStage + 128 * 128, mw, wx, wyb, &full_w[s], stream_once);
-              // the pass's term rows (8 per token, consecutive); rows past the end of the tensor arrive as zeros
-              const int arow = (row_begin + pass * tok_pass) * nt;
-              if (by_token) {
-                // (the tokens' term rows were seen complete during the set-up: no dependency to hold these back for)
-                for (int j = 0; j < n_rows_e; ++j)
-                  tma_load_2d(sW + s * kStage + kWStage + j * (8 * 128), &ma->box[0], ks * 128, s_tok[row_begin + j] * kTerms, &full_w[s]);
-              } else if (dep_ok) {
-                load_terms(ma, s, bi, ks * 128, arow);
-              } else {
-                pend_s[n_pend] = s;
-                pend_x[n_pend] = ks * 128;
-                pend_y[n_pend] = arow;
-                pend_b[n_pend] = bi;
-                if (++n_pend == kWStages) meet();
-              }
-              if (++s == kWStages) { s = 0; ph ^= 1u; }
+    int s = 0, cs = 0;
+    uint32_t ph = 0, cph = 0;
+    const uint32_t ring = smem_u32(sW), sc_ring = smem_u32(sSc), full_bar = smem_u32(full_w), sc_bar = smem_u32(full_sc);
+    // every weight byte is read once per call - unless items have several passes, each of which reads it again
+    const uint64_t stream_once = a.by_pass ? l2_policy_evict_normal() : l2_policy_evict_first();
+    for (int phase = a.ph_lo; phase < a.ph_hi; ++phase) {
+      const Phase P = phase == 0 ? P0 : P1;
+      const CUtensorMap* mw = phase == 0 ? &tmap_w13 : &tmap_w2;
+      const CUtensorMap* msc = phase == 0 ? &tmap_s13 : &tmap_s2;
+      for (int it = P.begin; it < P.end; ++it) {
+        const int ti = it / P.tiles, e = warp_uniform(touched[ti]);
+        const int tile = warp_uniform(t_tile[ti]) + it % P.tiles;
+        const int n_pass = warp_uniform((t_end[ti] - t_begin[ti] + tok_pass - 1) / tok_pass);
+        const int wrow_a = phase == 0 ? e * P.R + tile * 128 : e * P.R + tile * kTile;
+        const int wrow_b = phase == 0 ? e * P.R + a.I + tile * 128 : wrow_a + 128;
+        for (int pass = 0; pass < n_pass; ++pass) {
+          for (int ks = 0; ks < P.n_steps; ++ks) {
+            if (!P.direct && (ks & 1) == 0) {  // 16 scale bytes per weight row cover two K steps
+              mbar_wait_warp(&empty_sc[cs], cph ^ 1u, a.status);
+              const uint32_t bar = sc_bar + cs * 8, dst = sc_ring + cs * kScStage;
+              mbar_expect_tx_elect(bar, kScStage);
+              // 128 rows x 16 scale bytes; tile-contiguous layout: tile (row / 128, ks / 2) is 128 consecutive rows of 16 bytes
+              const int sx = a.blocked ? 0 : ks * 8;
+              const int sya = a.blocked ? ((wrow_a >> 7) * (P.n_steps >> 1) + (ks >> 1)) * 128 : wrow_a;
+              const int syb = a.blocked ? ((wrow_b >> 7) * (P.n_steps >> 1) + (ks >> 1)) * 128 : wrow_b;
+              tma_load_2d_hint_elect(dst, msc, sx, sya, bar, stream_once);
+              tma_load_2d_hint_elect(dst + 128 * 16, msc, sx, syb, bar, stream_once);
+              if (++cs == kScStages) { cs = 0; cph ^= 1u; }
             }
+            mbar_wait_warp(&empty_w[s], ph ^ 1u, a.status);
+            const uint32_t bar = full_bar + s * 8, dst = ring + s * kStage;
+            mbar_expect_tx_elect(bar, kWStage);
+            // 128 rows x 128 bytes of codes; tile-contiguous layout: tile (row / 128, ks) is 128 consecutive rows of 128 bytes
+            const int wx = a.blocked ? 0 : ks * 128;
+            const int wya = a.blocked ? ((wrow_a >> 7) * P.n_steps + ks) * 128 : wrow_a;
+            const int wyb = a.blocked ? ((wrow_b >> 7) * P.n_steps + ks) * 128 : wrow_b;
+            tma_load_2d_hint_elect(dst, mw, wx, wya, bar, stream_once);
+            tma_load_2d_hint_elect(dst + 128 * 128, mw, wx, wyb, bar, stream_once);
+            if (++s == kWStages) { s = 0; ph ^= 1u; }
           }
         }
       }
-      if (n_pend > 0) meet();
     }
     if constexpr (kFused) {
       // Once this CTA's last addition to and last read of the counters are behind it (the epilogue warps say so;
@@ -689,6 +632,57 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
           f.sync[kSyncExit] = 0;
           f.sync[kSyncSplit] = 0;
           if (a.own_status) *a.status = 0;  // every wait of this call is over; nobody reads this word on the host
+        }
+      }
+    }
+  } else if (role == kTermWarp) {
+    // =========================== term rows: likewise ===========================
+    const bool tok_rows = kFused || a.tok != nullptr;  // by token, seen complete during the set-up; or by sorted row
+    if (!kFused) pdl_wait();  // the kernel that splits the token rows is complete: their terms, cleared counters
+    fence_proxy_async_all();  // (one-launch layer: the rows were written through the generic proxy, TMA reads through the async one)
+    int s = 0, dep_e = -1;
+    uint32_t ph = 0;
+    const uint32_t part = smem_u32(sW) + kWStage, full_bar = smem_u32(full_w);
+    for (int phase = a.ph_lo; phase < a.ph_hi; ++phase) {
+      const Phase P = phase_of(phase, a, s_misc + 1);
+      const TermMaps* ma = phase == 0 ? &tmap_a1 : &tmap_a2;
+      const bool by_token = !kQ && tok_rows && phase == 0;
+      for (int it = P.begin; it < P.end; ++it) {
+        const int ti = it / P.tiles;
+        const int row_begin = warp_uniform(t_begin[ti]), n_rows_e = warp_uniform(t_end[ti]) - row_begin;
+        const int n_pass = (n_rows_e + tok_pass - 1) / tok_pass;
+        if (phase == 1 && a.ph_lo == 0) {  // (one projection per launch: the launch before this one has published all rows)
+          const int e = warp_uniform(touched[ti]);
+          if (e != dep_e) {
+            counter_wait_ge_warp(a.done + e, need_done, a.status);
+            fence_proxy_async_all();  // the rows were written through the generic proxy
+            dep_e = e;
+          }
+        }
+        for (int pass = 0; pass < n_pass; ++pass) {
+          const int row0 = row_begin + pass * tok_pass, n_tok = min(tok_pass, n_rows_e - pass * tok_pass);
+          const int bi = op_box(n_tok * nt);  // box of 8 << bi operand rows; rows past the end of the tensor arrive as zeros
+          int tok = 0, t4[4] = {0, 0, 0, 0};  // by token: lane j has the pass's token j, the first four are known to be uniform
+          if (by_token) {
+            if (lane < n_tok) tok = kFused ? s_tok[row0 + lane] : __ldcg(a.tok + row0 + lane);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) t4[j] = warp_uniform(lane == j ? tok : 0);
+          }
+          for (int ks = 0; ks < P.n_steps; ++ks) {
+            mbar_wait_warp(&empty_w[s], ph ^ 1u, a.status);
+            const uint32_t bar = full_bar + s * 8, dst = part + s * kStage;
+            mbar_expect_tx_elect(bar, static_cast<uint32_t>((by_token ? n_tok * 8 : 8 << bi) * 128));
+            if (by_token) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (j < n_tok) tma_load_2d_elect(dst + j * (8 * 128), &ma->box[0], ks * 128, t4[j] * kTerms, bar);
+              for (int j = 4; j < n_tok; ++j)
+                tma_load_2d_elect(dst + j * (8 * 128), &ma->box[0], ks * 128, warp_uniform(lane == j ? tok : 0) * kTerms, bar);
+            } else {
+              tma_load_2d_elect(dst, &ma->box[bi], ks * 128, row0 * nt, bar);
+            }
+            if (++s == kWStages) { s = 0; ph ^= 1u; }
+          }
         }
       }
     }
@@ -787,7 +781,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
               if (st == 0) counter_wait_ge(a.done + touched[ti], need_done, a.status);
               asm volatile("bar.sync 3, 128;" ::: "memory");
             }
-            const bool by_token = kFused && phase == 0;  // the tokens' scale bytes are stored by token, not by sorted row
+            const bool by_token = (kFused || a.tok != nullptr) && phase == 0;  // the tokens' scale bytes are stored by token, not by sorted row
             const int row0 = row_begin + pass * tok_pass;
             const int n_rows = min(tok_pass, row_end - row0) * nt;  // operand rows that exist
             // rows are n_blk bytes each and consecutive: one contiguous range, copied 16 bytes at a time
@@ -801,8 +795,11 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
             } else
             for (int i = st; i < n_vec; i += 128) {
               const int r = i / n_chunk, c = i % n_chunk;
-              const uint4* from = by_token ? reinterpret_cast<const uint4*>(src_sf) + (s_tok[row0 + (r >> 3)] * kTerms + (r & 7)) * n_chunk + c
-                                           : src + i;
+              const uint4* from = src + i;
+              if (by_token) {
+                const int t = kFused ? s_tok[row0 + (r >> 3)] : __ldcg(a.tok + row0 + (r >> 3));
+                from = reinterpret_cast<const uint4*>(src_sf) + (t * kTerms + (r & 7)) * n_chunk + c;
+              }
               reinterpret_cast<uint4*>(sSfa)[r * n_chunk + (c ^ (r & cmask))] = __ldcg(from);
             }
             asm volatile("bar.sync 3, 128;" ::: "memory");
@@ -1282,18 +1279,30 @@ bool native_shape_ok(const moe_shape_t& sh, const void* w13, const void* w2) {
 
 namespace {
 // kQ: the quantised-activation variant (one operand row per token instead of kTerms)
+// scratch: operand rows of the intermediate and of the token rows, each followed by its scale bytes; the counters
+struct NatScratch {
+  uint8_t *aq2, *sf2, *aq1, *sf1;
+  int* done;
+};
+NatScratch nat_scratch(void* scratch, const moe_shape_t& sh, size_t rows) {
+  NatScratch L;
+  L.aq2 = static_cast<uint8_t*>(scratch);
+  L.sf2 = L.aq2 + align_up(rows * (sh.I / 2), kAlign);
+  L.aq1 = L.sf2 + align_up(rows * (sh.I / 32), kAlign);
+  L.sf1 = L.aq1 + align_up(rows * (sh.H / 2), kAlign);
+  L.done = reinterpret_cast<int*>(L.sf1 + align_up(rows * (sh.H / 32), kAlign));
+  return L;
+}
+// tok: null, or the token of every sorted row - the token rows' terms then lie by token (see launch_expert_ffn_native_tokens)
 template <bool kQ>
 int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
-                      void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst) {
+                      void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, const int* tok = nullptr) {
   if (!nat_attr_once()) return MOE_ERR_CUDA;
   const size_t S = static_cast<size_t>(sh.T) * sh.k;
   const size_t rows = S * (kQ ? 1 : kTerms);  // operand rows
-  // scratch: operand rows of the intermediate and of the token rows, each followed by its scale bytes; the counters
-  uint8_t* aq2 = static_cast<uint8_t*>(scratch);
-  uint8_t* sf2 = aq2 + align_up(rows * (sh.I / 2), kAlign);
-  uint8_t* aq1 = sf2 + align_up(rows * (sh.I / 32), kAlign);
-  uint8_t* sf1 = aq1 + align_up(rows * (sh.H / 2), kAlign);
-  int* done = reinterpret_cast<int*>(sf1 + align_up(rows * (sh.H / 32), kAlign));
+  const NatScratch L = nat_scratch(scratch, sh, rows);
+  uint8_t *aq2 = L.aq2, *sf2 = L.sf2, *aq1 = L.aq1, *sf1 = L.sf1;
+  int* done = L.done;
   CUtensorMap tm_w13, tm_w2, tm_s13, tm_s2;
   TermMaps tm_a1, tm_a2;
   for (int i = 0; i < kTermBoxes; ++i)
@@ -1301,16 +1310,19 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
         !nat_map(&tm_a2.box[i], aq2, sh.I / 2, rows, 128, 8u << i, CU_TENSOR_MAP_SWIZZLE_128B))
       return MOE_ERR_CUDA;
   if (!weight_maps(w, sh, &tm_w13, &tm_s13, &tm_w2, &tm_s2)) return MOE_ERR_CUDA;
-  const size_t per_block = kQ ? 4 : 8;  // threads per 32-element block
-  const size_t split_threads = S * (sh.H / 32) * per_block > static_cast<size_t>(sh.E) ? S * (sh.H / 32) * per_block : static_cast<size_t>(sh.E);
-  const dim3 split_grid(static_cast<unsigned>((split_threads + 1023) / 1024));
-  int* own_word = status.own ? status.word : nullptr;
-  if ((kQ ? launch_pdl(native_quant_rows_kernel, split_grid, dim3(1024), 0, st, x_perm, aq1, sf1, done, static_cast<int>(S), sh.H, sh.E, own_word)
-          : launch_pdl(native_split_kernel, split_grid, dim3(1024), 0, st, x_perm, aq1, sf1, done, static_cast<int>(S), sh.H, sh.E, own_word)) !=
-      cudaSuccess)
-    return MOE_ERR_CUDA;
+  if (tok == nullptr) {
+    const size_t per_block = kQ ? 4 : 8;  // threads per 32-element block
+    const size_t split_threads = S * (sh.H / 32) * per_block > static_cast<size_t>(sh.E) ? S * (sh.H / 32) * per_block : static_cast<size_t>(sh.E);
+    const dim3 split_grid(static_cast<unsigned>((split_threads + 1023) / 1024));
+    int* own_word = status.own ? status.word : nullptr;
+    if ((kQ ? launch_pdl(native_quant_rows_kernel, split_grid, dim3(1024), 0, st, x_perm, aq1, sf1, done, static_cast<int>(S), sh.H, sh.E, own_word)
+            : launch_pdl(native_split_kernel, split_grid, dim3(1024), 0, st, x_perm, aq1, sf1, done, static_cast<int>(S), sh.H, sh.E, own_word)) !=
+        cudaSuccess)
+      return MOE_ERR_CUDA;
+  }
   NatArgs a;
   a.sf1 = sf1;
+  a.tok = tok;
   a.aq2 = aq2;
   a.sf2 = sf2;
   a.done = done;
@@ -1341,7 +1353,7 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
                    FusedArgs{}) != cudaSuccess)
       return MOE_ERR_CUDA;
   }
-  note_kernel(kQ ? "ffn_native_mxf4_quantised_activations" : "ffn_native_mxf4_block_scaled", two ? 3 : 2);
+  note_kernel(kQ ? "ffn_native_mxf4_quantised_activations" : "ffn_native_mxf4_block_scaled", two ? 3 : (tok != nullptr ? 1 : 2));
   return MOE_OK;
 }
 }  // namespace
@@ -1349,6 +1361,14 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
 int launch_expert_ffn_native(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
                              void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst) {
   return launch_native_ffn<false>(x_perm, offsets, w, sh, scratch, y_perm, status, st, row_dst);
+}
+FrontSplit native_front_split(const __nv_bfloat16* x, const moe_shape_t& sh, void* scratch, StatusRef status) {
+  const NatScratch L = nat_scratch(scratch, sh, static_cast<size_t>(sh.T) * sh.k * kTerms);
+  return FrontSplit{x, L.aq1, L.sf1, L.done, sh.E, sh.H, status.own ? status.word : nullptr};
+}
+int launch_expert_ffn_native_tokens(const int* tok, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh, void* scratch,
+                                    float* y_perm, StatusRef status, cudaStream_t st) {
+  return launch_native_ffn<false>(nullptr, offsets, w, sh, scratch, y_perm, status, st, nullptr, tok);
 }
 int launch_expert_ffn_native_q(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
                                void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst) {
@@ -1394,6 +1414,7 @@ int launch_forward_fused(const float* logits, const __nv_bfloat16* x, const Expe
   if (!weight_maps(w, sh, &tm_w13, &tm_s13, &tm_w2, &tm_s2)) return MOE_ERR_CUDA;
   NatArgs a;
   a.sf1 = nullptr;
+  a.tok = nullptr;
   a.aq2 = aq2;
   a.sf2 = sf2;
   a.done = sync;

@@ -622,9 +622,11 @@ __global__ void __launch_bounds__(256) twoterm_scatter_kernel(const __nv_bfloat1
                                                              const int* __restrict__ inv_perm, const int* __restrict__ offsets,
                                                              uint8_t* __restrict__ xq, uint8_t* __restrict__ sfx, int T, int k, int H,
                                                              int E, int max_tok, int sf_step, int chunks, uint8_t* __restrict__ marks,
-                                                             int* __restrict__ flags) {
+                                                             int* __restrict__ flags, int offsets_late) {
   extern __shared__ int s_tt_tables[];
-  // (behind the sort of the same call, which waited for the router before it let this kernel start: expert_offsets is complete)
+  // expert_offsets is read here and, as it starts, by the gate/up grid: complete where the sort of the same call waited for
+  // the router before it let this kernel start, to be waited for where one kernel routes and sorts
+  if (offsets_late) pdl_wait();
   pdl_launch_dependents();
   const TtTables tab = tt_tables<false>(s_tt_tables, offsets, E, max_tok);
   pdl_wait();
@@ -1329,7 +1331,7 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
     const size_t want = (static_cast<size_t>(sh.T) * parts + 7) / 8;
     rc = launch_pdl(guard ? twoterm_scatter_kernel<true> : twoterm_scatter_kernel<false>, dim3(static_cast<unsigned>(want < most ? want : most)), dim3(256), table_bytes, st, in.x,
                     in.ids, in.inv_perm, offsets, base + L.xq, base + L.sfx, sh.T, sh.k, sh.H, sh.E, geo.max_tok, geo.sf_step, chunks,
-                    marks, flags);
+                    marks, flags, in.offsets_late ? 1 : 0);
   } else {
     const size_t want = (S * parts + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
     rc = launch_pdl(guard ? twoterm_split_kernel<false, true> : twoterm_split_kernel<false, false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256), table_bytes, st, in.x,

@@ -62,6 +62,25 @@ MOE_DEVINL void counter_wait_ge(const int* p, int need, int* status) {
     __nanosleep(64);
   }
 }
+// The same by a whole convergent warp (see mbar_wait_warp)
+MOE_DEVINL void counter_wait_ge_warp(const int* p, int need, int* status) {
+  const long long t0 = clock64();
+  int spins = 0;
+  while (true) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    if (__all_sync(0xffffffffu, v >= need)) return;
+    const long long waited = clock64() - t0;
+    if (__any_sync(0xffffffffu, waited > kWaitLimitCycles)) {
+      if (status != nullptr) atomicExch(status, static_cast<int>(MOE_ERR_TIMEOUT));
+      return;
+    }
+    if (((++spins) & 63) == 0 &&
+        __any_sync(0xffffffffu, waited > 2000000 && status != nullptr && *reinterpret_cast<volatile int*>(status) != 0))
+      return;
+    __nanosleep(64);
+  }
+}
 // orders this thread's generic-proxy accesses with its asynchronous-proxy (TMA) accesses, global memory included
 MOE_DEVINL void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 MOE_DEVINL void prefetch_tmap(const void* tmap) { asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory"); }
@@ -122,6 +141,27 @@ MOE_DEVINL void split_terms(float (&r)[NB][4], Store store) {
       store(nb, t, bytes, se);
     }
   }
+}
+
+// Rows [0, n_rows) of bf16 -> 8 E2M1 term rows each with their scale bytes; thread gt of the grid, 8 threads per 32-element block
+// (whole warps call it together)
+MOE_DEVINL void split_row_blocks(const __nv_bfloat16* __restrict__ x, uint8_t* __restrict__ aq, uint8_t* __restrict__ aq_sf, int n_rows, int H,
+                                 long long gt) {
+  const int n_blk = H / 32;
+  const long long task = gt >> 3;  // (row, block); the grid is padded to whole warps, so whole tasks are in or out
+  const int sub = static_cast<int>(gt & 7);
+  const bool live = task < static_cast<long long>(n_rows) * n_blk;
+  const int p = live ? static_cast<int>(task / n_blk) : 0, b = live ? static_cast<int>(task % n_blk) : 0;
+  const uint2 v = __ldcg(reinterpret_cast<const uint2*>(x + static_cast<size_t>(p) * H + b * 32 + sub * 4));
+  float r[1][4] = {{__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
+                   __uint_as_float(v.y & 0xFFFF0000u)}};
+  split_terms<1>(r, [&](int, int t, uint32_t bytes, int se) {
+    if (live) {
+      const size_t row = static_cast<size_t>(p) * kTerms + t;
+      *reinterpret_cast<uint16_t*>(aq + row * (H / 2) + b * 16 + sub * 2) = static_cast<uint16_t>(bytes);
+      if (sub == 0) aq_sf[row * n_blk + b] = static_cast<uint8_t>(se + 127);
+    }
+  });
 }
 
 }  // namespace moe

@@ -2,6 +2,7 @@
 // All three are integer / bandwidth work: warp shuffles, shared-memory histograms, prefix scans and
 // 16-byte vector copies.  Results are bit-defined (see include/moe_b200.h).
 #include "moe_common.cuh"
+#include "moe_mxf4_device.cuh"
 #include "moe_route_device.cuh"
 
 namespace moe {
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(1024) route_kernel(const float* __restrict__ l
 
 int launch_route(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* counters,
                  cudaStream_t st) {
+  if (route_sort_ok(T, E)) return launch_route_sort(logits, T, E, k, ids, w, offsets, nullptr, nullptr, false, nullptr, nullptr, false, st);
   // One CTA up to a round of its 32 warps.  (64 tokens: 19 us in two rounds of one CTA, 7 us on eight.)
   const bool single = T <= 32;
   const int nw = single ? 32 : 8;
@@ -124,6 +126,129 @@ int launch_route(const float* logits, int T, int E, int k, int* ids, float* w, i
     note_kernel("route_topk_multi_cta", launches);
   }
   return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+}
+
+// ---- routing and sort of batches that one cluster routes (up to 256 tokens and 256 experts), and the split of their rows ----
+// A warp per token, tokens in order over the cluster's CTAs (as many as there are eights of tokens: the warps of a CTA share its
+// issue slots).  The warps that chose an expert are the bits of a mask, so a CTA's count of it is a population count and
+// a slot's rank the one of the bits below its warp's; the counts meet through distributed shared memory.  Latency is all
+// there is to it: one launch without anything to clear in front, where the general route takes a memset, a router whose last
+// CTA scans, and a sort (64 tokens and the split of their rows: 9 us until the expert FFN's weights start to stream, 26 before).
+// With more than a token per warp it is no faster than those (333 tokens in two rounds: 12 us, and 13 to the end of the
+// general sort).
+// The CTAs behind the first cluster (kSplit) split the token rows, which depends on no routing, meanwhile.
+constexpr int kFrontMaxE = 256, kFrontCluster = 8;
+template <bool kSplit>
+__global__ void __launch_bounds__(1024) route_sort_kernel(const float* __restrict__ logits, int T, int E, int k, int* __restrict__ ids,
+                                                          float* __restrict__ w, int* __restrict__ offsets, int* __restrict__ order,
+                                                          int* __restrict__ inv_perm, int order_tokens, int* __restrict__ offsets2, int late,
+                                                          const FrontSplit f) {
+  __shared__ unsigned s_mask[kFrontMaxE];
+  __shared__ int s_cnt[kFrontMaxE], s_base[kFrontMaxE], s_tot[kFrontMaxE / 32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  unsigned n_cta, rank;
+  asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n_cta));
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  pdl_launch_dependents();  // (whatever comes next waits before it reads)
+  if (kSplit && blockIdx.x >= n_cta) {
+    pdl_wait();
+    const long long gt = static_cast<long long>(blockIdx.x - n_cta) * blockDim.x + tid;
+    for (long long i = gt; i < f.n_done; i += static_cast<long long>(gridDim.x - n_cta) * blockDim.x) f.done[i] = 0;
+    if (gt == 0 && f.status_clear != nullptr) *f.status_clear = 0;
+    split_row_blocks(f.x, f.aq, f.sf, T, f.H, gt);
+    return;
+  }
+  // this kernel may have started while the one before it still reads what is about to be overwritten: only the logits are read
+  // before the wait, and not where that one may write them (what moe_route promises above 32 tokens)
+  if (late) pdl_wait();
+  if (tid < kFrontMaxE) s_mask[tid] = 0u;
+  __syncthreads();
+  const int per_cta = (T + static_cast<int>(n_cta) - 1) / static_cast<int>(n_cta);  // at most 32
+  const int t = static_cast<int>(rank) * per_cta + wid;
+  const bool live = wid < per_cta && t < T;
+  int my_id = -1;
+  float wt = 0.0f;
+  if (live) {
+    float my_v;
+    warp_topk_256(logits + static_cast<size_t>(t) * E, E, k, lane, &my_id, &my_v);
+    wt = warp_softmax_selected(my_v, k, lane);
+  }
+  if (!late) pdl_wait();
+  const bool mine = live && lane < k;
+  if (mine) {
+    ids[static_cast<size_t>(t) * k + lane] = my_id;
+    w[static_cast<size_t>(t) * k + lane] = wt;
+    atomicOr(&s_mask[my_id], 1u << wid);
+  }
+  __syncthreads();
+  if (tid < E) s_cnt[tid] = __popc(s_mask[tid]);
+  if (n_cta > 1)
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  int total = 0, before = 0, ex = 0;
+  if (tid < kFrontMaxE) {
+    if (tid < E) {
+      for (unsigned c = 0; c < n_cta; ++c) {
+        uint32_t at;
+        int v;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(&s_cnt[tid])), "r"(c));
+        asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+        total += v;
+        before += c < rank ? v : 0;
+      }
+    }
+    int warp_total;
+    ex = warp_excl_scan(total, lane, &warp_total);
+    if (lane == 0) s_tot[wid] = warp_total;
+  }
+  __syncthreads();
+  if (tid < E) {
+    for (int i = 0; i < wid; ++i) ex += s_tot[i];
+    s_base[tid] = ex + before;
+    if (rank == 0) {
+      offsets[tid] = ex;
+      if (tid == E - 1) offsets[E] = ex + total;
+    }
+  }
+  if (rank == 0 && tid < 2 && offsets2 != nullptr) offsets2[tid] = tid == 0 ? 0 : T;
+  if (n_cta > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");  // (the other CTAs' counts have been read)
+  __syncthreads();
+  if (order != nullptr && mine) {
+    const int p = s_base[my_id] + __popc(s_mask[my_id] & ((1u << wid) - 1u)), slot = t * k + lane;
+    inv_perm[slot] = p;
+    order[p] = order_tokens ? t : slot;
+  }
+  if (n_cta > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+bool route_sort_ok(int T, int E) { return E <= kFrontMaxE && T <= 32 * kFrontCluster; }
+
+int launch_route_sort(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* order, int* inv_perm,
+                      bool order_tokens, int* offsets2, const FrontSplit* split, bool late, cudaStream_t st) {
+  int n_cta = 1;
+  while (n_cta < kFrontCluster && n_cta * 8 < T) n_cta *= 2;
+  long long extra = 0;
+  if (split != nullptr) {
+    extra = (static_cast<long long>(T) * (split->H / 32) * 8 + 1023) / 1024;
+    extra = (extra + n_cta - 1) / n_cta * n_cta;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(n_cta + extra));
+  cfg.blockDim = dim3(1024);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(n_cta);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  if (cudaLaunchKernelEx(&cfg, split != nullptr ? route_sort_kernel<true> : route_sort_kernel<false>, logits, T, E, k, ids, w, offsets, order,
+                         inv_perm, order_tokens ? 1 : 0, offsets2, late || T > 32 ? 1 : 0, split != nullptr ? *split : FrontSplit{}) != cudaSuccess)
+    return MOE_ERR_CUDA;
+  note_kernel(order != nullptr ? "route_topk_and_sort_one_cluster" : "route_topk_one_cluster", 1);
+  return MOE_OK;
 }
 
 // =================================================================================================

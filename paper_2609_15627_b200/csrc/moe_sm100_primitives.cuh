@@ -122,6 +122,32 @@ MOE_DEVINL void tma_load_2d_hint(void* dst, const void* tmap, int x, int y, uint
       "l"(tmap), "r"(smem_u32(bar)), "r"(x), "r"(y), "l"(policy)
       : "memory");
 }
+// The same and the expected bytes from a whole convergent warp, issued by one elected lane (see umma_commit_elect), with
+// shared-memory addresses as integers
+MOE_DEVINL void mbar_expect_tx_elect(uint32_t bar, uint32_t bytes) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar), "r"(bytes)
+      : "memory");
+}
+MOE_DEVINL void tma_load_2d_elect(uint32_t dst, const void* tmap, int x, int y, uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n\t}" ::"r"(dst),
+      "l"(tmap), "r"(bar), "r"(x), "r"(y)
+      : "memory");
+}
+MOE_DEVINL void tma_load_2d_hint_elect(uint32_t dst, const void* tmap, int x, int y, uint32_t bar, uint64_t policy) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], "
+      "[%2], %5;\n\t}" ::"r"(dst),
+      "l"(tmap), "r"(bar), "r"(x), "r"(y), "l"(policy)
+      : "memory");
+}
 // Output row `row` of the expert FFN: in the caller's y_perm [rows, stride], or - expert-parallel sharding - wherever the
 // table says (a row of the buffer of the rank that finishes the row's token, possibly in a peer GPU's memory)
 MOE_DEVINL float* y_row(float* y, float* const* row_dst, size_t row, int stride) {

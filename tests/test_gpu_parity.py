@@ -430,6 +430,24 @@ def test_forward_small_shapes(T, H, I, E, k, one_launch):
     _check_forward(wl, d, None, one_launch)
 
 
+# One cluster of 1, 2, 4 or 8 CTAs of up to 32 tokens routes and sorts; beyond that the general route and sort
+@pytest.mark.parametrize("T,E,k", [(2, 16, 2), (31, 256, 8), (32, 256, 8), (33, 100, 6), (64, 256, 8), (65, 40, 32), (128, 64, 3), (129, 64, 8),
+                                   (255, 256, 8), (256, 100, 1), (256, 256, 6), (257, 100, 6), (8, 256, 8), (9, 7, 7), (1000, 256, 6)])
+def test_forward_routes_and_sorts_as_the_calls_do(T, E, k):
+    H, I = 512, 512
+    wl = inputs.Workload("sort", T, H, I, E, k)
+    d = inputs.make_workload(wl, seed=21)
+    wdev = weights_dev(d)
+    out, ids, w, _ = _run_forward(wl, d, wdev)
+    rids, rw, roff = O.route(d["logits"], k)
+    assert np.array_equal(ids.cpu().numpy(), rids) and np.array_equal(w.cpu().numpy().view(np.uint32), rw.view(np.uint32))
+    buf, out4 = run_layer(wl, d, wdev)
+    assert np.array_equal(buf.expert_offsets.cpu().numpy(), roff)
+    _, perm, inv = O.permute(d["x"], rids, roff)
+    assert np.array_equal(buf.perm.cpu().numpy(), perm) and np.array_equal(buf.inv_perm.cpu().numpy(), inv)
+    assert torch.equal(out.view(torch.int16), out4.view(torch.int16))
+
+
 @pytest.mark.parametrize("T,H,I,E,k", [
     (2, 1024, 512, 16, 4), (2, 2048, 1024, 64, 8), (3, 1024, 512, 32, 6), (4, 512, 512, 8, 2), (4, 1024, 512, 32, 8),
     (2, 512, 512, 16, 16),          # 32 slots, every expert touched by both tokens
