@@ -193,6 +193,10 @@ int permute_and_ffn(const void* x, const int32_t* ids, const int32_t* offsets, c
                                    twoterm_guarded(*shape, w), base + L.act_off, y_perm, status.word, st);
 }
 
+// whether the front of such a call is one launch (see below), which reads logits and rows once
+bool front_in_one(const moe_shape_t& s, const ExpertWeights& w) {
+  return route_sort_ok(s.T, s.E) && (twoterm_chosen(s, w) || (native_shape_ok(s, w.w13, w.w2) && s.H % 512 == 0));
+}
 // Routing, sort and expert FFN of such a call.  Where one cluster routes and the expert FFN is the two-term or the native
 // kernel, routing and sort are one launch, and the native kernel takes the tokens' rows as that launch splits them beside it, once
 // per token and not per slot; otherwise moe_route and the above.  Same bits.  `offsets2` (may be null) receives {0, T}; `late`:
@@ -203,8 +207,8 @@ int route_and_ffn(const float* logits, const void* x, int32_t* ids, float* topk_
   int rc;
   const moe_shape_t& s = *shape;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const bool twoterm = twoterm_chosen(s, w), native = !twoterm && native_shape_ok(s, w.w13, w.w2) && s.H % 512 == 0;
-  if (!route_sort_ok(s.T, s.E) || !(twoterm || native)) {
+  const bool twoterm = twoterm_chosen(s, w);
+  if (!front_in_one(s, w)) {
     if (offsets2 != nullptr && (rc = launch_shared_offsets(offsets2, s.T, st)) != MOE_OK) return rc;
     if ((rc = moe_route(logits, s.T, s.E, s.k, ids, topk_w, offsets, ws, ws_bytes, cuda_stream)) != MOE_OK) return rc;
     return permute_and_ffn(x, ids, offsets, w, shape, x_perm, perm, inv_perm, y_perm, status_word, ws, ws_bytes, cuda_stream);
@@ -726,7 +730,14 @@ unsigned char* logits_staging() {
   }
   return buf;
 }
-constexpr size_t kDirectOutBytes = 64 * 1024;  // outputs up to this size are written to pinned host memory by the kernel
+// A buffer of the caller as the device addresses it, where it can (pinned host memory under unified addressing), or null
+void* device_view(const void* host) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, host) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer != nullptr && aligned(at.devicePointer, 16))
+    return at.devicePointer;
+  cudaGetLastError();  // pageable memory: not an error of this call
+  return nullptr;
+}
 int forward_host_impl(const float* logits_host, const void* x_host_bf16, const ExpertWeights& w, const moe_shape_t* shape,
                       void* out_host_bf16, int32_t* status_word, void* ws, size_t ws_bytes, void* cuda_stream) {
   int rc;
@@ -739,39 +750,28 @@ int forward_host_impl(const float* logits_host, const void* x_host_bf16, const E
   float* d_logits = reinterpret_cast<float*>(base + L.logits);
   void* d_x = base + L.x;
   void* d_out = base + L.out;
-  // A small output goes straight to the caller's buffer where the device can address it (pinned host memory under
-  // unified addressing): the last kernel's stores cross the bus instead of a copy operation enqueued after it.
-  bool direct = false;
+  // The output goes straight to the caller's buffer where the device can address it: the last kernel's stores cross the bus
+  // instead of a copy operation enqueued after it (4096-wide rows: 16 tokens 244 -> 234 us a call with the next one, 256 tokens 742 -> 731, 1300 tokens 1223 -> 1207).
   const size_t out_bytes = static_cast<size_t>(s.T) * s.H * 2;
-  if (out_bytes <= kDirectOutBytes) {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, out_host_bf16) == cudaSuccess && at.type == cudaMemoryTypeHost &&
-        at.devicePointer != nullptr && aligned(at.devicePointer, 16)) {
-      d_out = at.devicePointer;
-      direct = true;
-    } else {
-      cudaGetLastError();  // pageable memory: not an error of this call
-    }
-  }
-  // Likewise a single token row is read where it lies: the few CTAs that split it fetch 512 bytes each across the bus,
-  // which costs the kernel less than a copy operation in front of it costs the call.
-  bool x_direct = false;
-  if (s.T == 1 && decode_one_ok(s, w.w13, w.w2)) {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, x_host_bf16) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer != nullptr &&
-        aligned(at.devicePointer, 16)) {
-      d_x = at.devicePointer;
-      x_direct = true;
-    } else {
-      cudaGetLastError();
-    }
-  }
+  void* out_view = device_view(out_host_bf16);
+  const bool direct = out_view != nullptr;
+  if (direct) d_out = out_view;
+  // Likewise what a kernel reads once is read where it lies: a single token's row (the few CTAs that split it fetch 512 bytes
+  // each), and the logits and rows of a batch whose front is one launch (up to 256 tokens).
+  const bool one = s.T == 1 && decode_one_ok(s, w.w13, w.w2), front = s.T > 1 && front_in_one(s, w);
+  void* x_view = one || front ? device_view(x_host_bf16) : nullptr;
+  const bool x_direct = x_view != nullptr;
+  if (x_direct) d_x = x_view;
+  void* logits_view = front ? device_view(logits_host) : nullptr;
   // This call owns its workspace's contents: it clears the counter block of moe_forward itself.  Small logits go through
   // a page-locked staging buffer of this thread that ends in zeros, so that one copy brings both (the call waits for the
   // stream before it returns, so the buffer is free again by then).
+  // (with more than one token no kernel uses the counter block)
   const size_t lg_bytes = static_cast<size_t>(s.T) * s.E * 4, lg_span = L.inner - L.logits;
-  unsigned char* stage = lg_span <= kStageLogitsBytes ? logits_staging() : nullptr;
-  if (stage != nullptr) {
+  unsigned char* stage = logits_view == nullptr && lg_span <= kStageLogitsBytes ? logits_staging() : nullptr;
+  if (logits_view != nullptr) {
+    d_logits = static_cast<float*>(logits_view);
+  } else if (stage != nullptr) {
     memcpy(stage, logits_host, lg_bytes);
     memset(stage + lg_bytes, 0, lg_span - lg_bytes + kForwardSyncBytes);  // (an earlier, larger batch may have left logits there)
     if (cudaMemcpyAsync(d_logits, stage, lg_span + kForwardSyncBytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return MOE_ERR_CUDA;
