@@ -153,6 +153,17 @@ int moe_combine(const float* y_perm, const int32_t* inv_perm, const float* topk_
                 void* out_bf16 /* [T,H] */, void* cuda_stream);
 
 /*
+ * The four calls above one after the other on the caller's buffers: moe_route, moe_permute, moe_expert_ffn and moe_combine with these
+ * arguments, every buffer written as they write it, the same errors; `ws` moe_workspace_bytes().  One call into the library
+ * where a caller with no use for the steps would make four, and one launch less to wait for where one kernel routes and
+ * sorts (T <= 256, E <= 256).
+ */
+int moe_layer(const float* logits, const void* x_bf16, const uint8_t* w13, const uint8_t* w13_scale, const uint8_t* w2,
+              const uint8_t* w2_scale, const moe_shape_t* shape, int32_t* topk_ids, float* topk_w, int32_t* expert_offsets,
+              void* x_perm_bf16, int32_t* perm, int32_t* inv_perm, float* y_perm, void* out_bf16, int32_t* status_word, void* ws,
+              size_t ws_bytes, void* cuda_stream);
+
+/*
  * One-time load check of E8M0 scale bytes (paper: scale layout and value traps, "test real
  * nonconstant scales").  Counts bytes outside [0,128] into *bad_count (device int32, overwritten).
  */

@@ -302,6 +302,31 @@ int moe_combine(const float* y_perm, const int32_t* inv_perm, const float* topk_
                         static_cast<cudaStream_t>(cuda_stream));
 }
 
+int moe_layer(const float* logits, const void* x_bf16, const uint8_t* w13, const uint8_t* w13_scale, const uint8_t* w2,
+              const uint8_t* w2_scale, const moe_shape_t* shape, int32_t* topk_ids, float* topk_w, int32_t* expert_offsets,
+              void* x_perm_bf16, int32_t* perm, int32_t* inv_perm, float* y_perm, void* out_bf16, int32_t* status_word, void* ws,
+              size_t ws_bytes, void* cuda_stream) {
+  int rc = check_shape(shape);
+  if (rc != MOE_OK) return rc;
+  const moe_shape_t& s = *shape;
+  if (!route_sort_ok(s.T, s.E)) {
+    if ((rc = moe_route(logits, s.T, s.E, s.k, topk_ids, topk_w, expert_offsets, ws, ws_bytes, cuda_stream)) != MOE_OK) return rc;
+    if ((rc = moe_permute(x_bf16, topk_ids, expert_offsets, shape, x_perm_bf16, perm, inv_perm, ws, ws_bytes, cuda_stream)) != MOE_OK) return rc;
+  } else {
+    if (!aligned(logits, 16) || !aligned(x_bf16, 16) || !aligned(topk_ids, 16) || !aligned(topk_w, 16) || !aligned(expert_offsets, 16) ||
+        !aligned(x_perm_bf16, 16) || !aligned(perm, 16) || !aligned(inv_perm, 16))
+      return MOE_ERR_INVALID_ARG;
+    if (check_ws(ws, ws_bytes, ws_layout(s).total) != MOE_OK) return MOE_ERR_WORKSPACE;
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    if ((rc = launch_route_sort(logits, s.T, s.E, s.k, topk_ids, topk_w, expert_offsets, perm, inv_perm, false, nullptr, nullptr, false, st)) != MOE_OK ||
+        (rc = launch_gather_rows(static_cast<const __nv_bfloat16*>(x_bf16), perm, s, static_cast<__nv_bfloat16*>(x_perm_bf16), st)) != MOE_OK)
+      return rc;
+  }
+  if ((rc = moe_expert_ffn(x_perm_bf16, expert_offsets, w13, w13_scale, w2, w2_scale, shape, y_perm, status_word, ws, ws_bytes, cuda_stream)) != MOE_OK)
+    return rc;
+  return moe_combine(y_perm, inv_perm, topk_w, shape, out_bf16, cuda_stream);
+}
+
 // ---- router projection, shared expert, join: the whole FFN block ---------------------------------------------
 int moe_router_logits(const void* x_bf16, const void* w_router_bf16, int32_t T, int32_t H, int32_t E, float* logits,
                       int32_t* status_word, void* cuda_stream) {

@@ -230,6 +230,8 @@ struct FrontSplit {
 bool route_sort_ok(int T, int E);
 int launch_route_sort(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* order, int* inv_perm,
                       bool order_tokens, int* offsets2, const FrontSplit* split, bool late, cudaStream_t st);
+// the rows alone, in the order of a sort that is done (perm: slot of every sorted row)
+int launch_gather_rows(const __nv_bfloat16* x, const int* perm, const moe_shape_t& s, __nv_bfloat16* x_perm, cudaStream_t st);
 // (x_perm null: the sort alone, no rows are copied)
 int launch_permute(const __nv_bfloat16* x, const int* ids, const int* offsets, const moe_shape_t& s,
                    __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st,

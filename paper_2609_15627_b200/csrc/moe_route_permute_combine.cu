@@ -426,6 +426,15 @@ __global__ void __launch_bounds__(256) permute_gather_kernel(const __nv_bfloat16
   }
 }
 
+int launch_gather_rows(const __nv_bfloat16* x, const int* perm, const moe_shape_t& sh, __nv_bfloat16* x_perm, cudaStream_t st) {
+  const int S = sh.T * sh.k, grid = min((S + 7) / 8, sm_count() * 16);
+  if (launch_pdl(permute_gather_kernel, dim3(grid), dim3(256), 0, st, x, perm, S, sh.H, sh.k, x_perm, static_cast<const int*>(nullptr),
+                 static_cast<const int*>(nullptr)) != cudaSuccess)
+    return MOE_ERR_CUDA;
+  note_kernel("permute_gather_rows", 1);
+  return MOE_OK;
+}
+
 int launch_permute(const __nv_bfloat16* x, const int* ids, const int* offsets, const moe_shape_t& sh,
                    __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st, const int* range_lo,
                    const int* range_hi) {
