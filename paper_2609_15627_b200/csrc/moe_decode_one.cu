@@ -9,8 +9,12 @@
 //   * The token row is split into its eight E2M1 term rows by the first H/256 CTAs - the earliest to start - 8 blocks of
 //     32 elements each, about a microsecond (splitting the whole row in every CTA was tried: several microseconds of
 //     issue time).  They store kCopies copies to global memory and count themselves in; every CTA with an item fetches
-//     the rows K step by K step with its weight stages (TMA, four copies of each row, one per lane quadrant of the
-//     accumulator) and their scale bytes straight into registers on the way to tensor memory.
+//     the rows K step by K step with its weight stages (TMA) and their scale bytes straight into registers on the way to
+//     tensor memory.
+//   * In both projections the weights are the A operand (M = 128 rows) and the 8 term rows the B operand (N = 16, the smallest),
+//     so the eight terms of a result are eight registers of one thread: nothing is summed over lanes, and the 32 lanes
+//     of a warp are one scale block of the intermediate (one token of 8 experts of 4096 x 2048, top-8: 27.2 -> 26.1 us a layer; with
+//     the rows as A, four copies of each for the four lane quadrants, their sums took three exchanges over lanes per chunk).
 //   * The down projection is split along K, so that it needs no other CTA's part of the intermediate: the two CTAs of a
 //     thread-block cluster hold neighbouring 128-wide slices of the expert's intermediate (gate/up tiles 2p and 2p + 1),
 //     exchange their E2M1 term rows through distributed shared memory (st.shared::cluster, one cluster barrier), and
@@ -32,7 +36,7 @@
 //
 // Warp roles (320 threads, one CTA per SM, clusters of two CTAs):
 //   warp 0      lane 0 issues all TMA loads (weights, weight scale bytes, the token's term rows) of both projections
-//   warp 1      allocates tensor memory, issues the MMAs (kind::mxf4.block_scale, M = 128 term rows, N = 256 weight rows)
+//   warp 1      allocates tensor memory, issues the MMAs (kind::mxf4.block_scale, M = 128 weight rows, N = 16)
 //   warps 2..5  move weight scale bytes shared memory -> tensor memory
 //   warps 6..9  epilogue, one per lane quadrant: scale factors of the token's terms -> tensor memory; gate/up
 //               accumulator -> SwiGLU -> bf16 -> term rows into both CTAs of the pair; down accumulators -> partial
@@ -58,16 +62,16 @@ MOE_DEVINL unsigned long long trace_time() {
 
 namespace {
 
-constexpr int kTile = 256;             // weight rows per MMA (N)
+constexpr int kTile = 256;             // weight rows per stage: two MMA tiles
 constexpr int kWStage = kTile * 128;   // 32 KB: 256 weight rows x one K step (256 elements = 128 packed bytes)
 constexpr int kWStages = 4;
 constexpr int kScStage = kTile * 16;   // 4 KB: 256 rows x 16 scale bytes (two K steps)
 constexpr int kScStages = 3;
 constexpr int kSfGroups = 3;           // tensor-memory groups of weight scale factors: 4 words x 8 columns each
-constexpr int kATile = 128 * 128;      // 16 KB: span of one A operand (128 rows x 128 bytes)
 constexpr int kOneThreads = 10 * 32;
 constexpr uint32_t kOneTmemCols = 512;
-constexpr uint32_t kColD = 0, kColSfAct = 256, kColSfW = 384;  // accumulator | scale factors of the term rows | of the weights
+// accumulators of the down projection's sub-tiles (16 columns each) | scale factors of the term rows | of the weights | gate, up
+constexpr uint32_t kColD = 0, kColSfAct = 256, kColSfW = 384, kColGate = 480, kColUp = 496;
 // The token's term rows and their scale bytes are written kCopies times (16 KB + 1 KB each at H = 4096) and CTA i reads
 // copy i % kCopies: every CTA with an item fetches them at the same moment, and with a single copy each cache line is
 // asked for by hundreds of requesters at once.
@@ -94,14 +98,9 @@ struct OneArgs {
 struct OneSmem {
   uint32_t ring, a1, a2, sc, sf2, logit, route, bars, misc, total;
 };
-// A operand of the gate/up projection: the token's 8 term rows of one K step, 4 copies (one per lane quadrant of the
-// accumulator, so that each epilogue warp finds the token in its own quadrant), fetched by TMA with every stage of the
-// weight ring.  Row 32 q + t of ring stage s sits at (s / 4) * 16 KB + (s % 4) * 1 KB + q * 4 KB + t * 128: four stages
-// interleave inside one 16 KB operand span, each using the 8-row group the others leave empty.  The MMA of a stage
-// reads 128 rows from its own base (up to 3 KB past the span); rows it does not own hold other stages' data and feed
-// accumulator lanes nobody reads.
-__host__ __device__ inline uint32_t a1_slot(int s) { return static_cast<uint32_t>((s >> 2) * kATile + (s & 3) * 1024); }
-__host__ __device__ inline uint32_t a1_bytes(int) { return static_cast<uint32_t>((kWStages + 3) / 4) * kATile + 4096; }
+// B operand of the gate/up projection: the token's 8 term rows of one K step, 1 KB per ring stage; the MMAs read 16 rows from
+// there, of which the upper 8 - the next stage's, or the padding behind the last - feed columns nobody reads.
+constexpr int kA1Stage = 8 * 128;
 constexpr int kA2Bytes = 2048;  // B operand of the down projection: the 8 term rows of one K step (N = 16 reads 16 rows)
 __host__ __device__ inline OneSmem one_smem(int E, int H) {
   OneSmem m;
@@ -109,7 +108,8 @@ __host__ __device__ inline OneSmem one_smem(int E, int H) {
   m.ring = off;
   off += kWStages * kWStage;
   m.a1 = off;
-  off += a1_bytes(H);
+  off += (kWStages + 1) * kA1Stage;
+  off = (off + 1023u) & ~1023u;
   m.a2 = off;  // the term rows of the pair's slice of the intermediate, row t at t * 128 (1024-byte aligned)
   off += kA2Bytes;
   m.sc = off;
@@ -139,9 +139,7 @@ MOE_DEVINL uint32_t map_to_cta(uint32_t local_smem_addr, uint32_t cta_rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_smem_addr), "r"(cta_rank));
   return r;
 }
-MOE_DEVINL void st_cluster_u16(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(addr), "h"(static_cast<unsigned short>(v)) : "memory");
-}
+MOE_DEVINL void st_cluster_u32(uint32_t addr, uint32_t v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 MOE_DEVINL void st_cluster_u8(uint32_t addr, uint32_t v) {
   asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
@@ -174,9 +172,8 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
   uint64_t* empty_sc = full_sc + kScStages;   // [kScStages] scale warps -> producer
   uint64_t* sf_full = empty_sc + kScStages;   // [kSfGroups] scale warps -> MMA
   uint64_t* sf_free = sf_full + kSfGroups;    // [kSfGroups] MMA done -> scale warps
-  uint64_t* acc_full = sf_free + kSfGroups;   // [2, the second unused] MMA -> epilogue
-  uint64_t* acc_empty = acc_full + 2;         // [2, the second unused] epilogue -> MMA
-  uint64_t* act_ready = acc_empty + 2;        // epilogue warps -> MMA: an A operand and its scale factors are in place
+  uint64_t* acc_full = sf_free + kSfGroups;   // MMA -> epilogue
+  uint64_t* act_ready = acc_full + 1;         // epilogue warps -> MMA: an A operand and its scale factors are in place
   uint64_t* route_ready = act_ready + 1;      // routing warp -> producer
   uint64_t* split_ready = route_ready + 1;    // routing warp -> producer: the token's term rows are complete in global memory
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + sm.misc);
@@ -218,7 +215,7 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
     for (int s = 0; s < kWStages; ++s) { mbar_init(&full_w[s], 1); mbar_init(&empty_w[s], 1); }
     for (int s = 0; s < kScStages; ++s) { mbar_init(&full_sc[s], 1); mbar_init(&empty_sc[s], 4); }
     for (int s = 0; s < kSfGroups; ++s) { mbar_init(&sf_full[s], 4); mbar_init(&sf_free[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 4); }
+    mbar_init(acc_full, 1);
     mbar_init(act_ready, 4);
     mbar_init(route_ready, 1);
     mbar_init(split_ready, 1);
@@ -235,27 +232,9 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
   const int q = wid & 3;                         // tensor-memory lane quadrant this warp may access; also its scheduler
   const uint32_t lane_base = static_cast<uint32_t>(q * 32) << 16;
   const int jl = lane >> 3, tl = lane & 7;
-  const int cb = 16 * (tl & 1) + 8 * ((tl >> 1) & 1) + 4 * (tl >> 2);  // column offset a lane ends up with (see reduce8)
   const uint32_t sA2_u = smem_u32(sA2), sSf2_u = smem_u32(sSf2);
   const int n_blk = a.H / 32;
   const int n_split_ctas = n_blk / 8;            // the first CTAs (the earliest to start) split the token row, 8 blocks each
-
-  // Accumulator lane = term row.  A 32x32b load hands each lane 32 columns of its row; three exchange rounds over the
-  // 8 lanes of the token (each halves the columns a lane keeps) leave lane t with the 8-term sums of 4 consecutive
-  // columns, at offset cb of the 32.
-  auto reduce8 = [&](const uint32_t (&vc)[32], float (&o)[4]) {
-    float a16[16], a8[8];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const float lo = __uint_as_float(vc[k]), hi = __uint_as_float(vc[16 + k]);
-      a16[k] = ((tl & 1) ? hi : lo) + __shfl_xor_sync(0xffffffffu, (tl & 1) ? lo : hi, 1);
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      a8[k] = ((tl & 2) ? a16[8 + k] : a16[k]) + __shfl_xor_sync(0xffffffffu, (tl & 2) ? a16[k] : a16[8 + k], 2);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) o[k] = ((tl & 4) ? a8[4 + k] : a8[k]) + __shfl_xor_sync(0xffffffffu, (tl & 4) ? a8[k] : a8[4 + k], 4);
-  };
 
   // Every thread waits for the kernel launched before this one on the stream (logits and the token row may be its
   // outputs; the counter block is clear once it has completed) and looks at the two words nobody ever writes.
@@ -304,7 +283,7 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
             if (++cs == kScStages) { cs = 0; cph ^= 1u; }
           }
           mbar_wait(&empty_w[s], ph ^ 1u, a.status);
-          mbar_expect_tx(&full_w[s], phase == 0 ? kWStage + 4 * 1024 : kWStage);
+          mbar_expect_tx(&full_w[s], phase == 0 ? kWStage + kA1Stage : kWStage);
           const int wx = blocked ? 0 : ks * 128;
           const int wya = blocked ? ((wrow_a >> 7) * n_steps + ks) * 128 : wrow_a;
           const int wyb = blocked ? ((wrow_b >> 7) * n_steps + ks) * 128 : wrow_b;
@@ -317,9 +296,7 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
               fence_proxy_async_all();  // the rows were written through the generic proxy, TMA reads through the async one
               MOE_TP(20);
             }
-#pragma unroll
-            for (int qq = 0; qq < 4; ++qq)
-              tma_load_2d(sA1 + a1_slot(s) + qq * 4096, &tmap_a1, ks * 128, (item % kCopies) * kTerms, &full_w[s]);
+            tma_load_2d(sA1 + s * kA1Stage, &tmap_a1, ks * 128, (item % kCopies) * kTerms, &full_w[s]);
           }
           if (++s == kWStages) { s = 0; ph ^= 1u; }
         }
@@ -332,7 +309,7 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
       uint32_t ph = 0, sph = 0;
       const uint32_t d_addr = tmem_base + kColD;
       const uint32_t ring = smem_u32(sW), a1 = smem_u32(sA1), a2_addr = smem_u32(sA2);
-      // ---- gate/up: one accumulator over all K steps ----
+      // ---- gate/up: 128 gate rows and the 128 matching up rows, an accumulator each over all K steps ----
       mbar_wait_warp(act_ready, 0u, a.status);
       tc_fence_after_sync();
       if (lane == 0) MOE_TP(21);
@@ -343,9 +320,13 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
         tc_fence_after_sync();
         if (ks == 0 && lane == 0) MOE_TP(7);
         // scale words: 4 columns apart for the term rows, 8 for the 256 weight rows of a group
-        umma_mxf4_step<4, 8>(d_addr, umma_desc_k_sw128(a1 + a1_slot(s)), umma_desc_k_sw128(ring + static_cast<uint32_t>(s * kWStage)),
-                             idesc_mxf4(), tmem_base + kColSfAct + static_cast<uint32_t>(ks * 8),
-                             tmem_base + kColSfW + static_cast<uint32_t>(slotg * 32 + (ks & 1) * 16), ks != 0 ? 1u : 0u);
+#pragma unroll
+        for (uint32_t b = 0; b < 2; ++b)
+          umma_mxf4_step<8, 4>(tmem_base + (b == 0 ? kColGate : kColUp),
+                               umma_desc_k_sw128(ring + static_cast<uint32_t>(s * kWStage) + b * (128u * 128u)),
+                               umma_desc_k_sw128(a1 + static_cast<uint32_t>(s * kA1Stage)), idesc_mxf4(16u),
+                               tmem_base + kColSfW + static_cast<uint32_t>(slotg * 32 + (ks & 1) * 16) + b * 4,
+                               tmem_base + kColSfAct + static_cast<uint32_t>(ks * 8), ks != 0 ? 1u : 0u);
         umma_commit_elect(&empty_w[s]);
         if (++s == kWStages) { s = 0; ph ^= 1u; }
         if ((ks & 1) == 1) {
@@ -353,14 +334,11 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
           if (++slotg == kSfGroups) { slotg = 0; sph ^= 1u; }
         }
       }
-      umma_commit_elect(&acc_full[0]);
+      umma_commit_elect(acc_full);
       if (lane == 0) MOE_TP(8);
-      // ---- down: a single K step.  The operands change places: the 128 weight rows of a sub-tile are the M side, the
-      // 8 term rows of the pair's slice the N side (N = 16, the smallest; its upper 8 rows are never looked at), so the
-      // accumulator of a sub-tile is 16 columns and those of all H/256 sub-tiles of this CTA sit side by side in the
-      // 256 columns: no accumulator is handed back and forth with the epilogue, which reads them all once at the end ----
+      // ---- down: a single K step; the accumulators of all H/256 sub-tiles of this CTA sit side by side in the 256 columns: none
+      // is handed back and forth with the epilogue, which reads them all once at the end ----
       mbar_wait_warp(act_ready, 1u, a.status);
-      mbar_wait_warp(&acc_empty[0], 0u, a.status);  // the gate/up accumulator has been read
       tc_fence_after_sync();
       if (lane == 0) MOE_TP(9);
       for (int n = 0; n < n_t1; ++n) {
@@ -378,7 +356,7 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
         if (++s == kWStages) { s = 0; ph ^= 1u; }
         if (++slotg == kSfGroups) { slotg = 0; sph ^= 1u; }
       }
-      umma_commit_elect(&acc_full[0]);
+      umma_commit_elect(acc_full);
       if (lane == 0) MOE_TP(10);
     }
   } else {
@@ -541,47 +519,47 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
       // times, and its first real use, which is on the critical path, would otherwise pay for fetching it.
       for (int sweep = 0; sweep < 2; ++sweep) {
         const bool dry = sweep == 0;
-        // ---- gate/up accumulator: gate chunk q and up chunk 4 + q of the 8 chunks of 32 columns ----
+        // ---- gate/up accumulators: lane = i, the 8 terms in 8 columns ----
         if (!dry) {
-          mbar_wait(&acc_full[0], 0u, a.status);
+          mbar_wait(acc_full, 0u, a.status);
           if (wid == 6 && lane == 0) MOE_TP(13);
         }
         __syncwarp();  // tcgen05.ld is warp-collective
         tc_fence_after_sync();
-        float gsel[4], usel[4];
-        {
-          uint32_t vg[32], vu[32];
-          tmem_ld_32x32(tmem_base + lane_base + kColD + static_cast<uint32_t>(32 * q), vg);
-          tmem_ld_32x32(tmem_base + lane_base + kColD + static_cast<uint32_t>(32 * (4 + q)), vu);
-          tmem_ld_wait();
-          tc_fence_before_sync();
-          __syncwarp();
-          if (!dry && lane == 0) mbar_arrive(&acc_empty[0]);  // the accumulator is free for the down projection
-          reduce8(vg, gsel);
-          reduce8(vu, usel);
-        }
+        uint32_t vv[32];  // 16 columns of gate, 16 of up
+        tmem_ld_32x32(tmem_base + lane_base + kColGate, vv);
+        tmem_ld_wait();
         {
           // SwiGLU, bf16 rounding (the intermediate is defined as a bf16 value) and the 8-term split of this warp's block
           // of 32: block q of this CTA's four = 16-byte chunk rank * 4 + q of the pair's 128-byte K step.  The rows go
           // to this CTA's operand and to the partner's.
-          float r[1][4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const float sv = __fdividef(gsel[c], 1.0f + __expf(-gsel[c])) * usel[c];
-            r[0][c] = __bfloat162float(__float2bfloat16_rn(sv));
+          auto sum8 = [&](int o) {
+            auto f = [&](int i) { return __uint_as_float(vv[o + i]); };
+            return ((f(0) + f(1)) + (f(2) + f(3))) + ((f(4) + f(5)) + (f(6) + f(7)));
+          };
+          const float g = sum8(0), u = sum8(16);
+          float r = __bfloat162float(__float2bfloat16_rn(__fdividef(g, 1.0f + __expf(-g)) * u));
+          const uint32_t keep = r != r ? 0u : 0x7FFFFFFFu;  // (a NaN does not take part in its block's maximum)
+          uint32_t word = 0u, sb = 0u;  // nibble t: code of term t
+#pragma unroll 1
+          for (int t = 0; t < kTerms; ++t) {
+            const uint32_t amax = __reduce_max_sync(0xffffffffu, __float_as_uint(r) & keep);
+            const int se = amax != 0u ? term_exp(__uint_as_float(amax)) : 0;
+            float qv, unused;
+            word |= (e2m1_pair(r * pow2f(-se), 0.0f, &qv, &unused) & 15u) << (4 * t);
+            r = fmaf(-qv, pow2f(se), r);
+            if (tl == t) sb = static_cast<uint32_t>(se + 127);
           }
-          const bool live = !dry && jl == 0;
-          split_terms<1>(r, [&](int, int t, uint32_t bytes, int se) {
-            if (live) {
-              const uint32_t off = static_cast<uint32_t>(t * 128) + ((chunk ^ static_cast<uint32_t>(t)) << 4) + static_cast<uint32_t>(cb >> 1);
-              asm volatile("st.shared.u16 [%0], %1;" ::"r"(sA2_u + off), "h"(static_cast<unsigned short>(bytes)) : "memory");
-              st_cluster_u16(peer_a2 + off, bytes);
-              if (tl == 0) {
-                sSf2[t * 8 + static_cast<int>(chunk)] = static_cast<uint8_t>(se + 127);
-                st_cluster_u8(peer_sf2 + static_cast<uint32_t>(t * 8) + chunk, static_cast<uint32_t>(se + 127));
-              }
+          word = transpose_8x8_nibbles(word, lane);  // lane: eight consecutive values of term tl
+          if (!dry) {
+            const uint32_t off = static_cast<uint32_t>(tl * 128) + ((chunk ^ static_cast<uint32_t>(tl)) << 4) + static_cast<uint32_t>(jl * 4);
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(sA2_u + off), "r"(word) : "memory");
+            st_cluster_u32(peer_a2 + off, word);
+            if (jl == 0) {
+              sSf2[tl * 8 + static_cast<int>(chunk)] = static_cast<uint8_t>(sb);
+              st_cluster_u8(peer_sf2 + static_cast<uint32_t>(tl * 8) + chunk, sb);
             }
-          });
+          }
         }
         if (!dry) {
           if (wid == 6 && lane == 0) MOE_TP(14);
@@ -605,7 +583,7 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
         }
         // ---- down accumulators, all sub-tiles at once: lane = weight row of the sub-tile, 16 columns per sub-tile of
         // which the first 8 are the 8 terms; their sum, in ascending term order, is the row's partial sum ----
-        if (!dry) mbar_wait(&acc_full[0], 1u, a.status);
+        if (!dry) mbar_wait(acc_full, 1u, a.status);
         __syncwarp();
         tc_fence_after_sync();
         for (int u0 = 0; u0 < (dry ? 2 : 2 * n_t1); u0 += 2) {  // two sub-tiles (32 columns) per load
