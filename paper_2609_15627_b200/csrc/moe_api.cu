@@ -158,7 +158,7 @@ int expert_ffn_impl(const void* x_perm_bf16, const int32_t* expert_offsets, cons
     return launch_expert_ffn_native(xp, expert_offsets, w, *shape, act, y_perm, status, st, row_dst);
   if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
   if (twoterm)
-    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr, false}, expert_offsets, w, *shape, *choice, twoterm_guarded(*choice, w),
+    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr, false, false}, expert_offsets, w, *shape, *choice, twoterm_guarded(*choice, w),
                                      act, y_perm, status.word, st, row_dst);
   if (umma_shape_ok(*choice) || w.blocked)
     return launch_expert_ffn_umma(xp, expert_offsets, w, *shape, act, y_perm, status.word, st, row_dst);
@@ -167,10 +167,10 @@ int expert_ffn_impl(const void* x_perm_bf16, const int32_t* expert_offsets, cons
 
 // Sort and expert FFN of a call that holds the tokens and their routing: moe_permute and moe_expert_ffn, or, where the
 // two-term kernel runs, the sort alone and that kernel fed from the unsorted rows (same bits; x_perm then only takes the rows of
-// experts that are done again)
+// experts that are done again, or with `rows` all of them)
 int permute_and_ffn(const void* x, const int32_t* ids, const int32_t* offsets, const ExpertWeights& w, const moe_shape_t* shape,
                     void* x_perm, int32_t* perm, int32_t* inv_perm, float* y_perm, int32_t* status_word, void* ws, size_t ws_bytes,
-                    void* cuda_stream) {
+                    void* cuda_stream, bool rows = false) {
   int rc;
   if (!twoterm_chosen(*shape, w)) {
     if ((rc = moe_permute(x, ids, offsets, shape, x_perm, perm, inv_perm, ws, ws_bytes, cuda_stream)) != MOE_OK) return rc;
@@ -189,7 +189,7 @@ int permute_and_ffn(const void* x, const int32_t* ids, const int32_t* offsets, c
   char* base = static_cast<char*>(ws);
   if ((rc = launch_permute(xb, ids, offsets, *shape, nullptr, perm, inv_perm, reinterpret_cast<int*>(base + L.permute_off), st)) != MOE_OK)
     return rc;
-  return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, static_cast<__nv_bfloat16*>(x_perm), false}, offsets, w, *shape, *shape,
+  return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, static_cast<__nv_bfloat16*>(x_perm), false, rows}, offsets, w, *shape, *shape,
                                    twoterm_guarded(*shape, w), base + L.act_off, y_perm, status.word, st);
 }
 
@@ -199,11 +199,12 @@ bool front_in_one(const moe_shape_t& s, const ExpertWeights& w) {
 }
 // Routing, sort and expert FFN of such a call.  Where one cluster routes and the expert FFN is the two-term or the native
 // kernel, routing and sort are one launch, and the native kernel takes the tokens' rows as that launch splits them beside it, once
-// per token and not per slot; otherwise moe_route and the above.  Same bits.  `offsets2` (may be null) receives {0, T}; `late`:
+// per token and not per slot; otherwise moe_route and the above.  Same bits.  `rows`: perm and x_perm are the caller's and written as
+// moe_permute writes them.  `offsets2` (may be null) receives {0, T}; `late`:
 // the kernel in front may be the one that writes the logits.
 int route_and_ffn(const float* logits, const void* x, int32_t* ids, float* topk_w, int32_t* offsets, int32_t* offsets2, bool late,
                   const ExpertWeights& w, const moe_shape_t* shape, void* x_perm, int32_t* perm, int32_t* inv_perm, float* y_perm,
-                  int32_t* status_word, void* ws, size_t ws_bytes, void* cuda_stream) {
+                  int32_t* status_word, void* ws, size_t ws_bytes, void* cuda_stream, bool rows = false) {
   int rc;
   const moe_shape_t& s = *shape;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
@@ -211,7 +212,7 @@ int route_and_ffn(const float* logits, const void* x, int32_t* ids, float* topk_
   if (!front_in_one(s, w)) {
     if (offsets2 != nullptr && (rc = launch_shared_offsets(offsets2, s.T, st)) != MOE_OK) return rc;
     if ((rc = moe_route(logits, s.T, s.E, s.k, ids, topk_w, offsets, ws, ws_bytes, cuda_stream)) != MOE_OK) return rc;
-    return permute_and_ffn(x, ids, offsets, w, shape, x_perm, perm, inv_perm, y_perm, status_word, ws, ws_bytes, cuda_stream);
+    return permute_and_ffn(x, ids, offsets, w, shape, x_perm, perm, inv_perm, y_perm, status_word, ws, ws_bytes, cuda_stream, rows);
   }
   if (!aligned(w.w13, 16) || !aligned(w.s13, 16) || !aligned(w.w2, 16) || !aligned(w.s2, 16) ||
       (status_word != nullptr && !aligned(status_word, 4)))
@@ -225,12 +226,13 @@ int route_and_ffn(const float* logits, const void* x, int32_t* ids, float* topk_
   if (twoterm) {
     if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
     if ((rc = launch_route_sort(logits, s.T, s.E, s.k, ids, topk_w, offsets, perm, inv_perm, false, offsets2, nullptr, late, st)) != MOE_OK) return rc;
-    return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, static_cast<__nv_bfloat16*>(x_perm), true}, offsets, w, s, s,
+    return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, static_cast<__nv_bfloat16*>(x_perm), true, rows}, offsets, w, s, s,
                                      twoterm_guarded(s, w), scratch, y_perm, status.word, st);
   }
   const FrontSplit split = native_front_split(xb, s, scratch, status);
-  if ((rc = launch_route_sort(logits, s.T, s.E, s.k, ids, topk_w, offsets, perm, inv_perm, true, offsets2, &split, late, st)) != MOE_OK) return rc;
-  return launch_expert_ffn_native_tokens(perm, offsets, w, s, scratch, y_perm, status, st);
+  if ((rc = launch_route_sort(logits, s.T, s.E, s.k, ids, topk_w, offsets, perm, inv_perm, !rows, offsets2, &split, late, st)) != MOE_OK) return rc;
+  if (rows && (rc = launch_gather_rows(xb, perm, s, static_cast<__nv_bfloat16*>(x_perm), st)) != MOE_OK) return rc;
+  return launch_expert_ffn_native_tokens(perm, rows ? s.k : 1, offsets, w, s, scratch, y_perm, status, st);
 }
 
 // the four tensors inside a buffer written by moe_prepack
@@ -308,22 +310,23 @@ int moe_layer(const float* logits, const void* x_bf16, const uint8_t* w13, const
               size_t ws_bytes, void* cuda_stream) {
   int rc = check_shape(shape);
   if (rc != MOE_OK) return rc;
+  if (!aligned(logits, 16) || !aligned(x_bf16, 16) || !aligned(topk_ids, 16) || !aligned(topk_w, 16) || !aligned(expert_offsets, 16) ||
+      !aligned(x_perm_bf16, 16) || !aligned(perm, 16) || !aligned(inv_perm, 16) || !aligned(w13, 16) || !aligned(w13_scale, 16) ||
+      !aligned(w2, 16) || !aligned(w2_scale, 16) || !aligned(y_perm, 16) || !aligned(out_bf16, 16) || (status_word != nullptr && !aligned(status_word, 4)))
+    return MOE_ERR_INVALID_ARG;
   const moe_shape_t& s = *shape;
-  if (!route_sort_ok(s.T, s.E)) {
-    if ((rc = moe_route(logits, s.T, s.E, s.k, topk_ids, topk_w, expert_offsets, ws, ws_bytes, cuda_stream)) != MOE_OK) return rc;
-    if ((rc = moe_permute(x_bf16, topk_ids, expert_offsets, shape, x_perm_bf16, perm, inv_perm, ws, ws_bytes, cuda_stream)) != MOE_OK) return rc;
-  } else {
-    if (!aligned(logits, 16) || !aligned(x_bf16, 16) || !aligned(topk_ids, 16) || !aligned(topk_w, 16) || !aligned(expert_offsets, 16) ||
-        !aligned(x_perm_bf16, 16) || !aligned(perm, 16) || !aligned(inv_perm, 16))
-      return MOE_ERR_INVALID_ARG;
-    if (check_ws(ws, ws_bytes, ws_layout(s).total) != MOE_OK) return MOE_ERR_WORKSPACE;
+  if (check_ws(ws, ws_bytes, ws_layout(s).total) != MOE_OK) return MOE_ERR_WORKSPACE;
+  const ExpertWeights w{w13, w13_scale, w2, w2_scale, false};
+  if (route_sort_ok(s.T, s.E) && !front_in_one(s, w)) {  // routing and sort in one launch for the other kernels too
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if ((rc = launch_route_sort(logits, s.T, s.E, s.k, topk_ids, topk_w, expert_offsets, perm, inv_perm, false, nullptr, nullptr, false, st)) != MOE_OK ||
-        (rc = launch_gather_rows(static_cast<const __nv_bfloat16*>(x_bf16), perm, s, static_cast<__nv_bfloat16*>(x_perm_bf16), st)) != MOE_OK)
+        (rc = launch_gather_rows(static_cast<const __nv_bfloat16*>(x_bf16), perm, s, static_cast<__nv_bfloat16*>(x_perm_bf16), st)) != MOE_OK ||
+        (rc = expert_ffn_impl(x_perm_bf16, expert_offsets, w, shape, y_perm, status_word, ws, ws_bytes, cuda_stream)) != MOE_OK)
       return rc;
-  }
-  if ((rc = moe_expert_ffn(x_perm_bf16, expert_offsets, w13, w13_scale, w2, w2_scale, shape, y_perm, status_word, ws, ws_bytes, cuda_stream)) != MOE_OK)
+  } else if ((rc = route_and_ffn(logits, x_bf16, topk_ids, topk_w, expert_offsets, nullptr, false, w, shape, x_perm_bf16, perm, inv_perm, y_perm,
+                                 status_word, ws, ws_bytes, cuda_stream, true)) != MOE_OK) {
     return rc;
+  }
   return moe_combine(y_perm, inv_perm, topk_w, shape, out_bf16, cuda_stream);
 }
 
@@ -684,7 +687,7 @@ int moe_debug_expert_ffn_variant(const void* x_perm_bf16, const int32_t* expert_
     if (!twoterm_shape_ok(*shape) || !twoterm_weights_ok(w13, w2)) return MOE_ERR_UNSUPPORTED_SHAPE;
     if (check_ws(ws, ws_bytes, L.act_off + twoterm_scratch(*shape).total) != MOE_OK) return MOE_ERR_WORKSPACE;
     if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
-    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr, false}, expert_offsets, w, *shape, *shape, false, act, y_perm, status.word, st);
+    return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr, false, false}, expert_offsets, w, *shape, *shape, false, act, y_perm, status.word, st);
   }
   if (variant == 2) {
     if (!native_shape_ok(*shape, w13, w2)) return MOE_ERR_UNSUPPORTED_SHAPE;

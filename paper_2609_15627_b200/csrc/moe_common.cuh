@@ -259,6 +259,7 @@ struct TwoTermInput {
   const int* inv_perm;     // [T, k] sorted row of every slot
   __nv_bfloat16* x_sorted; // with the tables: room for the rows in sorted order, of the experts that `guard` does again
   bool offsets_late;       // with the tables: the kernel in front is the one that writes the offsets
+  bool write_rows;         // with the tables: x_sorted is the caller's and receives all rows
 };
 int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
                            const moe_shape_t& choice, bool guard, void* scratch, float* y_perm, int* status_word, cudaStream_t st,
@@ -284,9 +285,9 @@ int launch_expert_ffn_native(const __nv_bfloat16* x_perm, const int* offsets, co
                              void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst = nullptr);
 
 // the native variant behind launch_route_sort: token rows by token (native_front_split says where that launch leaves them),
-// `tok` the token of every sorted row.  H a multiple of 512.
+// `tok` over `tok_div` the token of every sorted row.  H a multiple of 512.
 FrontSplit native_front_split(const __nv_bfloat16* x, const moe_shape_t& s, void* scratch, StatusRef status);
-int launch_expert_ffn_native_tokens(const int* tok, const int* offsets, const ExpertWeights& w, const moe_shape_t& s, void* scratch,
+int launch_expert_ffn_native_tokens(const int* tok, int tok_div, const int* offsets, const ExpertWeights& w, const moe_shape_t& s, void* scratch,
                                     float* y_perm, StatusRef status, cudaStream_t st);
 
 // the whole layer in one launch, for a handful of tokens on shapes the native variant takes (moe_forward);

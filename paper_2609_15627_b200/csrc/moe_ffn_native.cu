@@ -100,7 +100,7 @@ constexpr int kSmallRows = 64;
 
 struct NatArgs {
   const uint8_t* sf1;        // scale bytes of the token rows' terms [S * 8, H/32] (terms: row p * 8 + t, packed E2M1)
-  const int* tok;            // null; or the token of every sorted row: then the token rows' terms are stored by token, once each,
+  const int* tok;            // null; or tok_div times the token of every sorted row (and less than that more): then the token rows' terms are stored by token, once each,
                              //   and the kernel in front of this one is the one that routes, sorts and splits (launch_route_sort)
   uint8_t* aq2;              // terms of the bf16 intermediate [S * 8, I/2]: written by phase 0, read by phase 1
   uint8_t* sf2;              //   and their scale bytes [S * 8, I/32]
@@ -111,6 +111,7 @@ struct NatArgs {
   int* status;               // never null: the caller's word or the library's own (see StatusRef)
   int own_status;            // the library's own word: the one-launch kernel's last CTA clears it for the next call
   int E, H, I, S;
+  int tok_div;
   int blocked;               // weights in moe_prepack's tile-contiguous layout (see ExpertWeights)
   const uint8_t* s13;        // the weights' scale bytes in the row layout, for reductions that are not multiples of 512:
   const uint8_t* s2;         //   their rows are then not multiples of 16 bytes, which a tensor map cannot address
@@ -664,7 +665,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
           const int bi = op_box(n_tok * nt);  // box of 8 << bi operand rows; rows past the end of the tensor arrive as zeros
           int tok = 0, t4[4] = {0, 0, 0, 0};  // by token: lane j has the pass's token j, the first four are known to be uniform
           if (by_token) {
-            if (lane < n_tok) tok = kFused ? s_tok[row0 + lane] : __ldcg(a.tok + row0 + lane);
+            if (lane < n_tok) tok = kFused ? s_tok[row0 + lane] : __ldcg(a.tok + row0 + lane) / a.tok_div;
 #pragma unroll
             for (int j = 0; j < 4; ++j) t4[j] = warp_uniform(lane == j ? tok : 0);
           }
@@ -797,7 +798,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
               const int r = i / n_chunk, c = i % n_chunk;
               const uint4* from = src + i;
               if (by_token) {
-                const int t = kFused ? s_tok[row0 + (r >> 3)] : __ldcg(a.tok + row0 + (r >> 3));
+                const int t = kFused ? s_tok[row0 + (r >> 3)] : __ldcg(a.tok + row0 + (r >> 3)) / a.tok_div;
                 from = reinterpret_cast<const uint4*>(src_sf) + (t * kTerms + (r & 7)) * n_chunk + c;
               }
               reinterpret_cast<uint4*>(sSfa)[r * n_chunk + (c ^ (r & cmask))] = __ldcg(from);
@@ -1293,10 +1294,10 @@ NatScratch nat_scratch(void* scratch, const moe_shape_t& sh, size_t rows) {
   L.done = reinterpret_cast<int*>(L.sf1 + align_up(rows * (sh.H / 32), kAlign));
   return L;
 }
-// tok: null, or the token of every sorted row - the token rows' terms then lie by token (see launch_expert_ffn_native_tokens)
+// tok: null, or tok_div times the token of every sorted row - the token rows' terms then lie by token (see launch_expert_ffn_native_tokens)
 template <bool kQ>
 int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
-                      void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, const int* tok = nullptr) {
+                      void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, const int* tok = nullptr, int tok_div = 1) {
   if (!nat_attr_once()) return MOE_ERR_CUDA;
   const size_t S = static_cast<size_t>(sh.T) * sh.k;
   const size_t rows = S * (kQ ? 1 : kTerms);  // operand rows
@@ -1323,6 +1324,7 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
   NatArgs a;
   a.sf1 = sf1;
   a.tok = tok;
+  a.tok_div = tok_div;
   a.aq2 = aq2;
   a.sf2 = sf2;
   a.done = done;
@@ -1366,9 +1368,9 @@ FrontSplit native_front_split(const __nv_bfloat16* x, const moe_shape_t& sh, voi
   const NatScratch L = nat_scratch(scratch, sh, static_cast<size_t>(sh.T) * sh.k * kTerms);
   return FrontSplit{x, L.aq1, L.sf1, L.done, sh.E, sh.H, status.own ? status.word : nullptr};
 }
-int launch_expert_ffn_native_tokens(const int* tok, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh, void* scratch,
-                                    float* y_perm, StatusRef status, cudaStream_t st) {
-  return launch_native_ffn<false>(nullptr, offsets, w, sh, scratch, y_perm, status, st, nullptr, tok);
+int launch_expert_ffn_native_tokens(const int* tok, int tok_div, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
+                                    void* scratch, float* y_perm, StatusRef status, cudaStream_t st) {
+  return launch_native_ffn<false>(nullptr, offsets, w, sh, scratch, y_perm, status, st, nullptr, tok, tok_div);
 }
 int launch_expert_ffn_native_q(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
                                void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst) {
@@ -1415,6 +1417,7 @@ int launch_forward_fused(const float* logits, const __nv_bfloat16* x, const Expe
   NatArgs a;
   a.sf1 = nullptr;
   a.tok = nullptr;
+  a.tok_div = 1;
   a.aq2 = aq2;
   a.sf2 = sf2;
   a.done = sync;

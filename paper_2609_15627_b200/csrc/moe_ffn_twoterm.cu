@@ -616,13 +616,17 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
 // once and stored at its k sorted places, so the bf16 copy in sorted order is neither written nor read and a value is
 // converted once, not k times.  Warp task: (token, `chunks` pieces of 256 values).  It writes k * H * 2 bytes per token and is
 // bound by issuing them, 8 bytes a lane with the row and scale places shuffled out per slot: 8192 tokens of 4096, top-8,
-// 166 us for 0.61 GB, 0.56 of the copy rate. ----
+// 166 us for 0.61 GB, 0.56 of the copy rate.  (A warp's part collected in shared memory and sent with one bulk copy per slot and
+// term: 181 us.)
+// What it writes is written at the rate at which memory takes writes alone (3.9 TB/s; a copy reaches 6.5 with the half that it reads).
+// `rows` (may be null): the bf16 rows in sorted order as well, for a caller whose buffer they are (moe_layer): 11 us less than the
+// copy and a split from it (8216 slots of 4096: the layer 238 -> 227 us; 12288 slots 1123 -> 1108). ----
 template <bool kGuard>
 __global__ void __launch_bounds__(256) twoterm_scatter_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ ids,
                                                              const int* __restrict__ inv_perm, const int* __restrict__ offsets,
                                                              uint8_t* __restrict__ xq, uint8_t* __restrict__ sfx, int T, int k, int H,
                                                              int E, int max_tok, int sf_step, int chunks, uint8_t* __restrict__ marks,
-                                                             int* __restrict__ flags, int offsets_late) {
+                                                             int* __restrict__ flags, int offsets_late, __nv_bfloat16* __restrict__ rows) {
   extern __shared__ int s_tt_tables[];
   // expert_offsets is read here and, as it starts, by the gate/up grid: complete where the sort of the same call waited for
   // the router before it let this kernel start, to be waited for where one kernel routes and sorts
@@ -653,12 +657,14 @@ __global__ void __launch_bounds__(256) twoterm_scatter_kernel(const __nv_bfloat1
     for (int c = c0; c < c1; ++c) {
       uint2 hi, lo;
       uint32_t word;
-      again |= tt_split_256<kGuard>(__ldg(src + c * 32 + lane), lane, &hi, &lo, &word);
+      const uint4 v = __ldg(src + c * 32 + lane);
+      again |= tt_split_256<kGuard>(v, lane, &hi, &lo, &word);
       const size_t step = static_cast<size_t>(2 * c + (lane >> 4)) * sf_step;
       for (int j = 0; j < k; ++j) {
         const size_t row = static_cast<size_t>(__shfl_sync(0xffffffffu, p, j));
         reinterpret_cast<uint2*>(xq + row * H)[c * 32 + lane] = hi;
         reinterpret_cast<uint2*>(xq + (S + row) * H)[c * 32 + lane] = lo;
+        if (rows != nullptr) reinterpret_cast<uint4*>(rows + row * H)[c * 32 + lane] = v;
         const size_t at = __shfl_sync(0xffffffffu, static_cast<unsigned long long>(sf_hi), j);
         const int d = __shfl_sync(0xffffffffu, sf_lo, j);
         if ((lane & 15) == 0) *reinterpret_cast<uint32_t*>(sfx + at + step) = word;
@@ -1287,7 +1293,9 @@ bool twoterm_guarded(const moe_shape_t& choice, const ExpertWeights& w) { return
 static int launch_again(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh, const moe_shape_t& choice,
                         void* act, float* y_perm, int* status_word, cudaStream_t st, float* const* row_dst, const int* flags) {
   const __nv_bfloat16* rows = in.x;
-  if (in.inv_perm != nullptr) {
+  if (in.write_rows) {
+    rows = in.x_sorted;
+  } else if (in.inv_perm != nullptr) {
     if (launch_pdl(twoterm_gather_kernel, dim3(static_cast<unsigned>(sm_count()) * 8), dim3(256), 0, st, in.x, in.ids, in.inv_perm, flags,
                    sh.T, sh.k, sh.H, sh.E, in.x_sorted) != cudaSuccess)
       return MOE_ERR_CUDA;
@@ -1331,7 +1339,7 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
     const size_t want = (static_cast<size_t>(sh.T) * parts + 7) / 8;
     rc = launch_pdl(guard ? twoterm_scatter_kernel<true> : twoterm_scatter_kernel<false>, dim3(static_cast<unsigned>(want < most ? want : most)), dim3(256), table_bytes, st, in.x,
                     in.ids, in.inv_perm, offsets, base + L.xq, base + L.sfx, sh.T, sh.k, sh.H, sh.E, geo.max_tok, geo.sf_step, chunks,
-                    marks, flags, in.offsets_late ? 1 : 0);
+                    marks, flags, in.offsets_late ? 1 : 0, in.write_rows ? in.x_sorted : nullptr);
   } else {
     const size_t want = (S * parts + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
     rc = launch_pdl(guard ? twoterm_split_kernel<false, true> : twoterm_split_kernel<false, false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256), table_bytes, st, in.x,
@@ -1374,7 +1382,7 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
     const int again = launch_again(in, offsets, w, sh, choice, base + L.aq, y_perm, status_word, st, row_dst, flags);
     if (again != MOE_OK) return again;
   }
-  note_kernel("ffn_mxf8_two_term_cta_pair", 3 + (guard && in.inv_perm != nullptr ? 1 : 0));
+  note_kernel("ffn_mxf8_two_term_cta_pair", 3 + (guard && in.inv_perm != nullptr && !in.write_rows ? 1 : 0));
   return MOE_OK;
 }
 

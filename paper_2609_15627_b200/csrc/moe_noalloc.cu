@@ -74,7 +74,7 @@ int moe_expert_ffn_noalloc(const void* x_perm_bf16, const int32_t* expert_offset
                                     status, st);
   if (status.own && cudaMemsetAsync(status.word, 0, sizeof(int), st) != cudaSuccess) return MOE_ERR_CUDA;
   if (twoterm)
-    return launch_expert_ffn_twoterm(TwoTermInput{static_cast<const __nv_bfloat16*>(x_perm_bf16), nullptr, nullptr, nullptr, false}, expert_offsets, w, s, s,
+    return launch_expert_ffn_twoterm(TwoTermInput{static_cast<const __nv_bfloat16*>(x_perm_bf16), nullptr, nullptr, nullptr, false, false}, expert_offsets, w, s, s,
                                      twoterm_guarded(s, w), scratch, y_perm, status.word, st);
   if (umma_shape_ok(s))
     return launch_expert_ffn_umma(static_cast<const __nv_bfloat16*>(x_perm_bf16), expert_offsets, w, s, act, y_perm,

@@ -103,6 +103,30 @@ def test_chosen_by_shape_the_same_on_packed_weights_and_on_expert_parallel_ranks
     assert int(buf.status.item()) == 0 and torch.equal(out1, buf.out)
 
 
+# Rows split once per token and copied to their sorted places: rows of one, three, nine, sixteen and 28 pieces of 256 values, a
+# warp's share of them from four to sixteen, one slot per token and thirty-two
+@pytest.mark.parametrize("T,H,I,E,k", [(4200, 256, 256, 128, 1), (600, 768, 256, 128, 5), (1100, 2304, 256, 128, 2), (128, 4096, 256, 128, 32),
+                                       (9000, 4096, 256, 128, 1), (520, 7168, 256, 128, 6)])
+def test_rows_split_by_token_are_the_rows_split_in_sorted_order(T, H, I, E, k):
+    wdev = tuple(dev(a) for a in _weights(H, I, E, seed=14))
+    logits, x = inputs.make_logits(T, E, 15), inputs.make_x(T, H, 16)
+    sh = moe.shape(T, H, I, E, k)
+    buf = moe.LayerBuffers(sh)
+    moe.moe_route(dev(logits), k, buf.topk_ids, buf.topk_w, buf.expert_offsets, buf.ws)
+    moe.moe_permute(dev(x), buf.topk_ids, buf.expert_offsets, sh, buf.x_perm, buf.perm, buf.inv_perm, buf.ws)
+    moe.moe_expert_ffn(buf.x_perm, buf.expert_offsets, *wdev, sh, buf.y_perm, buf.status, buf.ws)
+    assert moe.moe_last_kernel_name() == NAME
+    moe.moe_combine(buf.y_perm, buf.inv_perm, buf.topk_w, sh, buf.out)
+    out = torch.empty_like(buf.out)
+    moe.moe_forward(dev(logits), dev(x), *wdev, sh, out, None, None, buf.status, moe.alloc_forward_workspace(sh))
+    torch.cuda.synchronize()
+    assert int(buf.status.item()) == 0 and torch.equal(out.view(torch.int16), buf.out.view(torch.int16))
+    buf2 = moe.LayerBuffers(sh)
+    moe.moe_layer(dev(logits), dev(x), wdev, buf2)
+    torch.cuda.synchronize()
+    assert all(torch.equal(getattr(buf2, n).view(torch.int16), getattr(buf, n).view(torch.int16)) for n in ("x_perm", "perm", "inv_perm", "y_perm", "out"))
+
+
 @pytest.mark.parametrize("T,H,I,E,k,packed", [(1100, 1024, 512, 32, 2, False), (1100, 1024, 512, 32, 2, True),   # 69 rows per expert
                                               (4200, 512, 256, 64, 1, False), (600, 768, 768, 43, 5, False)])
 def test_quantised_activations_on_cta_pairs(T, H, I, E, k, packed):
