@@ -225,14 +225,14 @@ int route_and_ffn(const float* logits, const void* x, int32_t* ids, float* topk_
   char* scratch = static_cast<char*>(ws) + L.act_off;
   if (twoterm) {
     if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
-    if ((rc = launch_route_sort(logits, s.T, s.E, s.k, ids, topk_w, offsets, perm, inv_perm, false, offsets2, nullptr, late, st)) != MOE_OK) return rc;
+    if ((rc = launch_route_sort(logits, s.T, s.E, s.k, ids, topk_w, offsets, perm, inv_perm, offsets2, nullptr, late, st)) != MOE_OK) return rc;
     return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, static_cast<__nv_bfloat16*>(x_perm), true, rows}, offsets, w, s, s,
                                      twoterm_guarded(s, w), scratch, y_perm, status.word, st);
   }
   const FrontSplit split = native_front_split(xb, s, scratch, status);
-  if ((rc = launch_route_sort(logits, s.T, s.E, s.k, ids, topk_w, offsets, perm, inv_perm, !rows, offsets2, &split, late, st)) != MOE_OK) return rc;
+  if ((rc = launch_route_sort(logits, s.T, s.E, s.k, ids, topk_w, offsets, rows ? perm : nullptr, inv_perm, offsets2, &split, late, st)) != MOE_OK) return rc;
   if (rows && (rc = launch_gather_rows(xb, perm, s, static_cast<__nv_bfloat16*>(x_perm), st)) != MOE_OK) return rc;
-  return launch_expert_ffn_native_tokens(perm, rows ? s.k : 1, offsets, w, s, scratch, y_perm, status, st);
+  return launch_expert_ffn_native_tokens(offsets, w, s, scratch, y_perm, status, st);
 }
 
 // the four tensors inside a buffer written by moe_prepack
@@ -319,7 +319,7 @@ int moe_layer(const float* logits, const void* x_bf16, const uint8_t* w13, const
   const ExpertWeights w{w13, w13_scale, w2, w2_scale, false};
   if (route_sort_ok(s.T, s.E) && !front_in_one(s, w)) {  // routing and sort in one launch for the other kernels too
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if ((rc = launch_route_sort(logits, s.T, s.E, s.k, topk_ids, topk_w, expert_offsets, perm, inv_perm, false, nullptr, nullptr, false, st)) != MOE_OK ||
+    if ((rc = launch_route_sort(logits, s.T, s.E, s.k, topk_ids, topk_w, expert_offsets, perm, inv_perm, nullptr, nullptr, false, st)) != MOE_OK ||
         (rc = launch_gather_rows(static_cast<const __nv_bfloat16*>(x_bf16), perm, s, static_cast<__nv_bfloat16*>(x_perm_bf16), st)) != MOE_OK ||
         (rc = expert_ffn_impl(x_perm_bf16, expert_offsets, w, shape, y_perm, status_word, ws, ws_bytes, cuda_stream)) != MOE_OK)
       return rc;

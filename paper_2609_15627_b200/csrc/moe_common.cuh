@@ -43,6 +43,14 @@ inline size_t native_scratch_bytes(const moe_shape_t& s) {
          align_up(8 * S * (s.H / 32), kAlign) + align_up(static_cast<size_t>(s.E) * 4, kAlign);
 }
 
+// beside it, in moe_workspace_bytes() alone: the term rows by token of batches whose front is one launch (see launch_route_sort)
+constexpr int kFrontMaxTok = 256, kFrontMaxE = 256;
+inline size_t native_token_bytes(const moe_shape_t& s) {
+  if (s.T > kFrontMaxTok || s.E > kFrontMaxE) return 0;
+  return align_up(static_cast<size_t>(8) * s.T * (s.H / 2), kAlign) + align_up(static_cast<size_t>(8) * s.T * (s.H / 32), kAlign) +
+         align_up(static_cast<size_t>(s.T) * s.k * 4, kAlign);
+}
+
 // scratch of the quantised-activation variant: one operand row per sorted row (codes and scale bytes of the token rows
 // and of the intermediate) and the per-expert counters
 inline size_t native_q_scratch_bytes(const moe_shape_t& s) {
@@ -148,7 +156,7 @@ inline WsLayout ws_layout(const moe_shape_t& s) {
   off += align_up((static_cast<size_t>(s.E) + 8) * 4, kAlign);
   L.act_off = off;  // bf16 act[S,I], or the scratch of the native variant
   const size_t act_bytes = align_up(S * s.I * 2, kAlign);
-  const size_t nat_bytes = native_batch_ok(s) ? native_scratch_bytes(s) : 0;
+  const size_t nat_bytes = native_batch_ok(s) ? native_scratch_bytes(s) + native_token_bytes(s) : 0;
   const size_t twoterm_bytes = twoterm_batch_ok(s) ? twoterm_scratch(s).total : 0;
   size_t ffn_bytes = act_bytes > nat_bytes ? act_bytes : nat_bytes;
   ffn_bytes = ffn_bytes > twoterm_bytes ? ffn_bytes : twoterm_bytes;
@@ -217,19 +225,20 @@ void note_kernel(const char* name, int launches);
 int launch_route(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* counters,
                  cudaStream_t st);
 // Routing and stable sort in one launch, for batches that one thread-block cluster routes; beside it, where `split` is given, the
-// tokens' rows are split into E2M1 term rows, stored by token (split->n_done counters are cleared).  `order` (null: the
-// routing alone) receives slot t * k + j of every sorted row, or with `order_tokens` its token; offsets2 (may be null) {0, T};
-// `late`: the kernel in front may be the one that writes the logits.
+// tokens' rows are split into E2M1 term rows, stored by token (split->n_done counters are cleared).  inv_perm null: the routing
+// alone; perm, offsets2 ({0, T}) may be null; `late`: the kernel in front may be the one that writes the logits.
 struct FrontSplit {
   const __nv_bfloat16* x;
   uint8_t *aq, *sf;   // [T * 8, H / 2], [T * 8, H / 32]
   int* done;
   int n_done, H;
   int* status_clear;  // the library's own status word, or null
+  int* tok;           // token of every sorted row, the top bit set where its expert has more than `most` rows
+  int most;
 };
 bool route_sort_ok(int T, int E);
-int launch_route_sort(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* order, int* inv_perm,
-                      bool order_tokens, int* offsets2, const FrontSplit* split, bool late, cudaStream_t st);
+int launch_route_sort(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* perm, int* inv_perm, int* offsets2,
+                      const FrontSplit* split, bool late, cudaStream_t st);
 // the rows alone, in the order of a sort that is done (perm: slot of every sorted row)
 int launch_gather_rows(const __nv_bfloat16* x, const int* perm, const moe_shape_t& s, __nv_bfloat16* x_perm, cudaStream_t st);
 // (x_perm null: the sort alone, no rows are copied)
@@ -284,10 +293,10 @@ int launch_expert_ffn_native_q(const __nv_bfloat16* x_perm, const int* offsets, 
 int launch_expert_ffn_native(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
                              void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst = nullptr);
 
-// the native variant behind launch_route_sort: token rows by token (native_front_split says where that launch leaves them),
-// `tok` over `tok_div` the token of every sorted row.  H a multiple of 512.
+// the native variant behind launch_route_sort: token rows by token (native_front_split says where that launch leaves them).  H a
+// multiple of 512.
 FrontSplit native_front_split(const __nv_bfloat16* x, const moe_shape_t& s, void* scratch, StatusRef status);
-int launch_expert_ffn_native_tokens(const int* tok, int tok_div, const int* offsets, const ExpertWeights& w, const moe_shape_t& s, void* scratch,
+int launch_expert_ffn_native_tokens(const int* offsets, const ExpertWeights& w, const moe_shape_t& s, void* scratch,
                                     float* y_perm, StatusRef status, cudaStream_t st);
 
 // the whole layer in one launch, for a handful of tokens on shapes the native variant takes (moe_forward);

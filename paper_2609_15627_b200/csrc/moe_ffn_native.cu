@@ -100,8 +100,9 @@ constexpr int kSmallRows = 64;
 
 struct NatArgs {
   const uint8_t* sf1;        // scale bytes of the token rows' terms [S * 8, H/32] (terms: row p * 8 + t, packed E2M1)
-  const int* tok;            // null; or tok_div times the token of every sorted row (and less than that more): then the token rows' terms are stored by token, once each,
-                             //   and the kernel in front of this one is the one that routes, sorts and splits (launch_route_sort)
+  const int* tok;            // null; or the token of every sorted row (and a top bit): then the rows' terms are also stored by
+                             //   token, and only there for experts with at most tok_rows rows
+  const uint8_t* sf_tok;     //   scale bytes of those
   uint8_t* aq2;              // terms of the bf16 intermediate [S * 8, I/2]: written by phase 0, read by phase 1
   uint8_t* sf2;              //   and their scale bytes [S * 8, I/32]
   int* done;                 // [E] epilogue warps that have published a gate/up item of the expert
@@ -111,7 +112,7 @@ struct NatArgs {
   int* status;               // never null: the caller's word or the library's own (see StatusRef)
   int own_status;            // the library's own word: the one-launch kernel's last CTA clears it for the next call
   int E, H, I, S;
-  int tok_div;
+  int tok_rows;
   int blocked;               // weights in moe_prepack's tile-contiguous layout (see ExpertWeights)
   const uint8_t* s13;        // the weights' scale bytes in the row layout, for reductions that are not multiples of 512:
   const uint8_t* s2;         //   their rows are then not multiples of 16 bytes, which a tensor map cannot address
@@ -295,6 +296,34 @@ __global__ void __launch_bounds__(1024) native_quant_rows_kernel(const __nv_bflo
   }
 }
 
+// ---- the rows' terms by token -> in sorted order, where the router has set the top bit of the row's token: its expert has more
+// rows than are fetched by token.  A box of 8 rows takes the TMA unit 99 cycles, one of 128 rows 340, so fetching one by one is for
+// passes of a few tokens (110 tokens, heavily uneven experts: 437 us a layer with all rows by token).  A CTA per sorted row, a
+// warp per term. ----
+__global__ void __launch_bounds__(kTerms * 32) native_expand_kernel(const uint8_t* __restrict__ from, const uint8_t* __restrict__ sf_from,
+                                                                   const int* __restrict__ tok, int H, uint8_t* __restrict__ aq,
+                                                                   uint8_t* __restrict__ sf) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int p = static_cast<int>(blockIdx.x), v = __ldcg(tok + p);
+  if (v >= 0) return;
+  const size_t lane = threadIdx.x & 31, t = (static_cast<size_t>(v & 0x7FFFFFFF) * kTerms + (threadIdx.x >> 5)), r = static_cast<size_t>(p) * kTerms + (threadIdx.x >> 5);
+  const uint4* src = reinterpret_cast<const uint4*>(from + t * (H / 2));
+  uint4* dst = reinterpret_cast<uint4*>(aq + r * (H / 2));
+  const int n = H / 32, n_sf = H / 512;  // pieces of 16 bytes
+  uint4 c[4], s = {};
+  if (static_cast<int>(lane) < n_sf) s = __ldcg(reinterpret_cast<const uint4*>(sf_from + t * n) + lane);
+  for (int i = static_cast<int>(lane); i < n; i += 4 * 32) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i + 32 * u < n) c[u] = __ldcg(src + i + 32 * u);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i + 32 * u < n) dst[i + 32 * u] = c[u];
+  }
+  if (static_cast<int>(lane) < n_sf) reinterpret_cast<uint4*>(sf + r * n)[lane] = s;
+}
+
 // kFused = false: the expert FFN (moe_expert_ffn).  kFused = true: the whole layer in this one launch (see FusedArgs);
 // the differences are the set-up, where the gate/up items' operand rows come from, which rows their epilogue writes,
 // and the reduction over slots after the down items.
@@ -305,8 +334,8 @@ template <bool kFused, bool kQ = false>
 __global__ void __launch_bounds__(kNatThreads, 1)
 ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_constant__ CUtensorMap tmap_s13,
                   const __grid_constant__ TermMaps tmap_a1, const __grid_constant__ CUtensorMap tmap_w2,
-                  const __grid_constant__ CUtensorMap tmap_s2, const __grid_constant__ TermMaps tmap_a2, const NatArgs a,
-                  const FusedArgs f) {
+                  const __grid_constant__ CUtensorMap tmap_s2, const __grid_constant__ TermMaps tmap_a2,
+                  const __grid_constant__ CUtensorMap tmap_tok, const NatArgs a, const FusedArgs f) {
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
   const NatSmem sm = nat_smem(a.E, a.H > a.I ? a.H : a.I);
@@ -638,7 +667,8 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
     }
   } else if (role == kTermWarp) {
     // =========================== term rows: likewise ===========================
-    const bool tok_rows = kFused || a.tok != nullptr;  // by token, seen complete during the set-up; or by sorted row
+    // a pass's rows: by token (at most kFusedMaxTok in the one-launch layer), or in sorted order
+    const int tok_rows = kQ ? 0 : (kFused ? tok_pass : (a.tok != nullptr ? a.tok_rows : 0));
     if (!kFused) pdl_wait();  // the kernel that splits the token rows is complete: their terms, cleared counters
     fence_proxy_async_all();  // (one-launch layer: the rows were written through the generic proxy, TMA reads through the async one)
     int s = 0, dep_e = -1;
@@ -647,11 +677,11 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
     for (int phase = a.ph_lo; phase < a.ph_hi; ++phase) {
       const Phase P = phase_of(phase, a, s_misc + 1);
       const TermMaps* ma = phase == 0 ? &tmap_a1 : &tmap_a2;
-      const bool by_token = !kQ && tok_rows && phase == 0;
       for (int it = P.begin; it < P.end; ++it) {
         const int ti = it / P.tiles;
         const int row_begin = warp_uniform(t_begin[ti]), n_rows_e = warp_uniform(t_end[ti]) - row_begin;
         const int n_pass = (n_rows_e + tok_pass - 1) / tok_pass;
+        const bool by_token = phase == 0 && n_rows_e <= tok_rows;
         if (phase == 1 && a.ph_lo == 0) {  // (one projection per launch: the launch before this one has published all rows)
           const int e = warp_uniform(touched[ti]);
           if (e != dep_e) {
@@ -665,7 +695,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
           const int bi = op_box(n_tok * nt);  // box of 8 << bi operand rows; rows past the end of the tensor arrive as zeros
           int tok = 0, t4[4] = {0, 0, 0, 0};  // by token: lane j has the pass's token j, the first four are known to be uniform
           if (by_token) {
-            if (lane < n_tok) tok = kFused ? s_tok[row0 + lane] : __ldcg(a.tok + row0 + lane) / a.tok_div;
+            if (lane < n_tok) tok = kFused ? s_tok[row0 + lane] : __ldcg(a.tok + row0 + lane) & 0x7FFFFFFF;
 #pragma unroll
             for (int j = 0; j < 4; ++j) t4[j] = warp_uniform(lane == j ? tok : 0);
           }
@@ -676,9 +706,9 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
             if (by_token) {
 #pragma unroll
               for (int j = 0; j < 4; ++j)
-                if (j < n_tok) tma_load_2d_elect(dst + j * (8 * 128), &ma->box[0], ks * 128, t4[j] * kTerms, bar);
+                if (j < n_tok) tma_load_2d_elect(dst + j * (8 * 128), &tmap_tok, ks * 128, t4[j] * kTerms, bar);
               for (int j = 4; j < n_tok; ++j)
-                tma_load_2d_elect(dst + j * (8 * 128), &ma->box[0], ks * 128, warp_uniform(lane == j ? tok : 0) * kTerms, bar);
+                tma_load_2d_elect(dst + j * (8 * 128), &tmap_tok, ks * 128, warp_uniform(lane == j ? tok : 0) * kTerms, bar);
             } else {
               tma_load_2d_elect(dst, &ma->box[bi], ks * 128, row0 * nt, bar);
             }
@@ -782,7 +812,8 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
               if (st == 0) counter_wait_ge(a.done + touched[ti], need_done, a.status);
               asm volatile("bar.sync 3, 128;" ::: "memory");
             }
-            const bool by_token = (kFused || a.tok != nullptr) && phase == 0;  // the tokens' scale bytes are stored by token, not by sorted row
+            // the tokens' scale bytes as their rows, by token or by sorted row
+            const bool by_token = !kQ && phase == 0 && (kFused || (a.tok != nullptr && row_end - row_begin <= a.tok_rows));
             const int row0 = row_begin + pass * tok_pass;
             const int n_rows = min(tok_pass, row_end - row0) * nt;  // operand rows that exist
             // rows are n_blk bytes each and consecutive: one contiguous range, copied 16 bytes at a time
@@ -798,8 +829,8 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
               const int r = i / n_chunk, c = i % n_chunk;
               const uint4* from = src + i;
               if (by_token) {
-                const int t = kFused ? s_tok[row0 + (r >> 3)] : __ldcg(a.tok + row0 + (r >> 3)) / a.tok_div;
-                from = reinterpret_cast<const uint4*>(src_sf) + (t * kTerms + (r & 7)) * n_chunk + c;
+                const int t = kFused ? s_tok[row0 + (r >> 3)] : __ldcg(a.tok + row0 + (r >> 3)) & 0x7FFFFFFF;
+                from = reinterpret_cast<const uint4*>(kFused ? f.sf1 : a.sf_tok) + (t * kTerms + (r & 7)) * n_chunk + c;
               }
               reinterpret_cast<uint4*>(sSfa)[r * n_chunk + (c ^ (r & cmask))] = __ldcg(from);
             }
@@ -915,9 +946,9 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
         }
       };
       if (phase == 0) {
-        // SwiGLU and the rounding to bf16 (the intermediate is defined as a bf16 value) of every token, then the accumulators
-        // are handed back and the 8-term split overlaps the next item's MMAs
-        float v[kMaxTokPass];
+        // every token's two sums, then the accumulators are handed back; SwiGLU, the rounding to bf16 (the intermediate is defined as
+        // a bf16 value) and the 8-term split overlap the next item's MMAs
+        float v[kMaxTokPass], v2[kMaxTokPass];
 #pragma unroll
         for (int g4 = 0; g4 < kMaxTokPass / 4; ++g4) {
           if (4 * g4 < n_tok) {
@@ -927,8 +958,8 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
             tmem_ld_wait();
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              const float g = sum8(gv + 8 * j), u = sum8(uv + 8 * j);
-              v[4 * g4 + j] = __bfloat162float(__float2bfloat16_rn(__fdividef(g, 1.0f + __expf(-g)) * u));
+              v[4 * g4 + j] = sum8(gv + 8 * j);
+              v2[4 * g4 + j] = sum8(uv + 8 * j);
             }
           }
         }
@@ -941,7 +972,9 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
           uint32_t keep[4], word[4], sb[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            r[j] = g4 == 0 ? v[j] : (g4 == 1 ? v[4 + j] : (g4 == 2 ? v[8 + j] : v[12 + j]));
+            const float g = g4 == 0 ? v[j] : (g4 == 1 ? v[4 + j] : (g4 == 2 ? v[8 + j] : v[12 + j]));
+            const float u = g4 == 0 ? v2[j] : (g4 == 1 ? v2[4 + j] : (g4 == 2 ? v2[8 + j] : v2[12 + j]));
+            r[j] = __bfloat162float(__float2bfloat16_rn(__fdividef(g, 1.0f + __expf(-g)) * u));
             keep[j] = r[j] != r[j] ? 0u : 0x7FFFFFFFu;  // (a NaN does not take part in its block's maximum)
             word[j] = 0u;
             sb[j] = 0u;
@@ -980,24 +1013,30 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
           }
         }
       } else {
-#pragma unroll 1
-        for (int g4 = 0; 4 * g4 < n_tok; ++g4) {
-          uint32_t va[32], vb[32];
-          tmem_ld_32x32(d0 + static_cast<uint32_t>(32 * g4), va);
-          tmem_ld_32x32(d1 + static_cast<uint32_t>(32 * g4), vb);
-          tmem_ld_wait();
+        float s0[kMaxTokPass], s1[kMaxTokPass];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int tok = 4 * g4 + j;
-            const float s0 = sum8(va + 8 * j), s1 = sum8(vb + 8 * j);
-            if (!dry && tok < n_tok) {
-              float* dst = y_row(a.y, a.row_dst, static_cast<size_t>(row0 + tok), out_stride) + tile * kTile + 32 * q + lane;
-              dst[0] = s0;
-              dst[128] = s1;
+        for (int g4 = 0; g4 < kMaxTokPass / 4; ++g4) {
+          if (4 * g4 < n_tok) {
+            uint32_t va[32], vb[32];
+            tmem_ld_32x32(d0 + static_cast<uint32_t>(32 * g4), va);
+            tmem_ld_32x32(d1 + static_cast<uint32_t>(32 * g4), vb);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              s0[4 * g4 + j] = sum8(va + 8 * j);
+              s1[4 * g4 + j] = sum8(vb + 8 * j);
             }
           }
         }
         release();
+#pragma unroll
+        for (int tok = 0; tok < kMaxTokPass; ++tok) {
+          if (!dry && tok < n_tok) {
+            float* dst = y_row(a.y, a.row_dst, static_cast<size_t>(row0 + tok), out_stride) + tile * kTile + 32 * q + lane;
+            dst[0] = s0[tok];
+            dst[128] = s1[tok];
+          }
+        }
       }
     };
     // Quantised-activation variant: accumulator lane = operand row = token.  The warp of quadrant q owns tokens
@@ -1294,10 +1333,23 @@ NatScratch nat_scratch(void* scratch, const moe_shape_t& sh, size_t rows) {
   L.done = reinterpret_cast<int*>(L.sf1 + align_up(rows * (sh.H / 32), kAlign));
   return L;
 }
-// tok: null, or tok_div times the token of every sorted row - the token rows' terms then lie by token (see launch_expert_ffn_native_tokens)
+// An expert of up to four rows takes them by token, of more in sorted order, which a kernel copies them to first - where there can
+// be none of more than eight, all by token (for that copy's launch in the chain costs 3 us).
+int tok_rows(const moe_shape_t& sh) { return sh.T <= 8 ? 8 : 4; }
+// the rows' terms by token and the tokens of the sorted rows, behind the scratch above
+struct NatTokens {
+  uint8_t *aq, *sf;
+  int* tok;
+};
+NatTokens nat_tokens(void* scratch, const moe_shape_t& sh) {
+  uint8_t* aq = static_cast<uint8_t*>(scratch) + native_scratch_bytes(sh);
+  uint8_t* sf = aq + align_up(static_cast<size_t>(kTerms) * sh.T * (sh.H / 2), kAlign);
+  return NatTokens{aq, sf, reinterpret_cast<int*>(sf + align_up(static_cast<size_t>(kTerms) * sh.T * (sh.H / 32), kAlign))};
+}
+// by_token: the rows' terms are those that launch_route_sort left (see launch_expert_ffn_native_tokens)
 template <bool kQ>
 int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
-                      void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, const int* tok = nullptr, int tok_div = 1) {
+                      void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, bool by_token = false) {
   if (!nat_attr_once()) return MOE_ERR_CUDA;
   const size_t S = static_cast<size_t>(sh.T) * sh.k;
   const size_t rows = S * (kQ ? 1 : kTerms);  // operand rows
@@ -1311,7 +1363,7 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
         !nat_map(&tm_a2.box[i], aq2, sh.I / 2, rows, 128, 8u << i, CU_TENSOR_MAP_SWIZZLE_128B))
       return MOE_ERR_CUDA;
   if (!weight_maps(w, sh, &tm_w13, &tm_s13, &tm_w2, &tm_s2)) return MOE_ERR_CUDA;
-  if (tok == nullptr) {
+  if (!by_token) {
     const size_t per_block = kQ ? 4 : 8;  // threads per 32-element block
     const size_t split_threads = S * (sh.H / 32) * per_block > static_cast<size_t>(sh.E) ? S * (sh.H / 32) * per_block : static_cast<size_t>(sh.E);
     const dim3 split_grid(static_cast<unsigned>((split_threads + 1023) / 1024));
@@ -1323,8 +1375,19 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
   }
   NatArgs a;
   a.sf1 = sf1;
-  a.tok = tok;
-  a.tok_div = tok_div;
+  a.tok = nullptr;
+  a.sf_tok = nullptr;
+  a.tok_rows = tok_rows(sh);
+  CUtensorMap tm_tok = tm_a1.box[0];
+  const bool expand = by_token && sh.T > a.tok_rows;
+  if (by_token) {
+    const NatTokens t = nat_tokens(scratch, sh);
+    a.tok = t.tok;
+    a.sf_tok = t.sf;
+    if (!nat_map(&tm_tok, t.aq, sh.H / 2, static_cast<uint64_t>(sh.T) * kTerms, 128, 8, CU_TENSOR_MAP_SWIZZLE_128B)) return MOE_ERR_CUDA;
+    if (expand && launch_pdl(native_expand_kernel, dim3(static_cast<unsigned>(S)), dim3(kTerms * 32), 0, st, t.aq, t.sf, t.tok, sh.H, aq1, sf1) != cudaSuccess)
+      return MOE_ERR_CUDA;
+  }
   a.aq2 = aq2;
   a.sf2 = sf2;
   a.done = done;
@@ -1351,11 +1414,11 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
     a.ph_lo = two ? l : 0;
     a.ph_hi = two ? l + 1 : 2;
     if (launch_pdl(ffn_native_kernel<false, kQ>, dim3(sm_count()), dim3(kNatThreads),
-                   nat_smem(sh.E, sh.H > sh.I ? sh.H : sh.I).total + 1024, st, tm_w13, tm_s13, tm_a1, tm_w2, tm_s2, tm_a2, a,
+                   nat_smem(sh.E, sh.H > sh.I ? sh.H : sh.I).total + 1024, st, tm_w13, tm_s13, tm_a1, tm_w2, tm_s2, tm_a2, tm_tok, a,
                    FusedArgs{}) != cudaSuccess)
       return MOE_ERR_CUDA;
   }
-  note_kernel(kQ ? "ffn_native_mxf4_quantised_activations" : "ffn_native_mxf4_block_scaled", two ? 3 : (tok != nullptr ? 1 : 2));
+  note_kernel(kQ ? "ffn_native_mxf4_quantised_activations" : "ffn_native_mxf4_block_scaled", two ? 3 : (by_token && !expand ? 1 : 2));
   return MOE_OK;
 }
 }  // namespace
@@ -1366,11 +1429,12 @@ int launch_expert_ffn_native(const __nv_bfloat16* x_perm, const int* offsets, co
 }
 FrontSplit native_front_split(const __nv_bfloat16* x, const moe_shape_t& sh, void* scratch, StatusRef status) {
   const NatScratch L = nat_scratch(scratch, sh, static_cast<size_t>(sh.T) * sh.k * kTerms);
-  return FrontSplit{x, L.aq1, L.sf1, L.done, sh.E, sh.H, status.own ? status.word : nullptr};
+  const NatTokens t = nat_tokens(scratch, sh);
+  return FrontSplit{x, t.aq, t.sf, L.done, sh.E, sh.H, status.own ? status.word : nullptr, t.tok, tok_rows(sh)};
 }
-int launch_expert_ffn_native_tokens(const int* tok, int tok_div, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
-                                    void* scratch, float* y_perm, StatusRef status, cudaStream_t st) {
-  return launch_native_ffn<false>(nullptr, offsets, w, sh, scratch, y_perm, status, st, nullptr, tok, tok_div);
+int launch_expert_ffn_native_tokens(const int* offsets, const ExpertWeights& w, const moe_shape_t& sh, void* scratch, float* y_perm,
+                                    StatusRef status, cudaStream_t st) {
+  return launch_native_ffn<false>(nullptr, offsets, w, sh, scratch, y_perm, status, st, nullptr, true);
 }
 int launch_expert_ffn_native_q(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
                                void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst) {
@@ -1417,7 +1481,8 @@ int launch_forward_fused(const float* logits, const __nv_bfloat16* x, const Expe
   NatArgs a;
   a.sf1 = nullptr;
   a.tok = nullptr;
-  a.tok_div = 1;
+  a.sf_tok = nullptr;
+  a.tok_rows = 0;
   a.aq2 = aq2;
   a.sf2 = sf2;
   a.done = sync;
@@ -1448,7 +1513,7 @@ int launch_forward_fused(const float* logits, const __nv_bfloat16* x, const Expe
   f.T = sh.T;
   f.k = sh.k;
   if (launch_pdl(ffn_native_kernel<true>, dim3(grid), dim3(kNatThreads), nat_smem(sh.E, sh.H > sh.I ? sh.H : sh.I).total + 1024, st,
-                 tm_w13, tm_s13, tm_a1, tm_w2, tm_s2, tm_a2, a, f) != cudaSuccess)
+                 tm_w13, tm_s13, tm_a1, tm_w2, tm_s2, tm_a2, tm_a1.box[0], a, f) != cudaSuccess)
     return MOE_ERR_CUDA;
   note_kernel("layer_one_launch_mxf4_block_scaled", 1);
   return MOE_OK;

@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(1024) route_kernel(const float* __restrict__ l
 
 int launch_route(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* counters,
                  cudaStream_t st) {
-  if (route_sort_ok(T, E)) return launch_route_sort(logits, T, E, k, ids, w, offsets, nullptr, nullptr, false, nullptr, nullptr, false, st);
+  if (route_sort_ok(T, E)) return launch_route_sort(logits, T, E, k, ids, w, offsets, nullptr, nullptr, nullptr, nullptr, false, st);
   // One CTA up to a round of its 32 warps.  (64 tokens: 19 us in two rounds of one CTA, 7 us on eight.)
   const bool single = T <= 32;
   const int nw = single ? 32 : 8;
@@ -137,14 +137,14 @@ int launch_route(const float* logits, int T, int E, int k, int* ids, float* w, i
 // With more than a token per warp it is no faster than those (333 tokens in two rounds: 12 us, and 13 to the end of the
 // general sort).
 // The CTAs behind the first cluster (kSplit) split the token rows, which depends on no routing, meanwhile.
-constexpr int kFrontMaxE = 256, kFrontCluster = 8;
+constexpr int kFrontCluster = 8;
+static_assert(kFrontMaxTok == 32 * kFrontCluster, "a warp per token");
 template <bool kSplit>
 __global__ void __launch_bounds__(1024) route_sort_kernel(const float* __restrict__ logits, int T, int E, int k, int* __restrict__ ids,
-                                                          float* __restrict__ w, int* __restrict__ offsets, int* __restrict__ order,
-                                                          int* __restrict__ inv_perm, int order_tokens, int* __restrict__ offsets2, int late,
-                                                          const FrontSplit f) {
+                                                          float* __restrict__ w, int* __restrict__ offsets, int* __restrict__ perm,
+                                                          int* __restrict__ inv_perm, int* __restrict__ offsets2, int late, const FrontSplit f) {
   __shared__ unsigned s_mask[kFrontMaxE];
-  __shared__ int s_cnt[kFrontMaxE], s_base[kFrontMaxE], s_tot[kFrontMaxE / 32];
+  __shared__ int s_cnt[kFrontMaxE], s_all[kFrontMaxE], s_base[kFrontMaxE], s_tot[kFrontMaxE / 32];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   unsigned n_cta, rank;
   asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n_cta));
@@ -204,6 +204,7 @@ __global__ void __launch_bounds__(1024) route_sort_kernel(const float* __restric
   if (tid < E) {
     for (int i = 0; i < wid; ++i) ex += s_tot[i];
     s_base[tid] = ex + before;
+    s_all[tid] = total;
     if (rank == 0) {
       offsets[tid] = ex;
       if (tid == E - 1) offsets[E] = ex + total;
@@ -212,18 +213,19 @@ __global__ void __launch_bounds__(1024) route_sort_kernel(const float* __restric
   if (rank == 0 && tid < 2 && offsets2 != nullptr) offsets2[tid] = tid == 0 ? 0 : T;
   if (n_cta > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");  // (the other CTAs' counts have been read)
   __syncthreads();
-  if (order != nullptr && mine) {
+  if (inv_perm != nullptr && mine) {
     const int p = s_base[my_id] + __popc(s_mask[my_id] & ((1u << wid) - 1u)), slot = t * k + lane;
     inv_perm[slot] = p;
-    order[p] = order_tokens ? t : slot;
+    if (perm != nullptr) perm[p] = slot;
+    if (kSplit) f.tok[p] = s_all[my_id] > f.most ? t | static_cast<int>(0x80000000u) : t;
   }
   if (n_cta > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-bool route_sort_ok(int T, int E) { return E <= kFrontMaxE && T <= 32 * kFrontCluster; }
+bool route_sort_ok(int T, int E) { return E <= kFrontMaxE && T <= kFrontMaxTok; }
 
-int launch_route_sort(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* order, int* inv_perm,
-                      bool order_tokens, int* offsets2, const FrontSplit* split, bool late, cudaStream_t st) {
+int launch_route_sort(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* perm, int* inv_perm, int* offsets2,
+                      const FrontSplit* split, bool late, cudaStream_t st) {
   int n_cta = 1;
   while (n_cta < kFrontCluster && n_cta * 8 < T) n_cta *= 2;
   long long extra = 0;
@@ -244,10 +246,10 @@ int launch_route_sort(const float* logits, int T, int E, int k, int* ids, float*
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (cudaLaunchKernelEx(&cfg, split != nullptr ? route_sort_kernel<true> : route_sort_kernel<false>, logits, T, E, k, ids, w, offsets, order,
-                         inv_perm, order_tokens ? 1 : 0, offsets2, late || T > 32 ? 1 : 0, split != nullptr ? *split : FrontSplit{}) != cudaSuccess)
+  if (cudaLaunchKernelEx(&cfg, split != nullptr ? route_sort_kernel<true> : route_sort_kernel<false>, logits, T, E, k, ids, w, offsets, perm,
+                         inv_perm, offsets2, late || T > 32 ? 1 : 0, split != nullptr ? *split : FrontSplit{}) != cudaSuccess)
     return MOE_ERR_CUDA;
-  note_kernel(order != nullptr ? "route_topk_and_sort_one_cluster" : "route_topk_one_cluster", 1);
+  note_kernel(inv_perm != nullptr ? "route_topk_and_sort_one_cluster" : "route_topk_one_cluster", 1);
   return MOE_OK;
 }
 

@@ -433,9 +433,10 @@ def test_forward_small_shapes(T, H, I, E, k, one_launch):
 # One cluster of 1, 2, 4 or 8 CTAs of up to 32 tokens routes and sorts; beyond that the general route and sort
 @pytest.mark.parametrize("T,E,k", [(2, 16, 2), (31, 256, 8), (32, 256, 8), (33, 100, 6), (64, 256, 8), (65, 40, 32), (128, 64, 3), (129, 64, 8),
                                    (255, 256, 8), (256, 100, 1), (256, 256, 6), (257, 100, 6), (8, 256, 8), (9, 7, 7), (1000, 256, 6)])
-def test_forward_routes_and_sorts_as_the_calls_do(T, E, k):
+@pytest.mark.parametrize("skew", [False, True])   # (experts of more than four rows take theirs in sorted order, others by token)
+def test_forward_routes_and_sorts_as_the_calls_do(T, E, k, skew):
     H, I = 512, 512
-    wl = inputs.Workload("sort", T, H, I, E, k)
+    wl = inputs.Workload("sort", T, H, I, E, k, skew)
     d = inputs.make_workload(wl, seed=21)
     wdev = weights_dev(d)
     out, ids, w, _ = _run_forward(wl, d, wdev)
@@ -445,6 +446,14 @@ def test_forward_routes_and_sorts_as_the_calls_do(T, E, k):
     assert np.array_equal(buf.expert_offsets.cpu().numpy(), roff)
     _, perm, inv = O.permute(d["x"], rids, roff)
     assert np.array_equal(buf.perm.cpu().numpy(), perm) and np.array_equal(buf.inv_perm.cpu().numpy(), inv)
+    # the four calls one by one
+    buf2 = moe.LayerBuffers(buf.sh)
+    moe.moe_route(dev(d["logits"]), k, buf2.topk_ids, buf2.topk_w, buf2.expert_offsets, buf2.ws)
+    moe.moe_permute(dev(d["x"]), buf2.topk_ids, buf2.expert_offsets, buf2.sh, buf2.x_perm, buf2.perm, buf2.inv_perm, buf2.ws)
+    moe.moe_expert_ffn(buf2.x_perm, buf2.expert_offsets, *wdev, buf2.sh, buf2.y_perm, buf2.status, buf2.ws)
+    moe.moe_combine(buf2.y_perm, buf2.inv_perm, buf2.topk_w, buf2.sh, buf2.out)
+    torch.cuda.synchronize()
+    assert all(torch.equal(getattr(buf2, n).view(torch.int16), getattr(buf, n).view(torch.int16)) for n in ("x_perm", "perm", "inv_perm", "y_perm", "out"))
     assert torch.equal(out.view(torch.int16), out4.view(torch.int16))
 
 
