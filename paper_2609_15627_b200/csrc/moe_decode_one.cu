@@ -91,6 +91,7 @@ struct OneArgs {
   int own_status;           // the library's own status word: the last CTA clears it
   int E, H, I, k;
   int blocked;              // weights in moe_prepack's tile-contiguous layout
+  const uint8_t *s13, *s2, *shared_s13, *shared_s2;  // scale bytes, for contiguous tiles of them
   int n_shared;             // 1: slot k is the shared expert (its own tensor maps, expert 0 of them), added with weight 1
   int blocked_shared;       //    and its weights' layout
 };
@@ -275,11 +276,16 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
           if (phase == 1 || (it & 1) == 0) {  // 16 scale bytes per weight row cover two K steps
             mbar_wait(&empty_sc[cs], cph ^ 1u, a.status);
             mbar_expect_tx(&full_sc[cs], kScStage);
-            const int sx = blocked ? 0 : (ks >> 1) * 16;
-            const int sya = blocked ? ((wrow_a >> 7) * (n_steps >> 1) + (ks >> 1)) * 128 : wrow_a;
-            const int syb = blocked ? ((wrow_b >> 7) * (n_steps >> 1) + (ks >> 1)) * 128 : wrow_b;
-            tma_load_2d_hint(sSc + cs * kScStage, msc, sx, sya, &full_sc[cs], stream_once);
-            tma_load_2d_hint(sSc + cs * kScStage + 128 * 16, msc, sx, syb, &full_sc[cs], stream_once);
+            if (blocked) {  // 128 rows in one piece
+              const uint8_t* sc = shared ? (phase == 0 ? a.shared_s13 : a.shared_s2) : (phase == 0 ? a.s13 : a.s2);
+              const int half = n_steps >> 1;
+              bulk_g2s_hint(sSc + cs * kScStage, sc + static_cast<size_t>((wrow_a >> 7) * half + (ks >> 1)) * 2048, 2048u, &full_sc[cs], stream_once);
+              bulk_g2s_hint(sSc + cs * kScStage + 128 * 16, sc + static_cast<size_t>((wrow_b >> 7) * half + (ks >> 1)) * 2048, 2048u, &full_sc[cs],
+                            stream_once);
+            } else {
+              tma_load_2d_hint(sSc + cs * kScStage, msc, (ks >> 1) * 16, wrow_a, &full_sc[cs], stream_once);
+              tma_load_2d_hint(sSc + cs * kScStage + 128 * 16, msc, (ks >> 1) * 16, wrow_b, &full_sc[cs], stream_once);
+            }
             if (++cs == kScStages) { cs = 0; cph ^= 1u; }
           }
           mbar_wait(&empty_w[s], ph ^ 1u, a.status);
@@ -751,6 +757,10 @@ int launch_decode_one(const float* logits, const __nv_bfloat16* x, const ExpertW
   a.k = sh.k;
   a.blocked = w.blocked ? 1 : 0;
   a.n_shared = n_shared;
+  a.s13 = w.s13;
+  a.s2 = w.s2;
+  a.shared_s13 = shared != nullptr ? shared->s13 : nullptr;
+  a.shared_s2 = shared != nullptr ? shared->s2 : nullptr;
   a.blocked_shared = (shared != nullptr && shared->blocked) ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(sm_count() & ~1));

@@ -114,8 +114,8 @@ struct NatArgs {
   int E, H, I, S;
   int tok_rows;
   int blocked;               // weights in moe_prepack's tile-contiguous layout (see ExpertWeights)
-  const uint8_t* s13;        // the weights' scale bytes in the row layout, for reductions that are not multiples of 512:
-  const uint8_t* s2;         //   their rows are then not multiples of 16 bytes, which a tensor map cannot address
+  const uint8_t* s13;        // the weights' scale bytes, where no tensor map is used: contiguous tiles, and rows of reductions that are
+  const uint8_t* s2;         //   not multiples of 512 - then not multiples of 16 bytes, which a tensor map cannot address
   int ph_lo, ph_hi;          // projections this launch runs: [0, 2) = both; the large-batch schedule runs one per launch
   int by_pass;               // large-batch schedule: the list of experts is a list of (expert, pass) entries (see the set-up)
 };
@@ -621,12 +621,16 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
               mbar_wait_warp(&empty_sc[cs], cph ^ 1u, a.status);
               const uint32_t bar = sc_bar + cs * 8, dst = sc_ring + cs * kScStage;
               mbar_expect_tx_elect(bar, kScStage);
-              // 128 rows x 16 scale bytes; tile-contiguous layout: tile (row / 128, ks / 2) is 128 consecutive rows of 16 bytes
-              const int sx = a.blocked ? 0 : ks * 8;
-              const int sya = a.blocked ? ((wrow_a >> 7) * (P.n_steps >> 1) + (ks >> 1)) * 128 : wrow_a;
-              const int syb = a.blocked ? ((wrow_b >> 7) * (P.n_steps >> 1) + (ks >> 1)) * 128 : wrow_b;
-              tma_load_2d_hint_elect(dst, msc, sx, sya, bar, stream_once);
-              tma_load_2d_hint_elect(dst + 128 * 16, msc, sx, syb, bar, stream_once);
+              // 128 rows x 16 scale bytes; tile-contiguous layout: tile (row / 128, ks / 2) is 2 KB in one piece
+              if (a.blocked) {
+                const uint8_t* sc = phase == 0 ? a.s13 : a.s2;
+                const int half = P.n_steps >> 1;
+                bulk_g2s_hint_elect(dst, sc + static_cast<size_t>((wrow_a >> 7) * half + (ks >> 1)) * 2048, 2048u, bar, stream_once);
+                bulk_g2s_hint_elect(dst + 128 * 16, sc + static_cast<size_t>((wrow_b >> 7) * half + (ks >> 1)) * 2048, 2048u, bar, stream_once);
+              } else {
+                tma_load_2d_hint_elect(dst, msc, ks * 8, wrow_a, bar, stream_once);
+                tma_load_2d_hint_elect(dst + 128 * 16, msc, ks * 8, wrow_b, bar, stream_once);
+              }
               if (++cs == kScStages) { cs = 0; cph ^= 1u; }
             }
             mbar_wait_warp(&empty_w[s], ph ^ 1u, a.status);

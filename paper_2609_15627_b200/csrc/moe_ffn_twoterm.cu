@@ -805,9 +805,10 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
           for (int t = 0; t < kM; ++t) {
             const int row = weight_row(e, rt, t);
             const uint32_t dst = sf_base + (fs * kM + t) * 2048;
-            if (sf_tma)
-              tt_load_2d_hint(dst, &tmap_sc, a.blocked ? 0 : ks * (step_k / 32), a.blocked ? ((row >> 7) * (K / 512) + ks * step_k / 512) * 128 : row,
-                              raw_bar + fs * 8, pol);
+            if (sf_tma && a.blocked)  // 128 rows in one piece
+              bulk_g2s_hint_elect(dst, a.sc + static_cast<size_t>((row >> 7) * (K / 512) + ks * step_k / 512) * 2048, 2048u, raw_bar + fs * 8, pol);
+            else if (sf_tma)
+              tt_load_2d_hint(dst, &tmap_sc, ks * (step_k / 32), row, raw_bar + fs * 8, pol);
             else
               tt_bulk_g2s(dst, a.sc + static_cast<size_t>(row) * 8, 1024u, raw_bar + fs * 8);
           }
