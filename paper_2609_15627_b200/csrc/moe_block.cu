@@ -16,6 +16,7 @@
 //     number of CTAs (T/128 x E/64), not for the tensor-core rate.
 #include <cuda.h>
 
+#include "moe_mxf4_device.cuh"
 #include "moe_sm100_primitives.cuh"
 #include "moe_tmap.cuh"
 
@@ -28,11 +29,11 @@ constexpr int kGemvWarps = 8;
 
 __global__ void __launch_bounds__(kGemvWarps * 32) router_gemv_kernel(const __nv_bfloat16* __restrict__ x,
                                                                       const __nv_bfloat16* __restrict__ wr, int T, int H,
-                                                                      int E, float* __restrict__ logits) {
+                                                                      int E, float* __restrict__ logits, int beside) {
   extern __shared__ __align__(16) unsigned char smem_x[];  // [T][H] bf16
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   pdl_launch_dependents();
-  pdl_wait();  // x may be the output of the kernel before this one
+  if (!beside) pdl_wait();  // x may be the output of the kernel before this one
   const int n16 = T * H / 8;
   for (int i = tid; i < n16; i += blockDim.x) reinterpret_cast<uint4*>(smem_x)[i] = __ldg(reinterpret_cast<const uint4*>(x) + i);
   __syncthreads();
@@ -228,20 +229,26 @@ __global__ void __launch_bounds__(256) combine_shared_kernel(const float* __rest
 }
 
 __global__ void shared_offsets_kernel(int* offsets, int T) {
-  // waits BEFORE it releases its dependent: moe_route, launched next, reads the logits before its own wait, so the
-  // router projection two launches back must be complete by the time moe_route may start
+  // waits, and releases its dependent by ending only: what is launched behind it, whether that waits or not, starts when all that
+  // was launched before it has completed and the offsets are written
   pdl_wait();
-  pdl_launch_dependents();
   if (threadIdx.x == 0) {
     offsets[0] = 0;
     offsets[1] = T;
+    offsets[2] = 0;  // CTAs of the shared expert's last launch that are through
   }
+}
+// The kernels between the shared expert's and this one waited for the router's launch alone: whatever comes next is to wait for
+// the shared expert's CTAs, which count themselves (all of them have been running since before the router's)
+__global__ void shared_join_kernel(const int* finished, int n_cta, int* status) {
+  pdl_wait();
+  counter_wait_ge_warp(finished, n_cta, status);
 }
 
 }  // namespace
 
 int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, int T, int H, int E, float* logits, int* status,
-                         cudaStream_t st) {
+                         cudaStream_t st, bool beside) {
   if (T <= kGemvMaxTok && static_cast<size_t>(T) * H * 2 <= 160 * 1024) {
     const size_t smem = static_cast<size_t>(T) * H * 2;
     static PerDeviceFlag flag;
@@ -250,7 +257,7 @@ int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, 
         }))
       return MOE_ERR_CUDA;
     if (launch_pdl(router_gemv_kernel, dim3((E + kGemvWarps - 1) / kGemvWarps), dim3(kGemvWarps * 32), smem, st, x, w_router, T, H, E,
-                   logits) != cudaSuccess)
+                   logits, beside ? 1 : 0) != cudaSuccess)
       return MOE_ERR_CUDA;
     note_kernel("router_gemv_warp_per_expert", 1);
     return MOE_OK;
@@ -266,9 +273,14 @@ int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, 
       }))
     return MOE_ERR_CUDA;
   const dim3 grid((T + kRM - 1) / kRM, (E + cols - 1) / cols);
-  if (cols == 16) router_gemm_kernel<16><<<grid, kRThreads, smem, st>>>(tm_x, tm_w, T, H, E, logits, status);
-  else router_gemm_kernel<64><<<grid, kRThreads, smem, st>>>(tm_x, tm_w, T, H, E, logits, status);
-  if (cudaGetLastError() != cudaSuccess) return MOE_ERR_CUDA;
+  // (the kernel has no wait of its own: launched as a programmatic dependent it runs beside the launches in front of it)
+  const auto kernel = cols == 16 ? router_gemm_kernel<16> : router_gemm_kernel<64>;
+  if (beside) {
+    if (launch_pdl(kernel, grid, dim3(kRThreads), smem, st, tm_x, tm_w, T, H, E, logits, status) != cudaSuccess) return MOE_ERR_CUDA;
+  } else {
+    kernel<<<grid, kRThreads, smem, st>>>(tm_x, tm_w, T, H, E, logits, status);
+    if (cudaGetLastError() != cudaSuccess) return MOE_ERR_CUDA;
+  }
   note_kernel("router_gemm_tcgen05_128x64", 1);  // (also for tiles of 16 experts: callers know the kernel by this name)
   return MOE_OK;
 }
@@ -280,6 +292,12 @@ int launch_combine_shared(const float* y_perm, const int* inv_perm, const float*
                  sh.T, sh.H, sh.k, out) != cudaSuccess)
     return MOE_ERR_CUDA;
   note_kernel("combine_slot_order_fma_plus_shared", 1);
+  return MOE_OK;
+}
+
+int launch_shared_join(const int* finished, int n_cta, int* status, cudaStream_t st) {
+  if (launch_pdl(shared_join_kernel, dim3(1), dim3(32), 0, st, finished, n_cta, status) != cudaSuccess) return MOE_ERR_CUDA;
+  note_kernel("shared_expert_join", 1);
   return MOE_OK;
 }
 

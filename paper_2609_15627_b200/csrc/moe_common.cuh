@@ -270,9 +270,14 @@ struct TwoTermInput {
   bool offsets_late;       // with the tables: the kernel in front is the one that writes the offsets
   bool write_rows;         // with the tables: x_sorted is the caller's and receives all rows
 };
+// `again_later`: the launches of `guard` that do experts again are left to launch_twoterm_again, before anything reads y_perm.
+// `finished` (may be null), here and in launch_expert_ffn_native: every CTA of the last launch adds one when it is through; the
+// grid's size in *n_cta.
 int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
                            const moe_shape_t& choice, bool guard, void* scratch, float* y_perm, int* status_word, cudaStream_t st,
-                           float* const* row_dst = nullptr);
+                           float* const* row_dst = nullptr, bool again_later = false, int* finished = nullptr, int* n_cta = nullptr);
+int launch_twoterm_again(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& s, void* scratch, float* y_perm,
+                         int* status_word, cudaStream_t st);
 // chosen by the batch and the weights' alignment, where another kernel takes the shape as well: what one of those refuses
 // (rows too long for the streaming kernel, its only one) stays refused
 bool twoterm_chosen(const moe_shape_t& choice, const ExpertWeights& w);
@@ -291,7 +296,8 @@ bool native_q_shape_ok(const moe_shape_t& s, const void* w13, const void* w2);
 int launch_expert_ffn_native_q(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
                                void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst = nullptr);
 int launch_expert_ffn_native(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
-                             void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst = nullptr);
+                             void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst = nullptr,
+                             int* finished = nullptr, int* n_cta = nullptr);
 
 // the native variant behind launch_route_sort: token rows by token (native_front_split says where that launch leaves them).  H a
 // multiple of 512.
@@ -325,14 +331,16 @@ int launch_decode_one(const float* logits, const __nv_bfloat16* x, const ExpertW
                       cudaStream_t st, const ExpertWeights* shared = nullptr);
 
 // router projection, join with the shared expert, and the shared expert's offsets {0, T} (moe_block.cu)
+// `beside`: the logits are computed beside the launches in front, without waiting for them; x and w_router are complete
 int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, int T, int H, int E, float* logits, int* status,
-                         cudaStream_t st);
+                         cudaStream_t st, bool beside = false);
 // expert-parallel sharding: the table of output rows (see moe_ep_row_table)
 int launch_ep_row_table(const int* perm, const int* offsets, int k, int H, int e_begin, int e_end, float* const* owner_y, int world,
                         int tokens_per_rank, float** row_dst, cudaStream_t st, int max_rows);
 int launch_combine_shared(const float* y_perm, const int* inv_perm, const float* w, const float* y_shared, const moe_shape_t& s,
                           __nv_bfloat16* out, cudaStream_t st);
-int launch_shared_offsets(int* offsets2, int T, cudaStream_t st);
+int launch_shared_offsets(int* offsets2, int T, cudaStream_t st);  // offsets2: {0, T} and a counter, 0
+int launch_shared_join(const int* finished, int n_cta, int* status, cudaStream_t st);
 
 int sm_count();  // of the current device
 

@@ -116,6 +116,7 @@ struct NatArgs {
   int blocked;               // weights in moe_prepack's tile-contiguous layout (see ExpertWeights)
   const uint8_t* s13;        // the weights' scale bytes, where no tensor map is used: contiguous tiles, and rows of reductions that are
   const uint8_t* s2;         //   not multiples of 512 - then not multiples of 16 bytes, which a tensor map cannot address
+  int* finished;             // or null; every CTA adds one when its work is done
   int ph_lo, ph_hi;          // projections this launch runs: [0, 2) = both; the large-batch schedule runs one per launch
   int by_pass;               // large-batch schedule: the list of experts is a list of (expert, pass) entries (see the set-up)
 };
@@ -1207,6 +1208,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
   // ---- teardown ----
   tc_fence_before_sync();
   __syncthreads();
+  if (!kFused && tid == 0 && a.finished != nullptr) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(a.finished) : "memory");
   if (wid == 1) {
     tc_fence_after_sync();
     tmem_dealloc(tmem_base, kNatTmemCols);
@@ -1353,7 +1355,7 @@ NatTokens nat_tokens(void* scratch, const moe_shape_t& sh) {
 // by_token: the rows' terms are those that launch_route_sort left (see launch_expert_ffn_native_tokens)
 template <bool kQ>
 int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
-                      void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, bool by_token = false) {
+                      void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, bool by_token = false, int* finished = nullptr) {
   if (!nat_attr_once()) return MOE_ERR_CUDA;
   const size_t S = static_cast<size_t>(sh.T) * sh.k;
   const size_t rows = S * (kQ ? 1 : kTerms);  // operand rows
@@ -1379,6 +1381,7 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
   }
   NatArgs a;
   a.sf1 = sf1;
+  a.finished = finished;
   a.tok = nullptr;
   a.sf_tok = nullptr;
   a.tok_rows = tok_rows(sh);
@@ -1428,8 +1431,10 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
 }  // namespace
 
 int launch_expert_ffn_native(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
-                             void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst) {
-  return launch_native_ffn<false>(x_perm, offsets, w, sh, scratch, y_perm, status, st, row_dst);
+                             void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, int* finished,
+                             int* n_cta) {
+  if (n_cta != nullptr) *n_cta = sm_count();
+  return launch_native_ffn<false>(x_perm, offsets, w, sh, scratch, y_perm, status, st, row_dst, false, finished);
 }
 FrontSplit native_front_split(const __nv_bfloat16* x, const moe_shape_t& sh, void* scratch, StatusRef status) {
   const NatScratch L = nat_scratch(scratch, sh, static_cast<size_t>(sh.T) * sh.k * kTerms);
@@ -1484,6 +1489,7 @@ int launch_forward_fused(const float* logits, const __nv_bfloat16* x, const Expe
   if (!weight_maps(w, sh, &tm_w13, &tm_s13, &tm_w2, &tm_s2)) return MOE_ERR_CUDA;
   NatArgs a;
   a.sf1 = nullptr;
+  a.finished = nullptr;
   a.tok = nullptr;
   a.sf_tok = nullptr;
   a.tok_rows = 0;

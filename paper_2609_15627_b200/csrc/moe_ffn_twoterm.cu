@@ -83,6 +83,7 @@ struct TtArgs {
   int E, K, R, I, S;       // R weight rows per expert (2I or H)
   int blocked;             // weights in moe_prepack's tile-contiguous layout (see ExpertWeights)
   int max_tok, sf_step;    // of the pass geometry (see TwoTermGeometry)
+  int* finished;           // or null; every CTA adds one when its work is done
   int stages, t_bytes, sf_off;  // ring depth; token part of a stage, and where its scale factors begin (see tt_launch)
 };
 
@@ -832,7 +833,8 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     }
   } else if (wid == 2) {
     // =========================== tokens (likewise) ===========================
-    pdl_wait();  // the rows and scale factors are complete
+    if (first < total) pdl_wait();  // the rows and scale factors are complete.  (A CTA without items leaves at once: kernels further down
+                                    // the stream may be waiting for its SM to start beside this one, see moe_ffn_block.)
     int s = 0;
     uint32_t ph = 0;
     const uint32_t full_own = smem_u32(full), full_first = tt_first_addr(full);
@@ -1226,6 +1228,7 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
   // ---- teardown: neither CTA leaves while the other's MMAs may read its shared memory or arrive on its barriers ----
   tc_fence_before_sync();
   __syncthreads();
+  if (tid == 0 && a.finished != nullptr) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(a.finished) : "memory");
   tt_cluster_sync();
   if (wid == 1) {
     tc_fence_after_sync();
@@ -1309,7 +1312,7 @@ static int launch_again(const TwoTermInput& in, const int* offsets, const Expert
 
 int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
                               const moe_shape_t& choice, bool guard, void* scratch, float* y_perm, int* status_word, cudaStream_t st,
-                              float* const* row_dst) {
+                              float* const* row_dst, bool again_later, int* finished, int* n_cta) {
   const TwoTermGeometry geo = twoterm_geometry(choice);
   const TwoTermScratch L = twoterm_scratch(choice);
   uint8_t* base = static_cast<uint8_t*>(scratch);
@@ -1374,17 +1377,26 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
   a.R = 2 * sh.I;
   if (!(guard ? tt_launch<true, 2, false, true>(tm_w13, tm_s13, tm_x, a, st) : tt_launch<true, 2, false>(tm_w13, tm_s13, tm_x, a, st)))
     return MOE_ERR_CUDA;
+  a.finished = finished;
+  if (n_cta != nullptr) *n_cta = sm_count() & ~1;
   a.sc = w.s2;
   a.K = sh.I;
   a.R = sh.H;
   const bool two = geo.max_tok == 64 && sh.H % 512 == 0;
   if (!(two ? tt_launch<false, 2, false>(tm_w2, tm_s2, tm_a, a, st) : tt_launch<false, 1, false>(tm_w2, tm_s2, tm_a, a, st))) return MOE_ERR_CUDA;
-  if (guard) {
+  if (guard && !again_later) {
     const int again = launch_again(in, offsets, w, sh, choice, base + L.aq, y_perm, status_word, st, row_dst, flags);
     if (again != MOE_OK) return again;
   }
   note_kernel("ffn_mxf8_two_term_cta_pair", 3 + (guard && in.inv_perm != nullptr && !in.write_rows ? 1 : 0));
   return MOE_OK;
+}
+
+int launch_twoterm_again(const TwoTermInput& in, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh, void* scratch, float* y_perm,
+                         int* status_word, cudaStream_t st) {
+  const TwoTermScratch L = twoterm_scratch(sh);
+  uint8_t* base = static_cast<uint8_t*>(scratch);
+  return launch_again(in, offsets, w, sh, sh, base + L.aq, y_perm, status_word, st, nullptr, reinterpret_cast<const int*>(base + L.flags));
 }
 
 int launch_expert_ffn_q_pair(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,

@@ -131,3 +131,43 @@ def test_ffn_block_prefill_8k_sampled():
     wl = inputs.WORKLOADS["prefill_8k"]
     rng = np.random.default_rng(0)
     _check_block(wl, seed=9, sample=sorted(set([0, wl.T - 1] + rng.integers(0, wl.T, 30).tolist())))
+
+
+# Up to 256 tokens the shared expert, the router projection and the routing run beside one another: the block is its steps, bit for
+# bit, also where calls follow one another on one workspace and in a graph (17 tokens: router GEMM; above 32 the shared expert's
+# kernel is another)
+@pytest.mark.parametrize("T,H,I,E,k", [(4, 1024, 512, 32, 4), (17, 1024, 512, 64, 6), (48, 4096, 2048, 16, 6), (130, 4096, 2048, 32, 2), (256, 512, 512, 64, 8)])
+def test_ffn_block_is_its_steps(T, H, I, E, k):
+    routed = tuple(dev(a) for a in inputs.make_expert_weights(H, I, E, seed=0))
+    shared = tuple(dev(a) for a in inputs.make_expert_weights(H, I, 1, seed=21))
+    wr = dev(_router_weights(E, H, 3))
+    sh, sh1 = moe.shape(T, H, I, E, k), moe.shape(T, H, I, 1, 1)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    xs, want = [dev(inputs.make_x(T, H, 30 + i)) for i in range(3)], []
+    buf, lg, ys = moe.LayerBuffers(sh), torch.empty((T, E), device="cuda"), torch.empty((T, H), device="cuda")
+    off2, ws1 = torch.tensor([0, T], dtype=torch.int32, device="cuda"), moe.alloc_workspace(sh1)
+    for x in xs:
+        moe.moe_router_logits(x, wr, lg, st)
+        moe.moe_layer(lg, x, routed, buf)
+        moe.moe_expert_ffn(x, off2, *shared, sh1, ys, st, ws1)
+        moe.moe_combine_shared(buf.y_perm, buf.inv_perm, buf.topk_w, ys, sh, buf.out)
+        torch.cuda.synchronize()
+        want.append(buf.out.clone())
+    ws, ids, w = moe.alloc_block_workspace(sh), torch.empty((T, k), dtype=torch.int32, device="cuda"), torch.empty((T, k), device="cuda")
+    outs = [torch.empty((T, H), dtype=torch.bfloat16, device="cuda") for _ in range(9)]
+
+    def calls():
+        for i, o in enumerate(outs):
+            moe.moe_ffn_block(xs[i % 3], wr, routed, shared, sh, o, ids, w, st, ws)
+    calls()
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and all(torch.equal(o.view(torch.int16), want[i % 3].view(torch.int16)) for i, o in enumerate(outs))
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        calls()
+    for o in outs:
+        o.zero_()
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and all(torch.equal(o.view(torch.int16), want[i % 3].view(torch.int16)) for i, o in enumerate(outs))
