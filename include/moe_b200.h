@@ -209,8 +209,9 @@ int moe_expert_ffn_packed(const void* x_perm_bf16 /* [T*k,H] */, const int32_t* 
  *   - For T = 1 (k <= 32, E*4 <= 4*max(H,I) bytes) on shapes the decode-sized expert kernel takes,
  *     the call is ONE kernel launch: every CTA routes the token itself and sorts the slots, the first CTAs write the
  *     token's E2M1 term rows, every CTA runs its share of the gate/up and down items, and the CTA that finishes a
- *     column tile's last expert reduces that tile over the slots.  Any other shape runs the four calls back to back
- *     (from two tokens on they are the faster form).
+ *     column tile's last expert reduces that tile over the slots.  Any other shape runs the four calls' steps back to back;
+ *     up to 256 tokens and 256 experts routing and sort are one launch, beside which the tokens' rows are split into the term
+ *     rows of the decode-sized kernel, once per token.
  *   - ws: moe_forward_workspace_bytes() bytes, 256-byte aligned.  Its first moe_forward_sync_bytes() bytes are the
  *     kernel's completion counters: they must be ZERO when a call starts.  Clear them once (cudaMemsetAsync) before
  *     the first call that uses this ws; every call that returns MOE_OK and whose kernels ran to completion leaves them
@@ -234,12 +235,12 @@ int moe_forward_packed(const float* logits /* [T,E] */, const void* x_bf16 /* [T
 
 /*
  * moe_forward with HOST input and output for one batch: copies logits_host [T,E] and x_host [T,H] to
- * device buffers carved from `ws`, clears moe_forward's counters, runs moe_forward on `cuda_stream`,
- * copies out [T,H] bf16 back into out_host and waits for the stream.  Fewer stream operations where the sizes allow: an
- * output of at most 64 KB in page-locked memory that the device can address is written there by the last kernel itself;
- * a single token row in such memory is read there by the kernel; logits of at most 64 KB travel in one copy with the
- * zeros of moe_forward's counter block, through a page-locked staging buffer that the library allocates once per host
- * thread (the only allocation any entry point makes, on its first call).
+ * device buffers carved from `ws`, clears moe_forward's counters where they are used, runs moe_forward on `cuda_stream`,
+ * copies out [T,H] bf16 back into out_host and waits for the stream.  Fewer stream operations with page-locked memory that the
+ * device can address (16-byte aligned): the output is written there by the last kernel itself; a single token row, and the
+ * logits and rows of a batch whose routing, sort and split are one launch (see moe_forward), are read there by that launch.
+ * Otherwise logits of at most 64 KB travel in one copy with the zeros of moe_forward's counter block, through a page-locked
+ * staging buffer that the library allocates once per host thread (the only allocation any entry point makes, on its first call).
  * Weights stay device-resident (they are model state, not per-batch input).  For page-locked host
  * buffers the copies are asynchronous until the final wait.  ws must hold
  * moe_forward_host_workspace_bytes() bytes.  No counterpart in the paper: it is the end-to-end

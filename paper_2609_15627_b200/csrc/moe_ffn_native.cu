@@ -24,9 +24,10 @@
 // the same K step of the pass's term rows, each fetched by TMA with the 128-byte swizzle the MMA reads.
 //
 // Launches per call: native_split_kernel (token rows -> E2M1 terms, once per row; clears the per-expert completion
-// counters), then ffn_native_kernel, in which one persistent CTA per SM runs both projections back to back:
+// counters) - or, in calls that hold the routing, launch_route_sort, which leaves the terms by token, and from nine tokens on
+// native_expand_kernel - then ffn_native_kernel, in which one persistent CTA per SM runs both projections back to back:
 // phase 0 = gate/up + SwiGLU (work item = touched expert x 128 gate rows + the 128 matching up rows, so gate and up of
-// one i are two columns of the same accumulator lane), phase 1 = down (item = touched expert x 256 rows).  The weight
+// one i share a lane of the two accumulators), phase 1 = down (item = touched expert x 256 rows).  The weight
 // stream runs on across the phase change; a down item loads its term rows once the gate/up items of its expert - its
 // own and other CTAs' - have published theirs (one counter per expert, release/acquire through L2, bounded wait).
 // No gate/up item ever waits for another CTA, and a down item waits only for gate/up items of CTAs with a lower or
@@ -42,7 +43,7 @@
 //   warp 10     producer of the term rows (TMA): waits for the split, and in phase 1 for the expert's gate/up items, while the
 //               weights of the next steps are on their way
 // The producing warps run convergent and an elected lane issues: from lane 0 of a branch a load takes so long that a second
-// one per step and expert was felt (64 tokens whose rows are fetched one by one: 746 us a layer, now 478).
+// one per step and expert was felt (64 tokens whose rows are fetched one by one: 746 us a layer, from an elected lane 478).
 // Every wait is bounded and reports through the status word.
 //
 // The weights are read either in the checkpoint's row layout or in moe_prepack's tile-contiguous layout (one tensor
