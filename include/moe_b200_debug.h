@@ -32,6 +32,11 @@ int moe_debug_read_probe(const void* src, size_t bytes, void* sink, size_t sink_
  * nonsense (cta outside [0, n_ctas), n_touched outside [0, 1024], H or 2I not a multiple of 256). */
 int moe_debug_native_cta_share(int32_t n_ctas, int32_t cta, int32_t n_touched, int32_t H, int32_t I, int32_t* out4);
 
+/* Host, pure, diagnostic.  Where the decode-sized expert-FFN kernel keeps piece `piece` (16 bytes) of operand row `row`'s scale
+ * bytes in shared memory, for rows of n_pieces = K / 512 of them: a slot of [0, 128 * n_pieces), or -1 for arguments out of range
+ * (row outside [0, 128), n_pieces outside [1, 8], piece outside [0, n_pieces)). */
+int moe_debug_native_scale_slot(int32_t row, int32_t piece, int32_t n_pieces);
+
 /* Diagnostic: the one-launch kernel of moe_forward for any batch it can take (up to 4 tokens, T*k <= 32), where
  * moe_forward itself would run the four calls because they are faster from 2 tokens on.  Same arguments, workspace and
  * result as moe_forward; MOE_ERR_UNSUPPORTED_SHAPE if the kernel cannot take the shape.  For the tests. */

@@ -214,6 +214,11 @@ MOE_DEVINL Phase phase_of(int ph, const NatArgs& a, const int* shares) {
   return p;
 }
 
+// Where piece c (16 bytes) of operand row r's scale bytes lies in shared memory, rows of n_chunk pieces (n_chunk = K / 512): XORed
+// with the row against bank conflicts, in as many bits as leave it inside its row - those below n_chunk's lowest set one
+// (all of them at 1, 2, 4 and 8 pieces, none at 3, 5 and 7)
+__host__ __device__ inline int sf_slot(int r, int c, int n_chunk) { return r * n_chunk + (c ^ (r & ((n_chunk & -n_chunk) - 1))); }
+
 // entries of the list of experts with rows that a CTA keeps
 __host__ __device__ inline int touched_cap(int E) { return E > 32 ? E : 32; }
 struct NatSmem {
@@ -823,8 +828,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
             const int row0 = row_begin + pass * tok_pass;
             const int n_rows = min(tok_pass, row_end - row0) * nt;  // operand rows that exist
             // rows are n_blk bytes each and consecutive: one contiguous range, copied 16 bytes at a time
-            // (the 16-byte chunks of a row are XOR-swizzled with the row number against bank conflicts)
-            const int n_chunk = n_blk / 16, cmask = min(n_chunk, 8) - 1;
+            const int n_chunk = n_blk / 16;
             const int n_vec = n_rows * n_chunk;
             const uint4* src = reinterpret_cast<const uint4*>(src_sf + static_cast<size_t>(row0) * nt * n_blk);
             if (P.direct) {  // rows of n_blk = 8 (mod 16) bytes: 8 bytes at a time, rows plainly one after the other
@@ -838,7 +842,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
                 const int t = kFused ? s_tok[row0 + (r >> 3)] : __ldcg(a.tok + row0 + (r >> 3)) & 0x7FFFFFFF;
                 from = reinterpret_cast<const uint4*>(kFused ? f.sf1 : a.sf_tok) + (t * kTerms + (r & 7)) * n_chunk + c;
               }
-              reinterpret_cast<uint4*>(sSfa)[r * n_chunk + (c ^ (r & cmask))] = __ldcg(from);
+              reinterpret_cast<uint4*>(sSfa)[sf_slot(r, c, n_chunk)] = __ldcg(from);
             }
             asm volatile("bar.sync 3, 128;" ::: "memory");
             __syncwarp();
@@ -850,7 +854,7 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
               for (int c = 0; c < 4; ++c) {
                 const int r = 32 * c + lane;
                 const uint2 v = P.direct ? reinterpret_cast<const uint2*>(sSfa)[r * (n_blk / 8) + ks]
-                                         : *reinterpret_cast<const uint2*>(sSfa + (r * n_chunk + ((ks >> 1) ^ (r & cmask))) * 16 + (ks & 1) * 8);
+                                         : *reinterpret_cast<const uint2*>(sSfa + sf_slot(r, ks >> 1, n_chunk) * 16 + (ks & 1) * 8);
                 w[c] = v.x;
                 w[4 + c] = v.y;
               }
@@ -1531,6 +1535,11 @@ int launch_forward_fused(const float* logits, const __nv_bfloat16* x, const Expe
 }
 
 }  // namespace moe
+
+extern "C" int moe_debug_native_scale_slot(int32_t row, int32_t piece, int32_t n_pieces) {
+  if (row < 0 || row >= 128 || n_pieces < 1 || n_pieces > moe::kMaxK / 512 || piece < 0 || piece >= n_pieces) return -1;
+  return moe::sf_slot(row, piece, n_pieces);
+}
 
 extern "C" int moe_debug_native_cta_share(int32_t n_ctas, int32_t cta, int32_t n_touched, int32_t H, int32_t I, int32_t* out4) {
   if (out4 == nullptr || n_ctas < 1 || cta < 0 || cta >= n_ctas || n_touched < 0 || n_touched > 1024 || H < moe::kTile ||

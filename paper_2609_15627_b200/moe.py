@@ -16,7 +16,7 @@ EXPORTS = ("moe_workspace_bytes", "moe_status_string", "moe_last_kernel_name", "
            "moe_permute", "moe_expert_ffn", "moe_combine", "moe_validate_scales",
            "moe_forward_workspace_bytes", "moe_forward_sync_bytes", "moe_forward",
            "moe_forward_host_workspace_bytes", "moe_forward_host", "moe_expert_ffn_noalloc_max_bytes",
-           "moe_expert_ffn_noalloc", "moe_debug_native_cta_share", "moe_debug_read_probe", "moe_prepack_bytes", "moe_prepack",
+           "moe_expert_ffn_noalloc", "moe_debug_native_cta_share", "moe_debug_native_scale_slot", "moe_debug_read_probe", "moe_prepack_bytes", "moe_prepack",
            "moe_expert_ffn_packed", "moe_forward_packed", "moe_forward_host_packed", "moe_debug_forward_one_launch",
            "moe_debug_expert_ffn_variant", "moe_router_logits", "moe_combine_shared", "moe_ffn_block_workspace_bytes",
            "moe_ffn_block", "moe_expert_ffn_q_workspace_bytes", "moe_expert_ffn_q",
@@ -75,6 +75,8 @@ def lib():
         L.moe_expert_ffn_noalloc.argtypes = [vp, vp, vp, vp, vp, vp, C.POINTER(Shape), vp, vp, vp]
         L.moe_debug_native_cta_share.restype = C.c_int
         L.moe_debug_native_cta_share.argtypes = [i32, i32, i32, i32, i32, C.POINTER(C.c_int32)]
+        L.moe_debug_native_scale_slot.restype = C.c_int
+        L.moe_debug_native_scale_slot.argtypes = [i32, i32, i32]
         L.moe_prepack_bytes.restype = sz
         L.moe_prepack_bytes.argtypes = [C.POINTER(Shape)]
         L.moe_prepack.restype = C.c_int

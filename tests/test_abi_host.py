@@ -108,6 +108,15 @@ def test_missing_library_fails_loudly(monkeypatch):
         moe.lib()
 
 
+@pytest.mark.parametrize("n", range(1, 9))
+def test_scale_slots_are_a_permutation_of_each_row(L, n):
+    """Rows of n = K / 512 pieces: different threads write a pass's 128 rows, so no two pieces may share a slot and none may
+    leave its row (the slot after the last row's is another array)."""
+    for r in range(128):
+        assert sorted(L.moe_debug_native_scale_slot(r, c, n) for c in range(n)) == list(range(r * n, (r + 1) * n)), (r, n)
+    assert [L.moe_debug_native_scale_slot(*a) for a in ((128, 0, n), (-1, 0, n), (0, n, n), (0, -1, n), (0, 0, 0), (0, 0, 9))] == [-1] * 6
+
+
 def test_decode_ffn_work_split_keeps_waits_pointing_down(L):
     """The decode-sized expert-FFN kernel runs both projections in one grid: a down item waits on the device for the
     gate/up items of its expert.  The split must cover every item exactly once, and every gate/up item an expert's

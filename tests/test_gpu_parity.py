@@ -1075,6 +1075,39 @@ def test_ffn_native_pass_sizes(rows, H, I):
     check_y(buf.y_perm.cpu().numpy(), O.expert_ffn(x, off, *w, 1), "native pass sizes")
 
 
+# Reductions of 3, 5, 6 and 7 times 512, as H, as I and as both: the scale bytes of an operand row are then no power of two of
+# 16-byte pieces.  Passes from one token to all sixteen; rows in sorted order, by token, and in the one-launch kernel
+_ODD_512 = [(1536, 512), (512, 1536), (2560, 1536), (3072, 512), (512, 3584), (3584, 3072)]
+
+
+@pytest.mark.parametrize("H,I", _ODD_512)
+def test_ffn_native_reductions_that_are_no_power_of_two(H, I):
+    rows = (1, 16, 5, 0, 33, 8)
+    E, S = len(rows), sum(rows)
+    w = inputs.make_expert_weights(H, I, E, seed=13)
+    w = (w[0], inputs.index_scales(2 * I, H, E, lo=117, span=6), w[2], inputs.index_scales(H, I, E, lo=118, span=5))
+    x = inputs.bf16_bits_to_f32(inputs.make_x(S, H, seed=13))
+    x = inputs.f32_to_bf16_bits(x * np.exp2(np.arange(H) // 32 % 13 - 6).astype(np.float32))  # (every block its own scale)
+    off = np.concatenate([[0], np.cumsum(rows)]).astype(np.int32)
+    sh = moe.shape(S, H, I, E, 1)
+    want = O.expert_ffn(x, off, *w, 1)
+    wd = [dev(a) for a in w]
+    for weights in (wd, [moe.moe_prepack(*wd, sh)]):
+        buf = moe.LayerBuffers(sh)
+        (moe.moe_expert_ffn if len(weights) == 4 else moe.moe_expert_ffn_packed)(dev(x), dev(off), *weights, sh, buf.y_perm, buf.status, buf.ws)
+        torch.cuda.synchronize()
+        assert int(buf.status.item()) == 0
+        assert moe.moe_last_kernel_name() == "ffn_native_mxf4_block_scaled"
+        check_y(buf.y_perm.cpu().numpy(), want, "reduction of 512 times %d / %d" % (H // 512, I // 512))
+
+
+@pytest.mark.parametrize("H,I", _ODD_512)
+@pytest.mark.parametrize("T,one_launch,force", [(1, True, False), (3, True, True), (5, False, False), (24, False, False)])
+def test_forward_reductions_that_are_no_power_of_two(H, I, T, one_launch, force):
+    wl = inputs.Workload("odd512", T, H, I, 6, 3, True)
+    _check_forward(wl, inputs.make_workload(wl, seed=14), None, one_launch, force_one_launch=force)
+
+
 # ---- consecutive layer calls on one stream, sharing every buffer but the output ----
 # With programmatic dependent launch the next call's router may start while this call's combine is still
 # running; it must not overwrite the routing weights and the inverse permutation that combine reads.

@@ -71,6 +71,19 @@ def test_ffn_q_matches_its_oracle(case, packed):
     _check_rows(got, O.expert_ffn_q(xp, off, *w, k), (case, packed))
 
 
+# Reductions of 3, 5, 6 and 7 times 512 (scale bytes of an operand row: no power of two of 16-byte pieces), passes of 128 rows
+@pytest.mark.parametrize("H,I", [(1536, 512), (512, 1536), (2560, 3072), (3584, 1536)])
+@pytest.mark.parametrize("T", [9, 140])
+def test_ffn_q_reductions_that_are_no_power_of_two(H, I, T):
+    E, k = 3, 2
+    lg = inputs.make_logits(T, E, 4)
+    lg[:, 1] += 9.0                                  # a whole pass of 128 rows and more on one expert
+    w, xp, off = _problem(T, H, I, E, k, seed=H + I + T, logits=lg)
+    sh = moe.shape(T, H, I, E, k)
+    got = _run(tuple(dev(a) for a in w), xp, off, sh)
+    _check_rows(got, O.expert_ffn_q(xp, off, *w, k), (H, I, T))
+
+
 def test_ffn_q_all_rows_on_one_expert_and_empty_batch_edges():
     T, H, I, E, k = 200, 512, 512, 6, 1
     lg = np.full((T, E), -5.0, np.float32)
