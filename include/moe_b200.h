@@ -90,7 +90,8 @@ uint64_t moe_launch_count(void);
  * for the kernel launched just before it on the stream, and writes its outputs only after that kernel has
  * completed (so the outputs of one layer call may be the buffers the previous call's moe_combine still reads).
  * If that preceding kernel releases its dependents early (cudaTriggerProgrammaticLaunchCompletion /
- * griddepcontrol.launch_dependents), logits must not be among its outputs; moe_combine's are not.
+ * griddepcontrol.launch_dependents), logits must not be among its outputs; moe_combine's are not, and moe_router_logits
+ * releases nothing before it has ended.
  * Errors: INVALID_ARG (null/misaligned, T<1, k<1, k>E), UNSUPPORTED_SHAPE (E>1024, k>32), WORKSPACE.
  */
 int moe_route(const float* logits, int32_t T, int32_t E, int32_t k, int32_t* topk_ids /* [T,k] */,

@@ -331,8 +331,9 @@ int moe_layer(const float* logits, const void* x_bf16, const uint8_t* w13, const
 }
 
 // ---- router projection, shared expert, join: the whole FFN block ---------------------------------------------
-int moe_router_logits(const void* x_bf16, const void* w_router_bf16, int32_t T, int32_t H, int32_t E, float* logits,
-                      int32_t* status_word, void* cuda_stream) {
+namespace {
+int router_logits_impl(const void* x_bf16, const void* w_router_bf16, int32_t T, int32_t H, int32_t E, float* logits,
+                       int32_t* status_word, void* cuda_stream, RouterOrder order) {
   if (T < 1 || H < 1 || E < 1) return MOE_ERR_INVALID_ARG;
   if (H % 128 != 0 || E > 1024) return MOE_ERR_UNSUPPORTED_SHAPE;
   if (!aligned(x_bf16, 16) || !aligned(w_router_bf16, 16) || !aligned(logits, 16) ||
@@ -344,7 +345,13 @@ int moe_router_logits(const void* x_bf16, const void* w_router_bf16, int32_t T, 
   if (rc != MOE_OK) return rc;
   if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
   return launch_router_logits(static_cast<const __nv_bfloat16*>(x_bf16), static_cast<const __nv_bfloat16*>(w_router_bf16), T, H, E,
-                              logits, status.word, st);
+                              logits, status.word, st, order);
+}
+}  // namespace
+
+int moe_router_logits(const void* x_bf16, const void* w_router_bf16, int32_t T, int32_t H, int32_t E, float* logits,
+                      int32_t* status_word, void* cuda_stream) {
+  return router_logits_impl(x_bf16, w_router_bf16, T, H, E, logits, status_word, cuda_stream, RouterOrder::kAlone);
 }
 
 int moe_combine_shared(const float* y_perm, const int32_t* inv_perm, const float* topk_w, const float* y_shared,
@@ -530,7 +537,7 @@ int moe_ffn_block(const void* x_bf16, const void* w_router_bf16, const uint8_t* 
     // one-token kernel (its weights depend on no routing, so its stream starts first), added with weight 1 after the
     // routed slots' recurrence.  The kernel needs its counter block clear; this call owns the block.
     if (cudaMemsetAsync(base + L.one_sync, 0, kForwardSyncBytes, st) != cudaSuccess) return MOE_ERR_CUDA;
-    if ((rc = moe_router_logits(x_bf16, w_router_bf16, s.T, s.H, s.E, d_logits, status_word, st)) != MOE_OK) return rc;
+    if ((rc = router_logits_impl(x_bf16, w_router_bf16, s.T, s.H, s.E, d_logits, status_word, st, RouterOrder::kFront)) != MOE_OK) return rc;
     StatusRef status;
     if ((rc = resolve_status(status_word, &status)) != MOE_OK) return rc;
     const ExpertWeights shared{shared_w13, shared_w13_scale, shared_w2, shared_w2_scale, false};
@@ -557,7 +564,8 @@ int moe_ffn_block(const void* x_bf16, const void* w_router_bf16, const uint8_t* 
     rc = twoterm2 ? launch_expert_ffn_twoterm(in2, d_off2, shared, sh1, sh1, guard2, act2, d_ys, status_word, st, nullptr, true, d_off2 + 2, &n_cta2)
                   : launch_expert_ffn_native(xb, d_off2, shared, sh1, act2, d_ys, status, st, nullptr, d_off2 + 2, &n_cta2);
     if (rc != MOE_OK ||
-        (rc = launch_router_logits(xb, static_cast<const __nv_bfloat16*>(w_router_bf16), s.T, s.H, s.E, d_logits, status_word, st, true)) != MOE_OK ||
+        (rc = launch_router_logits(xb, static_cast<const __nv_bfloat16*>(w_router_bf16), s.T, s.H, s.E, d_logits, status_word, st,
+                                   RouterOrder::kBeside)) != MOE_OK ||
         (rc = route_and_ffn(d_logits, x_bf16, d_ids, d_w, d_off, nullptr, true, routed, shape, d_xp, d_perm, d_inv, d_y, status_word, inner,
                             L.inner_bytes, st)) != MOE_OK)
       return rc;
@@ -565,7 +573,7 @@ int moe_ffn_block(const void* x_bf16, const void* w_router_bf16, const uint8_t* 
     if (guard2 && (rc = launch_twoterm_again(in2, d_off2, shared, sh1, act2, d_ys, status_word, st)) != MOE_OK) return rc;
     return moe_combine_shared(d_y, d_inv, d_w, d_ys, shape, out_bf16, st);
   }
-  if ((rc = moe_router_logits(x_bf16, w_router_bf16, s.T, s.H, s.E, d_logits, status_word, st)) != MOE_OK) return rc;
+  if ((rc = router_logits_impl(x_bf16, w_router_bf16, s.T, s.H, s.E, d_logits, status_word, st, RouterOrder::kFront)) != MOE_OK) return rc;
   if ((rc = route_and_ffn(d_logits, x_bf16, d_ids, d_w, d_off, d_off2, true, routed, shape, d_xp, d_perm, d_inv, d_y, status_word, inner,
                           L.inner_bytes, st)) != MOE_OK)
     return rc;

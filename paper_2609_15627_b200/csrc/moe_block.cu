@@ -29,11 +29,12 @@ constexpr int kGemvWarps = 8;
 
 __global__ void __launch_bounds__(kGemvWarps * 32) router_gemv_kernel(const __nv_bfloat16* __restrict__ x,
                                                                       const __nv_bfloat16* __restrict__ wr, int T, int H,
-                                                                      int E, float* __restrict__ logits, int beside) {
+                                                                      int E, float* __restrict__ logits, RouterOrder order) {
   extern __shared__ __align__(16) unsigned char smem_x[];  // [T][H] bf16
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  pdl_launch_dependents();
-  if (!beside) pdl_wait();  // x may be the output of the kernel before this one
+  // (alone, the next kernel starts when this one has ended: moe_route and its like read the logits before they wait)
+  if (order != RouterOrder::kAlone) pdl_launch_dependents();
+  if (order != RouterOrder::kBeside) pdl_wait();  // x may be the output of the kernel before this one
   const int n16 = T * H / 8;
   for (int i = tid; i < n16; i += blockDim.x) reinterpret_cast<uint4*>(smem_x)[i] = __ldg(reinterpret_cast<const uint4*>(x) + i);
   __syncthreads();
@@ -248,7 +249,7 @@ __global__ void shared_join_kernel(const int* finished, int n_cta, int* status) 
 }  // namespace
 
 int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, int T, int H, int E, float* logits, int* status,
-                         cudaStream_t st, bool beside) {
+                         cudaStream_t st, RouterOrder order) {
   if (T <= kGemvMaxTok && static_cast<size_t>(T) * H * 2 <= 160 * 1024) {
     const size_t smem = static_cast<size_t>(T) * H * 2;
     static PerDeviceFlag flag;
@@ -257,7 +258,7 @@ int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, 
         }))
       return MOE_ERR_CUDA;
     if (launch_pdl(router_gemv_kernel, dim3((E + kGemvWarps - 1) / kGemvWarps), dim3(kGemvWarps * 32), smem, st, x, w_router, T, H, E,
-                   logits, beside ? 1 : 0) != cudaSuccess)
+                   logits, order) != cudaSuccess)
       return MOE_ERR_CUDA;
     note_kernel("router_gemv_warp_per_expert", 1);
     return MOE_OK;
@@ -275,7 +276,7 @@ int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, 
   const dim3 grid((T + kRM - 1) / kRM, (E + cols - 1) / cols);
   // (the kernel has no wait of its own: launched as a programmatic dependent it runs beside the launches in front of it)
   const auto kernel = cols == 16 ? router_gemm_kernel<16> : router_gemm_kernel<64>;
-  if (beside) {
+  if (order == RouterOrder::kBeside) {
     if (launch_pdl(kernel, grid, dim3(kRThreads), smem, st, tm_x, tm_w, T, H, E, logits, status) != cudaSuccess) return MOE_ERR_CUDA;
   } else {
     kernel<<<grid, kRThreads, smem, st>>>(tm_x, tm_w, T, H, E, logits, status);

@@ -331,9 +331,12 @@ int launch_decode_one(const float* logits, const __nv_bfloat16* x, const ExpertW
                       cudaStream_t st, const ExpertWeights* shared = nullptr);
 
 // router projection, join with the shared expert, and the shared expert's offsets {0, T} (moe_block.cu)
-// `beside`: the logits are computed beside the launches in front, without waiting for them; x and w_router are complete
+// Where the router projection stands in its stream.  kAlone: whatever comes next may read the logits as it starts.  kFront: what
+// comes next is this library's and waits before it reads them, so it may set up meanwhile.  kBeside: likewise, and the logits
+// are computed beside the launches in front, without waiting for them; x and w_router are complete.
+enum class RouterOrder : int { kAlone, kFront, kBeside };
 int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, int T, int H, int E, float* logits, int* status,
-                         cudaStream_t st, bool beside = false);
+                         cudaStream_t st, RouterOrder order);
 // expert-parallel sharding: the table of output rows (see moe_ep_row_table)
 int launch_ep_row_table(const int* perm, const int* offsets, int k, int H, int e_begin, int e_end, float* const* owner_y, int world,
                         int tokens_per_rank, float** row_dst, cudaStream_t st, int max_rows);

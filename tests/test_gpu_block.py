@@ -133,6 +133,49 @@ def test_ffn_block_prefill_8k_sampled():
     _check_block(wl, seed=9, sample=sorted(set([0, wl.T - 1] + rng.integers(0, wl.T, 30).tolist())))
 
 
+# The calls that read logits before they wait (up to 32 tokens) directly behind the projection that writes them, queued up in a
+# graph: every pair finds the logits of other tokens, or ones that choose other experts, in the buffer
+@pytest.mark.parametrize("T", [1, 2, 16, 17, 32])
+@pytest.mark.parametrize("call", ["route", "layer", "forward"])
+def test_what_follows_the_router_projection_reads_its_logits(T, call):
+    H, I, E, k = 4096, 256, 32, 4
+    sh = moe.shape(T, H, I, E, k)
+    w = tuple(dev(a) for a in inputs.make_expert_weights(H, I, E, seed=0))
+    wr, xs = dev(_router_weights(E, H, 5)), [dev(inputs.make_x(T, H, 50 + i)) for i in range(6)]
+    lg, buf, fws = torch.empty((T, E), device="cuda"), moe.LayerBuffers(sh), moe.alloc_forward_workspace(sh)
+    ids = [torch.zeros((T, k), dtype=torch.int32, device="cuda") for _ in xs]
+    outs = [torch.zeros((T, H), dtype=torch.bfloat16, device="cuda") for _ in xs]
+
+    def pair(x, ids, out):
+        moe.moe_router_logits(x, wr, lg, buf.status)
+        if call == "route":
+            moe.moe_route(lg, k, ids, buf.topk_w, buf.expert_offsets, buf.ws)
+        elif call == "layer":
+            buf.topk_ids, buf.out = ids, out
+            moe.moe_layer(lg, x, w, buf)
+        else:
+            moe.moe_forward(lg, x, *w, sh, out, ids, buf.topk_w, buf.status, fws)
+    want = []
+    for x, i, o in zip(xs, ids, outs):
+        pair(x, i, o)
+        torch.cuda.synchronize()
+        want.append((O.route(lg.cpu().numpy(), k)[0], o.clone()))
+        assert np.array_equal(i.cpu().numpy(), want[-1][0])
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for a in zip(xs, ids, outs):
+            pair(*a)
+    for _ in range(5):
+        lg.copy_(torch.arange(E, device="cuda").expand(T, E))
+        for t in (*ids, *outs):
+            t.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert int(buf.status.item()) == 0
+        for (wi, wo), i, o in zip(want, ids, outs):
+            assert np.array_equal(i.cpu().numpy(), wi) and torch.equal(o.view(torch.int16), wo.view(torch.int16))
+
+
 # Up to 256 tokens the shared expert, the router projection and the routing run beside one another: the block is its steps, bit for
 # bit, also where calls follow one another on one workspace and in a graph (17 tokens: router GEMM; above 32 the shared expert's
 # kernel is another)
