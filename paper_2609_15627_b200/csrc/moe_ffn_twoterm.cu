@@ -833,8 +833,11 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     }
   } else if (wid == 2) {
     // =========================== tokens (likewise) ===========================
-    if (first < total) pdl_wait();  // the rows and scale factors are complete.  (A CTA without items leaves at once: kernels further down
-                                    // the stream may be waiting for its SM to start beside this one, see moe_ffn_block.)
+    // The rows and scale factors are complete.  (A CTA without items leaves at once: kernels further down the stream may be waiting
+    // for its SM to start beside this one, see moe_ffn_block.  Where no CTA has any - an expert-parallel rank without rows -
+    // one pair waits all the same: each kernel of a stream waits for the one in front only, which must therefore not
+    // end before those in front of it.)
+    if (first < total || (total == 0 && pair == 0)) pdl_wait();
     int s = 0;
     uint32_t ph = 0;
     const uint32_t full_own = smem_u32(full), full_first = tt_first_addr(full);

@@ -77,6 +77,49 @@ def test_the_kernel_a_rank_runs_and_the_rows_it_writes():
     assert np.array_equal(table[p], want_addr)
 
 
+# A rank whose experts get no rows: its launches wait for one another all the same, so the calls queued behind them find their
+# buffers as they should (two-term kernel without and with the look for experts to be done again, eight-term kernel)
+@pytest.mark.parametrize("T,H,I,E,k,kernel", [(512, 1024, 512, 32, 2, "ffn_mxf8_two_term_cta_pair"), (1200, 1024, 512, 32, 2, "ffn_mxf8_two_term_cta_pair"),
+                                              (24, 1024, 512, 32, 2, "ffn_native_mxf4_block_scaled")])
+def test_a_rank_without_rows_between_calls_that_have_some(T, H, I, E, k, kernel):
+    sh, world = moe.shape(T, H, I, E, k), 4
+    wd = tuple(dev(a) for a in inputs.make_expert_weights(H, I, E, seed=2))
+    b = ep.RankBuffers(torch, moe, sh, world, 1)
+    spare = [torch.zeros_like(b.y_own) for _ in range(world - 1)]
+    b.owner_y.copy_(torch.tensor([t.data_ptr() for t in (spare[0], b.y_own, *spare[1:])], dtype=torch.int64))
+    local = ep.slice_weights(wd, b.e_begin, b.e_end)
+    steps = []
+    for i in range(6):
+        lg = inputs.make_logits(T, E, 60 + i)
+        lg[:, b.e_begin:b.e_end] += -50.0 if i % 2 == 0 else 1.0
+        steps.append((dev(lg), dev(inputs.make_x(T, H, 70 + i))))
+    for i, (lg, x) in enumerate(steps):  # the last step has rows: what it leaves is compared
+        ep.compute(moe, b, lg, x, local)
+        torch.cuda.synchronize()
+        assert moe.moe_last_kernel_name() == kernel and int(b.layer.status.item()) == 0
+        off = b.layer.expert_offsets
+        assert (int(off[b.e_end]) - int(off[b.e_begin]) == 0) == (i % 2 == 0)
+    want = [t.clone() for t in (b.y_own, *spare, b.layer.expert_offsets, b.layer.inv_perm)]
+
+    def check():
+        torch.cuda.synchronize()
+        assert int(b.layer.status.item()) == 0
+        assert all(torch.equal(t, v) for t, v in zip((b.y_own, *spare, b.layer.expert_offsets, b.layer.inv_perm), want))
+
+    def queue():
+        for lg, x in steps:
+            ep.compute(moe, b, lg, x, local)
+    for _ in range(3):
+        queue()
+    check()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        queue()
+    for _ in range(3):
+        g.replay()
+    check()
+
+
 def test_production_decode_shape_on_eight_ranks():
     wl = inputs.WORKLOADS["decode_c64"]
     w, logits, x = _layer(wl.T, wl.H, wl.I, wl.E, wl.k, seed=0)
