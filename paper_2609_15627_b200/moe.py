@@ -404,12 +404,12 @@ def moe_layer(logits, x, weights, buf, stream=None):
     sh = buf.sh
     stream = _stream(stream)
     T, E = logits.shape
-    if T == sh.T and E == sh.E and lib().moe_layer(  # the four calls in one, which takes a small layer's host time from four trips to one
-            _ptr(logits), _ptr(x), _ptr(w13), _ptr(s13), _ptr(w2), _ptr(s2), C.byref(sh), _ptr(buf.topk_ids), _ptr(buf.topk_w),
-            _ptr(buf.expert_offsets), _ptr(buf.x_perm), _ptr(buf.perm), _ptr(buf.inv_perm), _ptr(buf.y_perm), _ptr(buf.out),
-            _ptr(buf.status), _ptr(buf.ws), buf.ws.numel(), stream) == 0:
+    if T == sh.T and E == sh.E:  # the four calls in one, which takes a small layer's host time from four trips to one
+        _check(lib().moe_layer(_ptr(logits), _ptr(x), _ptr(w13), _ptr(s13), _ptr(w2), _ptr(s2), C.byref(sh), _ptr(buf.topk_ids),
+                               _ptr(buf.topk_w), _ptr(buf.expert_offsets), _ptr(buf.x_perm), _ptr(buf.perm), _ptr(buf.inv_perm),
+                               _ptr(buf.y_perm), _ptr(buf.out), _ptr(buf.status), _ptr(buf.ws), buf.ws.numel(), stream), "moe_layer")
         return buf.out
-    # (the call that fails says so itself)
+    # logits of another size than the buffers' shape: moe_route takes the logits' own
     moe_route(logits, sh.k, buf.topk_ids, buf.topk_w, buf.expert_offsets, buf.ws, stream)
     moe_permute(x, buf.topk_ids, buf.expert_offsets, sh, buf.x_perm, buf.perm, buf.inv_perm, buf.ws, stream)
     moe_expert_ffn(buf.x_perm, buf.expert_offsets, w13, s13, w2, s2, sh, buf.y_perm, buf.status, buf.ws, stream)

@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2609_15627_b200 import build_ext, moe
 
@@ -69,6 +70,36 @@ def test_argument_errors_are_found_on_the_host(L):
     assert L.moe_forward(fake, fake, fake, fake, fake, fake, C.byref(bad), fake, null, null, null, big, 1 << 30, null) == 2
     assert L.moe_forward(fake, fake, fake, fake, fake, fake, C.byref(sh), fake, null, null, null, big, 64, null) == 3
     assert L.moe_forward(fake, fake, fake, fake, fake, fake, C.byref(sh), fake, null, null, null, null, 1 << 30, null) == 3
+
+
+def test_layer_argument_errors_are_those_of_the_four_calls(L):
+    sh, bad = moe.shape(4, 256, 128, 8, 2), moe.shape(4, 200, 128, 8, 2)
+    fake, odd, null = C.c_void_p(0x1000), C.c_void_p(0x1004), C.c_void_p(0)
+
+    def call(shape=sh, ws=fake, ws_bytes=1 << 30, status=null, **at):  # at: argument number -> pointer
+        a = [fake] * 6 + [None if shape is None else C.byref(shape)] + [fake] * 8 + [status, ws, ws_bytes, null]
+        for i, p in at.items():
+            a[int(i[1:])] = p
+        return L.moe_layer(*a)
+    for i in (*range(6), *range(7, 15)):
+        assert call(**{"a%d" % i: null}) == 1 and call(**{"a%d" % i: odd}) == 1, i
+    assert call(status=C.c_void_p(0x1002)) == 1
+    assert call(shape=None) == 1 and call(shape=bad) == 2
+    assert call(shape=moe.shape(4, 256, 128, 8, 9)) == 1 and call(shape=moe.shape(4, 256, 128, 2048, 2)) == 2
+    assert call(ws=null) == 3 and call(ws=C.c_void_p(0x1010)) == 3 and call(ws_bytes=moe.moe_workspace_bytes(sh) - 1) == 3
+
+
+def test_layer_that_fails_raises_and_does_nothing_else(L, monkeypatch):
+    sh = moe.shape(4, 256, 128, 8, 2)
+    buf = moe.LayerBuffers(sh, device="cpu")             # validation fails before anything is dereferenced
+    def not_called(*a, **k):
+        raise AssertionError("a failed call was made again in parts")
+    for name in ("moe_route", "moe_permute", "moe_expert_ffn", "moe_combine"):
+        monkeypatch.setattr(moe, name, not_called)
+    w = tuple(torch.zeros(64, dtype=torch.uint8) for _ in range(4))
+    x = torch.zeros(4 * 256 + 1, dtype=torch.bfloat16)[1:]  # 2 bytes past an aligned address
+    with pytest.raises(moe.MoeError, match="moe_layer failed: invalid argument"):
+        moe.moe_layer(torch.zeros(4, 8), x, w, buf, stream=0)
 
 
 def test_prepack_sizes_and_argument_errors(L):
