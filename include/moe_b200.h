@@ -238,7 +238,7 @@ int moe_forward_packed(const float* logits /* [T,E] */, const void* x_bf16 /* [T
  * moe_forward with HOST input and output for one batch: copies logits_host [T,E] and x_host [T,H] to
  * device buffers carved from `ws`, clears moe_forward's counters where they are used, runs moe_forward on `cuda_stream`,
  * copies out [T,H] bf16 back into out_host and waits for the stream.  Fewer stream operations with page-locked memory that the
- * device can address (16-byte aligned): the output is written there by the last kernel itself; a single token row, and the
+ * device can address (the whole buffer, 16-byte aligned): the output is written there by the last kernel itself; a single token row, and the
  * logits and rows of a batch whose routing, sort and split are one launch (see moe_forward), are read there by that launch.
  * Otherwise logits of at most 64 KB travel in one copy with the zeros of moe_forward's counter block, through a page-locked
  * staging buffer that the library allocates once per host thread (the only allocation any entry point makes, on its first call).

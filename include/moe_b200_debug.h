@@ -37,6 +37,11 @@ int moe_debug_native_cta_share(int32_t n_ctas, int32_t cta, int32_t n_touched, i
  * (row outside [0, 128), n_pieces outside [1, 8], piece outside [0, n_pieces)). */
 int moe_debug_native_scale_slot(int32_t row, int32_t piece, int32_t n_pieces);
 
+/* Host, diagnostic.  Where the device addresses the host buffer [host, host + bytes) that moe_forward_host lets kernels read or
+ * write in place, or NULL where it copies: memory that is not page-locked from the first byte to the last, or not in one
+ * piece for the device, or not 16-byte aligned there. */
+void* moe_debug_host_view(const void* host, size_t bytes);
+
 /* Diagnostic: the one-launch kernel of moe_forward for any batch it can take (up to 4 tokens, T*k <= 32), where
  * moe_forward itself would run the four calls because they are faster from 2 tokens on.  Same arguments, workspace and
  * result as moe_forward; MOE_ERR_UNSUPPORTED_SHAPE if the kernel cannot take the shape.  For the tests. */

@@ -796,13 +796,19 @@ unsigned char* logits_staging() {
   }
   return buf;
 }
-// A buffer of the caller as the device addresses it, where it can (pinned host memory under unified addressing), or null
-void* device_view(const void* host) {
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, host) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer != nullptr && aligned(at.devicePointer, 16))
-    return at.devicePointer;
-  cudaGetLastError();  // pageable memory: not an error of this call
-  return nullptr;
+// A buffer of the caller as the device addresses it, where it can (pinned host memory under unified addressing), or null.  Memory is
+// pinned page by page, so a buffer whose last byte is not pinned, or lies elsewhere for the device, is left to the copies.
+void* device_view(const void* host, size_t bytes) {
+  const auto address = [](const void* p) -> char* {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeHost) return static_cast<char*>(at.devicePointer);
+    cudaGetLastError();  // pageable memory: not an error of this call
+    return nullptr;
+  };
+  if (bytes == 0) return nullptr;
+  char* first = address(host);
+  if (!aligned(first, 16) || address(static_cast<const char*>(host) + bytes - 1) != first + bytes - 1) return nullptr;
+  return first;
 }
 int forward_host_impl(const float* logits_host, const void* x_host_bf16, const ExpertWeights& w, const moe_shape_t* shape,
                       void* out_host_bf16, int32_t* status_word, void* ws, size_t ws_bytes, void* cuda_stream) {
@@ -819,21 +825,21 @@ int forward_host_impl(const float* logits_host, const void* x_host_bf16, const E
   // The output goes straight to the caller's buffer where the device can address it: the last kernel's stores cross the bus
   // instead of a copy operation enqueued after it (4096-wide rows: 16 tokens 244 -> 234 us a call with the next one, 256 tokens 742 -> 731, 1300 tokens 1223 -> 1207).
   const size_t out_bytes = static_cast<size_t>(s.T) * s.H * 2;
-  void* out_view = device_view(out_host_bf16);
+  void* out_view = device_view(out_host_bf16, out_bytes);
   const bool direct = out_view != nullptr;
   if (direct) d_out = out_view;
   // Likewise what a kernel reads once is read where it lies: a single token's row (the few CTAs that split it fetch 512 bytes
   // each), and the logits and rows of a batch whose front is one launch (up to 256 tokens).
   const bool one = s.T == 1 && decode_one_ok(s, w.w13, w.w2), front = s.T > 1 && front_in_one(s, w);
-  void* x_view = one || front ? device_view(x_host_bf16) : nullptr;
+  void* x_view = one || front ? device_view(x_host_bf16, out_bytes) : nullptr;  // (as large as the output)
   const bool x_direct = x_view != nullptr;
   if (x_direct) d_x = x_view;
-  void* logits_view = front ? device_view(logits_host) : nullptr;
+  const size_t lg_bytes = static_cast<size_t>(s.T) * s.E * 4, lg_span = L.inner - L.logits;
+  void* logits_view = front ? device_view(logits_host, lg_bytes) : nullptr;
   // This call owns its workspace's contents: it clears the counter block of moe_forward itself.  Small logits go through
   // a page-locked staging buffer of this thread that ends in zeros, so that one copy brings both (the call waits for the
   // stream before it returns, so the buffer is free again by then).
   // (with more than one token no kernel uses the counter block)
-  const size_t lg_bytes = static_cast<size_t>(s.T) * s.E * 4, lg_span = L.inner - L.logits;
   unsigned char* stage = logits_view == nullptr && lg_span <= kStageLogitsBytes ? logits_staging() : nullptr;
   if (logits_view != nullptr) {
     d_logits = static_cast<float*>(logits_view);
@@ -856,6 +862,8 @@ int forward_host_impl(const float* logits_host, const void* x_host_bf16, const E
   return MOE_OK;
 }
 }  // namespace
+
+void* moe_debug_host_view(const void* host, size_t bytes) { return device_view(host, bytes); }
 
 int moe_forward_host(const float* logits_host, const void* x_host_bf16, const uint8_t* w13, const uint8_t* w13_scale,
                      const uint8_t* w2, const uint8_t* w2_scale, const moe_shape_t* shape, void* out_host_bf16,

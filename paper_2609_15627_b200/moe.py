@@ -17,7 +17,7 @@ EXPORTS = ("moe_workspace_bytes", "moe_status_string", "moe_last_kernel_name", "
            "moe_forward_workspace_bytes", "moe_forward_sync_bytes", "moe_forward",
            "moe_forward_host_workspace_bytes", "moe_forward_host", "moe_expert_ffn_noalloc_max_bytes",
            "moe_expert_ffn_noalloc", "moe_debug_native_cta_share", "moe_debug_native_scale_slot", "moe_debug_read_probe", "moe_prepack_bytes", "moe_prepack",
-           "moe_expert_ffn_packed", "moe_forward_packed", "moe_forward_host_packed", "moe_debug_forward_one_launch",
+           "moe_expert_ffn_packed", "moe_forward_packed", "moe_forward_host_packed", "moe_debug_host_view", "moe_debug_forward_one_launch",
            "moe_debug_expert_ffn_variant", "moe_router_logits", "moe_combine_shared", "moe_ffn_block_workspace_bytes",
            "moe_ffn_block", "moe_expert_ffn_q_workspace_bytes", "moe_expert_ffn_q",
            "moe_ep_permute", "moe_ep_row_table", "moe_ep_expert_ffn", "moe_layer")
@@ -87,6 +87,8 @@ def lib():
         L.moe_forward_packed.argtypes = [vp, vp, vp, C.POINTER(Shape), vp, vp, vp, vp, vp, sz, vp]
         L.moe_forward_host_packed.restype = C.c_int
         L.moe_forward_host_packed.argtypes = [vp, vp, vp, C.POINTER(Shape), vp, vp, vp, sz, vp]
+        L.moe_debug_host_view.restype = vp
+        L.moe_debug_host_view.argtypes = [vp, sz]
         L.moe_debug_read_probe.restype = C.c_int
         L.moe_debug_read_probe.argtypes = [vp, sz, vp, sz, vp, vp]
         L.moe_forward_workspace_bytes.restype = sz

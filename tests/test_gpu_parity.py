@@ -664,6 +664,26 @@ def test_forward_host_sequence_of_shapes_and_pageable_buffers():
             assert_same_up_to_rounding(oh.numpy().view(np.uint16), bits(out4))
 
 
+def test_only_buffers_page_locked_to_their_last_byte_are_used_in_place():
+    """moe_forward_host hands such buffers to its kernels; a kernel must not reach a page that is not the device's."""
+    view, rt, page = moe.lib().moe_debug_host_view, torch.cuda.cudart(), 4096
+    torch.cuda.init()
+    raw = np.zeros(17 * page, np.uint8)
+    base = -(-raw.ctypes.data // page) * page
+    half, whole = 8 * page, 16 * page
+    assert view(base, whole) is None
+    assert int(rt.cudaHostRegister(base, half, 0)) == 0
+    try:
+        at = view(base, half)
+        assert at is not None and view(base + 64, half - 64) == at + 64 and view(base, 16) == at
+        assert view(base, half + 1) is None and view(base, whole) is None and view(base + half - 16, 32) is None
+        assert view(base + half, half) is None and view(base + 4, 64) is None and view(base, 0) is None
+    finally:
+        assert int(rt.cudaHostUnregister(base)) == 0
+    pinned = torch.zeros(3 * page + 100, dtype=torch.uint8).pin_memory()
+    assert view(pinned.data_ptr(), pinned.numel()) is not None
+
+
 # ---- moe_prepack and the calls that take its result ------------------------------------------------------
 
 def _tiles(a, tile_bytes):
