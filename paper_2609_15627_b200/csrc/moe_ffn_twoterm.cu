@@ -620,9 +620,10 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
 // 166 us for 0.61 GB, 0.56 of the copy rate.  (A warp's part collected in shared memory and sent with one bulk copy per slot and
 // term: 181 us.)
 // What it writes is written at the rate at which memory takes writes alone (3.9 TB/s; a copy reaches 6.5 with the half that it reads).
-// `rows` (may be null): the bf16 rows in sorted order as well, for a caller whose buffer they are (moe_layer): 11 us less than the
-// copy and a split from it (8216 slots of 4096: the layer 238 -> 227 us; 12288 slots 1123 -> 1108). ----
-template <bool kGuard>
+// kRows: into `rows` the bf16 rows in sorted order as well, for a caller whose buffer they are (moe_layer): 11 us less than the
+// copy and a split from it (8216 slots of 4096: the layer 238 -> 227 us; 12288 slots 1123 -> 1108).  (Asked at run time, slot by
+// slot, it took the form without it from 40 to 48 registers and made that of moe_forward's prompts spill.) ----
+template <bool kGuard, bool kRows>
 __global__ void __launch_bounds__(256) twoterm_scatter_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ ids,
                                                              const int* __restrict__ inv_perm, const int* __restrict__ offsets,
                                                              uint8_t* __restrict__ xq, uint8_t* __restrict__ sfx, int T, int k, int H,
@@ -665,7 +666,7 @@ __global__ void __launch_bounds__(256) twoterm_scatter_kernel(const __nv_bfloat1
         const size_t row = static_cast<size_t>(__shfl_sync(0xffffffffu, p, j));
         reinterpret_cast<uint2*>(xq + row * H)[c * 32 + lane] = hi;
         reinterpret_cast<uint2*>(xq + (S + row) * H)[c * 32 + lane] = lo;
-        if (rows != nullptr) reinterpret_cast<uint4*>(rows + row * H)[c * 32 + lane] = v;
+        if (kRows) reinterpret_cast<uint4*>(rows + row * H)[c * 32 + lane] = v;
         const size_t at = __shfl_sync(0xffffffffu, static_cast<unsigned long long>(sf_hi), j);
         const int d = __shfl_sync(0xffffffffu, sf_lo, j);
         if ((lane & 15) == 0) *reinterpret_cast<uint32_t*>(sfx + at + step) = word;
@@ -1344,9 +1345,11 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
     const int chunks = per_token >= static_cast<size_t>(n_chunk) ? 1 : (per_token <= 1 ? n_chunk : (n_chunk + static_cast<int>(per_token) - 1) / static_cast<int>(per_token));
     parts = (n_chunk + chunks - 1) / chunks;
     const size_t want = (static_cast<size_t>(sh.T) * parts + 7) / 8;
-    rc = launch_pdl(guard ? twoterm_scatter_kernel<true> : twoterm_scatter_kernel<false>, dim3(static_cast<unsigned>(want < most ? want : most)), dim3(256), table_bytes, st, in.x,
+    const auto scatter = in.write_rows ? (guard ? twoterm_scatter_kernel<true, true> : twoterm_scatter_kernel<false, true>)
+                                       : (guard ? twoterm_scatter_kernel<true, false> : twoterm_scatter_kernel<false, false>);
+    rc = launch_pdl(scatter, dim3(static_cast<unsigned>(want < most ? want : most)), dim3(256), table_bytes, st, in.x,
                     in.ids, in.inv_perm, offsets, base + L.xq, base + L.sfx, sh.T, sh.k, sh.H, sh.E, geo.max_tok, geo.sf_step, chunks,
-                    marks, flags, in.offsets_late ? 1 : 0, in.write_rows ? in.x_sorted : nullptr);
+                    marks, flags, in.offsets_late ? 1 : 0, in.x_sorted);
   } else {
     const size_t want = (S * parts + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
     rc = launch_pdl(guard ? twoterm_split_kernel<false, true> : twoterm_split_kernel<false, false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256), table_bytes, st, in.x,
