@@ -201,15 +201,19 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
   // ---- set-up: barriers, tensor memory, descriptors ----
   if (tid == 32 * 3) {
     prefetch_tmap(&tmap_w13);
-    prefetch_tmap(&tmap_s13);
     prefetch_tmap(&tmap_w2);
-    prefetch_tmap(&tmap_s2);
     prefetch_tmap(&tmap_a1);
+    if (!a.blocked) {  // (tiles have no maps of their scale bytes, see weight_maps)
+      prefetch_tmap(&tmap_s13);
+      prefetch_tmap(&tmap_s2);
+    }
     if (a.n_shared) {
       prefetch_tmap(&tmap_sw13);
-      prefetch_tmap(&tmap_ss13);
       prefetch_tmap(&tmap_sw2);
-      prefetch_tmap(&tmap_ss2);
+      if (!a.blocked_shared) {
+        prefetch_tmap(&tmap_ss13);
+        prefetch_tmap(&tmap_ss2);
+      }
     }
   }
   if (tid == 0) {

@@ -381,9 +381,9 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
   // ---- setup: touched experts, barriers, tensor memory ----
   if (tid == 32 * 3) {  // a warp with nothing to set up fetches the tensor maps
     prefetch_tmap(&tmap_w13);
-    prefetch_tmap(&tmap_s13);
     prefetch_tmap(&tmap_w2);
-    prefetch_tmap(&tmap_s2);
+    if (!a.blocked && a.H % 512 == 0) prefetch_tmap(&tmap_s13);  // (see weight_maps)
+    if (!a.blocked && a.I % 512 == 0) prefetch_tmap(&tmap_s2);
     for (int i = 0; i < kTermBoxes; ++i) {
       prefetch_tmap(&tmap_a1.box[i]);
       prefetch_tmap(&tmap_a2.box[i]);
@@ -1302,14 +1302,13 @@ bool bf16_map_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t rows
 bool weight_maps(const ExpertWeights& w, const moe_shape_t& sh, CUtensorMap* tm_w13, CUtensorMap* tm_s13, CUtensorMap* tm_w2,
                  CUtensorMap* tm_s2) {
   const uint64_t r13 = static_cast<uint64_t>(sh.E) * 2 * sh.I, r2 = static_cast<uint64_t>(sh.E) * sh.H;
-  if (w.blocked)  // every tile is [128 rows][128 or 16 bytes], tiles one after the other
-    return nat_map(tm_w13, w.w13, 128, r13 * (sh.H / 256), 128, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
-           nat_map(tm_w2, w.w2, 128, r2 * (sh.I / 256), 128, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
-           nat_map(tm_s13, w.s13, 16, r13 * (sh.H / 512), 16, 128, CU_TENSOR_MAP_SWIZZLE_NONE) &&
-           nat_map(tm_s2, w.s2, 16, r2 * (sh.I / 512), 16, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
-  // (scale rows that are not multiples of 16 bytes get no tensor map: the kernel loads them itself)
+  // No tensor map, and none that a kernel looks at, for scale bytes in tiles, which come as contiguous copies, and for
+  // scale rows that are not multiples of 16 bytes, which the kernel loads itself
   std::memset(tm_s13, 0, sizeof(*tm_s13));
   std::memset(tm_s2, 0, sizeof(*tm_s2));
+  if (w.blocked)  // every tile is [128 rows][128 bytes], tiles one after the other
+    return nat_map(tm_w13, w.w13, 128, r13 * (sh.H / 256), 128, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
+           nat_map(tm_w2, w.w2, 128, r2 * (sh.I / 256), 128, 128, CU_TENSOR_MAP_SWIZZLE_128B);
   return nat_map(tm_w13, w.w13, sh.H / 2, r13, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
          nat_map(tm_w2, w.w2, sh.I / 2, r2, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
          (sh.H % 512 != 0 || nat_map(tm_s13, w.s13, sh.H / 32, r13, 16, 128, CU_TENSOR_MAP_SWIZZLE_NONE)) &&
