@@ -214,3 +214,59 @@ def test_ffn_block_is_its_steps(T, H, I, E, k):
         g.replay()
     torch.cuda.synchronize()
     assert int(st.item()) == 0 and all(torch.equal(o.view(torch.int16), want[i % 3].view(torch.int16)) for i, o in enumerate(outs))
+
+
+# The same with what a network does around it: the rows are rewritten in place between calls, in stream order only; blocks of
+# them that two terms hold too little of, so that a shared expert on the two-term kernel is done again behind the join; and
+# without a status word, where the steps run one after the other
+@pytest.mark.parametrize("T,H,I,E,k,again", [(4, 1024, 512, 32, 4, False), (20, 1024, 512, 32, 4, False), (48, 4096, 2048, 16, 6, True),
+                                             (130, 4096, 2048, 32, 2, True)])
+@pytest.mark.parametrize("status", [True, False])
+def test_ffn_block_on_rows_rewritten_in_place(T, H, I, E, k, again, status):
+    routed = tuple(dev(a) for a in inputs.make_expert_weights(H, I, E, seed=0))
+    shared = tuple(dev(a) for a in inputs.make_expert_weights(H, I, 1, seed=21))
+    wr = dev(_router_weights(E, H, 3))
+    sh, sh1 = moe.shape(T, H, I, E, k), moe.shape(T, H, I, 1, 1)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    xs, want = [], []
+    for i in range(3):
+        xf = bf(inputs.make_x(T, H, 40 + i)).copy()
+        if i != 1:                       # 2^15 and eight values below 2^-14 of it, in a block of two rows
+            xf[[0, T - 1], 64 * i:64 * i + 32] = 64.0
+            xf[[0, T - 1], 64 * i + 5] = 2.0 ** 15
+            xf[[0, T - 1], 64 * i + 8:64 * i + 16] = 1.0 + 2.0 ** -7
+        xs.append(dev(inputs.f32_to_bf16_bits(xf)))
+    buf, lg = moe.LayerBuffers(sh), torch.empty((T, E), device="cuda")
+    ys, alone = torch.empty((T, H), device="cuda"), torch.empty((T, H), device="cuda")
+    off2, ws1 = torch.tensor([0, T], dtype=torch.int32, device="cuda"), moe.alloc_workspace(sh1)
+    for i, x in enumerate(xs):
+        moe.moe_router_logits(x, wr, lg, st)
+        moe.moe_layer(lg, x, routed, buf)
+        moe.moe_expert_ffn(x, off2, *shared, sh1, ys, st, ws1)
+        assert (moe.moe_last_kernel_name() == "ffn_mxf8_two_term_cta_pair") == again
+        moe.moe_combine_shared(buf.y_perm, buf.inv_perm, buf.topk_w, ys, sh, buf.out)
+        if again:
+            moe.moe_debug_expert_ffn_variant(x, off2, *shared, sh1, alone, st, ws1, moe.VARIANT_TWOTERM)
+            assert torch.equal(ys, alone) == (i == 1)
+        torch.cuda.synchronize()
+        want.append(buf.out.clone())
+    ws, ids, w = moe.alloc_block_workspace(sh), torch.empty((T, k), dtype=torch.int32, device="cuda"), torch.empty((T, k), device="cuda")
+    outs = [torch.empty((T, H), dtype=torch.bfloat16, device="cuda") for _ in range(7)]
+    x = torch.empty_like(xs[0])
+
+    def calls():
+        for i, o in enumerate(outs):
+            x.copy_(xs[i % 3])
+            moe.moe_ffn_block(x, wr, routed, shared, sh, o, ids, w, st if status else None, ws)
+    calls()
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and all(torch.equal(o.view(torch.int16), want[i % 3].view(torch.int16)) for i, o in enumerate(outs))
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        calls()
+    for o in outs:
+        o.zero_()
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and all(torch.equal(o.view(torch.int16), want[i % 3].view(torch.int16)) for i, o in enumerate(outs))

@@ -288,6 +288,37 @@ def test_whole_layer_and_expert_parallel_ranks_do_experts_again(I, kernel):
     assert int(buf.status.item()) == 0
 
 
+# moe_forward_host where the two-term kernel runs: rows and logits read in place up to 256 tokens (by the gather of experts that are
+# done again as well), the output written in place at any size; and the bf16 kernel's output
+@pytest.mark.parametrize("T,H,I,E,k,ffn,again", [(256, 512, 512, 64, 4, NAME, False), (256, 1024, 512, 64, 32, NAME, True), (300, 512, 512, 64, 4, NAME, False),
+                                                 (1300, 1024, 512, 64, 8, NAME, True), (1500, 512, 512, 8, 2, _UMMA, False)])
+def test_host_buffers_in_place_and_copied(T, H, I, E, k, ffn, again):
+    wdev = tuple(dev(a) for a in _weights(H, I, E, seed=61))
+    xf = inputs.bf16_bits_to_f32(inputs.make_x(T, H, 62))
+    if again:
+        xf[::5, 64] = 2.0 ** 20
+    x, logits = inputs.f32_to_bf16_bits(xf), inputs.make_logits(T, E, 63)
+    sh = moe.shape(T, H, I, E, k)
+    buf = moe.LayerBuffers(sh)
+    moe.moe_layer(dev(logits), dev(x), wdev, buf)
+    want = buf.out.clone()
+    moe.moe_expert_ffn(buf.x_perm, buf.expert_offsets, *wdev, sh, buf.y_perm, buf.status, buf.ws)
+    assert moe.moe_last_kernel_name() == ffn
+    if again:                                      # (it does some experts again: alone the kernel gives other bits)
+        alone = torch.empty_like(buf.y_perm)
+        moe.moe_debug_expert_ffn_variant(buf.x_perm, buf.expert_offsets, *wdev, sh, alone, buf.status, buf.ws, moe.VARIANT_TWOTERM)
+        assert not torch.equal(alone, buf.y_perm)
+    ws = moe.alloc_workspace(sh, host_path=True)
+    lh, xh = torch.from_numpy(logits), torch.from_numpy(x.view(np.int16))
+    for pin in (True, False):
+        oh = torch.zeros((T, H), dtype=torch.int16)
+        bufs = [t.pin_memory() for t in (lh, xh, oh)] if pin else [lh, xh, oh]
+        assert all((moe.lib().moe_debug_host_view(t.data_ptr(), t.numel() * t.element_size()) is not None) == pin for t in bufs)
+        ws.fill_(0x5A)
+        moe.moe_forward_host(bufs[0], bufs[1], *wdev, sh, bufs[2], buf.status, ws)
+        assert int(buf.status.item()) == 0 and torch.equal(bufs[2], want.view(torch.int16).cpu())
+
+
 # (33 and 97 rows per expert: passes of 64 and of 224 tokens; the quantised variant above 64)
 @pytest.mark.parametrize("T,k,H,I,quantised", [(2112, 2, 512, 512, False), (3100, 4, 512, 512, False), (3100, 4, 512, 512, True)])
 def test_offsets_may_come_from_the_launch_in_front(T, k, H, I, quantised):
