@@ -86,12 +86,13 @@ uint64_t moe_launch_count(void);
  *   fixed fp32 sequence: d = max(d,-80); n = rint(d*0x1.715476p+0f); r = fma(n,-0x1.62e4p-1f,d);
  *   r = fma(n,-0x1.7f7d1cp-20f,r); p = Horner/fma over 1/720,1/120,1/24,1/6,1/2,1,1 in r; EXP = p*2^n.
  *   expert_offsets [E+1] int32: exclusive prefix sum of the per-expert slot counts, [E] = T*k.
- * Launch order: for T <= 32 the kernel uses programmatic dependent launch.  It reads logits before it waits
- * for the kernel launched just before it on the stream, and writes its outputs only after that kernel has
- * completed (so the outputs of one layer call may be the buffers the previous call's moe_combine still reads).
- * If that preceding kernel releases its dependents early (cudaTriggerProgrammaticLaunchCompletion /
- * griddepcontrol.launch_dependents), logits must not be among its outputs; moe_combine's are not, and moe_router_logits
- * releases nothing before it has ended.
+ * Launch order: for T <= 32, and up to T = 256 with E <= 256, the kernel uses programmatic dependent launch.  It writes its
+ * outputs only after the kernel launched just before it on the stream has completed (so the outputs of one layer call
+ * may be the buffers the previous call's moe_combine still reads).  From 33 tokens on it reads logits after that as well; up
+ * to 32 tokens before.  So if that preceding kernel releases its dependents early
+ * (cudaTriggerProgrammaticLaunchCompletion / griddepcontrol.launch_dependents), the logits of T <= 32 must not be among its
+ * outputs; moe_combine's are not, and moe_router_logits releases nothing before it has ended.  The same holds for the
+ * logits of moe_layer and moe_forward.
  * Errors: INVALID_ARG (null/misaligned, T<1, k<1, k>E), UNSUPPORTED_SHAPE (E>1024, k>32), WORKSPACE.
  */
 int moe_route(const float* logits, int32_t T, int32_t E, int32_t k, int32_t* topk_ids /* [T,k] */,
@@ -264,7 +265,8 @@ int moe_forward_host_packed(const float* logits_host, const void* x_host_bf16, c
  *   - moe_router_logits: logits[t,e] = sum_h x[t,h] * w_router[e,h]; x [T,H] and w_router [E,H] bf16, fp32
  *     accumulation (each product is exact in fp32; the order of the sum is the kernel's), logits [T,E] fp32.  The paper
  *     states no precision for this step (it kept a vendor BLAS).  H a multiple of 128, E <= 1024.  Up to 16 tokens: one
- *     warp per expert streams w_router once; more: a tcgen05 GEMM on tiles of 128 tokens x 64 experts.
+ *     warp per expert streams w_router once; more: a tcgen05 GEMM on tiles of 128 tokens x 16 or 64 experts.
+ *     Calls that read the logits may follow directly, at any T.
  *   - The shared expert is one more expert in the routed experts' weight format, applied to every token with weight 1:
  *     tensors shaped as the routed ones with E = 1.  It needs no entry point of its own: moe_expert_ffn with x as
  *     x_perm, offsets {0, T} and shape {T, H, I, 1, 1} gives y_shared [T,H] fp32.

@@ -823,7 +823,9 @@ int forward_host_impl(const float* logits_host, const void* x_host_bf16, const E
   void* d_x = base + L.x;
   void* d_out = base + L.out;
   // The output goes straight to the caller's buffer where the device can address it: the last kernel's stores cross the bus
-  // instead of a copy operation enqueued after it (4096-wide rows: 16 tokens 244 -> 234 us a call with the next one, 256 tokens 742 -> 731, 1300 tokens 1223 -> 1207).
+  // instead of a copy operation enqueued after it (4096-wide rows: 16 tokens 244 -> 234 us a call with
+  // the next one, 256 tokens 742 -> 731; the output alone, 1300 tokens 1223 -> 1207, 4096 2928 -> 2881, 8192 5519 -> 5428, 32768
+  // 20948 -> 20636: the stores fill the bus as the copy does, and begin earlier).
   const size_t out_bytes = static_cast<size_t>(s.T) * s.H * 2;
   void* out_view = device_view(out_host_bf16, out_bytes);
   const bool direct = out_view != nullptr;

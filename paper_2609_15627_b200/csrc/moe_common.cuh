@@ -98,8 +98,9 @@ inline TwoTermScratch twoterm_scratch(const moe_shape_t& s) {
   L.total = off;
   return L;
 }
-// When it is chosen.  Measured on packed weights of 256 experts of 4096 x 2048, top-8, the expert-FFN call: 128 tokens 0.55
-// ms against 0.56 on the eight-term kernel, 333 tokens 0.58 against 0.86, 768 tokens 0.64 against 1.60; against the bf16
+// When it is chosen.  Measured on packed weights of 256 experts of 4096 x 2048, top-8, layers in a row: 64 tokens 527 us against
+// 446 on the eight-term kernel, 128 tokens 608 and 533, 333 tokens 641 and 886, 768 tokens 743 and 1573 (for the line between
+// them see twoterm_chosen); the expert-FFN call against the bf16
 // kernel 1024 tokens 0.69 and 1.96 ms, 4096 tokens 1.56 and 2.05, 8192 tokens 2.9 and 3.3; at I = 256 1027 tokens take 0.22
 // ms against 2.8 on the streaming kernel.  Below four rows per expert the eight-term kernel reads the weights as fast
 // as HBM delivers them, in one launch less; with fewer items than SMs the finer items of the other kernels fill more of the
@@ -369,12 +370,18 @@ inline bool once_per_device(PerDeviceFlag& f, F&& set) {
 // ---- programmatic dependent launch (host) ------------------------------------------------------
 // The kernel may start while its predecessor in the stream is still running; it must execute
 // griddepcontrol.wait before it reads anything the predecessor writes, and before it writes anything at all to
-// global memory.  Most kernels here wait first and then release their own dependent; route_kernel, native_split_kernel
-// and the expert-FFN kernels release theirs BEFORE they wait, so three or four neighbours of a chain (route, permute,
-// split, expert FFN) can be resident together.  That is safe because of the rule above: whatever a kernel does before
-// its wait only reads buffers that no kernel of the chain before it writes (logits, expert_offsets of a completed
-// router, the weights), and every global write comes after the wait, i.e. after everything launched earlier on the
-// stream has completed.
+// global memory.  Most kernels here wait first and then release their own dependent; route_kernel, route_sort_kernel,
+// native_split_kernel, native_quant_rows_kernel, native_expand_kernel, twoterm_scatter_kernel and the expert-FFN kernels
+// release theirs BEFORE they wait, so three or four neighbours of a chain (route, permute, split, expert FFN) can be
+// resident together.  That is safe because of the rule above: whatever a kernel does before its wait only reads buffers
+// that no kernel of the chain before it writes (logits, expert_offsets of a completed router, the weights), and every
+// global write comes after the wait, i.e. after everything launched earlier on the stream has completed - for the wait is
+// for the launch in front only, and that has waited in its turn, whether it had work or not.  shared_offsets_kernel and
+// shared_join_kernel release by ending; so does router_gemv_kernel but inside moe_ffn_block (see RouterOrder).
+// One launch waits for nothing: the router projection beside the shared expert (RouterOrder::kBeside).  It starts when all
+// CTAs of the launches in front have, the first of which ended before the next began; what it reads is complete by then,
+// and it writes the logits, which only the launch behind it reads.  But its end says nothing of the launches in front, so
+// those count their CTAs out and the join waits for the count.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};

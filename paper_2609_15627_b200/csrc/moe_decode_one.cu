@@ -407,8 +407,8 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
     // ---- the token row -> 8 E2M1 term rows.  Splitting the whole row in every CTA would cost several microseconds of
     // issue time (eight dependent terms for each of H/32 blocks), so the first H/256 CTAs - the earliest to start -
     // split 8 blocks of 32 elements each (warps 6 and 9, one block per group of 8 lanes, about a microsecond), store
-    // the codes and scale bytes to global memory and count themselves in; every CTA with an item then fetches the
-    // rows K step by K step with its weight stages (TMA, from L2; four copies of each row) ----
+    // the codes and scale bytes to global memory, kCopies times, and count themselves in; every CTA with an item then
+    // fetches the rows of one copy K step by K step with its weight stages (TMA, from L2, 1 KB a stage) ----
     if ((wid == 6 || wid == 9) && item < n_split_ctas) {
       const int b = item * 8 + (wid == 9 ? 4 : 0) + jl;
       const uint2 v = __ldg(reinterpret_cast<const uint2*>(a.x + b * 32 + tl * 4));
@@ -476,8 +476,9 @@ decode_one_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
     } else if (has_item) {
       // =========================== epilogue warps ===========================
       // ---- scale factors of the token's term rows -> tensor memory: K step ks owns two scale-factor blocks (its two
-      // scale words); column c of a block holds, in lane l of every quadrant, the word of operand row 32c + l, which
-      // for every c is term row l & 7 (the four copies).  Four K steps per store. ----
+      // scale words); column c of a block holds, in lane l of every quadrant, the word of operand row 32c + l.  The MMAs
+      // take 16 rows, of which the first 8 are the terms; every lane and column gets the word of term row l & 7, as one
+      // store has room for all.  Four K steps per store. ----
       __syncwarp();
       mbar_wait(split_ready, 0u, a.status);  // the first CTAs have written the scale bytes (and the rows) of the token's terms
       __syncwarp();

@@ -76,7 +76,7 @@ namespace moe {
 
 namespace {
 
-constexpr int kTile = 256;            // weight rows per item (N of the MMA)
+constexpr int kTile = 256;            // weight rows per item: two tiles of M = 128 (kQ: N of the MMA)
 constexpr int kKStep = 256;           // K elements per stage: one 128-byte swizzled row of packed codes per weight row
 constexpr int kWStage = kTile * 128;  // 32 KB of weights per stage, shared memory and HBM alike
 constexpr int kAStage = 128 * 128;    // 16 KB: the same K step of up to 128 term rows
@@ -92,7 +92,8 @@ constexpr int kNatThreads = 11 * 32;
 constexpr int kEpiWarp = 6;           // warps 6..9: warp % 4 = 2, 3, 0, 1 -> one tensor-memory lane quadrant each
 constexpr int kTermWarp = 10;
 constexpr uint32_t kNatTmemCols = 512;
-// tensor-memory columns: one 256-column accumulator; per K step two scale words per operand row, each its own
+// tensor-memory columns: 256 of accumulators, either weight tile's terms side by side (kQ: one accumulator, a column per weight
+// row); per K step two scale words per operand row, each its own
 // scale-factor block of 4 columns (a block covers 128 rows - rows 32c..32c+31 in column c - and must start on a
 // multiple of 4 columns); 3 groups of 4 words x 8 columns (256 weight rows) for the weight scales
 constexpr uint32_t kColD = 0, kColSfAct = 256, kColSfW = 384;
@@ -112,7 +113,7 @@ struct NatArgs {
   float* const* row_dst;     // or null; else output row p goes to row_dst[p] (see y_row)
   int* status;               // never null: the caller's word or the library's own (see StatusRef)
   int own_status;            // the library's own word: the one-launch kernel's last CTA clears it for the next call
-  int E, H, I, S;
+  int E, H, I;
   int tok_rows;
   int blocked;               // weights in moe_prepack's tile-contiguous layout (see ExpertWeights)
   const uint8_t* s13;        // the weights' scale bytes, where no tensor map is used: contiguous tiles, and rows of reductions that are
@@ -1410,12 +1411,11 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
   a.E = sh.E;
   a.H = sh.H;
   a.I = sh.I;
-  a.S = static_cast<int>(S);
   a.blocked = w.blocked ? 1 : 0;
   a.s13 = w.s13;
   a.s2 = w.s2;
-  // Batches whose experts have several passes: one launch per projection, shares balanced by passes (see pass_shares)
-  // (a CTA's blocks, one list entry each, must fit the list it keeps)
+  // Batches whose experts have several passes: one launch per projection, over blocks of (expert, pass, a few tiles) dealt
+  // round-robin (see the set-up; a CTA's blocks, one list entry each, must fit the list it keeps)
   const size_t ent_max = S / (kQ ? 128 : kMaxTokPass) + sh.E, grid_n = static_cast<size_t>(sm_count());
   const size_t bpe_max = static_cast<size_t>(std::max(2 * sh.I / kTile / block_tiles(2 * sh.I / kTile), sh.H / kTile / block_tiles(sh.H / kTile)));
   const bool two = kQ && S > static_cast<size_t>(kQOneLaunchRows) * sh.E &&
@@ -1508,7 +1508,6 @@ int launch_forward_fused(const float* logits, const __nv_bfloat16* x, const Expe
   a.E = sh.E;
   a.H = sh.H;
   a.I = sh.I;
-  a.S = static_cast<int>(S);
   a.blocked = w.blocked ? 1 : 0;
   a.s13 = w.s13;
   a.s2 = w.s2;

@@ -619,10 +619,12 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
 // bound by issuing them, 8 bytes a lane with the row and scale places shuffled out per slot: 8192 tokens of 4096, top-8,
 // 166 us for 0.61 GB, 0.56 of the copy rate.  (A warp's part collected in shared memory and sent with one bulk copy per slot and
 // term: 181 us.)
-// What it writes is written at the rate at which memory takes writes alone (3.9 TB/s; a copy reaches 6.5 with the half that it reads).
+// It writes at 3.9 TB/s, which is what torch's fill_ writes at - the only kernel of stores alone that was timed beside it; a copy
+// reaches 6.5 with the half that it reads.
 // kRows: into `rows` the bf16 rows in sorted order as well, for a caller whose buffer they are (moe_layer): 11 us less than the
 // copy and a split from it (8216 slots of 4096: the layer 238 -> 227 us; 12288 slots 1123 -> 1108).  (Asked at run time, slot by
-// slot, it took the form without it from 40 to 48 registers and made that of moe_forward's prompts spill.) ----
+// slot, it took the form without it from 40 to 48 registers and made that of moe_forward's prompts spill: 8192 tokens 160 us
+// and 158, 32768 skewed 610 and 604.) ----
 template <bool kGuard, bool kRows>
 __global__ void __launch_bounds__(256) twoterm_scatter_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ ids,
                                                              const int* __restrict__ inv_perm, const int* __restrict__ offsets,
@@ -1277,11 +1279,13 @@ bool tt_launch(const CUtensorMap& tm_w, const CUtensorMap& tm_sc, const TtTokMap
 
 bool twoterm_chosen(const moe_shape_t& choice, const ExpertWeights& w) {
   const long long S = static_cast<long long>(choice.T) * choice.k;
-  // Few rows per expert of large ones: this kernel loses more than the eight-term one where the weights' rows lie 2 KB apart,
-  // and both read moe_prepack's tiles alike (256 experts of 4096 x 2048, 4 / 5 / 6 / 7 / 8 rows, eight terms and two: rows of
-  // weights 595 us and 632, 611 and 636, 618 and 640, 636 and 649, 884 and 646; the whole call on tiles 568 and 567, 577 and
-  // 577, 598 and 580; with rows of 2048 elements two terms are ahead from 4 on, 374 us and 321).  One line for both layouts,
-  // so that they give the same bits.
+  // Few rows per expert of large ones: the eight-term kernel is ahead up to six, on weights in rows and in moe_prepack's tiles
+  // (256 experts of 4096 x 2048, top-8, layers in a row, 4 / 5 / 6 / 7 / 8 rows, eight terms and two: tiles 532 us and 602,
+  // 555 and 609, 574 and 615, 672 and 625, 672 and 631; rows 583 and 645, 615 and 670, 632 and 685, 733 and 694, 736 and 699).
+  // With H = 2048 the two meet about 5 (2048 x 2048, 4 / 5 / 6 / 8 rows: tiles 307 and 318, 311 and 314, 347 and 317, 396 and
+  // 334; rows 323 and 335, 329 and 338, 367 and 346, 424 and 350; after a pause, at higher clocks, two terms are ahead at 4 as
+  // well, 310 and 300): they stay with the line at 4 of twoterm_batch_ok.  One line for both layouts, so that they give
+  // the same bits.
   if (choice.H >= 4096 && choice.I >= 1024 && S <= 6LL * choice.E && native_shape_ok(choice, w.w13, w.w2)) return false;
   // A layer of small experts is done in a few rounds of either kernel, and the launches that look for experts to be done again
   // decide (L2 cold, this call / bf16 kernel: 64 experts of 512 x 512, 128 rows 59 us and 56, 200 rows 74 and 65; 32 of 1024 x
@@ -1336,7 +1340,7 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
   int* flags = reinterpret_cast<int*>(base + L.flags);
   const int n_chunk = sh.H / 256;
   int parts = (n_chunk + 7) / 8;  // pieces of a row, a mark each
-  const size_t most = static_cast<size_t>(sm_count()) * 8;  // CTAs of eight warps that fit the chip
+  const size_t most = static_cast<size_t>(sm_count()) * 8;  // CTAs of the scatter kernel at most (five or six of a SM's eight run at a time)
   const size_t table_bytes = static_cast<size_t>(kTtTableInts * (sh.E + 1)) * 4;
   cudaError_t rc;
   if (in.inv_perm != nullptr) {
