@@ -235,6 +235,11 @@ int route_and_ffn(const float* logits, const void* x, int32_t* ids, float* topk_
   return launch_expert_ffn_native_tokens(offsets, w, s, scratch, y_perm, status, st);
 }
 
+// whether the layer is one launch of one cluster: where the streaming kernel would take its expert FFN, whose bits that launch has
+bool small_layer(const moe_shape_t& s, const ExpertWeights& w) {
+  return layer_small_ok(s) && !w.blocked && stream_shape_ok(s) && !twoterm_chosen(s, w) && !native_shape_ok(s, w.w13, w.w2) && !umma_shape_ok(s);
+}
+
 // the four tensors inside a buffer written by moe_prepack
 ExpertWeights packed_view(const void* packed, const moe_shape_t& s) {
   const PackedLayout L = packed_layout(s);
@@ -317,6 +322,11 @@ int moe_layer(const float* logits, const void* x_bf16, const uint8_t* w13, const
   const moe_shape_t& s = *shape;
   if (check_ws(ws, ws_bytes, ws_layout(s).total) != MOE_OK) return MOE_ERR_WORKSPACE;
   const ExpertWeights w{w13, w13_scale, w2, w2_scale, false};
+  if (small_layer(s, w))
+    return launch_layer_small(logits, static_cast<const __nv_bfloat16*>(x_bf16), w, s,
+                              SmallLayerOut{topk_ids, expert_offsets, perm, inv_perm, topk_w, y_perm, static_cast<__nv_bfloat16*>(x_perm_bf16),
+                                            static_cast<__nv_bfloat16*>(out_bf16)},
+                              static_cast<cudaStream_t>(cuda_stream));
   if (route_sort_ok(s.T, s.E) && !front_in_one(s, w)) {  // routing and sort in one launch for the other kernels too
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if ((rc = launch_route_sort(logits, s.T, s.E, s.k, topk_ids, topk_w, expert_offsets, perm, inv_perm, nullptr, nullptr, false, st)) != MOE_OK ||
@@ -666,6 +676,11 @@ int forward_impl(const float* logits, const void* x_bf16, const ExpertWeights& w
   float* d_y = reinterpret_cast<float*>(base + L.y_perm);
   void* inner = base + L.inner;
   const size_t inner_bytes = ws_bytes - L.inner;
+  if (small_layer(*shape, w))
+    return launch_layer_small(logits, static_cast<const __nv_bfloat16*>(x_bf16), w, *shape,
+                              SmallLayerOut{d_ids, d_off, d_perm, d_inv, d_w, d_y, static_cast<__nv_bfloat16*>(d_xp),
+                                            static_cast<__nv_bfloat16*>(out_bf16)},
+                              st);
   if ((rc = route_and_ffn(logits, x_bf16, d_ids, d_w, d_off, nullptr, false, w, shape, d_xp, d_perm, d_inv, d_y, status_word, inner, inner_bytes,
                           st)) != MOE_OK)
     return rc;

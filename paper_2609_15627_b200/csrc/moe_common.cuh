@@ -286,6 +286,15 @@ bool twoterm_guarded(const moe_shape_t& choice, const ExpertWeights& w);
 // quantised activations, batches that fill the chip; scratch of q_pair_scratch
 int launch_expert_ffn_q_pair(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
                              void* scratch, float* y_perm, int* status_word, cudaStream_t st);
+// the whole layer in one launch of one cluster, for layers whose weights fit its shared memory; the streaming kernel's bits
+struct SmallLayerOut {
+  int *ids, *offsets, *perm, *inv_perm;
+  float *w, *y_perm;
+  __nv_bfloat16 *x_perm, *out;
+};
+bool layer_small_ok(const moe_shape_t& s);
+int launch_layer_small(const float* logits, const __nv_bfloat16* x, const ExpertWeights& w, const moe_shape_t& s, const SmallLayerOut& o,
+                       cudaStream_t st);
 int launch_combine(const float* y_perm, const int* inv_perm, const float* w, const moe_shape_t& s,
                    __nv_bfloat16* out, cudaStream_t st);
 int launch_validate_scales(const uint8_t* scales, size_t n, int* bad, cudaStream_t st);
@@ -370,7 +379,7 @@ inline bool once_per_device(PerDeviceFlag& f, F&& set) {
 // ---- programmatic dependent launch (host) ------------------------------------------------------
 // The kernel may start while its predecessor in the stream is still running; it must execute
 // griddepcontrol.wait before it reads anything the predecessor writes, and before it writes anything at all to
-// global memory.  Most kernels here wait first and then release their own dependent; route_kernel, route_sort_kernel,
+// global memory.  Most kernels here wait first and then release their own dependent; route_kernel, route_sort_kernel, layer_small_kernel,
 // native_split_kernel, native_quant_rows_kernel, native_expand_kernel, twoterm_scatter_kernel and the expert-FFN kernels
 // release theirs BEFORE they wait, so three or four neighbours of a chain (route, permute, split, expert FFN) can be
 // resident together.  That is safe because of the rule above: whatever a kernel does before its wait only reads buffers

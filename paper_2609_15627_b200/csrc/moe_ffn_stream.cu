@@ -13,7 +13,7 @@
 //
 // K elements are assigned to MMA k slots in a permuted order (identically for weights and activations);
 // only the summation order inside the dot product depends on it.
-#include "moe_sm100_primitives.cuh"
+#include "moe_stream_device.cuh"
 
 namespace moe {
 
@@ -38,14 +38,6 @@ struct FfnArgs {
   int E, K, R, I;             // R rows per expert (2I for stage 1, H for stage 2); I used by stage 1 only
   int n_stages;
 };
-
-MOE_DEVINL void mma_bf16_16x8x16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                 uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 
 }  // namespace
 
@@ -190,10 +182,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_stream_kernel(const FfnArgs a
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                   const uint4 v = __ldcg(src + q);  // 8 consecutive elements
-                  breg[j][4 * q + 0] = __byte_perm(v.x, v.z, 0x5410);  // elements (0,4)
-                  breg[j][4 * q + 1] = __byte_perm(v.x, v.z, 0x7632);  // elements (1,5)
-                  breg[j][4 * q + 2] = __byte_perm(v.y, v.w, 0x5410);  // elements (2,6)
-                  breg[j][4 * q + 3] = __byte_perm(v.y, v.w, 0x7632);  // elements (3,7)
+                  stream_activations(v, &breg[j][4 * q]);
                 }
               } else {
 #pragma unroll
@@ -211,16 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_stream_kernel(const FfnArgs a
               const uint4 wb = *reinterpret_cast<const uint4*>(codesB + g * (K / 2) + sc * 64 + t * 16);
               const uint32_t ma = scale_mult(scaleA[g * (K / 32) + sc * 4 + t]);
               const uint32_t mb = scale_mult(scaleB[g * (K / 32) + sc * 4 + t]);
-              const uint32_t wav[4] = {wa.x, wa.y, wa.z, wa.w};
-              const uint32_t wbv[4] = {wb.x, wb.y, wb.z, wb.w};
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                uint32_t pa[4], pb[4];
-                dequant8(wav[q], ma, a.k1, a.k2, pa);
-                dequant8(wbv[q], mb, a.k1, a.k2, pb);
-                mma_bf16_16x8x16(c, pa[0], pb[0], pa[1], pb[1], breg[j][4 * q + 0], breg[j][4 * q + 1]);
-                mma_bf16_16x8x16(c2, pa[2], pb[2], pa[3], pb[3], breg[j][4 * q + 2], breg[j][4 * q + 3]);
-              }
+              stream_group(c, c2, wa, wb, ma, mb, breg[j], a.k1, a.k2);
             }
           }
         }
@@ -242,14 +222,8 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_stream_kernel(const FfnArgs a
           const int r_a = row0 + 2 * t, r_b = r_a + 1;
           if (STAGE1) {
             const int i = tile * 8 + g;
-            if (r_a < row_end) {
-              const float v = (s.x / (1.0f + __expf(-s.x))) * s.z;
-              a.act[static_cast<size_t>(r_a) * a.I + i] = __float2bfloat16_rn(v);
-            }
-            if (r_b < row_end) {
-              const float v = (s.y / (1.0f + __expf(-s.y))) * s.w;
-              a.act[static_cast<size_t>(r_b) * a.I + i] = __float2bfloat16_rn(v);
-            }
+            if (r_a < row_end) a.act[static_cast<size_t>(r_a) * a.I + i] = stream_swiglu(s.x, s.z);
+            if (r_b < row_end) a.act[static_cast<size_t>(r_b) * a.I + i] = stream_swiglu(s.y, s.w);
           } else {
             const int n = tile * 16 + g;
             if (r_a < row_end) {

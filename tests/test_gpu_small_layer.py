@@ -1,0 +1,106 @@
+"""The layer in one launch of one cluster (layers whose weights fit its shared memory) against the four calls, every buffer bit for
+bit: few and many tokens, fewer experts than CTAs, several experts per CTA, experts without rows and with more than one block of
+eight, odd token counts, widths that are odd multiples of 128."""
+import numpy as np
+import pytest
+import torch
+
+from _gpu_util import bits, check_out, dev
+from oracle import moe_oracle as O
+from paper_2609_15627_b200 import inputs, moe
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [  # T, H, I, E, k
+    (1, 256, 128, 8, 2), (16, 256, 128, 8, 2), (32, 256, 128, 8, 4), (31, 128, 128, 3, 3), (8, 256, 128, 32, 8), (17, 128, 128, 64, 4),
+    (7, 384, 128, 9, 1), (5, 128, 640, 5, 2), (1, 1024, 128, 8, 8), (2, 128, 128, 60, 32)]
+
+
+def _weights(H, I, E, seed=0):
+    return tuple(dev(a) for a in inputs.make_expert_weights(H, I, E, seed=seed))
+
+
+@pytest.mark.parametrize("T,H,I,E,k", SHAPES)
+def test_small_layer_has_the_four_calls_bits(T, H, I, E, k):
+    sh, w = moe.shape(T, H, I, E, k), _weights(H, I, E)
+    logits, x = dev(inputs.make_logits(T, E, 11)), dev(inputs.make_x(T, H, 11))
+    b, c = moe.LayerBuffers(sh), moe.LayerBuffers(sh)
+    for buf in (b, c):
+        for v in (buf.x_perm, buf.y_perm, buf.out, buf.topk_w):
+            v.fill_(float("nan"))
+        for v in (buf.topk_ids, buf.expert_offsets, buf.perm, buf.inv_perm):
+            v.fill_(-7)
+    moe.moe_layer(logits, x, w, b)
+    assert moe.moe_last_kernel_name() == "layer_one_cluster"
+    moe.moe_route(logits, k, c.topk_ids, c.topk_w, c.expert_offsets, c.ws)
+    moe.moe_permute(x, c.topk_ids, c.expert_offsets, sh, c.x_perm, c.perm, c.inv_perm, c.ws)
+    moe.moe_expert_ffn(c.x_perm, c.expert_offsets, *w, sh, c.y_perm, c.status, c.ws)
+    assert moe.moe_last_kernel_name() == "ffn_stream_bulk_ring_mma16816"
+    moe.moe_combine(c.y_perm, c.inv_perm, c.topk_w, sh, c.out)
+    torch.cuda.synchronize()
+    for n in ("topk_ids", "topk_w", "expert_offsets", "x_perm", "perm", "inv_perm", "y_perm", "out"):
+        assert torch.equal(getattr(b, n), getattr(c, n)), n
+    out = torch.empty_like(b.out)
+    ids, wt, st = torch.empty_like(b.topk_ids), torch.empty_like(b.topk_w), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = moe.alloc_forward_workspace(sh)
+    moe.moe_forward(logits, x, *w, sh, out, ids, wt, st, ws)
+    packed = moe.moe_prepack(*w, sh)
+    out_p = torch.empty_like(out)
+    moe.moe_forward_packed(logits, x, packed, sh, out_p, None, None, st, ws)
+    torch.cuda.synchronize()
+    assert torch.equal(out, b.out) and torch.equal(out_p, b.out) and torch.equal(ids, b.topk_ids) and torch.equal(wt, b.topk_w) and int(st.item()) == 0
+
+
+def test_small_layer_against_the_oracle_with_equal_logits_and_infinities():
+    T, H, I, E, k = 9, 256, 128, 8, 3
+    sh, raw = moe.shape(T, H, I, E, k), inputs.make_expert_weights(H, I, E, seed=4)
+    logits, x = inputs.make_logits(T, E, 12), inputs.make_x(T, H, 12)
+    logits[2] = 0.0                                   # ties: the lowest ids
+    logits[3, :4] = np.float32(-3.0e38)
+    logits[5, 1] = np.float32(3.0e38)
+    buf = moe.LayerBuffers(sh)
+    moe.moe_layer(dev(logits), dev(x), tuple(dev(a) for a in raw), buf)
+    torch.cuda.synchronize()
+    r = O.forward_staged(logits, x, *raw, k)
+    assert np.array_equal(buf.topk_ids.cpu().numpy(), r["ids"]) and np.array_equal(buf.topk_w.cpu().numpy().view(np.uint32), r["w"].view(np.uint32))
+    check_out(bits(buf.out), r["out"], r["out_f32"], "small layer")
+    x[4, 7] = 0x7F80                                  # an infinite activation: that token's output is not finite, the others stay
+    want = buf.out.clone()
+    moe.moe_layer(dev(logits), dev(x), tuple(dev(a) for a in raw), buf)
+    torch.cuda.synchronize()
+    keep = torch.arange(T, device="cuda") != 4
+    assert torch.equal(buf.out[keep], want[keep]) and not bool(torch.isfinite(buf.out[4].float()).all())
+
+
+def test_small_layers_one_behind_the_other_in_a_graph():
+    """Each layer's rows are the one before's output and its logits are rewritten beside it: nothing of a launch may start early."""
+    T, H, I, E, k, n = 16, 256, 128, 8, 2, 40
+    sh, w = moe.shape(T, H, I, E, k), _weights(H, I, E)
+    lg = [dev(inputs.make_logits(T, E, 50 + i)) for i in range(n)]
+    x0 = dev(inputs.make_x(T, H, 1))
+    bufs = [moe.LayerBuffers(sh) for _ in range(2)]
+    cur_lg = torch.empty_like(lg[0])
+
+    def chain():
+        x = x0
+        for i in range(n):
+            cur_lg.copy_(lg[i])
+            x = moe.moe_layer(cur_lg, x, w, bufs[i & 1])
+        return x
+
+    chain()
+    torch.cuda.synchronize()
+    x = x0
+    for i in range(n):   # one at a time
+        x = moe.moe_layer(lg[i], x, w, bufs[i & 1]).clone()
+        torch.cuda.synchronize()
+    want = x
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            chain()
+        for _ in range(20):
+            g.replay()
+            s.synchronize()
+            assert torch.equal(bufs[(n - 1) & 1].out, want)
