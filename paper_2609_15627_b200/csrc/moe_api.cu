@@ -211,6 +211,26 @@ int route_and_ffn(const float* logits, const void* x, int32_t* ids, float* topk_
   const bool twoterm = twoterm_chosen(s, w);
   if (!front_in_one(s, w)) {
     if (offsets2 != nullptr && (rc = launch_shared_offsets(offsets2, s.T, st)) != MOE_OK) return rc;
+    if (route_permute_ok(s)) {
+      if (!aligned(w.w13, 16) || !aligned(w.s13, 16) || !aligned(w.w2, 16) || !aligned(w.s2, 16) ||
+          (status_word != nullptr && !aligned(status_word, 4)))
+        return MOE_ERR_INVALID_ARG;
+      const WsLayout L = ws_layout(s);
+      if (check_ws(ws, ws_bytes, L.total) != MOE_OK) return MOE_ERR_WORKSPACE;
+      char* base = static_cast<char*>(ws);
+      const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(x);
+      __nv_bfloat16* xp = static_cast<__nv_bfloat16*>(x_perm);
+      StatusRef status;
+      if ((rc = resolve_status(status_word, &status)) != MOE_OK) return rc;
+      if (twoterm && (rc = clear_own_status(status, st)) != MOE_OK) return rc;
+      if ((rc = launch_route_permute(logits, xb, s, ids, topk_w, offsets, twoterm ? nullptr : xp, perm, inv_perm,
+                                     reinterpret_cast<int*>(base + L.permute_off), st)) != MOE_OK)
+        return rc;
+      if (twoterm)
+        return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, xp, true, rows}, offsets, w, s, s, twoterm_guarded(s, w), base + L.act_off,
+                                         y_perm, status.word, st);
+      return expert_ffn_impl(x_perm, offsets, w, shape, y_perm, status_word, ws, ws_bytes, cuda_stream);
+    }
     if ((rc = moe_route(logits, s.T, s.E, s.k, ids, topk_w, offsets, ws, ws_bytes, cuda_stream)) != MOE_OK) return rc;
     return permute_and_ffn(x, ids, offsets, w, shape, x_perm, perm, inv_perm, y_perm, status_word, ws, ws_bytes, cuda_stream, rows);
   }

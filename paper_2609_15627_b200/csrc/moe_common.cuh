@@ -246,6 +246,11 @@ int launch_gather_rows(const __nv_bfloat16* x, const int* perm, const moe_shape_
 int launch_permute(const __nv_bfloat16* x, const int* ids, const int* offsets, const moe_shape_t& s,
                    __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st,
                    const int* range_lo = nullptr, const int* range_hi = nullptr);
+// routing and sort of batches that no cluster routes, in a call that makes both (x_perm null: no rows); offsets is written by the
+// sort, so what comes next waits before it reads it
+bool route_permute_ok(const moe_shape_t& s);
+int launch_route_permute(const float* logits, const __nv_bfloat16* x, const moe_shape_t& s, int* ids, float* w, int* offsets,
+                         __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st);
 // weight-streaming variant (any shape; the one for decode-sized batches)
 int launch_expert_ffn_stream(const __nv_bfloat16* x_perm, const int* offsets, const uint8_t* w13, const uint8_t* s13,
                              const uint8_t* w2, const uint8_t* s2, const moe_shape_t& s, __nv_bfloat16* act, float* y_perm,

@@ -66,6 +66,55 @@ MOE_DEVINL void warp_topk_256(const float* row, int E, int k, int lane, int* my_
   }
 }
 
+// The same for batches, where the instructions count and not one token's latency: a lane sorts its eight keys once (with their ids,
+// descending, the lower id first among equals), so a round looks at its head alone - about 330 instructions for a top-8
+// instead of 520.
+MOE_DEVINL void warp_topk_256_sorted(const float* row, int E, int k, int lane, int* my_id, float* my_v) {
+  unsigned key[8];
+  int id[8];  // beyond E: an id no one has, and the lowest key
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int idx = u * 32 + lane;
+    const float v = idx < E ? row[idx] : 0.0f;
+    const unsigned b = __float_as_uint(v == 0.0f ? 0.0f : v);
+    key[u] = idx < E ? ((b & 0x80000000u) ? ~b : (b | 0x80000000u)) : 0u;
+    id[u] = idx < E ? idx : 0x7FFFFFFF;
+  }
+  auto order = [&](int i, int j) {  // (i < j)
+    const bool swap = key[j] > key[i] || (key[j] == key[i] && id[j] < id[i]);
+    const unsigned ka = swap ? key[j] : key[i], kb = swap ? key[i] : key[j];
+    const int ia = swap ? id[j] : id[i], ib = swap ? id[i] : id[j];
+    key[i] = ka, key[j] = kb, id[i] = ia, id[j] = ib;
+  };
+  // Batcher's odd-even merge network for eight
+  order(0, 1), order(2, 3), order(4, 5), order(6, 7);
+  order(0, 2), order(1, 3), order(4, 6), order(5, 7);
+  order(1, 2), order(5, 6);
+  order(0, 4), order(1, 5), order(2, 6), order(3, 7);
+  order(2, 4), order(3, 5);
+  order(1, 2), order(3, 4), order(5, 6);
+  *my_id = 0;
+  *my_v = 0.0f;
+  for (int j = 0; j < k; ++j) {
+    const unsigned top = __reduce_max_sync(0xffffffffu, key[0]);
+    const unsigned win = __reduce_min_sync(0xffffffffu, key[0] == top ? static_cast<unsigned>(id[0]) : 0xffffffffu);
+    const bool mine = static_cast<unsigned>(id[0]) == win;
+    if (lane == j) {
+      *my_id = static_cast<int>(win);
+      *my_v = __uint_as_float((top & 0x80000000u) ? (top & 0x7fffffffu) : ~top);
+    }
+#pragma unroll
+    for (int u = 0; u < 7; ++u) {
+      key[u] = mine ? key[u + 1] : key[u];
+      id[u] = mine ? id[u + 1] : id[u];
+    }
+    if (mine) {
+      key[7] = 0u;
+      id[7] = 0x7FFFFFFF;
+    }
+  }
+}
+
 MOE_DEVINL void warp_topk(const float* row, int E, int k, int lane, int* my_id, float* my_v) {
   if (E <= 256) {
     warp_topk_256(row, E, k, lane, my_id, my_v);

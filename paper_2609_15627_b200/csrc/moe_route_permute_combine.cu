@@ -41,37 +41,48 @@ __device__ void block_offsets_scan(const int* counts, int E, int* offsets, int* 
   }
 }
 
-// single_block != 0: one CTA handles every token and builds the histogram in shared memory.
-// Otherwise the histogram is accumulated in g_counts[0..E) (zeroed before the launch) and the last
-// CTA to finish (ticket in g_counts[E]) scans it.
-__global__ void __launch_bounds__(1024) route_kernel(const float* __restrict__ logits, int T, int E, int k,
+// kSingle: one CTA handles every token and builds the histogram in shared memory.  Otherwise a warp per token and nothing
+// but its ids and weights: the histogram is another launch's (route_offsets_kernel or the sort), which reads the ids back in
+// chunks.  (With a global atomic per slot, 256 addresses for all, 8192 tokens took 37 us in a row of layers and 32768 129, with a
+// memset in front; without, and with the keys sorted, 17 and 48.)  zero: counters [0, n_zero) that the next launch adds to, or null.  kWide: more than 256 experts.
+template <bool kSingle, bool kWide>
+__global__ void __launch_bounds__(kSingle ? 1024 : 256, kSingle || kWide ? 1 : 6) route_kernel(const float* __restrict__ logits, int T, int E, int k,
                                                      int* __restrict__ ids, float* __restrict__ w,
-                                                     int* __restrict__ offsets, int* g_counts, int single_block) {
+                                                     int* __restrict__ offsets, int* zero, int n_zero) {
   extern __shared__ float sm_f[];
   const int nw = blockDim.x >> 5;
-  float* rows = sm_f;                                   // [nw][E]
-  int* s_counts = reinterpret_cast<int*>(sm_f + nw * E);  // [E]
-  int* s_misc = s_counts + E;                           // [32] + flag
+  float* rows = sm_f;                                   // [nw][E], more than 256 experts or one CTA
+  int* s_counts = reinterpret_cast<int*>(sm_f + nw * E);  // [E], one CTA
+  int* s_misc = s_counts + E;                           // [32]
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  // Programmatic dependent launch on both sides: moe_permute may start and waits before it reads; this kernel may
+  // Programmatic dependent launch on both sides: what comes next may start and waits before it reads; this kernel may
   // itself have started while the kernel before it (the previous layer call's moe_combine, which still reads the
-  // routing weights this kernel is about to overwrite) is running, so it reads only its input before it waits and
-  // writes nothing to global memory until then.
+  // routing weights this kernel is about to overwrite) is running, so it writes nothing to global memory before it waits, and reads the
+  // logits before only where one CTA routes (what moe_route promises: up to 32 tokens).
   pdl_launch_dependents();
   bool waited = false;
-  if (single_block) {
+  if (kSingle) {
     for (int e = tid; e < E; e += blockDim.x) s_counts[e] = 0;
     __syncthreads();
+  } else {
+    pdl_wait();
+    waited = true;
+    if (zero != nullptr && blockIdx.x == 0)
+      for (int e = tid; e < n_zero; e += blockDim.x) zero[e] = 0;
   }
   float* row = rows + wid * E;
   const int t0 = blockIdx.x * nw + wid;
   const int tstride = gridDim.x * nw;
   for (int t = t0; t < T; t += tstride) {
-    for (int e = lane; e < E; e += 32) row[e] = logits[static_cast<size_t>(t) * E + e];
-    __syncwarp();
     int my_id;
     float my_v;
-    warp_topk(row, E, k, lane, &my_id, &my_v);
+    if (!kSingle && !kWide) {
+      warp_topk_256_sorted(logits + static_cast<size_t>(t) * E, E, k, lane, &my_id, &my_v);
+    } else {
+      for (int e = lane; e < E; e += 32) row[e] = logits[static_cast<size_t>(t) * E + e];
+      __syncwarp();
+      warp_topk(row, E, k, lane, &my_id, &my_v);
+    }
     const float wt = warp_softmax_selected(my_v, k, lane);
     if (!waited) {
       pdl_wait();
@@ -80,52 +91,83 @@ __global__ void __launch_bounds__(1024) route_kernel(const float* __restrict__ l
     if (lane < k) {
       ids[static_cast<size_t>(t) * k + lane] = my_id;
       w[static_cast<size_t>(t) * k + lane] = wt;
-      if (my_id >= 0) atomicAdd(single_block ? &s_counts[my_id] : &g_counts[my_id], 1);
+      if (kSingle && my_id >= 0) atomicAdd(&s_counts[my_id], 1);
     }
     __syncwarp();
   }
   if (!waited) pdl_wait();  // warps without a token
-  if (single_block) {
-    __syncthreads();
-    block_offsets_scan(s_counts, E, offsets, s_misc);
-    return;
-  }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s_misc[32] = (atomicAdd(&g_counts[E], 1) == static_cast<int>(gridDim.x) - 1);
-  __syncthreads();
-  if (s_misc[32]) {
-    __threadfence();
-    for (int e = tid; e < E; e += blockDim.x) s_counts[e] = __ldcg(&g_counts[e]);
+  if (kSingle) {
     __syncthreads();
     block_offsets_scan(s_counts, E, offsets, s_misc);
   }
 }
 
+// expert_offsets from the ids: a histogram in shared memory per chunk, added to counts[0..E), which the router cleared; the last CTA
+// (ticket in counts[E]) scans them.
+constexpr int kOffsetsChunk = 4096;
+__global__ void __launch_bounds__(1024) route_offsets_kernel(const int* __restrict__ ids, int S, int E, int* __restrict__ offsets, int* counts) {
+  extern __shared__ int s_hist[];  // [E], then the scan's [32] and a flag
+  int* s_misc = s_hist + E;
+  const int tid = threadIdx.x;
+  for (int e = tid; e < E; e += blockDim.x) s_hist[e] = 0;
+  __syncthreads();
+  pdl_wait();
+  pdl_launch_dependents();
+  const int s0 = blockIdx.x * kOffsetsChunk + 4 * tid;  // (a chunk is four slots a thread)
+  int e4[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) e4[j] = s0 + j < S ? __ldg(ids + s0 + j) : -1;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (e4[j] >= 0) atomicAdd(&s_hist[e4[j]], 1);
+  __syncthreads();
+  for (int e = tid; e < E; e += blockDim.x)
+    if (s_hist[e] != 0) atomicAdd(&counts[e], s_hist[e]);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_misc[32] = atomicAdd(&counts[E], 1) == static_cast<int>(gridDim.x) - 1;
+  __syncthreads();
+  if (s_misc[32] == 0) return;
+  __threadfence();
+  for (int e = tid; e < E; e += blockDim.x) s_hist[e] = __ldcg(&counts[e]);
+  __syncthreads();
+  block_offsets_scan(s_hist, E, offsets, s_misc);
+}
+
+// the router alone (no offsets), a warp per token
+static int launch_route_ids(const float* logits, int T, int E, int k, int* ids, float* w, int* zero, int n_zero, cudaStream_t st) {
+  constexpr int nw = 8;
+  const size_t smem = E <= 256 ? 0 : (static_cast<size_t>(nw) * E + E + 40) * 4;
+  return launch_pdl(E <= 256 ? route_kernel<false, false> : route_kernel<false, true>, dim3((T + nw - 1) / nw), dim3(nw * 32), smem, st, logits, T, E, k, ids, w, static_cast<int*>(nullptr), zero,
+                    n_zero) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+}
+static bool route_attr_once() {
+  static PerDeviceFlag flag;
+  return once_per_device(flag, [] {
+    return cudaFuncSetAttribute(route_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess &&
+           cudaFuncSetAttribute(route_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess;
+  });
+}
+
 int launch_route(const float* logits, int T, int E, int k, int* ids, float* w, int* offsets, int* counters,
                  cudaStream_t st) {
   if (route_sort_ok(T, E)) return launch_route_sort(logits, T, E, k, ids, w, offsets, nullptr, nullptr, nullptr, nullptr, false, st);
+  if (!route_attr_once()) return MOE_ERR_CUDA;
   // One CTA up to a round of its 32 warps.  (64 tokens: 19 us in two rounds of one CTA, 7 us on eight.)
-  const bool single = T <= 32;
-  const int nw = single ? 32 : 8;
-  const size_t smem = (static_cast<size_t>(nw) * E + E + 40) * 4;
-  static PerDeviceFlag flag;
-  if (!once_per_device(flag, [] {
-        return cudaFuncSetAttribute(route_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess;
-      }))
-    return MOE_ERR_CUDA;
-  int launches = 1;
-  if (single) {
-    if (launch_pdl(route_kernel, dim3(1), dim3(nw * 32), smem, st, logits, T, E, k, ids, w, offsets, counters, 1) != cudaSuccess)
+  if (T <= 32) {
+    const size_t smem = (static_cast<size_t>(32) * E + E + 40) * 4;
+    if (launch_pdl(route_kernel<true, true>, dim3(1), dim3(1024), smem, st, logits, T, E, k, ids, w, offsets, static_cast<int*>(nullptr), 0) != cudaSuccess)
       return MOE_ERR_CUDA;
-    note_kernel("route_topk_single_cta", launches);
-  } else {
-    if (cudaMemsetAsync(counters, 0, (static_cast<size_t>(E) + 1) * 4, st) != cudaSuccess) return MOE_ERR_CUDA;
-    const int grid = (T + nw - 1) / nw;
-    route_kernel<<<grid, nw * 32, smem, st>>>(logits, T, E, k, ids, w, offsets, counters, 0);
-    note_kernel("route_topk_multi_cta", launches);
+    note_kernel("route_topk_single_cta", 1);
+    return MOE_OK;
   }
-  return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+  const int S = T * k, rc = launch_route_ids(logits, T, E, k, ids, w, counters, E + 1, st);
+  if (rc != MOE_OK) return rc;
+  if (launch_pdl(route_offsets_kernel, dim3((S + kOffsetsChunk - 1) / kOffsetsChunk), dim3(1024), (static_cast<size_t>(E) + 40) * 4, st, ids, S, E,
+                 offsets, counters) != cudaSuccess)
+    return MOE_ERR_CUDA;
+  note_kernel("route_topk_multi_cta", 2);
+  return MOE_OK;
 }
 
 // ---- routing and sort of batches that one cluster routes (up to 256 tokens and 256 experts), and the split of their rows ----
@@ -276,32 +318,61 @@ MOE_DEVINL void warp_copy_row(const __nv_bfloat16* src, __nv_bfloat16* dst, int 
 
 // Up to permute_direct slots: a CTA takes eight consecutive slots, counts the earlier slots of each one's expert directly
 // (an id is loaded once per CTA and compared with the eight experts) and copies their rows, one warp each; the sort is
-// stable by construction.  One launch where the chunked sort takes three, and a fourth for the rows.
-// The count is quadratic and the launches are not: the line lies where the two meet (256 experts, direct / chunked).  Short
+// stable by construction.  One launch where the chunked sort takes two, and a third for the rows.
+// The count is quadratic and the launches are not: the line lies where the two meet (256 experts, direct / chunked in three).  Short
 // rows or none to copy: 4096 slots 10 us and 15, 8192 13 and 17, 12288 21 and 17, 16384 29 and 19; with long ones beside
 // the count later (H = 4096): 8192 slots 21 and 31, 12288 29 and 36, 16384 37 and 42, 24576 59 and 56.
 constexpr int permute_direct(bool rows, int H) { return rows && H >= 2048 ? 16384 : 8192; }
-__global__ void __launch_bounds__(256, 8) permute_small_kernel(const __nv_bfloat16* __restrict__ x,
+// kOffsets: expert_offsets is not there yet.  Then the slots of smaller experts are counted as well, and the last CTA writes it.
+template <bool kOffsets>
+__global__ void __launch_bounds__(256, kOffsets ? 6 : 8) permute_small_kernel(const __nv_bfloat16* __restrict__ x,
                                                             const int* __restrict__ ids,
-                                                            const int* __restrict__ offsets, int S, int H, int k,
+                                                            int* __restrict__ offsets, int S, int H, int k,
                                                             __nv_bfloat16* __restrict__ x_perm,
                                                             int* __restrict__ perm, int* __restrict__ inv_perm,
-                                                            const int* __restrict__ range_lo, const int* __restrict__ range_hi) {
+                                                            const int* __restrict__ range_lo, const int* __restrict__ range_hi, int E) {
   __shared__ int s_cnt[8][8];  // [warp][slot of the CTA]
+  extern __shared__ int s_hist[];  // kOffsets: [E + 32]
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int s0 = blockIdx.x * 8, s = s0 + wid;
   pdl_wait();                // the router's ids and offsets are complete
   pdl_launch_dependents();   // the expert FFN may set up and start its weight stream
+  if (kOffsets && s0 >= S) {  // (one CTA more than the slots take)
+    for (int e = threadIdx.x; e < E; e += 256) s_hist[e] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < S; i += 256) atomicAdd(&s_hist[__ldg(ids + i)], 1);
+    __syncthreads();
+    block_offsets_scan(s_hist, E, offsets, s_hist + E);
+    return;
+  }
   int e8[8], c8[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     e8[j] = s0 + j < S ? __ldg(ids + s0 + j) : -1;
     c8[j] = 0;
   }
-  for (int q = 4 * threadIdx.x; q < s0; q += 4 * 256) {
-    const int4 v = __ldg(reinterpret_cast<const int4*>(ids + q));  // (s0 is a multiple of 8)
+  if constexpr (kOffsets) {  // slots of smaller experts, and earlier slots of the same one
+    for (int q = 4 * threadIdx.x; q < S; q += 4 * 256) {
+      int v[4];
+      if (q + 4 <= S) {
+        const int4 v4 = __ldg(reinterpret_cast<const int4*>(ids + q));
+        v[0] = v4.x, v[1] = v4.y, v[2] = v4.z, v[3] = v4.w;
+      } else {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) c8[j] += (v.x == e8[j]) + (v.y == e8[j]) + (v.z == e8[j]) + (v.w == e8[j]);
+        for (int u = 0; u < 4; ++u) v[u] = q + u < S ? __ldg(ids + q + u) : 0x7FFFFFFF;
+      }
+      const int same = q < s0 ? 1 : 0;  // (s0 is a multiple of 8: all four or none)
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c8[j] += v[u] < e8[j] + same;
+    }
+  } else {
+    for (int q = 4 * threadIdx.x; q < s0; q += 4 * 256) {
+      const int4 v = __ldg(reinterpret_cast<const int4*>(ids + q));  // (s0 is a multiple of 8)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) c8[j] += (v.x == e8[j]) + (v.y == e8[j]) + (v.z == e8[j]) + (v.w == e8[j]);
+    }
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -318,7 +389,7 @@ __global__ void __launch_bounds__(256, 8) permute_small_kernel(const __nv_bfloat
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) c += (j < wid && e8[j] == e);
-  const int p = offsets[e] + c;
+  const int p = kOffsets ? c : offsets[e] + c;
   if (lane == 0) {
     perm[p] = s;
     inv_perm[s] = p;
@@ -344,7 +415,9 @@ __global__ void __launch_bounds__(256) permute_count_kernel(const int* __restric
   for (int e = threadIdx.x; e < E; e += blockDim.x) block_counts[static_cast<size_t>(blockIdx.x) * E + e] = s_hist[e];
 }
 
-// Large S, pass 2: one warp per expert turns the per-chunk counts into per-chunk start positions.
+// Very large S (more than kSortChunks chunks), between the two passes: one warp per expert turns the per-chunk counts into per-chunk
+// start positions.
+constexpr int kSortChunks = 512;
 __global__ void __launch_bounds__(256) permute_scan_kernel(const int* __restrict__ offsets, int E, int nblk,
                                                            int* __restrict__ block_counts) {
   const int lane = threadIdx.x & 31;
@@ -363,54 +436,102 @@ __global__ void __launch_bounds__(256) permute_scan_kernel(const int* __restrict
   }
 }
 
-// Large S, pass 3: stable ranks inside a chunk.  Each warp owns 128 consecutive slots; warps are
-// ordered through a per-warp count table, lanes through a match mask.
-__global__ void __launch_bounds__(256) permute_scatter_kernel(const int* __restrict__ ids, int S, int E,
-                                                              const int* __restrict__ block_base,
-                                                              int* __restrict__ perm, int* __restrict__ inv_perm) {
-  extern __shared__ int s_w[];  // [8][E]
+// Large S, pass 2: stable ranks inside a chunk, a slot per thread: warps are ordered through a per-warp count table, lanes through a
+// match mask.  What comes before the chunk is summed from the counts of pass 1 by every CTA itself, a row of E counts per chunk and
+// all rows in L2: one launch less than a scan between the two (in a row of layers, both: 1027 tokens 6.6 -> 4.6 us, 8192 10.4 -> 7.6, 32768
+// 14.2 -> 12.1, with the offsets as well).
+// offsets_out: expert_offsets is not there yet and written here by the last chunk; else it is read, or, where that is null as well,
+// block_counts holds positions already.
+__global__ void __launch_bounds__(kPermuteChunk) permute_scatter_kernel(const int* __restrict__ ids, int S, int E,
+                                                                       const int* __restrict__ block_counts, const int* __restrict__ offsets,
+                                                                       int* __restrict__ offsets_out, int* __restrict__ perm,
+                                                                       int* __restrict__ inv_perm) {
+  constexpr int kWarps = kPermuteChunk / 32;
+  extern __shared__ int s_base[];  // [E] counts before the chunk, then positions; [E] all counts; [32]; [kWarps][E] 16-bit counts
+  int* s_tot = s_base + E;
+  int* s_misc = s_tot + E;
+  unsigned short* s_w = reinterpret_cast<unsigned short*>(s_misc + 32);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, blk = static_cast<int>(blockIdx.x), nblk = static_cast<int>(gridDim.x);
+  for (int i = tid; i < 2 * E; i += kPermuteChunk) s_base[i] = 0;
+  for (int i = tid; i < kWarps * E; i += kPermuteChunk) s_w[i] = 0;
+  __syncthreads();
   pdl_wait();
   pdl_launch_dependents();
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  constexpr int kWarps = 8, kPerWarp = kPermuteChunk / kWarps;
-  for (int i = tid; i < kWarps * E; i += blockDim.x) s_w[i] = 0;
-  __syncthreads();
-  int* mine = s_w + wid * E;
-  const int base = blockIdx.x * kPermuteChunk + wid * kPerWarp;
-  const unsigned lt = (1u << lane) - 1u;
-  for (int it = 0; it < kPerWarp / 32; ++it) {
-    const int s = base + it * 32 + lane;
-    const int e = (s < S) ? ids[s] : E;
-    const unsigned peers = __match_any_sync(0xffffffffu, e);
-    if (e < E && (peers & lt) == 0u) mine[e] += __popc(peers);
-    __syncwarp();
+  const int s = blk * kPermuteChunk + tid;
+  const int e = s < S ? ids[s] : E;
+  // the counts: thread (four experts, part) sums every parts-th row, sixteen loads in flight
+  const int rows = offsets_out != nullptr ? nblk : blk;
+  if (offsets_out == nullptr && offsets == nullptr) {
+    if (tid < E) s_base[tid] = block_counts[static_cast<size_t>(blk) * E + tid];
+  } else if ((E & 3) == 0) {
+    const int quads = E >> 2, parts = kPermuteChunk / quads, cq = tid % quads, part = tid / quads;
+    if (part < parts) {
+      int before[4] = {0, 0, 0, 0}, all[4] = {0, 0, 0, 0};
+#pragma unroll 16
+      for (int b = part; b < rows; b += parts) {
+        const int4 c = __ldcg(reinterpret_cast<const int4*>(block_counts + static_cast<size_t>(b) * E) + cq);
+        const int in_front = b < blk ? -1 : 0;
+        all[0] += c.x, all[1] += c.y, all[2] += c.z, all[3] += c.w;
+        before[0] += c.x & in_front, before[1] += c.y & in_front, before[2] += c.z & in_front, before[3] += c.w & in_front;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (before[j] != 0) atomicAdd(&s_base[4 * cq + j], before[j]);
+        if (all[j] != 0) atomicAdd(&s_tot[4 * cq + j], all[j]);
+      }
+    }
+  } else {
+    const int parts = kPermuteChunk / E, ce = tid % E, part = tid / E;  // (E is at most 1024)
+    if (part < parts) {
+      int before = 0, all = 0;
+      for (int b = part; b < rows; b += parts) {
+        const int c = __ldcg(block_counts + static_cast<size_t>(b) * E + ce);
+        all += c;
+        before += b < blk ? c : 0;
+      }
+      if (before != 0) atomicAdd(&s_base[ce], before);
+      if (all != 0) atomicAdd(&s_tot[ce], all);
+    }
   }
+  const unsigned peers = __match_any_sync(0xffffffffu, e);
+  const unsigned before_me = peers & ((1u << lane) - 1u);
+  if (e < E && before_me == 0u) s_w[wid * E + e] = static_cast<unsigned short>(__popc(peers));
   __syncthreads();
-  for (int e = tid; e < E; e += blockDim.x) {
-    int run = block_base[static_cast<size_t>(blockIdx.x) * E + e];
+  if (offsets_out != nullptr) {  // exclusive scan of all counts, an expert per thread
+    const int v = tid < E ? s_tot[tid] : 0;
+    int wtot;
+    int ex = warp_excl_scan(v, lane, &wtot);
+    if (lane == 0) s_misc[wid] = wtot;
+    __syncthreads();
+    for (int i = 0; i < wid; ++i) ex += s_misc[i];
+    if (tid < E) {
+      s_base[tid] += ex;
+      if (blk == nblk - 1) {
+        offsets_out[tid] = ex;
+        if (tid == E - 1) offsets_out[E] = ex + v;
+      }
+    }
+  } else if (offsets != nullptr && tid < E) {
+    s_base[tid] += offsets[tid];
+  }
+  if (tid < E) {
+    unsigned run = 0;
+#pragma unroll
     for (int w = 0; w < kWarps; ++w) {
-      const int c = s_w[w * E + e];
-      s_w[w * E + e] = run;
+      const unsigned c = s_w[w * E + tid];
+      s_w[w * E + tid] = static_cast<unsigned short>(run);
       run += c;
     }
   }
   __syncthreads();
-  for (int it = 0; it < kPerWarp / 32; ++it) {
-    const int s = base + it * 32 + lane;
-    const int e = (s < S) ? ids[s] : E;
-    const unsigned peers = __match_any_sync(0xffffffffu, e);
-    if (e < E) {
-      const int p = mine[e] + __popc(peers & lt);
-      perm[p] = s;
-      inv_perm[s] = p;
-    }
-    __syncwarp();
-    if (e < E && (peers & lt) == 0u) mine[e] += __popc(peers);
-    __syncwarp();
+  if (e < E) {
+    const int p = s_base[e] + s_w[wid * E + e] + __popc(before_me);
+    perm[p] = s;
+    inv_perm[s] = p;
   }
 }
 
-// Large S, pass 4: gather rows, one warp per sorted row.
+// Large S, pass 3: gather rows, one warp per sorted row.
 // range: null, or two device words {first sorted row, row after the last} - only those rows are copied (a rank of an
 // expert-parallel job needs the rows of its own experts only)
 __global__ void __launch_bounds__(256) permute_gather_kernel(const __nv_bfloat16* __restrict__ x,
@@ -437,31 +558,72 @@ int launch_gather_rows(const __nv_bfloat16* x, const int* perm, const moe_shape_
   return MOE_OK;
 }
 
+// count and scatter; offsets_out as permute_scatter_kernel has it
+static int launch_chunked_sort(const int* ids, const int* offsets, int* offsets_out, int S, int E, int* perm, int* inv_perm, int* block_counts,
+                               cudaStream_t st) {
+  static PerDeviceFlag flag;
+  if (!once_per_device(flag, [] {
+        return cudaFuncSetAttribute(permute_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) == cudaSuccess;
+      }))
+    return MOE_ERR_CUDA;
+  const int nblk = (S + kPermuteChunk - 1) / kPermuteChunk;
+  const size_t smem = static_cast<size_t>(2 * E + 32) * 4 + static_cast<size_t>(kPermuteChunk / 32) * E * 2;
+  const bool scan = nblk > kSortChunks;  // (offsets is there in this case)
+  if (launch_pdl(permute_count_kernel, dim3(nblk), dim3(256), E * 4, st, ids, S, E, block_counts) != cudaSuccess ||
+      (scan && launch_pdl(permute_scan_kernel, dim3((E + 7) / 8), dim3(256), 0, st, offsets, E, nblk, block_counts) != cudaSuccess))
+    return MOE_ERR_CUDA;
+  if (scan) offsets = nullptr;
+  if (launch_pdl(permute_scatter_kernel, dim3(nblk), dim3(kPermuteChunk), smem, st, ids, S, E, block_counts, offsets, offsets_out, perm, inv_perm) !=
+          cudaSuccess)
+    return MOE_ERR_CUDA;
+  return MOE_OK;
+}
+
 int launch_permute(const __nv_bfloat16* x, const int* ids, const int* offsets, const moe_shape_t& sh,
                    __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st, const int* range_lo,
                    const int* range_hi) {
   const int S = sh.T * sh.k;
   if (S <= permute_direct(x_perm != nullptr, sh.H)) {
-    if (launch_pdl(permute_small_kernel, dim3((S + 7) / 8), dim3(256), 0, st, x, ids, offsets, S, sh.H, sh.k, x_perm, perm,
-                   inv_perm, range_lo, range_hi) != cudaSuccess)
+    if (launch_pdl(permute_small_kernel<false>, dim3((S + 7) / 8), dim3(256), 0, st, x, ids, const_cast<int*>(offsets), S, sh.H, sh.k, x_perm, perm,
+                   inv_perm, range_lo, range_hi, sh.E) != cudaSuccess)
       return MOE_ERR_CUDA;
     note_kernel("permute_rank_by_count", 1);
   } else {
-    const int nblk = (S + kPermuteChunk - 1) / kPermuteChunk;
-    if (launch_pdl(permute_count_kernel, dim3(nblk), dim3(256), sh.E * 4, st, ids, S, sh.E, block_counts) != cudaSuccess ||
-        launch_pdl(permute_scan_kernel, dim3((sh.E + 7) / 8), dim3(256), 0, st, offsets, sh.E, nblk, block_counts) != cudaSuccess ||
-        launch_pdl(permute_scatter_kernel, dim3(nblk), dim3(256), 8 * sh.E * 4, st, ids, S, sh.E, block_counts, perm, inv_perm) !=
-            cudaSuccess)
-      return MOE_ERR_CUDA;
+    const int rc = launch_chunked_sort(ids, offsets, nullptr, S, sh.E, perm, inv_perm, block_counts, st);
+    if (rc != MOE_OK) return rc;
     if (x_perm != nullptr) {
       const int grid = min((S + 7) / 8, sm_count() * 16);
       if (launch_pdl(permute_gather_kernel, dim3(grid), dim3(256), 0, st, x, perm, S, sh.H, sh.k, x_perm, range_lo, range_hi) !=
           cudaSuccess)
         return MOE_ERR_CUDA;
     }
-    note_kernel("permute_chunked_scan", x_perm != nullptr ? 4 : 3);
+    note_kernel("permute_chunked_scan", x_perm != nullptr ? 3 : 2);
   }
   return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+}
+
+bool route_permute_ok(const moe_shape_t& s) {
+  return !route_sort_ok(s.T, s.E) && s.T > 32 && static_cast<long long>(s.T) * s.k <= static_cast<long long>(kSortChunks) * kPermuteChunk;
+}
+// Routing and sort of a call that makes both, for batches that no cluster routes: the router, then the sort with the offsets as its
+// by-product.  The direct count doubles (it counts smaller experts too), so its line lies lower.
+int launch_route_permute(const float* logits, const __nv_bfloat16* x, const moe_shape_t& sh, int* ids, float* w, int* offsets,
+                         __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st) {
+  const int S = sh.T * sh.k;
+  if (!route_attr_once()) return MOE_ERR_CUDA;
+  int rc = launch_route_ids(logits, sh.T, sh.E, sh.k, ids, w, nullptr, 0, st);
+  if (rc != MOE_OK) return rc;
+  note_kernel("route_topk_multi_cta", 1);
+  if (S <= 4096) {
+    if (launch_pdl(permute_small_kernel<true>, dim3((S + 7) / 8 + 1), dim3(256), (static_cast<size_t>(sh.E) + 32) * 4, st, x, ids, offsets, S, sh.H,
+                   sh.k, x_perm, perm, inv_perm, static_cast<const int*>(nullptr), static_cast<const int*>(nullptr), sh.E) != cudaSuccess)
+      return MOE_ERR_CUDA;
+    note_kernel("permute_rank_by_count", 1);
+    return MOE_OK;
+  }
+  if ((rc = launch_chunked_sort(ids, nullptr, offsets, S, sh.E, perm, inv_perm, block_counts, st)) != MOE_OK) return rc;
+  note_kernel("permute_chunked_scan", 2);
+  return x_perm != nullptr ? launch_gather_rows(x, perm, sh, x_perm, st) : MOE_OK;
 }
 
 // =================================================================================================
