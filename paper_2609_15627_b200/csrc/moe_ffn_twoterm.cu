@@ -520,36 +520,12 @@ MOE_DEVINL bool tt_split_256(const uint4& v, int lane, uint2* hi, uint2* lo, uin
   return __any_sync(0xffffffffu, n >= kTtLossyTokens || !finite);
 }
 
-// The quantised-activation variant's counterpart: 8 E2M1 codes per lane (native_quant_rows_kernel's arithmetic), scale word likewise
-MOE_DEVINL uint32_t tt_quant_256(const uint4& v, int lane, uint32_t* word) {
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  float amax = 0.0f;
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    amax = fmaxf(amax, fmaxf(fabsf(__uint_as_float(w[j] << 16)), fabsf(__uint_as_float(w[j] & 0xFFFF0000u))));
-  amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
-  amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
-  const int se = amax > 0.0f ? term_exp(amax) : 0;
-  const float inv = pow2f(-se);
-  uint32_t codes = 0u;
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    codes |= static_cast<uint32_t>(__nv_cvt_float2_to_fp4x2(make_float2(__uint_as_float(w[j] << 16) * inv, __uint_as_float(w[j] & 0xFFFF0000u) * inv),
-                                                            __NV_E2M1, cudaRoundNearest)) << (8 * j);
-  uint32_t sw = static_cast<uint32_t>(se + 127) << (8 * ((lane >> 2) & 3));
-  sw |= __shfl_xor_sync(0xffffffffu, sw, 4);
-  sw |= __shfl_xor_sync(0xffffffffu, sw, 8);
-  *word = sw;
-  return codes;
-}
-
 // ---- bf16 rows of the sorted order -> two E4M3 rows and their scale factors.  Warp task: (row, eight pieces of 256 values -
 // enough for the look-up of the row's place not to count, few enough for a short last round of the resident warps).  Bound by
 // issue (2 bytes read and 2 written per element; 12288 rows of 4096: 41 us; 54 with a look-up per four pieces, 49 with
 // conversion instructions, which kept their pipe 99.8 % busy). ----
-// kQ (quantised activations): one E2M1 term instead, rows of H / 2 bytes, two scale words per K step of 256.
 // kGuard: a byte per task into `marks` (see tt_split_256), and the experts' flags start at zero.
-template <bool kQ, bool kGuard>
+template <bool kGuard>
 __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ offsets,
                                                               uint8_t* __restrict__ xq, uint8_t* __restrict__ sfx, int S, int H, int E,
                                                               int max_tok, int sf_step, uint8_t* __restrict__ marks, int* __restrict__ flags) {
@@ -559,27 +535,24 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
   // reads rows).
   pdl_wait();
   pdl_launch_dependents();
-  const TtTables tab = tt_tables<kQ>(s_tt_tables, offsets, E, max_tok);
+  const TtTables tab = tt_tables<false>(s_tt_tables, offsets, E, max_tok);
   if (kGuard && blockIdx.x == 0)
     for (int e = threadIdx.x; e <= E; e += blockDim.x) flags[e] = 0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int n_chunk = H / 256, parts = (n_chunk + 7) / 8;
   const int p_begin = tab.off[0], n_task = (tab.off[E] - p_begin) * parts;
-  // (kQ: of either half warp, which holds one word of the step, one lane)
-  const bool sf_lane = (lane & 15) < (kQ ? 1 : 2), sf_is_lo = (lane & 1) != 0;  // in either half warp one lane stores the hi word, one the lo word
+  const bool sf_lane = (lane & 15) < 2, sf_is_lo = (lane & 1) != 0;  // in either half warp one lane stores the hi word, one the lo word
   const uint32_t sf_less = sf_is_lo ? 0x05050505u : 0u;
   for (int task = static_cast<int>(blockIdx.x) * 8 + wid; task < n_task; task += static_cast<int>(gridDim.x) * 8) {
     const int row = parts == 1 ? task : (parts == 2 ? task >> 1 : task / parts);
     const int p = p_begin + row, c0 = (task - row * parts) * 8, left = n_chunk - c0;
     // the expert: off[e] <= p < off[e + 1] (empty experts share a value with their successor)
     const int e = tt_find_expert(tab.off, E, p);
-    const TtSfPlace at = tt_sf_place<kQ>(p, e, tab, H, sf_step);
+    const TtSfPlace at = tt_sf_place<false>(p, e, tab, H, sf_step);
     const uint4* src = reinterpret_cast<const uint4*>(x + static_cast<size_t>(p) * H) + c0 * 32 + lane;
     uint2* dst_hi = reinterpret_cast<uint2*>(xq + static_cast<size_t>(p) * H) + c0 * 32 + lane;
     uint2* dst_lo = dst_hi + static_cast<size_t>(S) * H / 8;
-    uint32_t* dst_q = reinterpret_cast<uint32_t*>(xq + static_cast<size_t>(p) * (H / 2)) + c0 * 32 + lane;
-    uint8_t* sf = kQ ? sfx + at.hi + (lane >> 4) * at.lo + static_cast<size_t>(c0) * sf_step
-                     : sfx + at.hi + (sf_is_lo ? at.lo : 0) + static_cast<size_t>(2 * c0 + (lane >> 4)) * sf_step;
+    uint8_t* sf = sfx + at.hi + (sf_is_lo ? at.lo : 0) + static_cast<size_t>(2 * c0 + (lane >> 4)) * sf_step;
     bool again = false;
 #pragma unroll 1
     for (int cb = 0; cb < 8 && cb < left; cb += 4) {
@@ -591,25 +564,81 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
       for (int u = 0; u < 4; ++u)
         if (cb + u < left) {
           uint32_t word;
-          if constexpr (kQ) {
-            dst_q[u * 32] = tt_quant_256(v[u], lane, &word);
-            if (sf_lane) *reinterpret_cast<uint32_t*>(sf) = word;
-            sf += sf_step;
-          } else {
-            uint2 hi, lo;
-            again |= tt_split_256<kGuard>(v[u], lane, &hi, &lo, &word);
-            dst_hi[u * 32] = hi;
-            dst_lo[u * 32] = lo;
-            if (sf_lane) *reinterpret_cast<uint32_t*>(sf) = word - sf_less;
-            sf += 2 * sf_step;
-          }
+          uint2 hi, lo;
+          again |= tt_split_256<kGuard>(v[u], lane, &hi, &lo, &word);
+          dst_hi[u * 32] = hi;
+          dst_lo[u * 32] = lo;
+          if (sf_lane) *reinterpret_cast<uint32_t*>(sf) = word - sf_less;
+          sf += 2 * sf_step;
         }
       src += 128;
       dst_hi += 128;
       dst_lo += 128;
-      dst_q += 128;
     }
     if (kGuard && lane == 0) marks[static_cast<size_t>(p) * parts + (task - row * parts)] = again;
+  }
+}
+
+// ---- quantised activations (moe_expert_ffn_q): bf16 rows of the sorted order -> one E2M1 row of H / 2 bytes, two scale words per K
+// step of 256.  Warp task: (row, four pieces of 512 values), all their loads issued before the row's place is looked up, 16
+// values a lane so that a block is two lanes.  4096 tokens of 4096, top-8, in a row of layers: 84 -> 77 us (as a form of the kernel
+// above, eight values a lane); the 0.34 GB take 51 at the copy rate. ----
+// The quantised-activation variant's counterpart: 16 E2M1 codes per lane (native_quant_rows_kernel's arithmetic), scale word likewise
+MOE_DEVINL uint2 tt_quant_512(const uint4 (&v)[2], int lane, uint32_t* word) {
+  const uint32_t w[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
+  constexpr uint32_t kAbs = 0x7FFF7FFFu;
+  uint32_t m2 = w[0] & kAbs;
+#pragma unroll
+  for (int j = 1; j < 8; ++j) m2 = __vmaxu2(m2, w[j] & kAbs);  // (finite by this variant's domain: the bits order as the magnitudes)
+  m2 = __vmaxu2(m2, __shfl_xor_sync(0xffffffffu, m2, 1));
+  const uint32_t amax = max(m2 & 0xFFFFu, m2 >> 16) << 16;
+  const int se = amax != 0u ? term_exp(__uint_as_float(amax)) : 0;
+  const float inv = pow2f(-se);
+  uint32_t codes[2] = {0u, 0u};
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    codes[j >> 2] |= static_cast<uint32_t>(__nv_cvt_float2_to_fp4x2(make_float2(__uint_as_float(w[j] << 16) * inv, __uint_as_float(w[j] & 0xFFFF0000u) * inv),
+                                                                    __NV_E2M1, cudaRoundNearest)) << (8 * (j & 3));
+  uint32_t sw = static_cast<uint32_t>(se + 127) << (8 * ((lane >> 1) & 3));
+  sw |= __shfl_xor_sync(0xffffffffu, sw, 2);
+  sw |= __shfl_xor_sync(0xffffffffu, sw, 4);
+  *word = sw;
+  return make_uint2(codes[0], codes[1]);
+}
+
+__global__ void __launch_bounds__(256, 4) twoterm_quant_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ offsets,
+                                                              uint8_t* __restrict__ xq, uint8_t* __restrict__ sfx, int H, int E, int max_tok,
+                                                              int sf_step) {
+  extern __shared__ int s_tt_tables[];
+  pdl_wait();  // (as twoterm_split_kernel)
+  pdl_launch_dependents();
+  const TtTables tab = tt_tables<true>(s_tt_tables, offsets, E, max_tok);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int parts = (H + 2047) / 2048;
+  const int p_begin = tab.off[0], n_task = (tab.off[E] - p_begin) * parts;
+  for (int task = static_cast<int>(blockIdx.x) * 8 + wid; task < n_task; task += static_cast<int>(gridDim.x) * 8) {
+    const int row = parts == 1 ? task : (parts == 2 ? task >> 1 : task / parts);
+    const int p = p_begin + row, c0 = (task - row * parts) * 4;
+    const int left = H - c0 * 512 - lane * 16;  // values of the row from this lane's first on (a multiple of 16)
+    const uint4* src = reinterpret_cast<const uint4*>(x + static_cast<size_t>(p) * H) + c0 * 64 + lane * 2;
+    uint4 v[4][2];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) v[u][i] = left > u * 512 ? __ldcg(src + u * 64 + i) : make_uint4(0u, 0u, 0u, 0u);
+    // the expert: off[e] <= p < off[e + 1] (empty experts share a value with their successor)
+    const TtSfPlace at = tt_sf_place<true>(p, tt_find_expert(tab.off, E, p), tab, H, sf_step);
+    uint2* dst = reinterpret_cast<uint2*>(xq + static_cast<size_t>(p) * (H / 2)) + c0 * 32 + lane;
+    uint8_t* sf = sfx + at.hi + ((lane >> 3) & 1) * at.lo + static_cast<size_t>(2 * c0 + (lane >> 4)) * sf_step;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      uint32_t word;
+      const uint2 codes = tt_quant_512(v[u], lane, &word);
+      if (left > u * 512) {  // (of a last half piece, half of the lanes: words in whole eights)
+        dst[u * 32] = codes;
+        if ((lane & 7) == 0) *reinterpret_cast<uint32_t*>(sf + static_cast<size_t>(2 * u) * sf_step) = word;
+      }
+    }
   }
 }
 
@@ -1356,7 +1385,7 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
                     marks, flags, in.offsets_late ? 1 : 0, in.x_sorted);
   } else {
     const size_t want = (S * parts + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
-    rc = launch_pdl(guard ? twoterm_split_kernel<false, true> : twoterm_split_kernel<false, false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256), table_bytes, st, in.x,
+    rc = launch_pdl(guard ? twoterm_split_kernel<true> : twoterm_split_kernel<false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256), table_bytes, st, in.x,
                     offsets, base + L.xq, base + L.sfx, static_cast<int>(S), sh.H, sh.E, geo.max_tok, geo.sf_step, marks, flags);
   }
   if (rc != cudaSuccess) return MOE_ERR_CUDA;
@@ -1422,10 +1451,10 @@ int launch_expert_ffn_q_pair(const __nv_bfloat16* x_perm, const int* offsets, co
       return MOE_ERR_CUDA;
   if (!byte_map_2d(&tm_x.sf, base + L.sfx, 128, (L.sfa - L.sfx) / 128, 128, 4) || !byte_map_2d(&tm_a.sf, base + L.sfa, 128, (L.total - L.sfa) / 128, 128, 4))
     return MOE_ERR_CUDA;
-  const size_t want = (S * ((sh.H / 256 + 7) / 8) + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
-  if (launch_pdl(twoterm_split_kernel<true, false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256),
-                 static_cast<size_t>(kTtTableInts * (sh.E + 1)) * 4, st, x_perm, offsets, base + L.xq, base + L.sfx, static_cast<int>(S), sh.H,
-                 sh.E, kQPairTok, 2048, nullptr, nullptr) != cudaSuccess)
+  const size_t want = (S * ((sh.H + 2047) / 2048) + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
+  if (launch_pdl(twoterm_quant_kernel, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256),
+                 static_cast<size_t>(kTtTableInts * (sh.E + 1)) * 4, st, x_perm, offsets, base + L.xq, base + L.sfx, sh.H, sh.E, kQPairTok,
+                 2048) != cudaSuccess)
     return MOE_ERR_CUDA;
   TtArgs a = {};
   a.offsets = offsets;
