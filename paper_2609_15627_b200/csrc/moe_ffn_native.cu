@@ -1242,7 +1242,7 @@ EncodeTiledFn nat_encode_fn() {
 
 // byte tensor [rows][row_bytes], box [box_rows][box_bytes]
 bool nat_map(CUtensorMap* m, const void* base, uint64_t row_bytes, uint64_t rows, uint32_t box_bytes, uint32_t box_rows,
-             CUtensorMapSwizzle sw) {
+             CUtensorMapSwizzle sw, CUtensorMapL2promotion promotion = CU_TENSOR_MAP_L2_PROMOTION_L2_128B) {
   EncodeTiledFn fn = nat_encode_fn();
   if (fn == nullptr) return false;
   const cuuint64_t dims[2] = {row_bytes, rows};
@@ -1250,7 +1250,7 @@ bool nat_map(CUtensorMap* m, const void* base, uint64_t row_bytes, uint64_t rows
   const cuuint32_t box[2] = {box_bytes, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+            sw, promotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace
@@ -1310,8 +1310,12 @@ bool weight_maps(const ExpertWeights& w, const moe_shape_t& sh, CUtensorMap* tm_
   if (w.blocked)  // every tile is [128 rows][128 bytes], tiles one after the other
     return nat_map(tm_w13, w.w13, 128, r13 * (sh.H / 256), 128, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
            nat_map(tm_w2, w.w2, 128, r2 * (sh.I / 256), 128, 128, CU_TENSOR_MAP_SWIZZLE_128B);
-  return nat_map(tm_w13, w.w13, sh.H / 2, r13, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
-         nat_map(tm_w2, w.w2, sh.I / 2, r2, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
+  // Rows: L2 fetches 256 bytes of a row at a time, two K steps' worth, so memory opens a page half as often as for the 128 bytes of a
+  // box (eight-term kernel, layers in a row: block of 48 tokens 404 -> 388 us, 100 tokens 548 -> 529, 16 tokens 222 -> 216; tiles, which
+  // lie in one piece, do not care).  Not so the maps of codes_map_u4, half as wide: 2048 tokens 1001 -> 1025 us with 256.
+  constexpr CUtensorMapL2promotion k256 = CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
+  return nat_map(tm_w13, w.w13, sh.H / 2, r13, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B, k256) &&
+         nat_map(tm_w2, w.w2, sh.I / 2, r2, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B, k256) &&
          (sh.H % 512 != 0 || nat_map(tm_s13, w.s13, sh.H / 32, r13, 16, 128, CU_TENSOR_MAP_SWIZZLE_NONE)) &&
          (sh.I % 512 != 0 || nat_map(tm_s2, w.s2, sh.I / 32, r2, 16, 128, CU_TENSOR_MAP_SWIZZLE_NONE));
 }
