@@ -128,8 +128,8 @@ def _ptr(t):
 
 def _stream(stream):
     """The raw stream of a call: the caller's (a stream object, or its raw handle), or torch's current one."""
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:  # (the handle alone: a Stream object made for it takes longer than the rest of a small call's marshalling)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 
@@ -403,14 +403,17 @@ class LayerBuffers:
 def moe_layer(logits, x, weights, buf, stream=None):
     """route -> permute -> expert_ffn -> combine on device tensors; returns buf.out (enqueue only)."""
     w13, s13, w2, s2 = weights
-    sh = buf.sh
+    sh, out, ws = buf.sh, buf.out, buf.ws
     stream = _stream(stream)
     T, E = logits.shape
     if T == sh.T and E == sh.E:  # the four calls in one, which takes a small layer's host time from four trips to one
-        _check(lib().moe_layer(_ptr(logits), _ptr(x), _ptr(w13), _ptr(s13), _ptr(w2), _ptr(s2), C.byref(sh), _ptr(buf.topk_ids),
-                               _ptr(buf.topk_w), _ptr(buf.expert_offsets), _ptr(buf.x_perm), _ptr(buf.perm), _ptr(buf.inv_perm),
-                               _ptr(buf.y_perm), _ptr(buf.out), _ptr(buf.status), _ptr(buf.ws), buf.ws.numel(), stream), "moe_layer")
-        return buf.out
+        rc = (_lib or lib()).moe_layer(logits.data_ptr(), _ptr(x), _ptr(w13), _ptr(s13), _ptr(w2), _ptr(s2), sh, buf.topk_ids.data_ptr(),
+                                       buf.topk_w.data_ptr(), buf.expert_offsets.data_ptr(), buf.x_perm.data_ptr(), buf.perm.data_ptr(),
+                                       buf.inv_perm.data_ptr(), buf.y_perm.data_ptr(), out.data_ptr(), _ptr(buf.status), ws.data_ptr(),
+                                       ws.numel(), stream)
+        if rc != 0:
+            _check(rc, "moe_layer")
+        return out
     # logits of another size than the buffers' shape: moe_route takes the logits' own
     moe_route(logits, sh.k, buf.topk_ids, buf.topk_w, buf.expert_offsets, buf.ws, stream)
     moe_permute(x, buf.topk_ids, buf.expert_offsets, sh, buf.x_perm, buf.perm, buf.inv_perm, buf.ws, stream)
