@@ -520,7 +520,7 @@ MOE_DEVINL bool tt_split_256(const uint4& v, int lane, uint2* hi, uint2* lo, uin
   return __any_sync(0xffffffffu, n >= kTtLossyTokens || !finite);
 }
 
-// ---- bf16 rows of the sorted order -> two E4M3 rows and their scale factors.  Warp task: (row, eight pieces of 256 values -
+// ---- bf16 rows of the sorted order -> two E4M3 rows and their scale factors.  Warp task: (row, `chunks` pieces of 256 values; eight -
 // enough for the look-up of the row's place not to count, few enough for a short last round of the resident warps).  Bound by
 // issue (2 bytes read and 2 written per element; 12288 rows of 4096: 41 us; 54 with a look-up per four pieces, 49 with
 // conversion instructions, which kept their pipe 99.8 % busy). ----
@@ -528,7 +528,7 @@ MOE_DEVINL bool tt_split_256(const uint4& v, int lane, uint2* hi, uint2* lo, uin
 template <bool kGuard>
 __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ offsets,
                                                               uint8_t* __restrict__ xq, uint8_t* __restrict__ sfx, int S, int H, int E,
-                                                              int max_tok, int sf_step, uint8_t* __restrict__ marks, int* __restrict__ flags) {
+                                                              int max_tok, int sf_step, uint8_t* __restrict__ marks, int* __restrict__ flags, int chunks) {
   extern __shared__ int s_tt_tables[];
   // The first launch of a public call, so the kernel in front of it may be the one that writes expert_offsets: wait before
   // they are read here, and before the gate/up grid, which reads them as it starts, may start (it waits again before it
@@ -539,13 +539,13 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
   if (kGuard && blockIdx.x == 0)
     for (int e = threadIdx.x; e <= E; e += blockDim.x) flags[e] = 0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int n_chunk = H / 256, parts = (n_chunk + 7) / 8;
+  const int n_chunk = H / 256, parts = (n_chunk + chunks - 1) / chunks;
   const int p_begin = tab.off[0], n_task = (tab.off[E] - p_begin) * parts;
   const bool sf_lane = (lane & 15) < 2, sf_is_lo = (lane & 1) != 0;  // in either half warp one lane stores the hi word, one the lo word
   const uint32_t sf_less = sf_is_lo ? 0x05050505u : 0u;
   for (int task = static_cast<int>(blockIdx.x) * 8 + wid; task < n_task; task += static_cast<int>(gridDim.x) * 8) {
     const int row = parts == 1 ? task : (parts == 2 ? task >> 1 : task / parts);
-    const int p = p_begin + row, c0 = (task - row * parts) * 8, left = n_chunk - c0;
+    const int p = p_begin + row, c0 = (task - row * parts) * chunks, left = min(n_chunk - c0, chunks);
     // the expert: off[e] <= p < off[e + 1] (empty experts share a value with their successor)
     const int e = tt_find_expert(tab.off, E, p);
     const TtSfPlace at = tt_sf_place<false>(p, e, tab, H, sf_step);
@@ -1384,9 +1384,13 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
                     in.ids, in.inv_perm, offsets, base + L.xq, base + L.sfx, sh.T, sh.k, sh.H, sh.E, geo.max_tok, geo.sf_step, chunks,
                     marks, flags, in.offsets_late ? 1 : 0, in.x_sorted);
   } else {
+    // few rows (a block's shared expert, whose chain of launches the block waits for): shorter tasks, more warps (with the router's boxes:
+    // block of 48 tokens 390.4 -> 388.3 us, 120 tokens 605.7 -> 603.9)
+    const int chunks = S <= 512 ? 2 : 8;
+    parts = (n_chunk + chunks - 1) / chunks;
     const size_t want = (S * parts + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
     rc = launch_pdl(guard ? twoterm_split_kernel<true> : twoterm_split_kernel<false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256), table_bytes, st, in.x,
-                    offsets, base + L.xq, base + L.sfx, static_cast<int>(S), sh.H, sh.E, geo.max_tok, geo.sf_step, marks, flags);
+                    offsets, base + L.xq, base + L.sfx, static_cast<int>(S), sh.H, sh.E, geo.max_tok, geo.sf_step, marks, flags, chunks);
   }
   if (rc != cudaSuccess) return MOE_ERR_CUDA;
   TtArgs a = {};
