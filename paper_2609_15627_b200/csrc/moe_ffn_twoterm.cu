@@ -143,6 +143,57 @@ MOE_DEVINL TtPass tt_pass(int r_begin, int r_end, int pass, int max_tok) {
   p.N = p.stacked ? 2 * p.nr : (p.n + 31) & ~31;
   return p;
 }
+// Where the K steps in flight lie in the ring, and their barriers.  Usually in stages as large as the largest pass needs.  kFifo
+// (passes of at most 64 tokens, few rows per expert): in KB, one behind the other, as large as their own pass needs, or at the
+// start where the end has no room - with 16 rows of a term six steps instead of five (layers in a row, 333 tokens, 10 rows per
+// expert: tiles 659.5 -> 645 us, weights in rows 729 -> 706; 210 tokens 642 -> 633).
+// All roles of both CTAs step through the same sequence; step n of a fifo uses barrier n % kTtMaxStages.
+MOE_DEVINL int tt_fifo_kb(const TtPass& p, int kM) { return (kM * kTtTile + p.nr * 128 + 512 + 1023) >> 10; }
+template <bool kFifo>
+struct TtRing {
+  uint32_t stage;    // bytes of a stage
+  int stages, size;  // stages; KB (kFifo)
+  int s, off, n, free, freed;
+  uint32_t ph;
+  uint64_t taken;    // KB of the last eight steps, with what was skipped in front of them, the newest in the low byte
+  uint32_t addr;     // of the step that `take` or `next` found
+  int bar;
+  uint32_t parity;
+  MOE_DEVINL TtRing(uint32_t stage_bytes, int n_stages)
+      : stage(stage_bytes), stages(n_stages), size(static_cast<int>(stage_bytes * n_stages >> 10)), s(0), off(0), n(0), free(size), freed(0), ph(0),
+        taken(0), addr(0), bar(0), parity(0) {}
+  MOE_DEVINL void next(int kb) {  // consumer
+    if constexpr (kFifo) {
+      const int at = off + kb > size ? 0 : off;
+      off = at + kb;
+      addr = static_cast<uint32_t>(at) << 10;
+      bar = n & (kTtMaxStages - 1);
+      parity = static_cast<uint32_t>(n / kTtMaxStages) & 1u;
+      ++n;
+    } else {
+      addr = s * stage;
+      bar = s;
+      parity = ph;
+      if (++s == stages) { s = 0; ph ^= 1u; }
+    }
+  }
+  MOE_DEVINL void take(int kb, uint64_t* empty, int* status) {  // producer: the same, once it is free
+    if constexpr (kFifo) {
+      const int at = off + kb > size ? 0 : off, need = at == 0 && off != 0 ? size - off + kb : kb;
+      free -= need;
+      while (free < 0 || n - freed == kTtMaxStages) {
+        const int f = freed++;
+        free += static_cast<int>(taken >> (8 * (n - f - 1))) & 0xFF;
+        mbar_wait_warp(&empty[f & (kTtMaxStages - 1)], static_cast<uint32_t>(f / kTtMaxStages) & 1u, status);
+      }
+      taken = (taken << 8) | static_cast<uint64_t>(need);
+      next(kb);
+    } else {
+      mbar_wait_warp(&empty[s], ph ^ 1u, status);
+      next(kb);
+    }
+  }
+};
 // passes of experts < e, for all e: one warp
 MOE_DEVINL void tt_prefix(const int* offsets, int E, int max_tok, int* prefix, int lane) {
   int run = 0;
@@ -727,12 +778,13 @@ __global__ void __launch_bounds__(256) twoterm_gather_kernel(const __nv_bfloat16
 // kQ: quantised activations (moe_expert_ffn_q), one E2M1 term per value: dense 4-bit operands (kind::mxf4, K = 64), K steps of
 // 256, two scale words per row and step; every pass is of the separate form with one operand
 // kGuard (gate/up): blocks that the terms hold too little of are looked for
-template <bool STAGE1, int kM, bool kQ, bool kGuard>
+template <bool STAGE1, int kM, bool kQ, bool kGuard, bool kFifo>
 __global__ void __launch_bounds__(kTtThreads, 1)
 ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_sc,
                    const __grid_constant__ TtTokMaps tmap_t, const TtArgs a) {
   static_assert(!STAGE1 || kM == 2, "gate and up");
   static_assert(!kGuard || (STAGE1 && !kQ), "gate/up on two terms");
+  static_assert(!kFifo || !kQ, "stacked passes");
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
   const TtSmem sm = tt_smem(a.E, kM, a.stages, a.t_bytes);
@@ -816,8 +868,9 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
 
   if (wid == 0) {
     // =========================== weights (all lanes; the instructions are issued by an elected one) ===========================
-    int s = 0, fs = 0;
-    uint32_t ph = 0, fph = 0;
+    int fs = 0, kb = 0;
+    uint32_t fph = 0;
+    TtRing<kFifo> r(sm.stage, a.stages);
     const uint32_t sf_base = smem_u32(sSf), raw_bar = smem_u32(raw_sf), full_own = smem_u32(full), full_first = tt_first_addr(full);
     const uint64_t pol_once = l2_policy_evict_first(), pol_again = l2_policy_evict_normal();
     int g_known = -1, e = 0;
@@ -827,6 +880,7 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
       if (g != g_known) {
         e = warp_uniform(tt_find_expert(prefix, a.E, g));
         once = warp_uniform(prefix[e + 1] - prefix[e]) == 1;  // an expert of one pass is read once per call
+        if (kFifo) kb = warp_uniform(tt_fifo_kb(tt_pass<kQ>(s_off[e], s_off[e + 1], g - prefix[e], a.max_tok), kM));
         g_known = g;
       }
       const uint64_t pol = once ? pol_once : pol_again;
@@ -847,20 +901,19 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
           }
           if (++fs == kTtSfSlots) { fs = 0; fph ^= 1u; }
         }
-        mbar_wait_warp(&empty[s], ph ^ 1u, a.status);
-        if (rank == 0) tt_expect_tx(full_own + s * 8, 2 * kM * (kQ ? kTtTile : kTtTile / 2));  // both CTAs' (transactions count the packed bytes)
+        r.take(kb, empty, a.status);
+        if (rank == 0) tt_expect_tx(full_own + r.bar * 8, 2 * kM * (kQ ? kTtTile : kTtTile / 2));  // both CTAs' (transactions count the packed bytes)
 #pragma unroll
         for (int t = 0; t < kM; ++t) {
           // 128 rows x 128 codes; tile-contiguous layout: half of the rows of tile (row / 128, ks / 2)
           const int row = weight_row(e, rt, t);
           if constexpr (kQ)  // packed rows as they are: 128 rows x 128 bytes
-            tt_load_2d_hint(ring + s * sm.stage + t * kTtTile, &tmap_w, a.blocked ? 0 : ks * 128,
-                            a.blocked ? ((row >> 7) * n_steps + ks) * 128 : row, full_first + s * 8, pol);
+            tt_load_2d_hint(ring + r.addr + t * kTtTile, &tmap_w, a.blocked ? 0 : ks * 128,
+                            a.blocked ? ((row >> 7) * n_steps + ks) * 128 : row, full_first + r.bar * 8, pol);
           else
-            tt_load_2d_hint(ring + s * sm.stage + t * kTtTile, &tmap_w, a.blocked ? (ks & 1) * kTtK : ks * kTtK,
-                            a.blocked ? ((row >> 7) * (n_steps >> 1) + (ks >> 1)) * 128 : row, full_first + s * 8, pol);
+            tt_load_2d_hint(ring + r.addr + t * kTtTile, &tmap_w, a.blocked ? (ks & 1) * kTtK : ks * kTtK,
+                            a.blocked ? ((row >> 7) * (n_steps >> 1) + (ks >> 1)) * 128 : row, full_first + r.bar * 8, pol);
         }
-        if (++s == a.stages) { s = 0; ph ^= 1u; }
       }
     }
   } else if (wid == 2) {
@@ -870,8 +923,7 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     // one pair waits all the same: each kernel of a stream waits for the one in front only, which must therefore not
     // end before those in front of it.)
     if (first < total || (total == 0 && pair == 0)) pdl_wait();
-    int s = 0;
-    uint32_t ph = 0;
+    TtRing<kFifo> r(sm.stage, a.stages);
     const uint32_t full_own = smem_u32(full), full_first = tt_first_addr(full);
     const int sf_pitch = a.sf_step >> 7;  // scale factors as rows of 128 bytes: a box is one 512-byte chunk
     int g_known = -1;
@@ -883,15 +935,16 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
       const int chunks = p.N <= 128 ? 1 : 2;
       const int rows = p.N >> 1;  // this CTA's half of the operand
       const int row_hi = p.stacked ? p.row0 + rank * a.S : p.row0 + rank * rows;
+      const int kb = kFifo ? tt_fifo_kb(p, kM) : 0, sf_off = kFifo ? p.nr * 128 : a.sf_off;
       for (int ks = 0; ks < n_steps; ++ks) {
-        const uint32_t part = ring + s * sm.stage + kM * kTtTile, bar = full_first + s * 8;
         const int terms = kQ || p.stacked ? 1 : 2;  // operands of this CTA: one term of a stacked pass, hi and lo of a separate one
         const int words = kQ ? 2 : terms;          // sets of scale factor chunks
-        mbar_wait_warp(&empty[s], ph ^ 1u, a.status);
-        if (rank == 0) tt_expect_tx(full_own + s * 8, static_cast<uint32_t>(2 * (terms * rows * 128 + words * chunks * 512)));
+        r.take(kb, empty, a.status);
+        const uint32_t part = ring + r.addr + kM * kTtTile, bar = full_first + r.bar * 8;
+        if (rank == 0) tt_expect_tx(full_own + r.bar * 8, static_cast<uint32_t>(2 * (terms * rows * 128 + words * chunks * 512)));
         for (int t = 0; t < words; ++t)
           for (int c = 0; c < chunks; ++c)
-            tt_load_2d(part + a.sf_off + t * 1024 + c * 512, &tmap_t.sf, 0, (g * n_steps + ks) * sf_pitch + t * 8 + c * 4, bar);
+            tt_load_2d(part + sf_off + t * 1024 + c * 512, &tmap_t.sf, 0, (g * n_steps + ks) * sf_pitch + t * 8 + c * 4, bar);
         for (int t = 0; t < terms; ++t) {
           uint32_t dst = part + t * (rows * 128);
           int row = row_hi + t * a.S;
@@ -907,14 +960,14 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
           }
           if (rows & 16) tt_load_2d(dst, &tmap_t.box[2], ks * 128, row, bar);
         }
-        if (++s == a.stages) { s = 0; ph ^= 1u; }
       }
     }
   } else if (wid == 1) {
-    int s = 0, fs = 0, tog = 0;
-    uint32_t ph = 0, fph = 0, acc_ph[2] = {0u, 0u};
+    int fs = 0, tog = 0;
+    uint32_t fph = 0, acc_ph[2] = {0u, 0u};
     int g_known = -1;
     TtPass p = {};
+    TtRing<kFifo> r(sm.stage, a.stages);
     if (rank == 0) {
       // =========================== first CTA: MMA issuer, all lanes ===========================
       for (int w = first; w < total; w = next_item(w)) {
@@ -929,14 +982,16 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
         const uint32_t d0 = tmem_base + static_cast<uint32_t>(half) * kTtFull;
         const uint32_t d1 = d0 + (small ? kTtHalf : kTtFull);
         tc_fence_after_sync();
+        const int kb = kFifo ? tt_fifo_kb(p, kM) : 0, sf_off = kFifo ? p.nr * 128 : a.sf_off;
         for (int ks = 0; ks < n_steps; ++ks) {
           const uint32_t sf_col = tmem_base + kTtColSf + static_cast<uint32_t>(ks & 1) * (kQ ? kTtSfSetQ : kTtSfSet);
           const int si = ks & (grp_steps - 1);
           if (si == 0) mbar_wait_warp(&full_sf[fs], fph, a.status);
-          mbar_wait_warp(&full[s], ph, a.status);
+          r.next(kb);
+          mbar_wait_warp(&full[r.bar], r.parity, a.status);
           tc_fence_after_sync();
-          const uint32_t w_addr = ring + s * sm.stage, t_addr = w_addr + kM * kTtTile;
-          const uint32_t sfw = smem_u32(sSf) + static_cast<uint32_t>((fs * 4 + si * (kQ ? 2 : 1)) * kM) * 512, sft = t_addr + a.sf_off;
+          const uint32_t w_addr = ring + r.addr, t_addr = w_addr + kM * kTtTile;
+          const uint32_t sfw = smem_u32(sSf) + static_cast<uint32_t>((fs * 4 + si * (kQ ? 2 : 1)) * kM) * 512, sft = t_addr + sf_off;
           if constexpr (kQ) {
 #pragma unroll
             for (uint32_t w = 0; w < 2; ++w) {  // scale words of the step
@@ -961,8 +1016,7 @@ ffn_twoterm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
                               umma_desc_k_sw128(t_addr + (p.N >> 1) * 128), idesc, sf_col, sf_col + 4, sf_col + 16, 1u);
             }
           }
-          tt_commit(&empty[s]);
-          if (++s == a.stages) { s = 0; ph ^= 1u; }
+          tt_commit(&empty[r.bar]);
           if (si == grp_steps - 1) {
             tt_commit(&empty_sf[fs]);
             if (++fs == kTtSfSlots) { fs = 0; fph ^= 1u; }
@@ -1278,13 +1332,19 @@ bool twoterm_weights_ok(const void* w13, const void* w2) {  // the 4-bit tensor 
 
 namespace {
 
-template <bool STAGE1, int kM, bool kQ, bool kGuard = false>
+template <bool STAGE1, int kM, bool kQ, bool kGuard = false, bool kFifo = false>
 bool tt_launch(const CUtensorMap& tm_w, const CUtensorMap& tm_sc, const TtTokMaps& tm_t, TtArgs a, cudaStream_t st) {
   a.stages = 1;
-  while (a.stages < kTtMaxStages && tt_smem(a.E, kM, a.stages + 1, a.t_bytes).total + 1024 <= 227 * 1024) ++a.stages;
+  if (kFifo) {
+    // a ring of KB: "stages" of one KB without token parts (see TtRing)
+    const int kb = (227 * 1024 - 1024 - static_cast<int>(tt_smem(a.E, 0, 0, 0).total) - kTtSfSlots * kM * 2048) >> 10;
+    a.stages = 1;
+    a.t_bytes = kb * 1024 - kM * kTtTile;
+  }
+  while (!kFifo && a.stages < kTtMaxStages && tt_smem(a.E, kM, a.stages + 1, a.t_bytes).total + 1024 <= 227 * 1024) ++a.stages;
   static PerDeviceFlag flag;
   if (!once_per_device(flag, [] {
-        return cudaFuncSetAttribute(ffn_twoterm_kernel<STAGE1, kM, kQ, kGuard>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
+        return cudaFuncSetAttribute(ffn_twoterm_kernel<STAGE1, kM, kQ, kGuard, kFifo>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
       }))
     return false;
   cudaLaunchConfig_t cfg = {};
@@ -1301,7 +1361,7 @@ bool tt_launch(const CUtensorMap& tm_w, const CUtensorMap& tm_sc, const TtTokMap
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, ffn_twoterm_kernel<STAGE1, kM, kQ, kGuard>, tm_w, tm_sc, tm_t, a) == cudaSuccess;
+  return cudaLaunchKernelEx(&cfg, ffn_twoterm_kernel<STAGE1, kM, kQ, kGuard, kFifo>, tm_w, tm_sc, tm_t, a) == cudaSuccess;
 }
 
 }  // namespace
@@ -1351,6 +1411,7 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
                               const moe_shape_t& choice, bool guard, void* scratch, float* y_perm, int* status_word, cudaStream_t st,
                               float* const* row_dst, bool again_later, int* finished, int* n_cta) {
   const TwoTermGeometry geo = twoterm_geometry(choice);
+  const bool two = geo.max_tok == 64 && sh.H % 512 == 0;  // M tiles of a down item
   const TwoTermScratch L = twoterm_scratch(choice);
   uint8_t* base = static_cast<uint8_t*>(scratch);
   const uint64_t S = static_cast<uint64_t>(sh.T) * sh.k;
@@ -1418,15 +1479,23 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
   a.sc = w.s13;
   a.K = sh.H;
   a.R = 2 * sh.I;
-  if (!(guard ? tt_launch<true, 2, false, true>(tm_w13, tm_s13, tm_x, a, st) : tt_launch<true, 2, false>(tm_w13, tm_s13, tm_x, a, st)))
+  // Up to 16 rows per expert on average, where most passes have 16 or 32 rows (512 tokens, 16 rows: 703 -> 699 us); with 48 rows no step more
+  // fits and finding its place costs 1 % (2048 tokens 986 -> 999).  Where no other kernel does experts again: the kernel that does
+  // is for more rows, or small layers.
+  const bool fifo = !guard && geo.max_tok == 64 && two && S <= 16ull * choice.E;
+  if (!(guard  ? tt_launch<true, 2, false, true>(tm_w13, tm_s13, tm_x, a, st)
+        : fifo ? tt_launch<true, 2, false, false, true>(tm_w13, tm_s13, tm_x, a, st)
+               : tt_launch<true, 2, false>(tm_w13, tm_s13, tm_x, a, st)))
     return MOE_ERR_CUDA;
   a.finished = finished;
   if (n_cta != nullptr) *n_cta = sm_count() & ~1;
   a.sc = w.s2;
   a.K = sh.I;
   a.R = sh.H;
-  const bool two = geo.max_tok == 64 && sh.H % 512 == 0;
-  if (!(two ? tt_launch<false, 2, false>(tm_w2, tm_s2, tm_a, a, st) : tt_launch<false, 1, false>(tm_w2, tm_s2, tm_a, a, st))) return MOE_ERR_CUDA;
+  if (!(fifo  ? tt_launch<false, 2, false, false, true>(tm_w2, tm_s2, tm_a, a, st)
+        : two ? tt_launch<false, 2, false>(tm_w2, tm_s2, tm_a, a, st)
+              : tt_launch<false, 1, false>(tm_w2, tm_s2, tm_a, a, st)))
+    return MOE_ERR_CUDA;
   if (guard && !again_later) {
     const int again = launch_again(in, offsets, w, sh, choice, base + L.aq, y_perm, status_word, st, row_dst, flags);
     if (again != MOE_OK) return again;
