@@ -133,9 +133,10 @@ int moe_permute(const void* x_bf16, const int32_t* topk_ids, const int32_t* expe
 namespace {
 int expert_ffn_impl(const void* x_perm_bf16, const int32_t* expert_offsets, const ExpertWeights& w, const moe_shape_t* shape,
                     float* y_perm, int32_t* status_word, void* ws, size_t ws_bytes, void* cuda_stream,
-                    float* const* row_dst = nullptr, const moe_shape_t* choice = nullptr) {
+                    float* const* row_dst = nullptr, const moe_shape_t* choice = nullptr, bool offsets_late = false) {
   // `choice`: the shape that picks the kernel where it is not `shape` itself - a rank of an expert-parallel job runs the
-  // kernel the unsharded layer would run, so that the sharded result has the same bits
+  // kernel the unsharded layer would run, so that the sharded result has the same bits.  `offsets_late`: the launch in front may
+  // still be writing expert_offsets when it lets this one start (for the kernels that the calls of a known routing send here)
   if (choice == nullptr) choice = shape;
   if (!aligned(x_perm_bf16, 16) || !aligned(expert_offsets, 16) || !aligned(w.w13, 16) || !aligned(w.s13, 16) ||
       !aligned(w.w2, 16) || !aligned(w.s2, 16) || (row_dst == nullptr ? !aligned(y_perm, 16) : !aligned(row_dst, 8)))
@@ -155,7 +156,7 @@ int expert_ffn_impl(const void* x_perm_bf16, const int32_t* expert_offsets, cons
   if (rc != MOE_OK) return rc;
   const bool twoterm = twoterm_chosen(*choice, w);
   if (!twoterm && native_shape_ok(*choice, w.w13, w.w2))
-    return launch_expert_ffn_native(xp, expert_offsets, w, *shape, act, y_perm, status, st, row_dst);
+    return launch_expert_ffn_native(xp, expert_offsets, w, *shape, act, y_perm, status, st, row_dst, nullptr, nullptr, offsets_late);
   if ((rc = clear_own_status(status, st)) != MOE_OK) return rc;
   if (twoterm)
     return launch_expert_ffn_twoterm(TwoTermInput{xp, nullptr, nullptr, nullptr, false, false}, expert_offsets, w, *shape, *choice, twoterm_guarded(*choice, w),
@@ -229,7 +230,7 @@ int route_and_ffn(const float* logits, const void* x, int32_t* ids, float* topk_
       if (twoterm)
         return launch_expert_ffn_twoterm(TwoTermInput{xb, ids, inv_perm, xp, true, rows}, offsets, w, s, s, twoterm_guarded(s, w), base + L.act_off,
                                          y_perm, status.word, st);
-      return expert_ffn_impl(x_perm, offsets, w, shape, y_perm, status_word, ws, ws_bytes, cuda_stream);
+      return expert_ffn_impl(x_perm, offsets, w, shape, y_perm, status_word, ws, ws_bytes, cuda_stream, nullptr, nullptr, true);
     }
     if ((rc = moe_route(logits, s.T, s.E, s.k, ids, topk_w, offsets, ws, ws_bytes, cuda_stream)) != MOE_OK) return rc;
     return permute_and_ffn(x, ids, offsets, w, shape, x_perm, perm, inv_perm, y_perm, status_word, ws, ws_bytes, cuda_stream, rows);

@@ -246,8 +246,9 @@ int launch_gather_rows(const __nv_bfloat16* x, const int* perm, const moe_shape_
 int launch_permute(const __nv_bfloat16* x, const int* ids, const int* offsets, const moe_shape_t& s,
                    __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st,
                    const int* range_lo = nullptr, const int* range_hi = nullptr);
-// routing and sort of batches that no cluster routes, in a call that makes both (x_perm null: no rows); offsets is written by the
-// sort, so what comes next waits before it reads it
+// routing and sort of batches that no cluster routes, in a call that makes both (x_perm null: no rows).  offsets is written by the
+// sort, and up to 4096 slots by its last CTA after the launch has let its dependents go: whatever is launched next is told so
+// (offsets_late) or is a plain launch
 bool route_permute_ok(const moe_shape_t& s);
 int launch_route_permute(const float* logits, const __nv_bfloat16* x, const moe_shape_t& s, int* ids, float* w, int* offsets,
                          __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st);
@@ -273,7 +274,7 @@ struct TwoTermInput {
   const int* ids;          // [T, k] expert of every slot
   const int* inv_perm;     // [T, k] sorted row of every slot
   __nv_bfloat16* x_sorted; // with the tables: room for the rows in sorted order, of the experts that `guard` does again
-  bool offsets_late;       // with the tables: the kernel in front is the one that writes the offsets
+  bool offsets_late;       // with the tables: the kernel in front is the one that writes the offsets (likewise in launch_expert_ffn_native)
   bool write_rows;         // with the tables: x_sorted is the caller's and receives all rows
 };
 // `again_later`: the launches of `guard` that do experts again are left to launch_twoterm_again, before anything reads y_perm.
@@ -312,7 +313,7 @@ int launch_expert_ffn_native_q(const __nv_bfloat16* x_perm, const int* offsets, 
                                void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst = nullptr);
 int launch_expert_ffn_native(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& s,
                              void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst = nullptr,
-                             int* finished = nullptr, int* n_cta = nullptr);
+                             int* finished = nullptr, int* n_cta = nullptr, bool offsets_late = false);
 
 // the native variant behind launch_route_sort: token rows by token (native_front_split says where that launch leaves them).  H a
 // multiple of 512.
@@ -388,7 +389,8 @@ inline bool once_per_device(PerDeviceFlag& f, F&& set) {
 // native_split_kernel, native_quant_rows_kernel, native_expand_kernel, twoterm_scatter_kernel and the expert-FFN kernels
 // release theirs BEFORE they wait, so three or four neighbours of a chain (route, permute, split, expert FFN) can be
 // resident together.  That is safe because of the rule above: whatever a kernel does before its wait only reads buffers
-// that no kernel of the chain before it writes (logits, expert_offsets of a completed router, the weights), and every
+// that no kernel of the chain still in flight writes (logits, the weights, expert_offsets once the kernel that writes them has
+// been waited for by one that had not let its dependents go: see offsets_late), and every
 // global write comes after the wait, i.e. after everything launched earlier on the stream has completed - for the wait is
 // for the launch in front only, and that has waited in its turn, whether it had work or not.  shared_offsets_kernel and
 // shared_join_kernel release by ending; so does router_gemv_kernel but inside moe_ffn_block (see RouterOrder).

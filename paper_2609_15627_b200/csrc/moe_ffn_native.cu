@@ -254,9 +254,12 @@ __host__ __device__ inline NatSmem nat_smem(int E, int K) {
 // grid still occupies delays one of them - with at most (SMs - working FFN CTAs) CTAs here, only idle ones.
 __global__ void __launch_bounds__(1024) native_split_kernel(const __nv_bfloat16* __restrict__ x, uint8_t* __restrict__ aq,
                                                            uint8_t* __restrict__ aq_sf, int* __restrict__ done, int S, int H,
-                                                           int E, int* __restrict__ status_clear) {
-  pdl_launch_dependents();  // the FFN grid may set up and start its weight stream; it waits before it reads aq or done
+                                                           int E, int* __restrict__ status_clear, int offsets_late) {
+  // The FFN grid may set up and start its weight stream; it waits before it reads aq or done.  It reads expert_offsets as it starts:
+  // where the kernel in front writes them, after whatever lets its dependents go there, this kernel waits for it first.
+  if (!offsets_late) pdl_launch_dependents();
   pdl_wait();               // the sorted token rows of moe_permute are complete, and every earlier kernel on the stream
+  if (offsets_late) pdl_launch_dependents();
   const long long gt = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (gt < E) done[gt] = 0;
   // the library's own status word (caller passed none): whatever an earlier call left there is over, and the FFN grid
@@ -270,7 +273,7 @@ __global__ void __launch_bounds__(1024) native_split_kernel(const __nv_bfloat16*
 __global__ void __launch_bounds__(1024) native_quant_rows_kernel(const __nv_bfloat16* __restrict__ x, uint8_t* __restrict__ aq,
                                                                 uint8_t* __restrict__ aq_sf, int* __restrict__ done, int S, int H,
                                                                 int E, int* __restrict__ status_clear) {
-  pdl_launch_dependents();  // as native_split_kernel
+  pdl_launch_dependents();  // as native_split_kernel (the offsets are the caller's)
   pdl_wait();
   const long long gt = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (gt < E) done[gt] = 0;
@@ -434,8 +437,8 @@ ffn_native_kernel(const __grid_constant__ CUtensorMap tmap_w13, const __grid_con
     }
   } else if (!kFused && wid == 2) {
     // lane l looks at experts l, l + 32, ...: all loads are issued before any is used (one memory round trip);
-    // the second loop's loads hit L1.  expert_offsets was complete before the permute kernel let this chain start - where there
-    // is none, it is the kernel in front's.
+    // the second loop's loads hit L1.  expert_offsets was complete before the split kernel let this grid start (the kernel in front of
+    // that one had waited for what writes them, or the split has: offsets_late) - where there is no split, it is the kernel in front's.
     if (a.tok != nullptr) pdl_wait();
     const int n_it = (a.E + 31) / 32;
     unsigned has_mask = 0u;
@@ -1364,7 +1367,8 @@ NatTokens nat_tokens(void* scratch, const moe_shape_t& sh) {
 // by_token: the rows' terms are those that launch_route_sort left (see launch_expert_ffn_native_tokens)
 template <bool kQ>
 int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
-                      void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, bool by_token = false, int* finished = nullptr) {
+                      void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, bool by_token = false, int* finished = nullptr,
+                      bool offsets_late = false) {
   if (!nat_attr_once()) return MOE_ERR_CUDA;
   const size_t S = static_cast<size_t>(sh.T) * sh.k;
   const size_t rows = S * (kQ ? 1 : kTerms);  // operand rows
@@ -1384,7 +1388,8 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
     const dim3 split_grid(static_cast<unsigned>((split_threads + 1023) / 1024));
     int* own_word = status.own ? status.word : nullptr;
     if ((kQ ? launch_pdl(native_quant_rows_kernel, split_grid, dim3(1024), 0, st, x_perm, aq1, sf1, done, static_cast<int>(S), sh.H, sh.E, own_word)
-            : launch_pdl(native_split_kernel, split_grid, dim3(1024), 0, st, x_perm, aq1, sf1, done, static_cast<int>(S), sh.H, sh.E, own_word)) !=
+            : launch_pdl(native_split_kernel, split_grid, dim3(1024), 0, st, x_perm, aq1, sf1, done, static_cast<int>(S), sh.H, sh.E, own_word,
+                         offsets_late ? 1 : 0)) !=
         cudaSuccess)
       return MOE_ERR_CUDA;
   }
@@ -1440,9 +1445,9 @@ int launch_native_ffn(const __nv_bfloat16* x_perm, const int* offsets, const Exp
 
 int launch_expert_ffn_native(const __nv_bfloat16* x_perm, const int* offsets, const ExpertWeights& w, const moe_shape_t& sh,
                              void* scratch, float* y_perm, StatusRef status, cudaStream_t st, float* const* row_dst, int* finished,
-                             int* n_cta) {
+                             int* n_cta, bool offsets_late) {
   if (n_cta != nullptr) *n_cta = sm_count();
-  return launch_native_ffn<false>(x_perm, offsets, w, sh, scratch, y_perm, status, st, row_dst, false, finished);
+  return launch_native_ffn<false>(x_perm, offsets, w, sh, scratch, y_perm, status, st, row_dst, false, finished, offsets_late);
 }
 FrontSplit native_front_split(const __nv_bfloat16* x, const moe_shape_t& sh, void* scratch, StatusRef status) {
   const NatScratch L = nat_scratch(scratch, sh, static_cast<size_t>(sh.T) * sh.k * kTerms);
