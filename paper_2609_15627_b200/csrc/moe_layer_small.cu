@@ -1,12 +1,13 @@
 // The whole layer in one launch, for layers that fit the shared memory of one thread-block cluster: a few experts of a few
 // hundred rows, a few tokens.  Such a layer's kernels each last 3 to 6 us, nearly all of it launch and memory latency, so what
-// counts is how many of them follow one another.  Here every CTA of a cluster of eight keeps some experts' weights whole: their
-// copies into shared memory start before the kernel in front has ended; every CTA routes all tokens (a warp per token) and sorts
+// counts is how many of them follow one another.  Here every CTA of a cluster of eight keeps some experts' weights whole: while
+// they are copied into shared memory every CTA routes all tokens (a warp per token) and sorts
 // the slots (a thread per slot, by counting), so nothing is exchanged; a CTA then runs its own experts' rows through both
 // projections, the intermediate staying in its shared memory; the rows of y_perm meet at one cluster barrier, behind which
 // all CTAs reduce them.  Everything the four calls write is written.
-// 16 tokens, 8 experts of 256 x 128, top-2, layers in a row: 21.0 us in five launches -> 10.2 (the host's part of one call; in a
-// graph 13.8 -> 6.9).
+// 16 tokens, 8 experts of 256 x 128, top-2, layers in a row: 21.0 us in five launches -> 8.0 (in a graph 13.8 -> 7.6).  Copies of the
+// weights that started before the kernel in front had ended gave 7.35 (7.0); but that kernel may be the one that writes them, as it may
+// in front of the streaming kernel.
 //
 // The arithmetic is the streaming kernel's (moe_ffn_stream.cu), K group by K group in its order, so that the rows have the
 // same bits: there warp w holds the 128-element groups w, w + 16, .. of K and the warps' sums are added in order; up to
@@ -121,6 +122,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) layer_small_kernel(const Sma
   int* s_slot = reinterpret_cast<int*>(smem + m.slot);  // slot of a sorted row
   int* s_off = reinterpret_cast<int*>(smem + m.off);
   pdl_launch_dependents();  // (whatever comes next waits before it reads)
+  pdl_wait();  // the kernel in front may write the weights, the logits and the rows, and may still read what is written here
   const size_t n = static_cast<size_t>(a.H) * a.I;
   for (int e = rank, j = 0; e < a.E; e += kSmallCluster, ++j) {
     unsigned char* dst = smem + j * m.expert;
@@ -129,7 +131,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1) layer_small_kernel(const Sma
     copy_async(dst + m.w2, a.w2 + e * (n / 2), n / 2);
     copy_async(dst + m.s2, a.s2 + e * (n / 32), n / 32);
   }
-  pdl_wait();  // logits and rows may come from the kernel in front, which may also still read what is written here
   const int per_row = a.H / 8;
   for (int i = tid; i < a.T * per_row; i += kSmallThreads) {
     const int t = i / per_row, c = i - t * per_row;
@@ -230,9 +231,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) layer_small_kernel(const Sma
 }
 
 // (Where the streaming kernel would take the layer: the caller asks for that.)  What fits shared memory and, since the eight CTAs go
-// through all rows where the streaming kernel's 148 would, up to 128 slots (in a graph, this / five launches: one token of 8 experts
-// of 1024 x 128 11.4 us and 13.3, 8 tokens of 32 of 256 x 128, top-8 16.5 and 19.3, 16 of 64 of 128 x 128, top-4 19.3 and 20.4;
-// 32 tokens, 256 slots, of 8 of 256 x 128 23.5 and 21.5).
+// through all rows where the streaming kernel's 148 would, up to 128 slots (this / five launches, in a graph: one token of 8 experts
+// of 1024 x 128, top-8 13.8 us and 16.5, 8 tokens of 32 of 256 x 128, top-8 18.6 and 19.8; 32 tokens, 256 slots, of 8 of 256 x 128 24.1
+// and 21.5.  With seven or eight experts a CTA and 64 slots or more it is ahead only without a graph: 16 tokens of 64 of 128 x 128,
+// top-4 22.4 and 24.9, in a graph 22.1 and 20.5).
 bool layer_small_ok(const moe_shape_t& s) {
   return s.T <= kSmallMaxTok && s.T * s.k <= kSmallMaxSlots && s.E <= kSmallMaxE && s.H <= kSmallMaxK && s.I <= kSmallMaxK &&
          small_smem(s.T, s.H, s.I, s.E, s.k).total <= kSmallSmem;

@@ -104,3 +104,36 @@ def test_small_layers_one_behind_the_other_in_a_graph():
             g.replay()
             s.synchronize()
             assert torch.equal(bufs[(n - 1) & 1].out, want)
+
+
+def test_small_layer_reads_weights_that_the_kernel_in_front_writes():
+    """moe_combine lets its dependents go before it writes; here its output is the expert codes of the layer behind it."""
+    T, H, I, E, k = 16, 256, 128, 8, 2
+    sh, g = moe.shape(T, H, I, E, k), torch.Generator(device="cuda").manual_seed(9)
+    _, s13, _, s2 = _weights(H, I, E)
+    n13, n2 = E * H * I, E * H * I // 2               # bytes of the codes
+    Tc, Hc = 4096, 4096                               # a combine that writes for a while, the codes last
+    shc = moe.shape(Tc, Hc, 128, 1, 1)
+    ys = [torch.randn((Tc, Hc), device="cuda", generator=g).to(torch.bfloat16) for _ in range(2)]
+    inv, one = torch.arange(Tc, dtype=torch.int32, device="cuda"), torch.ones(Tc, device="cuda")
+
+    def codes(out):
+        tail = out.view(torch.uint8).reshape(-1)[-(n13 + n2):]
+        return tail[:n13].view(E, 2 * I, H // 2), s13, tail[n13:].view(E, H, I // 2), s2
+
+    logits, x = dev(inputs.make_logits(T, E, 13)), dev(inputs.make_x(T, H, 13))
+    b, want = moe.LayerBuffers(sh), []
+    for y in ys:
+        moe.moe_layer(logits, x, tuple(v.clone() for v in codes(y)), b)
+        torch.cuda.synchronize()
+        want.append(b.out.clone())
+    assert moe.moe_last_kernel_name() == "layer_one_cluster" and not torch.equal(want[0], want[1])
+    yf, out = [y.float() for y in ys], torch.zeros_like(ys[0])
+    w, got = codes(out), []
+    for i in (0, 1, 0, 1, 1, 0):
+        moe.moe_combine(yf[i], inv, one, shc, out)
+        moe.moe_layer(logits, x, w, b)
+        got.append((i, b.out.clone()))
+    torch.cuda.synchronize()
+    for i, o in got:
+        assert torch.equal(o, want[i])
