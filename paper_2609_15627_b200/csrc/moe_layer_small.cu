@@ -234,9 +234,12 @@ __global__ void __launch_bounds__(kSmallThreads, 1) layer_small_kernel(const Sma
 // through all rows where the streaming kernel's 148 would, up to 128 slots (this / five launches, in a graph: one token of 8 experts
 // of 1024 x 128, top-8 13.8 us and 16.5, 8 tokens of 32 of 256 x 128, top-8 18.6 and 19.8; 32 tokens, 256 slots, of 8 of 256 x 128 24.1
 // and 21.5.  With seven or eight experts a CTA and 64 slots or more it is ahead only without a graph: 16 tokens of 64 of 128 x 128,
-// top-4 22.4 and 24.9, in a graph 22.1 and 20.5).
+// top-4 22.4 and 24.9, in a graph 22.1 and 20.5).  And up to 2^20 weights times rows per CTA that has an expert (launched, and in a graph: 32
+// tokens of 8 of 512 x 128, top-4, which is that, 22.8 us and 25.9, 22.5 and 21.7; of 8 of 384 x 256, top-4, one and a half times that, 28.9 and
+// 28.2, 28.5 and 24.3; of 4 of 512 x 128, top-4, twice that, 27.2 and 24.6, 27.1 and 21.1).
 bool layer_small_ok(const moe_shape_t& s) {
   return s.T <= kSmallMaxTok && s.T * s.k <= kSmallMaxSlots && s.E <= kSmallMaxE && s.H <= kSmallMaxK && s.I <= kSmallMaxK &&
+         static_cast<long long>(s.T) * s.k * s.H * s.I <= (1LL << 20) * (s.E < kSmallCluster ? s.E : kSmallCluster) &&
          small_smem(s.T, s.H, s.I, s.E, s.k).total <= kSmallSmem;
 }
 

@@ -137,3 +137,22 @@ def test_small_layer_reads_weights_that_the_kernel_in_front_writes():
     torch.cuda.synchronize()
     for i, o in got:
         assert torch.equal(o, want[i])
+
+
+@pytest.mark.parametrize("T,H,I,E,k,one", [
+    (32, 512, 128, 8, 4, True), (32, 512, 128, 4, 4, False), (32, 512, 128, 4, 2, True), (31, 384, 256, 8, 4, False), (32, 640, 128, 3, 2, False)])
+def test_small_layer_up_to_a_cta_s_share_of_the_work(T, H, I, E, k, one):
+    """Either side of the line (2^20 weights times rows per CTA with an expert): the same bits by either path."""
+    sh, w = moe.shape(T, H, I, E, k), _weights(H, I, E)
+    logits, x = dev(inputs.make_logits(T, E, 15)), dev(inputs.make_x(T, H, 15))
+    b, c = moe.LayerBuffers(sh), moe.LayerBuffers(sh)
+    b.out.fill_(float("nan"))
+    moe.moe_layer(logits, x, w, b)
+    assert (moe.moe_last_kernel_name() == "layer_one_cluster") == one
+    moe.moe_route(logits, k, c.topk_ids, c.topk_w, c.expert_offsets, c.ws)
+    moe.moe_permute(x, c.topk_ids, c.expert_offsets, sh, c.x_perm, c.perm, c.inv_perm, c.ws)
+    moe.moe_expert_ffn(c.x_perm, c.expert_offsets, *w, sh, c.y_perm, c.status, c.ws)
+    assert moe.moe_last_kernel_name() == "ffn_stream_bulk_ring_mma16816"
+    moe.moe_combine(c.y_perm, c.inv_perm, c.topk_w, sh, c.out)
+    torch.cuda.synchronize()
+    assert torch.equal(b.out, c.out) and torch.equal(b.y_perm, c.y_perm)
