@@ -299,7 +299,8 @@ int moe_ffn_block(const void* x_bf16 /* [T,H] */, const void* w_router_bf16 /* [
  *     32 consecutive elements: amax = max |v|; s = the smallest integer in [-126, 126] with amax <= 6 * 2^s (s = 0 for
  *     an all-zero block); code = E2M1 value nearest to v / 2^s, ties to the even code; the contraction consumes
  *     E2M1(code) * 2^s.  Everything else as moe_expert_ffn: g, u in fp32, act = bf16_rne(silu(g) * u), y_perm fp32.
- *     Inputs with |v| > 2^126 are outside the domain.
+ *     Inputs with |v| > 2^126 are outside the domain; a NaN of x_perm counts for nothing in its block's maximum and takes
+ *     the code of 6.
  *   - Result: y_perm differs from moe_expert_ffn's by the quantisation error (about a quarter of the output's norm on
  *     the benchmark's inputs: one E2M1 term keeps two to three significant bits); against this variant's own oracle the
  *     result is the same - bit for bit on most rows - up to fp32 summation order, the fast exponential and division of the

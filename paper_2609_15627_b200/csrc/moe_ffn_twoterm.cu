@@ -635,13 +635,18 @@ __global__ void __launch_bounds__(256, 4) twoterm_split_kernel(const __nv_bfloat
 // values a lane so that a block is two lanes.  4096 tokens of 4096, top-8, in a row of layers: 84 -> 77 us (as a form of the kernel
 // above, eight values a lane); the 0.34 GB take 51 at the copy rate. ----
 // The quantised-activation variant's counterpart: 16 E2M1 codes per lane (native_quant_rows_kernel's arithmetic), scale word likewise
+MOE_DEVINL uint32_t max_bf16x2(uint32_t a, uint32_t b) {  // the larger of each pair, the number where the other is a NaN (as fmaxf)
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
 MOE_DEVINL uint2 tt_quant_512(const uint4 (&v)[2], int lane, uint32_t* word) {
   const uint32_t w[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
   constexpr uint32_t kAbs = 0x7FFF7FFFu;
-  uint32_t m2 = w[0] & kAbs;
+  uint32_t m2 = 0u;
 #pragma unroll
-  for (int j = 1; j < 8; ++j) m2 = __vmaxu2(m2, w[j] & kAbs);  // (finite by this variant's domain: the bits order as the magnitudes)
-  m2 = __vmaxu2(m2, __shfl_xor_sync(0xffffffffu, m2, 1));
+  for (int j = 0; j < 8; ++j) m2 = max_bf16x2(m2, w[j] & kAbs);
+  m2 = max_bf16x2(m2, __shfl_xor_sync(0xffffffffu, m2, 1));
   const uint32_t amax = max(m2 & 0xFFFFu, m2 >> 16) << 16;
   const int se = amax != 0u ? term_exp(__uint_as_float(amax)) : 0;
   const float inv = pow2f(-se);

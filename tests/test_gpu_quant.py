@@ -280,3 +280,32 @@ def test_ffn_q_stage_by_stage(T, H, I, E, k):
         W2 = table[_unpack_codes(w2[e]).astype(np.int64)] * np.repeat(np.ldexp(1.0, s2w[e].astype(np.int64) - 127), 32, axis=1)
         ref = a_gpu[rows] @ W2.T
         assert np.allclose(got[rows], ref, rtol=2e-6, atol=2e-6 * np.abs(ref).max())
+
+
+@pytest.mark.parametrize("rows,H,I,E,kernel", [(16, 512, 512, 4, "ffn_native_mxf4_quantised_activations"),
+                                               (75, 2048, 1024, 16, "ffn_mxf4_quantised_cta_pair"),
+                                               (150, 2304, 1024, 16, "ffn_mxf4_quantised_cta_pair")])
+def test_ffn_q_a_nan_leaves_its_block_s_scale_alone(rows, H, I, E, kernel):
+    """A NaN counts for nothing in its block's maximum and becomes the code of 6, whatever its sign: the bits of the same rows with 6 times
+    the other values' scale in its place (6 where a whole block is NaN)."""
+    S = rows * E
+    sh, w = moe.shape(S, H, I, E, 1), tuple(dev(a) for a in inputs.make_expert_weights(H, I, E, seed=7))
+    off = torch.arange(0, S + 1, rows, dtype=torch.int32, device="cuda")
+    x = inputs.make_x(S, H, 8)
+    rng = np.random.default_rng(2)
+    r = rng.choice(S, 40, replace=False)
+    b = rng.integers(0, H // 32, 40)
+    bad, same = x.copy(), inputs.bf16_bits_to_f32(x)
+    for i, (p, q) in enumerate(zip(r, b)):
+        blk = slice(32 * q, 32 * q + 32)
+        at = np.arange(32) if i % 5 == 4 else rng.choice(32, 1 + i % 3, replace=False)
+        bad[p, blk][at] = 0x7FC0 if i % 2 else 0xFF81
+        amax = np.abs(np.delete(same[p, blk], at)).max() if len(at) < 32 else 6.0
+        same[p, blk][at] = 6.0 * 2.0 ** np.ceil(np.log2(amax / 6.0))
+    ws, st, y = moe.alloc_ffn_q_workspace(sh), torch.zeros(1, dtype=torch.int32, device="cuda"), []
+    for v in (bad, inputs.f32_to_bf16_bits(same)):
+        y.append(torch.full((S, H), float("nan"), device="cuda"))
+        moe.moe_expert_ffn_q(dev(v), off, w, sh, y[-1], st, ws)
+        assert moe.moe_last_kernel_name() == kernel
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and bool(torch.isfinite(y[0]).all()) and torch.equal(y[0], y[1])
