@@ -407,12 +407,15 @@ def moe_layer(logits, x, weights, buf, stream=None):
     stream = _stream(stream)
     T, E = logits.shape
     if T == sh.T and E == sh.E:  # the four calls in one, which takes a small layer's host time from four trips to one
+        call = (_lib or lib()).moe_layer
         try:
-            rc = (_lib or lib()).moe_layer(logits.data_ptr(), _ptr(x), _ptr(w13), _ptr(s13), _ptr(w2), _ptr(s2), sh, buf.topk_ids.data_ptr(),
-                                           buf.topk_w.data_ptr(), buf.expert_offsets.data_ptr(), buf.x_perm.data_ptr(), buf.perm.data_ptr(),
-                                           buf.inv_perm.data_ptr(), buf.y_perm.data_ptr(), out.data_ptr(), _ptr(buf.status), ws.data_ptr(),
-                                           ws.numel(), stream)
-        except AttributeError as e:  # a buffer that is missing: what the library calls a null pointer
+            rc = call(logits.data_ptr(), _ptr(x), _ptr(w13), _ptr(s13), _ptr(w2), _ptr(s2), sh, buf.topk_ids.data_ptr(),
+                      buf.topk_w.data_ptr(), buf.expert_offsets.data_ptr(), buf.x_perm.data_ptr(), buf.perm.data_ptr(),
+                      buf.inv_perm.data_ptr(), buf.y_perm.data_ptr(), out.data_ptr(), _ptr(buf.status), ws.data_ptr(), ws.numel(), stream)
+        except AttributeError as e:
+            if e.obj is not None:
+                raise
+            # a buffer that is missing: what the library calls a null pointer
             raise MoeError("moe_layer failed: invalid argument (%s)" % e) from e
         if rc != 0:
             _check(rc, "moe_layer")
