@@ -73,19 +73,19 @@ def test_small_layer_against_the_oracle_with_equal_logits_and_infinities():
 
 
 def test_small_layers_one_behind_the_other_in_a_graph():
-    """Each layer's rows are the one before's output and its logits are rewritten beside it: nothing of a launch may start early."""
+    """Nothing but the layers' launches, each of which lets the next one start at once: a layer's rows are the one before's output, and
+    its output lies where the one before reads its rows, so neither reads nor writes may be early."""
     T, H, I, E, k, n = 16, 256, 128, 8, 2, 40
     sh, w = moe.shape(T, H, I, E, k), _weights(H, I, E)
     lg = [dev(inputs.make_logits(T, E, 50 + i)) for i in range(n)]
     x0 = dev(inputs.make_x(T, H, 1))
     bufs = [moe.LayerBuffers(sh) for _ in range(2)]
-    cur_lg = torch.empty_like(lg[0])
 
     def chain():
         x = x0
         for i in range(n):
-            cur_lg.copy_(lg[i])
-            x = moe.moe_layer(cur_lg, x, w, bufs[i & 1])
+            x = moe.moe_layer(lg[i], x, w, bufs[i & 1])
+            assert moe.moe_last_kernel_name() == "layer_one_cluster"
         return x
 
     chain()
