@@ -1450,9 +1450,11 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
                     in.ids, in.inv_perm, offsets, base + L.xq, base + L.sfx, sh.T, sh.k, sh.H, sh.E, geo.max_tok, geo.sf_step, chunks,
                     marks, flags, in.offsets_late ? 1 : 0, in.x_sorted);
   } else {
-    // few rows (a block's shared expert, whose chain of launches the block waits for): shorter tasks, more warps (with the router's boxes:
-    // block of 48 tokens 390.4 -> 388.3 us, 120 tokens 605.7 -> 603.9)
-    const int chunks = S <= 512 ? 2 : 8;
+    // few rows (a block's shared expert, whose chain of launches the block waits for): shorter tasks, more warps.  The call on one expert of
+    // 4096 x 2048 with pieces of eight and of two: 40 rows 30.2 us and 28.6, 120 rows 44.3 and 42.8, 225 rows 44.9 and 44.6; 256 rows 45.5
+    // and 46.1, 400 rows 64.9 and 67.6, 512 rows 61.2 and 61.7, 1024 rows 76.1 and 77.8 (of 7168 x 2048: 40 rows 36.2 and 34.3, 225 rows 59.2
+    // and 58.6, 256 rows 60.4 and 61.1; there 300 rows are the other way, 72.8 and 70.9).  Block of 48 tokens 372.2 and 370.2, of 120 tokens 550 and 548.
+    const int chunks = S < 256 ? 2 : 8;
     parts = (n_chunk + chunks - 1) / chunks;
     const size_t want = (S * parts + 7) / 8, resident = static_cast<size_t>(sm_count()) * 4;
     rc = launch_pdl(guard ? twoterm_split_kernel<true> : twoterm_split_kernel<false>, dim3(static_cast<unsigned>(want < resident ? want : resident)), dim3(256), table_bytes, st, in.x,

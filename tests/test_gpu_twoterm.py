@@ -58,6 +58,15 @@ def test_against_oracle(counts, H, I):
     check_y(_ffn(x, off, [dev(a) for a in w], H, I, E), O.expert_ffn(x, off, *w, 1), "two terms")
 
 
+@pytest.mark.parametrize("counts", [[3, 0, 122, 130], [3, 0, 123, 130]])
+@pytest.mark.parametrize("H", [256, 2304])
+def test_rows_split_in_short_and_in_long_tasks(counts, H):   # below 256 rows two pieces of 256 values a task, from there on eight
+    E, S, I = len(counts), sum(counts), 512
+    w, x = _weights(H, I, E, seed=S), inputs.make_x(S, H, seed=H)
+    off = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    check_y(_ffn(x, off, [dev(a) for a in w], H, I, E), O.expert_ffn(x, off, *w, 1), "two terms")
+
+
 def test_non_finite_tokens_stay_non_finite_and_to_themselves():
     H, I, counts = 512, 256, [40, 130]
     E, S = len(counts), sum(counts)
