@@ -93,7 +93,7 @@ constexpr int kRThreads = 6 * 32;
 
 template <int kRN>
 __global__ void __launch_bounds__(kRThreads, 1)
-router_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w, int T, int box_rows, int H, int E,
+router_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w, int T, int H, int E,
                    float* __restrict__ logits, int* status) {
   constexpr int kRBBytes = kRN * kRK * 2;
   extern __shared__ unsigned char smem_dyn[];
@@ -124,8 +124,8 @@ router_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
       uint32_t ph = 0;
       for (int kb = 0; kb < n_kb; ++kb) {
         mbar_wait(&empty[s], ph ^ 1u, status);
-        mbar_expect_tx(&full[s], static_cast<uint32_t>(box_rows) * kRK * 2 + kRBBytes);
-        tma_load_2d(sA + s * kRABytes, &tmap_x, kb * kRK, t0, &full[s]);   // rows past T inside the box arrive as zeros
+        mbar_expect_tx(&full[s], kRABytes + kRBBytes);
+        tma_load_2d(sA + s * kRABytes, &tmap_x, kb * kRK, t0, &full[s]);   // rows past T arrive as zeros
         tma_load_2d(sB + s * kRBBytes, &tmap_w, kb * kRK, e0, &full[s]);   // rows past E likewise
         if (++s == kRStages) { s = 0; ph ^= 1u; }
       }
@@ -264,12 +264,8 @@ int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, 
     return MOE_OK;
   }
   const int cols = router_cols(T);
-  // A box takes the TMA unit 85 cycles and 2 a row, zero rows included, and a CTA fetches 64 of them at H = 4096: a batch that fills no
-  // tile of 128 tokens comes in boxes of its own rows.  The operand's other rows are whatever shared memory holds; what they give
-  // is not stored.
-  const int box_rows = T >= kRM ? kRM : (T + 7) & ~7;
   CUtensorMap tm_x, tm_w;
-  if (!bf16_map_2d(&tm_x, x, H, T, kRK, static_cast<uint32_t>(box_rows)) || !bf16_map_2d(&tm_w, w_router, H, E, kRK, static_cast<uint32_t>(cols))) return MOE_ERR_CUDA;
+  if (!bf16_map_2d(&tm_x, x, H, T, kRK, kRM) || !bf16_map_2d(&tm_w, w_router, H, E, kRK, static_cast<uint32_t>(cols))) return MOE_ERR_CUDA;
   const size_t smem = kRStages * (kRABytes + static_cast<size_t>(cols) * kRK * 2) + 256 + 1024;
   static PerDeviceFlag flag;
   if (!once_per_device(flag, [] {
@@ -281,9 +277,9 @@ int launch_router_logits(const __nv_bfloat16* x, const __nv_bfloat16* w_router, 
   // (the kernel has no wait of its own: launched as a programmatic dependent it runs beside the launches in front of it)
   const auto kernel = cols == 16 ? router_gemm_kernel<16> : router_gemm_kernel<64>;
   if (order == RouterOrder::kBeside) {
-    if (launch_pdl(kernel, grid, dim3(kRThreads), smem, st, tm_x, tm_w, T, box_rows, H, E, logits, status) != cudaSuccess) return MOE_ERR_CUDA;
+    if (launch_pdl(kernel, grid, dim3(kRThreads), smem, st, tm_x, tm_w, T, H, E, logits, status) != cudaSuccess) return MOE_ERR_CUDA;
   } else {
-    kernel<<<grid, kRThreads, smem, st>>>(tm_x, tm_w, T, box_rows, H, E, logits, status);
+    kernel<<<grid, kRThreads, smem, st>>>(tm_x, tm_w, T, H, E, logits, status);
     if (cudaGetLastError() != cudaSuccess) return MOE_ERR_CUDA;
   }
   note_kernel("router_gemm_tcgen05_128x64", 1);  // (also for tiles of 16 experts: callers know the kernel by this name)
