@@ -86,9 +86,9 @@ uint64_t moe_launch_count(void);
  *   fixed fp32 sequence: d = max(d,-80); n = rint(d*0x1.715476p+0f); r = fma(n,-0x1.62e4p-1f,d);
  *   r = fma(n,-0x1.7f7d1cp-20f,r); p = Horner/fma over 1/720,1/120,1/24,1/6,1/2,1,1 in r; EXP = p*2^n.
  *   expert_offsets [E+1] int32: exclusive prefix sum of the per-expert slot counts, [E] = T*k.
- * Launch order: for T <= 32, and up to T = 256 with E <= 256, the kernel uses programmatic dependent launch.  It writes its
- * outputs only after the kernel launched just before it on the stream has completed (so the outputs of one layer call
- * may be the buffers the previous call's moe_combine still reads).  From 33 tokens on it reads logits after that as well; up
+ * Launch order: one kernel, or above 32 tokens where T > 256 or E > 256 two, by programmatic dependent launch.  Outputs
+ * are written only after the kernel launched just before on the stream has completed (so the outputs of one layer call
+ * may be the buffers the previous call's moe_combine still reads).  From 33 tokens on logits are read after that as well; up
  * to 32 tokens before.  So if that preceding kernel releases its dependents early
  * (cudaTriggerProgrammaticLaunchCompletion / griddepcontrol.launch_dependents), the logits of T <= 32 must not be among its
  * outputs; moe_combine's are not, and moe_router_logits releases nothing before it has ended.  The same holds for the
@@ -157,8 +157,11 @@ int moe_combine(const float* y_perm, const int32_t* inv_perm, const float* topk_
 /*
  * The four calls above one after the other on the caller's buffers: moe_route, moe_permute, moe_expert_ffn and moe_combine with these
  * arguments, every buffer written as they write it, the same errors; `ws` moe_workspace_bytes().  One call into the library
- * where a caller with no use for the steps would make four, and one launch less to wait for where one kernel routes and
- * sorts (T <= 256, E <= 256).
+ * where a caller with no use for the steps would make four, and fewer launches to wait for: one kernel routes and sorts (T <= 256,
+ * E <= 256), or the sort writes expert_offsets itself (larger ones, up to 2^19 slots), or the whole layer is one launch of one cluster of
+ * eight CTAs (T <= 32, T*k <= 128, where moe_expert_ffn would take the streaming kernel, the weights fit those CTAs' shared memory
+ * and T*k*H*I <= 2^20 * min(E, 8)).  That launch reads nothing, weights included, before what is in front of it has
+ * completed.
  */
 int moe_layer(const float* logits, const void* x_bf16, const uint8_t* w13, const uint8_t* w13_scale, const uint8_t* w2,
               const uint8_t* w2_scale, const moe_shape_t* shape, int32_t* topk_ids, float* topk_w, int32_t* expert_offsets,
@@ -211,9 +214,10 @@ int moe_expert_ffn_packed(const void* x_perm_bf16 /* [T*k,H] */, const int32_t* 
  *   - For T = 1 (k <= 32, E*4 <= 4*max(H,I) bytes) on shapes the decode-sized expert kernel takes,
  *     the call is ONE kernel launch: every CTA routes the token itself and sorts the slots, the first CTAs write the
  *     token's E2M1 term rows, every CTA runs its share of the gate/up and down items, and the CTA that finishes a
- *     column tile's last expert reduces that tile over the slots.  Any other shape runs the four calls' steps back to back;
+ *     column tile's last expert reduces that tile over the slots.  Any other shape runs the four calls' steps back to back,
+ *     or in one launch where moe_layer has one;
  *     up to 256 tokens and 256 experts routing and sort are one launch, beside which the tokens' rows are split into the term
- *     rows of the decode-sized kernel, once per token.
+ *     rows of the decode-sized kernel, once per token; above, the router and then a sort that writes the offsets.
  *   - ws: moe_forward_workspace_bytes() bytes, 256-byte aligned.  Its first moe_forward_sync_bytes() bytes are the
  *     kernel's completion counters: they must be ZERO when a call starts.  Clear them once (cudaMemsetAsync) before
  *     the first call that uses this ws; every call that returns MOE_OK and whose kernels ran to completion leaves them

@@ -200,7 +200,8 @@ bool front_in_one(const moe_shape_t& s, const ExpertWeights& w) {
 }
 // Routing, sort and expert FFN of such a call.  Where one cluster routes and the expert FFN is the two-term or the native
 // kernel, routing and sort are one launch, and the native kernel takes the tokens' rows as that launch splits them beside it, once
-// per token and not per slot; otherwise moe_route and the above.  Same bits.  `rows`: perm and x_perm are the caller's and written as
+// per token and not per slot; larger batches route and then sort with the offsets as the sort's by-product (route_permute_ok); what is left
+// takes moe_route and the above.  Same bits.  `rows`: perm and x_perm are the caller's and written as
 // moe_permute writes them.  `offsets2` (may be null) receives {0, T}; `late`:
 // the kernel in front may be the one that writes the logits.
 int route_and_ffn(const float* logits, const void* x, int32_t* ids, float* topk_w, int32_t* offsets, int32_t* offsets2, bool late,

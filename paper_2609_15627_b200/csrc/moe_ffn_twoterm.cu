@@ -1341,9 +1341,8 @@ template <bool STAGE1, int kM, bool kQ, bool kGuard = false, bool kFifo = false>
 bool tt_launch(const CUtensorMap& tm_w, const CUtensorMap& tm_sc, const TtTokMaps& tm_t, TtArgs a, cudaStream_t st) {
   a.stages = 1;
   if (kFifo) {
-    // a ring of KB: "stages" of one KB without token parts (see TtRing)
+    // the whole ring is one stage of `kb` KB, whose nominal token part is what the weight tiles leave (TtRing only takes its size from it)
     const int kb = (227 * 1024 - 1024 - static_cast<int>(tt_smem(a.E, 0, 0, 0).total) - kTtSfSlots * kM * 2048) >> 10;
-    a.stages = 1;
     a.t_bytes = kb * 1024 - kM * kTtTile;
   }
   while (!kFifo && a.stages < kTtMaxStages && tt_smem(a.E, kM, a.stages + 1, a.t_bytes).total + 1024 <= 227 * 1024) ++a.stages;
@@ -1489,7 +1488,7 @@ int launch_expert_ffn_twoterm(const TwoTermInput& in, const int* offsets, const 
   // Up to 16 rows per expert on average, where most passes have 16 or 32 rows (512 tokens, 16 rows: 703 -> 699 us); with 48 rows no step more
   // fits and finding its place costs 1 % (2048 tokens 986 -> 999).  Where no other kernel does experts again: the kernel that does
   // is for more rows, or small layers.
-  const bool fifo = !guard && geo.max_tok == 64 && two && S <= 16ull * choice.E;
+  const bool fifo = !guard && two && S <= 16ull * choice.E;
   if (!(guard  ? tt_launch<true, 2, false, true>(tm_w13, tm_s13, tm_x, a, st)
         : fifo ? tt_launch<true, 2, false, false, true>(tm_w13, tm_s13, tm_x, a, st)
                : tt_launch<true, 2, false>(tm_w13, tm_s13, tm_x, a, st)))

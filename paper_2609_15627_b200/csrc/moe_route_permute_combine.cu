@@ -174,10 +174,9 @@ int launch_route(const float* logits, int T, int E, int k, int* ids, float* w, i
 // A warp per token, tokens in order over the cluster's CTAs (as many as there are eights of tokens: the warps of a CTA share its
 // issue slots).  The warps that chose an expert are the bits of a mask, so a CTA's count of it is a population count and
 // a slot's rank the one of the bits below its warp's; the counts meet through distributed shared memory.  Latency is all
-// there is to it: one launch without anything to clear in front, where the general route takes a memset, a router whose last
-// CTA scans, and a sort (64 tokens and the split of their rows: 9 us until the expert FFN's weights start to stream, 26 before).
-// With more than a token per warp it is no faster than those (333 tokens in two rounds: 12 us, and 13 to the end of the
-// general sort).
+// there is to it: one launch, where larger batches take a router and a sort (64 tokens and the split of their rows: 9 us until the
+// expert FFN's weights start to stream; 26 with a memset, a router whose last CTA scanned, and a sort).  Not for more than a token per
+// warp: 333 tokens in two rounds took 12 us, and those three launches 13 to the end of the sort.
 // The CTAs behind the first cluster (kSplit) split the token rows, which depends on no routing, meanwhile.
 constexpr int kFrontCluster = 8;
 static_assert(kFrontMaxTok == 32 * kFrontCluster, "a warp per token");
@@ -319,9 +318,11 @@ MOE_DEVINL void warp_copy_row(const __nv_bfloat16* src, __nv_bfloat16* dst, int 
 // Up to permute_direct slots: a CTA takes eight consecutive slots, counts the earlier slots of each one's expert directly
 // (an id is loaded once per CTA and compared with the eight experts) and copies their rows, one warp each; the sort is
 // stable by construction.  One launch where the chunked sort takes two, and a third for the rows.
-// The count is quadratic and the launches are not: the line lies where the two meet (256 experts, direct / chunked in three).  Short
-// rows or none to copy: 4096 slots 10 us and 15, 8192 13 and 17, 12288 21 and 17, 16384 29 and 19; with long ones beside
-// the count later (H = 4096): 8192 slots 21 and 31, 12288 29 and 36, 16384 37 and 42, 24576 59 and 56.
+// The count is quadratic and the launches are not.  moe_route and moe_permute one after the other in a graph, 256 experts, top-8, direct /
+// chunked: H = 256: 4096 slots 12.0 us and 15.4, 6144 14.4 and 15.3, 8192 17.8 and 15.4, 12288 22.5 and 17.0; H = 1024: 8192 slots 17.5 and
+// 17.8, 12288 23.1 and 19.8; H = 2048: 8192 slots 18.6 and 20.0, 12288 24.3 and 23.0, 16384 34.2 and 27.5; H = 4096: 8192 slots 23.0 and
+// 26.8, 12288 33.6 and 34.1, 16384 42.2 and 41.7, 24576 64.1 and 57.5.  The two lines were set when the chunked sort had a scan between its
+// launches; they lie where H = 1024 and H = 4096 meet now, and 256 and 2048 meet earlier, near 6800 and 11000 slots.
 constexpr int permute_direct(bool rows, int H) { return rows && H >= 2048 ? 16384 : 8192; }
 // kOffsets: expert_offsets is not there yet.  Then the slots of smaller experts are counted as well, and the last CTA writes it.
 template <bool kOffsets>
@@ -606,7 +607,9 @@ bool route_permute_ok(const moe_shape_t& s) {
   return !route_sort_ok(s.T, s.E) && s.T > 32 && static_cast<long long>(s.T) * s.k <= static_cast<long long>(kSortChunks) * kPermuteChunk;
 }
 // Routing and sort of a call that makes both, for batches that no cluster routes: the router, then the sort with the offsets as its
-// by-product.  The direct count doubles (it counts smaller experts too), so its line lies lower.
+// by-product.  The direct count doubles (it counts smaller experts too), so its line lies lower.  Whole layers in a graph, direct / chunked:
+// two-term kernel, 256 experts of 256 x 256, top-8: 2072 slots 36.4 us and 39.6, 4096 39.6 and 41.2, 6144 44.7 and 43.5, 8192 59.9 and 54.5; with
+// rows, 64 experts of 4096 x 256, top-2: 2072 slots 72.8 and 75.6, 4096 106.0 and 106.6, 6144 136.7 and 135.2.
 int launch_route_permute(const float* logits, const __nv_bfloat16* x, const moe_shape_t& sh, int* ids, float* w, int* offsets,
                          __nv_bfloat16* x_perm, int* perm, int* inv_perm, int* block_counts, cudaStream_t st) {
   const int S = sh.T * sh.k;
